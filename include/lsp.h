@@ -50,7 +50,11 @@ typedef enum lsp_status {
 
 /* How sin/cos of the phase are produced in the O(N_t N_f) loop. */
 typedef enum lsp_sincos_mode {
-    LSP_SINCOS_AUTO = 0,   /* the library's choice (currently RECUR3_X2)                 */
+    LSP_SINCOS_AUTO = 0,   /* the library's choice: RECUR3_X2 on small calls, and on larger
+                              ones, when freqs_per_thread, split and batch_rhs are 0 too
+                              and the tuning table has no entry for the size, the same
+                              sums as a matrix product on the tensor cores (FP32
+                              accuracy from split FP16 operands)                     */
     LSP_SINCOS_MUFU = 1,   /* hardware sin/cos (SFU) of every phase (Sec. 4.3's choice)  */
     LSP_SINCOS_RECUR = 2,  /* SFU seed per strip of adjacent frequencies, then the
                               angle-addition rotation by (cos, sin)(2 pi t_j df) on FMA */
@@ -249,9 +253,11 @@ lsp_status lsp_press_rybicki(lsp_ctx *ctx, const double *t, const double *X, int
  * (= RECUR3_X2) sin/cos mode the groups run the packed strip.  Each
  * (frequency, realization) is computed exactly as the one-at-a-time kernel
  * with the same strip length would.
- * A work item sums over all samples of its curve in FP32 (the batch does not
- * split N_t), so curves far beyond 10^6 samples are better served by
- * lsp_periodogram, which bounds each running sum to 16,384 samples.
+ * Under AUTO, batches with work enough run on the tensor cores, whose FP32
+ * running sums cover at most 16,384 samples each.  A strip kernel's work item
+ * sums over all samples of its curve in FP32 (the batch does not split N_t), so
+ * with a sin/cos mode asked for curves far beyond 10^6 samples are better
+ * served by lsp_periodogram.
  * At least one output must be given.  Arrays may be host or device pointers
  * (metadata is read on the host in either case); the sin/cos mode and strip
  * length follow the context's options (the naive FP32 phase is not offered).

@@ -150,36 +150,6 @@ struct GStrip<F, kRecur3x2> {
     }
 };
 
-// p from the six sums (weights summing to 1, data variance 1), in FP64.
-// Data the prep kernels refuse are reported through the status word (this
-// path has no allocation-free form that would need NaN outputs instead).
-__device__ __forceinline__ float gls_value(double XC, double XS, double C, double S, double CCp, double CSp,
-                                           double n) {
-    const double CC = CCp - C * C;
-    const double SS = (1.0 - CCp) - S * S;
-    const double CS = CSp - C * S;
-    const double A = CC - SS, B = 2.0 * CS;
-    const double T = CC + SS;
-    const double R = sqrt(A * A + B * B);
-    double c2 = 1.0, s2 = 0.0;
-    if (R > 0.0) {
-        const double iR = 1.0 / R;
-        c2 = A * iR;
-        s2 = B * iR;
-    }
-    const double z2 = XC * XC + XS * XS;
-    const double cross = c2 * (XC * XC - XS * XS) + s2 * (2.0 * XC * XS);
-    const double num1 = fmax(0.5 * (z2 + cross), 0.0);
-    const double num2 = fmax(0.5 * (z2 - cross), 0.0);
-    const double den1 = 0.5 * (T + R);
-    const double den2 = 0.5 * (T - R);
-    const double thr = 0x1p-24;
-    double p = 0.0;
-    if (den1 > thr) p += num1 / den1;
-    if (den2 > thr) p += num2 / den2;
-    return (float)(0.5 * n * p);
-}
-
 template <int F, int MODE>
 __global__ void __launch_bounds__(kGlsThreads)
 gls_main_kernel(const uint4* __restrict__ recA, const float4* __restrict__ recB, const float* __restrict__ q,

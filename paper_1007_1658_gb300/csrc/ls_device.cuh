@@ -108,9 +108,7 @@ __device__ __forceinline__ void merge_chunks(const float* __restrict__ part, int
 // A term whose denominator is below N 2^-16 is taken as zero.  A NaN among
 // the sums (non-finite data, or data the prep kernels refused) gives NaN: the
 // clamps and threshold tests below would otherwise turn it into 0.
-__device__ __forceinline__ float periodogram_value(float XC, float XS, float CC, float CS, float n) {
-    const float A = 2.f * CC - n;
-    const float B = 2.f * CS;
+__device__ __forceinline__ float periodogram_value2(float XC, float XS, float A, float B, float n) {
     const float R = sqrtf(A * A + B * B);
     float c2 = 1.f, s2 = 0.f;
     if (R > 0.f) {
@@ -129,6 +127,42 @@ __device__ __forceinline__ float periodogram_value(float XC, float XS, float CC,
     if (den2 > thr) P += num2 / den2;
     const float probe = z2 + R;
     return probe == probe ? 0.5f * P : probe;
+}
+
+// The same from the sums of Eq. 8.
+__device__ __forceinline__ float periodogram_value(float XC, float XS, float CC, float CS, float n) {
+    return periodogram_value2(XC, XS, 2.f * CC - n, 2.f * CS, n);
+}
+
+// The floating-mean form: p from the six sums (weights summing to 1, data
+// variance 1), in FP64, as P = (n / 2) p.  Data the prep kernels refuse are
+// reported through the status word (this path has no allocation-free form that
+// would need NaN outputs instead).
+__device__ __forceinline__ float gls_value(double XC, double XS, double C, double S, double CCp, double CSp,
+                                           double n) {
+    const double CC = CCp - C * C;
+    const double SS = (1.0 - CCp) - S * S;
+    const double CS = CSp - C * S;
+    const double A = CC - SS, B = 2.0 * CS;
+    const double T = CC + SS;
+    const double R = sqrt(A * A + B * B);
+    double c2 = 1.0, s2 = 0.0;
+    if (R > 0.0) {
+        const double iR = 1.0 / R;
+        c2 = A * iR;
+        s2 = B * iR;
+    }
+    const double z2 = XC * XC + XS * XS;
+    const double cross = c2 * (XC * XC - XS * XS) + s2 * (2.0 * XC * XS);
+    const double num1 = fmax(0.5 * (z2 + cross), 0.0);
+    const double num2 = fmax(0.5 * (z2 - cross), 0.0);
+    const double den1 = 0.5 * (T + R);
+    const double den2 = 0.5 * (T - R);
+    const double thr = 0x1p-24;
+    double p = 0.0;
+    if (den1 > thr) p += num1 / den1;
+    if (den2 > thr) p += num2 / den2;
+    return (float)(0.5 * n * p);
 }
 
 // The four running sums of Eq. 8 for a strip of F adjacent frequencies

@@ -144,6 +144,180 @@ void lsp::host::finish_shape(const lsp_ctx* ctx, MainShape& s, int occ_in, int64
     s.split = (int)((N + s.chunk - 1) / s.chunk);
 }
 
+// Terms of a call from which the tensor cores run it.  Whole calls, strips
+// against tensor cores: 3000 x 6000 50.1 / 54.7 us, 5000 x 10,000 62.9 / 62.2,
+// 7000 x 14,000 77.9 / 67.8, 10,000 x 20,000 96.8 / 68.6; floating mean 5000 x
+// 10,000 84.3 / 85.0, 7000 x 14,000 97.2 / 91.8; 100,000 x 300 98.5 / 102.7.
+static constexpr double kTcMinTerms = 6e7;
+bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f) {
+    const lsp_options& o = ctx->opt;
+    if (o.sincos_mode != LSP_SINCOS_AUTO || o.phase_mode != LSP_PHASE_FIXED64 || o.freqs_per_thread || o.split)
+        return false;
+    return (double)N * (double)N_f >= kTcMinTerms && !tuned(ctx, N, N_f);
+}
+
+lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_out, bool launch,
+                                int* launches) {
+    const int cols = lsp::tc_cols(N_f);
+    const int64_t per = (int64_t)lsp::kTcRows * cols, blocks = (N_f + per - 1) / per;
+    const int sums = gls ? 3 : 2;
+    const int64_t units = (N + lsp::kTcUnit - 1) / lsp::kTcUnit;
+    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    lsp::TcArgs a{};
+    a.slot_floats = 128 * (int64_t)cols;
+    // at most 1 GiB of partial tiles at a time
+    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - sms) / sums);
+    const int64_t step = std::min(blocks, most);
+    lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)(step * sums + sms) * (size_t)a.slot_floats * 4);
+    if (rs != LSP_OK || !launch) return rs;
+    a.cols = cols;
+    a.kinds[0] = gls ? lsp::kTcRecQ : lsp::kTcRec;
+    a.kinds[1] = gls ? lsp::kTcW2 : lsp::kTcOne2;
+    a.kinds[2] = lsp::kTcW1;
+    a.n0 = N;
+    a.recA = (const uint4*)ctx->recA.p;
+    a.recB = (const float4*)ctx->recB.p;
+    a.recE = (const float2*)ctx->recE.p;
+    a.q = (const float*)ctx->recQ.p;
+    a.qmax = (const float*)ctx->qmax.p;
+    a.part = (float*)ctx->tc_part.p;
+    a.status = ctx->status_d;
+    const bool timing = ctx->opt.timing != 0;
+    for (int64_t fb = 0; fb < blocks; fb += step) {
+        a.fb0 = (int)fb;
+        a.nblk = (int)std::min(step, blocks - fb);
+        a.n_tiles = a.nblk * sums;
+        a.work = (int64_t)a.n_tiles * units * lsp::tc_unit_cost(cols);
+        a.ctas = (int)std::min<int64_t>(sms, (int64_t)a.n_tiles * units);
+        LSP_CUDA(ctx, lsp::launch_tc_sums(a, ctx->stream));
+        if (timing && fb + step >= blocks) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
+        lsp::TcFinal f{};
+        f.nf0 = N_f;
+        f.P = P_out;
+        f.bins = (lsp::TcBin*)ctx->tc_bins.p;
+        f.n_bins = (unsigned*)ctx->qmax.p + 1;
+        LSP_CUDA(ctx, lsp::launch_tc_final(gls ? lsp::kTcGls : lsp::kTcClassic, a, f, ctx->stream));
+        *launches += 2;
+        if (gls && fb + step >= blocks) {
+            LSP_CUDA(ctx, lsp::launch_tc_refine(a, f, sms, ctx->stream));
+            ++*launches;
+        }
+    }
+    return LSP_OK;
+}
+
+// A tile costs about one unit's time beside its units, so many short curves stay
+// with the strips; a few of them do not fill the GPU either way, and there a
+// strip's serial pass over its curve is the longer.  Whole calls, strips against
+// tensor cores: 8 curves of 100 .. 500 samples 126 / 86 us, 100 of them 133 / 108,
+// 100 x 8 realizations (900 tiles) 180 / 226; 100 x 8 of 200 .. 1500 samples 330 /
+// 305, of 400 .. 5000 samples 1704 / 516.
+static bool tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real) {
+    double tiles = 0.0, units = 0.0, terms = 0.0;
+    for (size_t c = 0; c < nf.size(); ++c) {
+        if (nf[c] == 0) continue;
+        const double n = (double)(off[c + 1] - off[c]);
+        const double t = std::ceil((double)nf[c] / (lsp::kTcRows * lsp::tc_cols(nf[c]))) * (n_real + 1);
+        tiles += t;
+        units += t * std::ceil(n / lsp::kTcUnit);
+        terms += n * (double)nf[c] * n_real;
+    }
+    return terms >= 1e6 && (tiles <= 300.0 || units >= 5.0 * tiles);
+}
+
+bool lsp::host::use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf,
+                             int n_real) {
+    const lsp_options& o = ctx->opt;
+    return o.sincos_mode == LSP_SINCOS_AUTO && o.phase_mode == LSP_PHASE_FIXED64 && !o.freqs_per_thread &&
+           !o.batch_rhs && tc_batch_pays(off, nf, n_real);
+}
+
+void lsp::host::TcPlan::pack(void* p) const {
+    char* b = (char*)p;
+    std::memcpy(b, tiles.data(), tiles.size() * sizeof(lsp::TcTile));
+    b += tiles.size() * sizeof(lsp::TcTile);
+    std::memcpy(b, pre.data(), pre.size() * 8);
+    std::memcpy(b + pre.size() * 8, data.data(), data.size() * 4);
+}
+
+lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, const std::vector<int64_t>& off,
+                                     const std::vector<int64_t>& nf, int n_real) {
+    TcPlan p;
+    const int shared = form == lsp::kTcClassic ? 1 : 2;
+    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    // at most 4 GiB of partial tiles at a time
+    const int64_t most = (int64_t(1) << 30) / (128 * lsp::kTcMaxCols) - sms;
+    TcChunk cur{0, 0, 0, 0, 0, 0};
+    p.pre.push_back(0);
+    auto flush = [&]() {
+        if (cur.n == 0) return;
+        p.chunks.push_back(cur);
+        p.max_slot_floats = std::max(p.max_slot_floats, (cur.n + sms) * 128 * (int64_t)cur.cols);
+        cur = TcChunk{(int64_t)p.tiles.size(), 0, (int64_t)p.data.size(), 0, 0, 0};
+        p.pre.push_back(0);
+    };
+    auto add = [&](int c, int r, int64_t fb, int kind, int64_t units, int cols, int wt, int ct) {
+        p.tiles.push_back({c, r, (int32_t)fb, kind, wt, ct, cols, 0});
+        cur.work += units * lsp::tc_unit_cost(cols);
+        p.pre.push_back(cur.work);
+        cur.cols = std::max(cur.cols, cols);
+        return (int)cur.n++;
+    };
+    for (int c = 0; c < (int)nf.size(); ++c) {
+        if (nf[c] == 0) continue;
+        const int cols = lsp::tc_cols(nf[c]);
+        const int64_t per = (int64_t)lsp::kTcRows * cols, blocks = (nf[c] + per - 1) / per;
+        const int64_t units = (off[c + 1] - off[c] + lsp::kTcUnit - 1) / lsp::kTcUnit;
+        // blocks b, realizations r of this curve, as many at a time as fit a chunk
+        const int64_t bstep = std::min(blocks, std::max<int64_t>(1, most / (shared + 1)));
+        const int64_t rstep = std::min<int64_t>(n_real, std::max<int64_t>(1, most / bstep - shared));
+        for (int64_t b0 = 0; b0 < blocks; b0 += bstep)
+            for (int64_t r0 = 0; r0 < n_real; r0 += rstep) {
+                const int64_t b1 = std::min(blocks, b0 + bstep), r1 = std::min<int64_t>(n_real, r0 + rstep);
+                if (cur.n + (b1 - b0) * (shared + r1 - r0) > most) flush();
+                for (int64_t b = b0; b < b1; ++b) {
+                    int wt = -1, ct = -1;
+                    if (form == lsp::kTcClassic) wt = add(c, 0, b, lsp::kTcOne2, units, cols, -1, -1);
+                    if (form == lsp::kTcGls) {
+                        wt = add(c, 0, b, lsp::kTcW2, units, cols, -1, -1);
+                        ct = add(c, 0, b, lsp::kTcW1, units, cols, -1, -1);
+                    }
+                    for (int64_t r = r0; r < r1; ++r) {
+                        p.data.push_back(add(c, (int)r, b, data, units, cols, wt, ct));
+                        ++cur.nd;
+                    }
+                }
+            }
+    }
+    flush();
+    return p;
+}
+
+cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int form, lsp::TcArgs a,
+                              lsp::TcFinal f, cudaStream_t st) {
+    const lsp::TcTile* tiles = (const lsp::TcTile*)d_plan;
+    const int64_t* pre = (const int64_t*)(tiles + p.tiles.size());
+    const int* data = (const int*)(pre + p.pre.size());
+    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    for (size_t x = 0; x < p.chunks.size(); ++x) {
+        const TcChunk& c = p.chunks[x];
+        a.tiles = tiles + c.t0;
+        a.pre = pre + c.t0 + (int64_t)x;
+        a.n_tiles = (int)c.n;
+        a.cols = c.cols;
+        a.work = c.work;
+        a.ctas = (int)std::min<int64_t>(sms, c.work / lsp::tc_unit_cost(0));
+        a.slot_floats = 128 * (int64_t)c.cols;
+        f.data_tiles = data + c.d0;
+        f.n_data = (int)c.nd;
+        cudaError_t e = lsp::launch_tc_sums(a, st);
+        if (e == cudaSuccess) e = lsp::launch_tc_final(form, a, f, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (form == lsp::kTcGls && !p.chunks.empty()) return lsp::launch_tc_refine(a, f, sms, st);
+    return cudaSuccess;
+}
+
 extern "C" {
 
 void lsp_default_options(lsp_options* opt) {
@@ -240,7 +414,16 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
     if ((rs = where(ctx, t, &t_dev)) != LSP_OK || (rs = where(ctx, X, &x_dev)) != LSP_OK ||
         (rs = where(ctx, P_out, &p_dev)) != LSP_OK)
         return rs;
-    const MainShape s = choose_shape(ctx, N_t, N_f);
+    const bool tc = use_tc(ctx, N_t, N_f);
+    MainShape s{};
+    int tc_launches = 2;
+    if (tc) {
+        s.split = 1;
+        if ((rs = ensure(ctx, ctx->recE, (size_t)N_t * 8)) != LSP_OK) return rs;
+        if ((rs = tc_single(ctx, false, N_t, N_f, nullptr, false, nullptr)) != LSP_OK) return rs;
+    } else {
+        s = choose_shape(ctx, N_t, N_f);
+    }
     if ((rs = ensure(ctx, ctx->recA, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recB, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->stats, sizeof(CurveStats))) != LSP_OK) return rs;
@@ -272,19 +455,23 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
         NvtxRange r("lsp_periodogram.prep");
         LSP_CUDA(ctx, lsp::launch_prep_stats(td, xd, nullptr, N_t, 1, stats, ctx->status_d,
                                              (lsp::StatPart*)ctx->stat_parts.p, (unsigned*)ctx->stat_counters.p, st));
+        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f), nullptr};
         LSP_CUDA(ctx, lsp::launch_prep_records(td, xd, nullptr, N_t, 1, N_t, nullptr, nullptr, f_0, df, stats,
                                                (uint4*)ctx->recA.p, (float4*)ctx->recB.p,
                                                s.mode == lsp::kModeNaive ? (float2*)ctx->recN.p : nullptr, nullptr,
-                                               st, nullptr, nullptr, ctx->status_d));
+                                               st, nullptr, nullptr, ctx->status_d, tc ? &tp : nullptr));
     }
     if (timing) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    {
+    if (tc) {
+        NvtxRange r("lsp_periodogram.main");
+        if ((rs = tc_single(ctx, false, N_t, N_f, pd, true, &tc_launches)) != LSP_OK) return rs;
+    } else {
         NvtxRange r("lsp_periodogram.main");
         LSP_CUDA(ctx, lsp::launch_main(s, (const uint4*)ctx->recA.p, (const float4*)ctx->recB.p,
                                        (const float2*)ctx->recN.p, N_t, N_f, f_0, df, (float*)ctx->part.p, pd, st));
     }
-    if (timing) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
-    ctx->last_launches = 3;
+    if (timing && !tc) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
+    ctx->last_launches = tc ? tc_launches : 3;
     if (s.split > 1) {
         NvtxRange r("lsp_periodogram.finalize");
         LSP_CUDA(ctx, lsp::launch_finalize(s, (const float*)ctx->part.p, N_t, N_f, pd, st));
@@ -293,7 +480,7 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
     if (timing) {
         LSP_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
         ctx->timing_valid = true;
-        ctx->has_finalize = s.split > 1;
+        ctx->has_finalize = tc || s.split > 1;
     }
     if (!p_dev) {
         LSP_CUDA(ctx, cudaMemcpyAsync(P_out, pd, (size_t)N_f * 4, cudaMemcpyDeviceToHost, st));
@@ -327,6 +514,7 @@ lsp_status lsp_sync(lsp_ctx* ctx, double timeout_s) {
         if (flags & lsp::kStatusPhaseRange)
             return fail(ctx, LSP_ERR_INVALID_ARG,
                         "(t - t_min) f_0 or (t - t_min) df reaches 2^52 turns: beyond the exact fixed-point phase");
+        if (flags & lsp::kStatusWait) return fail(ctx, LSP_ERR_CUDA, "a wait for the tensor cores ran out");
         return fail(ctx, LSP_ERR_DEGENERATE, "X has zero variance");
     }
     return LSP_OK;
@@ -375,7 +563,7 @@ void lsp_destroy(lsp_ctx* ctx) {
     DeviceGuard guard(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_plan(ctx);
-    DevBuf* bufs[] = {&ctx->recQ,   &ctx->dy_stage, &ctx->pr_acc, &ctx->pr_z0, &ctx->pr_z1,
+    DevBuf* bufs[] = {&ctx->recE, &ctx->qmax, &ctx->tc_part, &ctx->tc_bins, &ctx->b_recE, &ctx->b_qmax, &ctx->b_tc, &ctx->recQ,   &ctx->dy_stage, &ctx->pr_acc, &ctx->pr_z0, &ctx->pr_z1,
                       &ctx->recA,   &ctx->recB,   &ctx->recN,   &ctx->part,    &ctx->stats,  &ctx->t_stage,
                       &ctx->x_stage, &ctx->p_stage, &ctx->stat_parts, &ctx->stat_counters, &ctx->b_recA,
                       &ctx->b_recB,  &ctx->b_xr,   &ctx->b_stats, &ctx->b_items, &ctx->b_head, &ctx->b_maxkey,

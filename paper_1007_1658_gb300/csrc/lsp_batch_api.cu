@@ -106,6 +106,15 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
             tile = lsp::kTile;
         }
     }
+    const bool tc = !shape && use_tc_batch(ctx, off, nf, n_real);
+    TcPlan tcp;
+    if (tc) {
+        mode = lsp::kModeTensor;
+        F = lsp::kTcMaxCols;
+        R = 1;
+        tailF = 0;
+        tile = lsp::kTcUnit;
+    }
     const bool xrec = n_real == 1;  // x travels inside the sample records
     // with four groups of realizations or more per pattern, CC and CS come from
     // one window pass per pattern (4 FMA-pipe ops per term) instead of from every
@@ -119,8 +128,10 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
     // 67.1 / 68.0, 8 groups 104.2 / 108.6; at R = 4, 3 groups 26.3 / 25.4,
     // 4 groups 33.2 / 33.6.
     const bool use_win = R > 1 && n_real >= 4 * R;
-    if ((R > 1 ? lsp::mrhs_occupancy(mode, F, R, tile, use_win) : lsp::batch_occupancy(mode, F, xrec, tailF, tile)) <= 0 ||
-        (use_win && lsp::window_occupancy(mode, F) <= 0))
+    if (!tc && (R > 1 ? lsp::mrhs_occupancy(mode, F, R, tile, use_win) : lsp::batch_occupancy(mode, F, xrec, tailF, tile)) <= 0)
+        return fail(ctx, LSP_ERR_UNSUPPORTED, "batch shape (mode %d, F %d, R %d, tail %d, tile %d) is not built", mode,
+                    F, R, tailF, tile);
+    if (use_win && lsp::window_occupancy(mode, F) <= 0)
         return fail(ctx, LSP_ERR_UNSUPPORTED, "batch shape (mode %d, F %d, R %d, tail %d, tile %d) is not built", mode,
                     F, R, tailF, tile);
     const int64_t per_block = lsp::freqs_per_block(F);
@@ -152,6 +163,7 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
     if (!p_dev && (rs = ensure(ctx, ctx->b_P, (size_t)n_real * (size_t)P_total * 4)) != LSP_OK) return rs;
     if (!m_dev && (rs = ensure(ctx, ctx->b_maxP, n_out * 4)) != LSP_OK) return rs;
     if (!a_dev && (rs = ensure(ctx, ctx->b_argmax, n_out * 4)) != LSP_OK) return rs;
+    if (tc && (rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
     if (use_win) {
         if ((rs = ensure(ctx, ctx->b_win, (size_t)nf_total * 8)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->b_woff, ((size_t)n_curves + 1) * 8)) != LSP_OK) return rs;
@@ -165,7 +177,8 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
                                            ctx->b_recA.p, ctx->b_recB.p, ctx->b_xr.p, ctx->b_stats.p,
                                            ctx->b_head.p, ctx->b_seed.p, ctx->b_maxkey.p,
                                            use_win ? ctx->b_win.p : nullptr, use_win ? ctx->b_woff.p : nullptr,
-                                           ctx->b_items.p};
+                                           tc ? ctx->b_recE.p : nullptr, tc ? ctx->b_tc.p : nullptr,
+                                           tc ? ctx->tc_part.p : nullptr, ctx->b_items.p};
     BatchPlan& pl = ctx->plan;
     const bool same = pl.valid && pl.n_curves == n_curves && pl.n_real == n_real && pl.mode == mode &&
                       pl.F == F && pl.R == R && pl.tailF == tailF && pl.tile == tile && pl.noise == noise &&
@@ -184,7 +197,14 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         const bool tails = R == 1 && tailF > 0 && F > tailF;
         const int64_t tail_block = lsp::freqs_per_block(tails ? tailF : 1);
         std::vector<lsp::BatchItem> items;
+        if (tc) {
+            tcp = plan_tc(ctx, lsp::kTcClassic, n_real == 1 ? lsp::kTcRec : lsp::kTcRow, off, nf, n_real);
+            if (tcp.tiles.size() >= (size_t)(1u << 31)) return fail(ctx, LSP_ERR_INVALID_ARG, "batch too large");
+            if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
+            if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
+        }
         for (int c : order) {
+            if (tc) break;
             const int64_t nfb = tails ? nf[c] / per_block : (nf[c] + per_block - 1) / per_block;
             for (int64_t fb = 0; fb < nfb; ++fb)
                 for (int r = 0; r < n_real; r += R) items.push_back({c, r, (int32_t)fb, std::min(R, n_real - r)});
@@ -205,13 +225,16 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         }
         const size_t n_win = items.size() - n_main;
         if (items.size() >= (size_t)(1u << 31)) return fail(ctx, LSP_ERR_INVALID_ARG, "batch too large");
-        const size_t item_bytes = items.size() * sizeof(lsp::BatchItem);
+        const size_t item_bytes = tc ? tcp.bytes() : items.size() * sizeof(lsp::BatchItem);
         const size_t woff_bytes = woff.size() * sizeof(int64_t);
         const void* old_items = ctx->b_items.p;
-        if ((rs = ensure(ctx, ctx->b_items, item_bytes + 16)) != LSP_OK) return rs;
+        if (!tc && (rs = ensure(ctx, ctx->b_items, item_bytes + 16)) != LSP_OK) return rs;
         if ((rs = ensure_pinned(ctx, item_bytes + woff_bytes + 64)) != LSP_OK) return rs;
         LSP_CUDA(ctx, cudaStreamSynchronize(st));  // the pinned buffer may still feed an earlier copy
-        if (!items.empty()) {
+        if (tc) {
+            tcp.pack(ctx->pinned);
+            LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_tc.p, ctx->pinned, item_bytes, cudaMemcpyHostToDevice, st));
+        } else if (!items.empty()) {
             std::memcpy(ctx->pinned, items.data(), item_bytes);
             LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_items.p, ctx->pinned, item_bytes, cudaMemcpyHostToDevice, st));
         }
@@ -222,8 +245,12 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         }
         std::vector<const void*> ptrs2 = ptrs;
         ptrs2.back() = ctx->b_items.p;
+        if (tc) {
+            ptrs2[ptrs2.size() - 3] = ctx->b_tc.p;
+            ptrs2[ptrs2.size() - 2] = ctx->tc_part.p;
+        }
         (void)old_items;
-        const int occ =
+        const int occ = tc ? 1 :
             R > 1 ? lsp::mrhs_occupancy(mode, F, R, tile, use_win) : lsp::batch_occupancy(mode, F, xrec, tailF, tile);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)occ * ctx->sms, (int64_t)n_main));
         const int grid_w = use_win ? (int)std::max<int64_t>(
@@ -246,10 +273,11 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
                                        ctx->status_d, nullptr, nullptr, cst);
         if (e == cudaSuccess) {
             const int64_t max_n = off[order[0] + 1] - off[order[0]];
+            const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, d_nf, 0, nullptr};
             e = lsp::launch_prep_records(d_t, d_X, d_off, 0, n_curves, max_n, d_f0, d_df, 0.0, 0.0,
                                          (const lsp::CurveStats*)ctx->b_stats.p, (uint4*)ctx->b_recA.p,
                                          (float4*)ctx->b_recB.p, nullptr, noise ? nullptr : (float*)ctx->b_xr.p,
-                                         cst, nullptr, nullptr, ctx->status_d);
+                                         cst, nullptr, nullptr, ctx->status_d, tc ? &tprep : nullptr);
         }
         if (e == cudaSuccess && noise)
             e = lsp::launch_noise_prep(d_off, n_curves, n_real, (const uint64_t*)ctx->b_seed.p, total,
@@ -259,7 +287,25 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
                                    (unsigned*)ctx->b_head.p + 1, d_off, d_nf, (const int64_t*)ctx->b_woff.p,
                                    (const uint4*)ctx->b_recA.p, (const float4*)ctx->b_recB.p,
                                    (float2*)ctx->b_win.p, cst);
-        if (e == cudaSuccess && n_main > 0 && R > 1)
+        if (e == cudaSuccess && tc) {
+            lsp::TcArgs a{};
+            a.off = d_off;
+            a.recA = (const uint4*)ctx->b_recA.p;
+            a.recB = (const float4*)ctx->b_recB.p;
+            a.recE = (const float2*)ctx->b_recE.p;
+            a.xr = (const float*)ctx->b_xr.p;
+            a.total = total;
+            a.part = (float*)ctx->tc_part.p;
+            a.status = ctx->status_d;
+            lsp::TcFinal f{};
+            f.nf = d_nf;
+            f.P = d_P;
+            f.P_off = d_poff;
+            f.P_total = P_total;
+            f.maxkey = (unsigned long long*)ctx->b_maxkey.p;
+            f.n_curves = n_curves;
+            e = run_tc(ctx, tcp, ctx->b_tc.p, lsp::kTcClassic, a, f, cst);
+        } else if (e == cudaSuccess && n_main > 0 && R > 1)
             e = lsp::launch_mrhs(mode, F, R, tile, grid, (const lsp::BatchItem*)ctx->b_items.p, (int)n_main,
                                  (unsigned*)ctx->b_head.p, d_off, d_nf, total, n_curves, (const uint4*)ctx->b_recA.p,
                                  (const float4*)ctx->b_recB.p, (const float*)ctx->b_xr.p, d_P, d_poff, P_total,
@@ -300,9 +346,10 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         pl.f0 = f0v;
         pl.df = dfv;
         pl.p_off = poff;
-        pl.n_items = (int)n_main;
+        pl.n_items = tc ? (int)tcp.tiles.size() : (int)n_main;
         pl.grid = grid;
-        pl.kernels = 3 + (noise ? 1 : 0) + ((d_maxP || d_argmax) ? 1 : 0) + (n_main == 0 ? -1 : 0) + (n_win > 0 ? 1 : 0);
+        pl.kernels = 3 + (noise ? 1 : 0) + ((d_maxP || d_argmax) ? 1 : 0) + (n_main == 0 ? -1 : 0) + (n_win > 0 ? 1 : 0) +
+                     2 * (int)tcp.chunks.size();
     }
 
     // ---- run: new seed, one graph launch, outputs back if they live on the host ----

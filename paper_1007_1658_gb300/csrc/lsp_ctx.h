@@ -12,6 +12,7 @@
 
 #include "lsp.h"
 #include "lsp_kernels.cuh"
+#include "tc_sums.cuh"
 
 namespace lsp {
 namespace host {
@@ -89,6 +90,8 @@ struct lsp_ctx {
     // single-curve workspace
     lsp::host::DevBuf recA, recB, recN, part, stats, t_stage, x_stage, p_stage, stat_parts, stat_counters;
     lsp::host::DevBuf recQ, dy_stage;  // floating-mean periodogram: sqrt(w_j), staged errors
+    lsp::host::DevBuf recE, qmax, tc_part, tc_bins;  // tensor-core path: coarse rotations, largest q, partial tiles, bins formed again
+    lsp::host::DevBuf b_recE, b_qmax, b_tc;  // its batch form: the same per curve, and the packed tile list
     lsp::host::DevBuf pr_acc, pr_z0, pr_z1;  // Press-Rybicki: FP64 grid, FFT ping-pong buffers
     // batch workspace
     lsp::host::DevBuf b_recA, b_recB, b_xr, b_stats, b_items, b_head, b_maxkey, b_seed, b_off, b_nf, b_f0,
@@ -305,6 +308,48 @@ void finish_shape(const lsp_ctx* ctx, lsp::MainShape& s, int occ, int64_t N, int
 
 // Autotuned entry for this size bucket, or null.
 const TuneEntry* tuned(const lsp_ctx* ctx, int64_t N, int64_t N_f);
+
+// Whether a single-curve call of this size runs on the tensor cores: the
+// options leave the choice to the library (AUTO, no strip length, no split) and
+// the tuning table has no entry for it.
+bool use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f);
+
+// The sums and the finalize pass of one curve on the tensor cores, its records
+// and recE in place, in blocks of frequencies whose partial tiles fit the
+// workspace (grown here; call before any kernel is queued with launch = false).
+lsp_status tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_out, bool launch, int* launches);
+
+// The tiles of a batch on the tensor cores, in chunks whose partial tiles fit
+// the workspace: tiles [t0, t0 + n) of the list, their cost prefix sums at
+// pre[t0 + chunk] (n + 1 values), the data tiles' indices within the chunk at
+// data[d0, d0 + nd).
+struct TcChunk {
+    int64_t t0, n, d0, nd, work;
+    int cols;
+};
+struct TcPlan {
+    std::vector<lsp::TcTile> tiles;
+    std::vector<int64_t> pre;
+    std::vector<int> data;
+    std::vector<TcChunk> chunks;
+    int64_t max_slot_floats = 0;  // largest workspace of a chunk, in floats
+    size_t bytes() const { return tiles.size() * sizeof(lsp::TcTile) + pre.size() * 8 + data.size() * 4; }
+    // tiles, then prefix sums, then indices, as one block
+    void pack(void* p) const;
+};
+// Data tiles of kind `data` for every (curve, realization), with the pattern's
+// sums the form needs (kTcClassic: h = 2; kTcGls: h = 2 and h = 1).
+TcPlan plan_tc(const lsp_ctx* ctx, int form, int data, const std::vector<int64_t>& off,
+               const std::vector<int64_t>& nf, int n_real);
+
+// Launches every chunk of a packed plan at d_plan (args: records and samples in
+// place, part the workspace; fin: outputs) on `st`.
+cudaError_t run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int form, lsp::TcArgs args,
+                   lsp::TcFinal fin, cudaStream_t st);
+
+// Whether a batch runs on the tensor cores: the options leave the choice to the
+// library, and the batch is of a size where they are faster.
+bool use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real);
 
 // Release the cached batch graph.
 void drop_plan(lsp_ctx* ctx);

@@ -66,8 +66,19 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
             (ws = where(ctx, P_out, &p_dev)) != LSP_OK || (dy && (ws = where(ctx, dy, &dy_dev)) != LSP_OK))
             return ws;
     }
-    const MainShape s = choose_gls_shape(ctx, N_t, N_f);
     lsp_status rs;
+    const bool tc = use_tc(ctx, N_t, N_f);
+    MainShape s{};
+    int tc_launches = 2;
+    if (tc) {
+        s.split = 1;
+        if ((rs = ensure(ctx, ctx->recE, (size_t)N_t * 8)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->qmax, 16)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins)) != LSP_OK) return rs;
+        if ((rs = tc_single(ctx, true, N_t, N_f, nullptr, false, nullptr)) != LSP_OK) return rs;
+    } else {
+        s = choose_gls_shape(ctx, N_t, N_f);
+    }
     if ((rs = ensure(ctx, ctx->recA, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recB, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recQ, (size_t)N_t * 4)) != LSP_OK) return rs;
@@ -106,19 +117,23 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
         NvtxRange r("lsp_periodogram_gls.prep");
         LSP_CUDA(ctx, lsp::launch_prep_stats(td, xd, nullptr, N_t, 1, stats, ctx->status_d,
                                              (lsp::StatPart*)ctx->stat_parts.p, (unsigned*)ctx->stat_counters.p, st,
-                                             dyd));
+                                             dyd, tc ? (float*)ctx->qmax.p : nullptr));
+        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f), (float*)ctx->qmax.p};
         LSP_CUDA(ctx, lsp::launch_prep_records(td, xd, nullptr, N_t, 1, N_t, nullptr, nullptr, f_0, df, stats,
                                                (uint4*)ctx->recA.p, (float4*)ctx->recB.p, nullptr, nullptr, st, dyd,
-                                               (float*)ctx->recQ.p, ctx->status_d));
+                                               (float*)ctx->recQ.p, ctx->status_d, tc ? &tp : nullptr));
     }
     if (timing) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    {
+    if (tc) {
+        NvtxRange r("lsp_periodogram_gls.main");
+        if ((rs = tc_single(ctx, true, N_t, N_f, pd, true, &tc_launches)) != LSP_OK) return rs;
+    } else {
         NvtxRange r("lsp_periodogram_gls.main");
         LSP_CUDA(ctx, lsp::launch_gls(s, (const uint4*)ctx->recA.p, (const float4*)ctx->recB.p,
                                       (const float*)ctx->recQ.p, N_t, N_f, (float*)ctx->part.p, pd, st));
     }
-    if (timing) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
-    ctx->last_launches = 3;
+    if (timing && !tc) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
+    ctx->last_launches = tc ? tc_launches : 3;
     if (s.split > 1) {
         NvtxRange r("lsp_periodogram_gls.finalize");
         LSP_CUDA(ctx, lsp::launch_gls_finalize(s, (const float*)ctx->part.p, N_t, N_f, pd, st));
@@ -127,7 +142,7 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
     if (timing) {
         LSP_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
         ctx->timing_valid = true;
-        ctx->has_finalize = s.split > 1;
+        ctx->has_finalize = tc || s.split > 1;
     }
     if (!p_dev) {
         LSP_CUDA(ctx, cudaMemcpyAsync(P_out, pd, (size_t)N_f * 4, cudaMemcpyDeviceToHost, st));
@@ -222,6 +237,8 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         if (R > 1 && lsp::gls_mrhs_occupancy(F, R) <= 0)
             return fail(ctx, LSP_ERR_UNSUPPORTED, "batch_rhs = %d is not built for the floating-mean form", R);
     }
+    const bool tc = use_tc_batch(ctx, off, nf, n_real);
+    TcPlan tcp;
     const int64_t per_block = lsp::gls_batch_freqs_per_block(F);
     std::vector<int> order(n_curves);
     for (int c = 0; c < n_curves; ++c) order[c] = c;
@@ -229,7 +246,12 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
                      [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
     // longest curve first, each curve's realizations together (in groups of R)
     std::vector<lsp::BatchItem> items;
+    if (tc) {
+        tcp = plan_tc(ctx, lsp::kTcGls, noise ? lsp::kTcRowQ : lsp::kTcRecQ, off, nf, n_real);
+        if (tcp.tiles.size() >= (size_t)(1u << 31)) return fail(ctx, LSP_ERR_INVALID_ARG, "batch too large");
+    }
     for (int c : order) {
+        if (tc) break;
         const int64_t nfb = (nf[c] + per_block - 1) / per_block;
         for (int r = 0; r < n_real; r += R)
             for (int64_t fb = 0; fb < nfb; ++fb) items.push_back({c, r, (int32_t)fb, std::min(R, n_real - r)});
@@ -244,7 +266,15 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
     if ((rs = ensure(ctx, ctx->b_head, 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->b_maxkey, n_out * 8)) != LSP_OK) return rs;
     if (noise && (rs = ensure(ctx, ctx->b_gx, (size_t)n_real * (size_t)total * 4)) != LSP_OK) return rs;
-    if ((rs = ensure(ctx, ctx->b_items, items.size() * sizeof(lsp::BatchItem) + 16)) != LSP_OK) return rs;
+    if (tc) {
+        if ((rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->b_qmax, (size_t)n_curves * 4 + 4)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
+    } else if ((rs = ensure(ctx, ctx->b_items, items.size() * sizeof(lsp::BatchItem) + 16)) != LSP_OK) {
+        return rs;
+    }
     if (!p_dev && (rs = ensure(ctx, ctx->b_P, (size_t)n_real * (size_t)P_total * 4)) != LSP_OK) return rs;
     if (!m_dev && (rs = ensure(ctx, ctx->b_maxP, n_out * 4)) != LSP_OK) return rs;
     if (!a_dev && (rs = ensure(ctx, ctx->b_argmax, n_out * 4)) != LSP_OK) return rs;
@@ -252,10 +282,13 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
     float* d_maxP = maxP_out ? (m_dev ? maxP_out : (float*)ctx->b_maxP.p) : nullptr;
     int32_t* d_argmax = argmax_out ? (a_dev ? argmax_out : (int32_t*)ctx->b_argmax.p) : nullptr;
 
-    const size_t item_bytes = items.size() * sizeof(lsp::BatchItem);
+    const size_t item_bytes = tc ? tcp.bytes() : items.size() * sizeof(lsp::BatchItem);
     if ((rs = ensure_pinned(ctx, item_bytes + 64)) != LSP_OK) return rs;
     LSP_CUDA(ctx, cudaStreamSynchronize(st));  // the pinned buffer may still feed an earlier copy
-    if (!items.empty()) {
+    if (tc) {
+        tcp.pack(ctx->pinned);
+        LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_tc.p, ctx->pinned, item_bytes, cudaMemcpyHostToDevice, st));
+    } else if (!items.empty()) {
         std::memcpy(ctx->pinned, items.data(), item_bytes);
         LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_items.p, ctx->pinned, item_bytes, cudaMemcpyHostToDevice, st));
     }
@@ -269,11 +302,12 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
     LSP_CUDA(ctx, cudaMemsetAsync(ctx->b_maxkey.p, 0, n_out * 8, st));
     lsp::CurveStats* stats = (lsp::CurveStats*)ctx->b_stats.p;
     LSP_CUDA(ctx, lsp::launch_prep_stats(d_t, d_X, d_off, 0, n_curves, stats, ctx->status_d, nullptr, nullptr, st,
-                                         d_dy));
+                                         d_dy, tc ? (float*)ctx->b_qmax.p : nullptr));
+    const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, d_nf, 0, (float*)ctx->b_qmax.p};
     const int64_t max_n = off[order[0] + 1] - off[order[0]];
     LSP_CUDA(ctx, lsp::launch_prep_records(d_t, d_X, d_off, 0, n_curves, max_n, d_f0, d_df, 0.0, 0.0, stats,
                                            (uint4*)ctx->b_recA.p, (float4*)ctx->b_recB.p, nullptr, nullptr, st,
-                                           d_dy, (float*)ctx->b_xr.p, ctx->status_d));
+                                           d_dy, (float*)ctx->b_xr.p, ctx->status_d, tc ? &tprep : nullptr));
     int launches = 2;
     if (noise) {
         LSP_CUDA(ctx, lsp::launch_gls_noise_prep(d_off, n_curves, n_real, seed, total, d_dy, (const float*)ctx->b_xr.p,
@@ -281,7 +315,31 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         ++launches;
     }
     if (timing) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[1], st));
-    if (!items.empty()) {
+    if (tc) {
+        NvtxRange r("lsp_batch_gls.main");
+        lsp::TcArgs a{};
+        a.off = d_off;
+        a.recA = (const uint4*)ctx->b_recA.p;
+        a.recB = (const float4*)ctx->b_recB.p;
+        a.recE = (const float2*)ctx->b_recE.p;
+        a.q = (const float*)ctx->b_xr.p;
+        a.qmax = (const float*)ctx->b_qmax.p;
+        a.xr = noise ? (const float*)ctx->b_gx.p : nullptr;
+        a.total = total;
+        a.part = (float*)ctx->tc_part.p;
+        a.status = ctx->status_d;
+        lsp::TcFinal f{};
+        f.nf = d_nf;
+        f.P = d_P;
+        f.P_off = d_poff;
+        f.P_total = P_total;
+        f.maxkey = (unsigned long long*)ctx->b_maxkey.p;
+        f.n_curves = n_curves;
+        f.bins = (lsp::TcBin*)ctx->tc_bins.p;
+        f.n_bins = (unsigned*)ctx->b_qmax.p + n_curves;
+        LSP_CUDA(ctx, run_tc(ctx, tcp, ctx->b_tc.p, lsp::kTcGls, a, f, st));
+        launches += 2 * (int)tcp.chunks.size() + 1;
+    } else if (!items.empty()) {
         NvtxRange r("lsp_batch_gls.main");
         // the packed form when the work is many times the longest curve's, per
         // SM sub-partition: its throughput then counts, not one warp's speed on

@@ -13,6 +13,7 @@ enum : int {
     kStatusDegenerate = 2,
     kStatusBadWeight = 4,   // a per-sample error that is not finite and > 0
     kStatusPhaseRange = 8,  // |t - t_min| f_0 or |t - t_min| df reaches 2^52 turns
+    kStatusWait = 16,       // a wait for the tensor cores ran out (never seen)
 };
 
 // Per-curve statistics written by prep_stats (Sec. 3 normalization, FP64).
@@ -52,7 +53,19 @@ int prep_stats_slices(int n_curves, int64_t n0);
 // dy (optional, floating-mean periodogram): per-sample errors, weights 1/dy^2.
 cudaError_t launch_prep_stats(const double* t, const double* X, const int64_t* off, int64_t n0,
                               int n_curves, CurveStats* stats, int* status, StatPart* parts,
-                              unsigned* counters, cudaStream_t st, const double* dy = nullptr);
+                              unsigned* counters, cudaStream_t st, const double* dy = nullptr,
+                              float* qmax = nullptr);
+
+// What the tensor-core path needs beside the records: recE[j] = (cos, sin)(2 pi
+// cols u_j) with cols the curve's fine offsets (`cols`, or from nf[curve]), and
+// the largest q of each curve (n_curves floats and one word more, zeroed by
+// launch_prep_stats).
+struct TcPrep {
+    float2* recE;
+    const int64_t* nf;
+    int cols;
+    float* qmax;
+};
 
 // X may be null (noise batches): then only t_ref is computed and x_hat = 0.
 // xout, if given, receives x_hat as a plain FP32 array (batch layout).
@@ -67,12 +80,14 @@ cudaError_t launch_prep_records(const double* t, const double* X, const int64_t*
                                 int n_curves, int64_t max_n, const double* f0, const double* df,
                                 double f0_single, double df_single, const CurveStats* stats,
                                 uint4* recA, float4* recB, float2* recN, float* xout, cudaStream_t st,
-                                const double* dy = nullptr, float* qout = nullptr, int* status = nullptr);
+                                const double* dy = nullptr, float* qout = nullptr, int* status = nullptr,
+                                const TcPrep* tc = nullptr);
 
 // Kernel modes (how sin/cos and the phase are formed in the O(N_t N_f) loop).
 // kModeRecur3x2 is RECUR3 with the (cos, sin) pair carried through packed
 // FP32x2 FMA (FFMA2); its results are bit-identical to kModeRecur3.
-enum : int { kModeMufu = 1, kModeRecur = 2, kModeNaive = 3, kModeRecur3 = 4, kModeRecur3x2 = 5 };
+// kModeTensor (batches only, never a strip kernel's): the tensor-core sums of tc_sums.cu.
+enum : int { kModeMufu = 1, kModeRecur = 2, kModeNaive = 3, kModeRecur3 = 4, kModeRecur3x2 = 5, kModeTensor = 6 };
 
 struct MainShape {
     int mode;      // kMode*

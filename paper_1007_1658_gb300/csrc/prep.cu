@@ -8,6 +8,7 @@
 #include <cmath>
 
 #include "lsp_kernels.cuh"
+#include "tc_sums.cuh"
 
 namespace lsp {
 namespace {
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(kStatsThreads)
 prep_stats_kernel(const double* __restrict__ t, const double* __restrict__ X,
                   const int64_t* __restrict__ off, int64_t n0, CurveStats* __restrict__ stats,
                   int* __restrict__ status, StatPart* __restrict__ parts, unsigned* __restrict__ counters,
-                  const double* __restrict__ dy) {
+                  const double* __restrict__ dy, float* __restrict__ qmax) {
     __shared__ double sh[33];
     __shared__ int last;
     const int c = blockIdx.y, g = blockIdx.x, G = gridDim.x;
@@ -185,6 +186,10 @@ prep_stats_kernel(const double* __restrict__ t, const double* __restrict__ X,
         r.t_ref = bad ? 0.0 : tmin;
         r.pad = dy ? tot_n : var;
         stats[c] = r;
+        if (qmax) {
+            qmax[c] = 0.f;
+            if (c == 0) qmax[gridDim.y] = 0.f;  // the counter of TcFinal::n_bins
+        }
         if (bad & 1) atomicOr(status, kStatusNonFinite);
         else if (bad) atomicOr(status, kStatusBadWeight);
         else if (!ok) atomicOr(status, kStatusDegenerate);
@@ -229,7 +234,7 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
                     double f0s, double dfs, const CurveStats* __restrict__ stats,
                     uint4* __restrict__ recA, float4* __restrict__ recB, float2* __restrict__ recN,
                     float* __restrict__ xout, const double* __restrict__ dy, float* __restrict__ qout,
-                    int* __restrict__ status) {
+                    int* __restrict__ status, const TcPrep tc) {
     const int c = blockIdx.y;
     const int64_t b = off ? off[c] : 0;
     const int64_t e = off ? off[c + 1] : n0;
@@ -239,6 +244,8 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // 1/sqrt(sum of weights): the weight sum from the stats, or N without errors
     const float isw = qout ? (float)rsqrt(dy ? st.pad : (double)(e - b)) : 0.f;
+    const int cols = tc.recE ? (tc.nf ? tc_cols(tc.nf[c]) : tc.cols) : 0;
+    float qm = 0.f;
     for (int64_t j = b + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < e; j += stride) {
         const double tt = t[j] - st.t_ref;
         const uint64_t u = frac_turns64(tt, df);
@@ -252,6 +259,7 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
             // equal weights without dy), x = q (X - mean_w) / sd_w, so sum x^2 = 1
             const float q = dy ? isw / (float)dy[j] : isw;
             qout[j] = q;
+            qm = fmaxf(qm, q);
             // without X (noise realizations, normalized later per realization) x_hat = 0
             xh = X ? (float)((X[j] - st.mean) * st.inv_sd) * q : 0.f;
         } else {
@@ -266,6 +274,16 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
         recB[j] = make_float4(xh, cs, sn, 2.f * cs);
         if (recN) recN[j] = make_float2(xh, __double2float_rn(tt));
         if (xout) xout[j] = xh;
+        if (tc.recE) {
+            float es, ec;
+            rotation_of(u * (uint64_t)cols, &ec, &es);
+            tc.recE[j] = make_float2(ec, es);
+        }
+    }
+    if (tc.qmax) {  // q >= 0: ordered as its bits
+        unsigned m = __float_as_uint(qm);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0 && m) atomicMax(reinterpret_cast<unsigned*>(tc.qmax) + c, m);
     }
 }
 
@@ -279,11 +297,12 @@ int prep_stats_slices(int n_curves, int64_t n0) {
 
 cudaError_t launch_prep_stats(const double* t, const double* X, const int64_t* off, int64_t n0,
                               int n_curves, CurveStats* stats, int* status, StatPart* parts,
-                              unsigned* counters, cudaStream_t st, const double* dy) {
+                              unsigned* counters, cudaStream_t st, const double* dy, float* qmax) {
     // without slice scratch every curve gets one CTA
     const int G = (parts && counters) ? prep_stats_slices(n_curves, n0) : 1;
     dim3 grid((unsigned)G, (unsigned)n_curves);
-    prep_stats_kernel<<<grid, kStatsThreads, 0, st>>>(t, X, off, n0, stats, status, parts, counters, dy);
+    prep_stats_kernel<<<grid, kStatsThreads, 0, st>>>(t, X, off, n0, stats, status, parts, counters, dy,
+                                                      qmax);
     return cudaGetLastError();
 }
 
@@ -291,13 +310,14 @@ cudaError_t launch_prep_records(const double* t, const double* X, const int64_t*
                                 int n_curves, int64_t max_n, const double* f0, const double* df,
                                 double f0_single, double df_single, const CurveStats* stats,
                                 uint4* recA, float4* recB, float2* recN, float* xout, cudaStream_t st,
-                                const double* dy, float* qout, int* status) {
+                                const double* dy, float* qout, int* status, const TcPrep* tc) {
     int64_t bx = (max_n + 255) / 256;
     if (bx > 4096) bx = 4096;
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)n_curves);
     prep_records_kernel<<<grid, 256, 0, st>>>(t, X, off, n0, f0, df, f0_single, df_single, stats,
-                                              recA, recB, recN, xout, dy, qout, status);
+                                              recA, recB, recN, xout, dy, qout, status,
+                                              tc ? *tc : TcPrep{nullptr, nullptr, 0, nullptr});
     return cudaGetLastError();
 }
 

@@ -1,0 +1,764 @@
+// tc_sums.cu -- the periodogram's sums on the tensor cores.
+//
+// Every frequency of a uniform grid is a coarse frequency plus or minus a fine
+// offset, f = f_a +- f_b, and exp(2 pi i f t) = exp(2 pi i f_a t)
+// exp(+- 2 pi i f_b t): the sums of Eq. 8 over the samples j,
+//     sum_j y_j e^{2 pi i f_a t_j} cos 2 pi f_b t_j,  ... sin 2 pi f_b t_j,
+// are a real matrix product A^T B with A[j][2a, 2a+1] = y_j (cos, sin)(2 pi f_a
+// t_j) and B[j][2b, 2b+1] = (cos, sin)(2 pi f_b t_j); its four entries for
+// (a, b) give the complex sums at f_a + f_b and f_a - f_b, so a term still
+// costs two multiply-adds per sum, and the operands cost 64 + cols/2 complex
+// values per sample for 64 cols terms.  With y = x_hat this is XC + i XS; the
+// tau sums CC - SS + 2i CS are the same product with y = 1 at doubled phases.
+// Phases are the exact 64-bit fixed-point turns of the strip kernels.
+//
+// FP32 accuracy from FP16 operands: a value v is split into hi = fp16(v) and
+// lo = fp16(v - hi) (22 bits, error at most 2^-24 for |v| <= 1), and the
+// product runs as hi hi + hi lo + lo hi, each exact, accumulated in FP32 by
+// the tensor core.  That accumulation truncates: every product is cut at a
+// quarter ulp of the accumulator and every step rounds toward zero, which
+// shrinks a coherent sum by ~1.5e-7 per 64 samples.  So an accumulator takes
+// only kTcUnit samples; then its values are added in FP32 (round to nearest)
+// to running sums in registers while the next unit accumulates in the other
+// half of tensor memory.
+//
+// What bounds it: with cols = 256 the three MMAs of 16 samples take 390 cycles
+// (24 a sample for 16,384 terms), the operands 192 complex values a sample.
+#include "ls_device.cuh"
+#include "tc_device.cuh"
+#include "tc_sums.cuh"
+
+#include <cooperative_groups.h>
+#include <cuda_fp16.h>
+
+namespace lsp {
+namespace {
+
+constexpr int kStage = 64;                         // samples of one operand stage
+constexpr int kAbytes = 128 * kStage * 2;          // one half (hi or lo) of A: 128 rows
+constexpr int kBbytes = kTcMaxCols * kStage * 2;   // one half of B
+constexpr int kStageBytes = 2 * kAbytes + 2 * kBbytes;
+constexpr int kSbo = kStage * 16;                  // bytes of one 8-row group of an operand
+constexpr int kGenWarps = 16;
+constexpr size_t kSmem = 2 * (size_t)kStageBytes + sizeof(float) * 12 * kGenWarps * 32;
+
+// (cos, sin) of a 64-bit fixed-point turn: quadrant and 30-bit remainder of the
+// top word, then the Taylor series on [-pi/4, pi/4] (truncation below 2e-9).
+__device__ __forceinline__ float2 turn_cos_sin(uint64_t ph) {
+    const uint32_t top = (uint32_t)(ph >> 32);
+    const uint32_t qd = (top + 0x20000000u) >> 30;
+    const float x = (float)(int32_t)(top - (qd << 30)) * 1.4629180792671596e-9f;  // 2 pi / 2^32
+    const float w = x * x;
+    float s = fmaf(w, 2.7557319223985893e-6f, -1.9841269841269841e-4f);
+    s = fmaf(w, s, 8.3333333333333333e-3f);
+    s = fmaf(w, s, -1.6666666666666667e-1f);
+    s = fmaf(x * w, s, x);
+    float c = fmaf(w, -2.7557319223985888e-7f, 2.4801587301587302e-5f);
+    c = fmaf(w, c, -1.3888888888888889e-3f);
+    c = fmaf(w, c, 4.1666666666666664e-2f);
+    c = fmaf(w, c, -0.5f);
+    c = fmaf(w, c, 1.f);
+    const float cc = (qd & 1) ? s : c, ss = (qd & 1) ? c : s;
+    return make_float2(__uint_as_float(__float_as_uint(cc) ^ (((qd + 1) & 2) << 30)),
+                       __uint_as_float(__float_as_uint(ss) ^ ((qd & 2) << 30)));
+}
+
+// A rotation and its products, scalar.
+__device__ __forceinline__ float2 cmul(float2 z, float2 e) {
+    return make_float2(fmaf(-z.y, e.y, z.x * e.x), fmaf(z.y, e.x, z.x * e.y));
+}
+__device__ __forceinline__ float2 csquare(float2 e) {
+    return make_float2(fmaf(-e.y, e.y, e.x * e.x), (e.x + e.x) * e.y);
+}
+
+// Two neighbouring complex values in the lanes of packed FP32: a product with
+// one rotation is four packed operations, and (re, re') and (im, im') are the
+// pairs that an FP16 word of an operand row holds.
+struct Pair {
+    float2 re, im;
+};
+__device__ __forceinline__ Pair mul_pair(const Pair& z, float2 e) {
+    const float2 c = make_float2(e.x, e.x), s = make_float2(e.y, e.y), n = make_float2(-e.y, -e.y);
+    Pair r;
+    r.re = __ffma2_rn(z.im, n, __fmul2_rn(z.re, c));
+    r.im = __ffma2_rn(z.im, c, __fmul2_rn(z.re, s));
+    return r;
+}
+
+// Eight consecutive values of an operand row group, split into their FP16
+// halves, 16 bytes each.
+__device__ __forceinline__ void split_pair(float2 v, uint32_t& hi, uint32_t& lo) {
+    const __half2 a = __floats2half2_rn(v.x, v.y);
+    const float2 f = __half22float2(a);
+    const float2 d = __ffma2_rn(f, make_float2(-1.f, -1.f), v);
+    const __half2 b = __floats2half2_rn(d.x, d.y);
+    hi = *reinterpret_cast<const uint32_t*>(&a);
+    lo = *reinterpret_cast<const uint32_t*>(&b);
+}
+
+__device__ __forceinline__ void store_group(const Pair (&z)[4], unsigned char* re_hi, unsigned char* re_lo,
+                                            unsigned char* im_hi, unsigned char* im_lo) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split_pair(z[i].re, h[i], l[i]);
+    *reinterpret_cast<uint4*>(re_hi) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(re_lo) = make_uint4(l[0], l[1], l[2], l[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split_pair(z[i].im, h[i], l[i]);
+    *reinterpret_cast<uint4*>(im_hi) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(im_lo) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// z, z e, ... z e^7 from e, e^2, e^4.
+__device__ __forceinline__ void powers8(float2 z, float2 e, float2 e2, float2 e4, Pair (&p)[4]) {
+    const float2 z1 = cmul(z, e);
+    p[0].re = make_float2(z.x, z1.x);
+    p[0].im = make_float2(z.y, z1.y);
+    p[1] = mul_pair(p[0], e2);
+    p[2] = mul_pair(p[0], e4);
+    p[3] = mul_pair(p[1], e4);
+}
+
+// Records of every thread's next sample, filled with cp.async a stage ahead: a
+// thread reads what it copied itself, so no barrier is needed.
+struct Ahead {
+    uint4 uv[kGenWarps * 32];
+    float4 B[kGenWarps * 32];
+    float2 E[kGenWarps * 32];
+    float q[kGenWarps * 32], x[kGenWarps * 32];
+};
+
+struct TileInfo {
+    int64_t b, n;       // samples [b, b + n)
+    uint32_t k0;        // first frequency index
+    int cols, kind;
+    float scale;        // power of two on y, so that its FP16 halves keep their bits
+    const float* x;     // realization row
+};
+
+__device__ __forceinline__ TileInfo tile_info(const TcArgs& a, int t) {
+    TileInfo f;
+    int curve = 0, real = 0, fb;
+    if (a.tiles) {
+        const TcTile w = a.tiles[t];
+        curve = w.curve;
+        real = w.real;
+        fb = w.fblock;
+        f.kind = w.kind;
+        f.cols = w.cols;
+        f.b = a.off[curve];
+        f.n = a.off[curve + 1] - f.b;
+    } else {
+        const int s = t / a.nblk;
+        fb = a.fb0 + (t - s * a.nblk);
+        f.kind = s == 0 ? a.kinds[0] : s == 1 ? a.kinds[1] : a.kinds[2];
+        f.cols = a.cols;
+        f.b = 0;
+        f.n = a.n0;
+    }
+    f.k0 = (uint32_t)fb * (uint32_t)(kTcRows * f.cols);
+    f.x = a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr;
+    // |x_hat| <= sqrt(n); |q x_hat| <= qmax; q^2 <= qmax^2: scaled to at most 2^14
+    int ex = 0;
+    if (f.kind == kTcRec || f.kind == kTcRow) {
+        ex = 14 - (33 - __clz((int)min(f.n, (int64_t)0x7fffffff))) / 2;
+    } else if (f.kind >= kTcW1) {
+        int eq;
+        frexpf(a.qmax[curve], &eq);  // qmax < 2^eq
+        ex = 14 - (f.kind >= kTcRecQ ? eq : 2 * eq);
+    }
+    f.scale = ldexpf(1.f, min(max(ex, -100), 100));
+    return f;
+}
+
+// The factor that undoes the mean shrinking of a unit's accumulation (see
+// above): 1 + 3 ulp.
+constexpr float kUnitGain = 1.f + 0x1.8p-22f;
+
+// A running sum covers at most this many units (16,384 samples); then it is
+// added to the piece's slot, so that its rounding error does not grow with the
+// length of the curve (382,003 samples in runs of any length: 8e-7 of the
+// result's norm from the 64-bit one, against 4e-7 with the strip kernels).
+constexpr int kRunUnits = 128;
+
+// Sixteen warps form the operands and drain the accumulators, in two sets that
+// take every other stage (a set's fixed latencies -- waits, record fetch, proxy
+// fence -- then pass while the other works), each thread 16 coarse rows and up
+// to 32 fine offsets of one sample; warp 16 issues the MMAs (issuing blocks
+// while the queue is full, so a warp that also forms operands would make the
+// two take turns: 5.4 us for 128 samples against 3.7).  The register split
+// comes from setmaxnreg: 640 threads at 96 registers launch, 512 x 112 + 128 x
+// 24 of those 61,440 are kept.  Barriers, two of each: filled and empty
+// (operand stages), full and drained (accumulators).  Nothing waits for another
+// CTA, and every wait has a limit, after which the CTA stops waiting, says so
+// in the status word and runs to its end.
+__global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) {
+    extern __shared__ __align__(128) unsigned char stages[];
+    Ahead& ahead = *reinterpret_cast<Ahead*>(stages + 2 * kStageBytes);
+    __shared__ uint64_t filled[2], empty[2], full[2], drained[2];
+    __shared__ uint32_t tbase;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&filled[i], kGenWarps / 2);
+            tc::mbar_init(&empty[i], 1);
+            tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&drained[i], kGenWarps);
+        }
+    }
+    if (warp == 0) tc::tmem_alloc(&tbase, 512);
+    tc::fence_operands();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tb = tbase;
+
+    const int64_t lo = tc_bound(a.work, a.ctas, blockIdx.x), hi = tc_bound(a.work, a.ctas, blockIdx.x + 1);
+    const int64_t cost0 = a.tiles ? 0 : (a.n0 + kTcUnit - 1) / kTcUnit * tc_unit_cost(a.cols);
+    // first tile that reaches beyond lo
+    int t = 0;
+    if (a.tiles) {
+        int h = a.n_tiles;
+        while (t < h) {
+            const int m = (t + h) >> 1;
+            if (a.pre[m + 1] > lo) h = m;
+            else t = m + 1;
+        }
+    } else {
+        t = (int)(lo / cost0);
+    }
+    bool ok = true;
+    uint32_t group = 0;  // units so far
+    // the next piece of a tile in this CTA's range: its tile, first sample and length
+    TileInfo f;
+    int64_t j0 = 0;
+    int left = 0;
+    auto next_piece = [&]() {
+        for (; t < a.n_tiles; ++t) {
+            const int64_t p = a.tiles ? a.pre[t] : (int64_t)t * cost0;
+            if (p >= hi) return false;
+            f = tile_info(a, t);
+            int64_t u0, u1;
+            tc_units(p, (f.n + kTcUnit - 1) / kTcUnit, tc_unit_cost(f.cols), lo, hi, &u0, &u1);
+            if (u0 >= u1) continue;
+            j0 = f.b + u0 * kTcUnit;
+            left = (int)(min(f.n, u1 * kTcUnit) - u0 * kTcUnit);
+            return true;
+        }
+        return false;
+    };
+
+    if (warp >= kGenWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+        if (warp == kGenWarps && lane == 0) {
+            uint32_t uses[2] = {0, 0};
+            for (; next_piece(); ++t) {
+                const uint32_t id = tc::instr_desc(f.cols);
+                for (int m = 0; m < left; m += kTcUnit, ++group) {
+                    const uint32_t d = tb + (group & 1) * 256u;
+                    if (group >= 2) ok = ok && tc::mbar_wait(&drained[group & 1], ((group >> 1) - 1) & 1);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const int rest = left - m - s * kStage;
+                        if (rest <= 0) break;
+                        ok = ok && tc::mbar_wait(&filled[s], uses[s]++ & 1);
+                        tc::fence_after_sync();
+                        const uint32_t sa = tc::smem_addr(stages) + s * kStageBytes, sb = sa + 2 * kAbytes;
+                        const int ks = (min(rest, kStage) + 15) / 16;
+                        uint32_t acc = s;
+                        for (int pass = 0; pass < 3; ++pass) {  // hi lo, lo hi, hi hi
+                            const uint32_t qa = sa + (pass == 1 ? kAbytes : 0), qb = sb + (pass == 0 ? kBbytes : 0);
+                            for (int k = 0; k < ks; ++k) {
+                                tc::mma_f16(d, tc::operand_desc(qa + k * 256, 128, kSbo),
+                                            tc::operand_desc(qb + k * 256, 128, kSbo), id, acc);
+                                acc = 1;
+                            }
+                        }
+                        tc::mma_commit(&empty[s]);
+                    }
+                    tc::mma_commit(&full[group & 1]);
+                }
+            }
+        }
+        __syncwarp();
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        const int set = tid / (kStage * 4), grp = (tid / kStage) & 3, js = tid & (kStage - 1);
+        const int quad = warp & 3, cg = warp >> 2;  // this warp's lanes and columns of the accumulators
+        unsigned char* const Ah = stages + set * kStageBytes + js * 16;
+        unsigned char* const Bh = Ah + 2 * kAbytes;
+        uint32_t uses = 0;
+        for (; next_piece(); ++t) {
+            const bool twice = f.kind == kTcOne2 || f.kind == kTcW2;
+            const int nb = f.cols >> 1;  // fine offsets of one sign
+            auto fetch = [&](int j) {    // sample j of the piece
+                if (j < left) {
+                    dev::cp_async16(&ahead.uv[tid], a.recA + j0 + j);
+                    dev::cp_async16(&ahead.B[tid], a.recB + j0 + j);
+                    dev::cp_async8(&ahead.E[tid], a.recE + j0 + j);
+                    if (f.kind >= kTcW1) dev::cp_async4(&ahead.q[tid], a.q + j0 + j);
+                    if (f.kind == kTcRow || f.kind == kTcRowQ) dev::cp_async4(&ahead.x[tid], f.x + j0 + j);
+                } else {  // beyond the piece: zeros, and y = 0 below
+                    ahead.uv[tid] = make_uint4(0, 0, 0, 0);
+                    ahead.B[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    ahead.E[tid] = make_float2(0.f, 0.f);
+                    ahead.q[tid] = ahead.x[tid] = 0.f;
+                }
+                dev::cp_async_commit();
+            };
+            float run[64];
+#pragma unroll
+            for (int i = 0; i < 64; ++i) run[i] = 0.f;
+            // adds a finished unit's accumulators to the running sums
+            auto drain = [&](uint32_t g) {
+                ok = ok && tc::mbar_wait(&full[g & 1], (g >> 1) & 1);
+                __syncwarp();
+                tc::fence_after_sync();
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (cg * 64 + c * 32 < f.cols) {  // columns from f.cols on are read as they are and never stored
+                        uint32_t r[32];
+                        tc::tmem_ld32(r, tb + (g & 1) * 256u + ((uint32_t)quad << 21) + (uint32_t)(cg * 64 + c * 32));
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            run[c * 32 + i] = fmaf(__uint_as_float(r[i]), kUnitGain, run[c * 32 + i]);
+                    }
+                }
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&drained[g & 1]);
+            };
+            // the running sums into this piece's slot: columns of the tile, rows contiguous
+            float* const out = a.part + (size_t)(t + (int)blockIdx.x) * (size_t)a.slot_floats +
+                               (size_t)(cg * 64) * 128 + quad * 32 + lane;
+            auto flush = [&](bool add) {
+                const float inv = 1.f / f.scale;
+#pragma unroll
+                for (int i = 0; i < 64; ++i)
+                    if (cg * 64 + i < f.cols) out[i * 128] = fmaf(run[i], inv, add ? out[i * 128] : 0.f);
+            };
+            fetch(set * kStage + js);
+            for (int m = 0; m < left; m += kTcUnit, ++group) {
+                const int jm = m + set * kStage;  // this set's stage of the unit
+                if (jm < left) {
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    const uint4 uv = ahead.uv[tid];
+                    const float4 B = ahead.B[tid];
+                    float2 e1 = make_float2(B.y, B.z), E = ahead.E[tid];
+                    float y = jm + js < left ? f.scale : 0.f;
+                    if (f.kind >= kTcW1) {
+                        const float q = ahead.q[tid];
+                        y *= q;
+                        if (f.kind <= kTcW2) y *= q;
+                    }
+                    if ((f.kind & 3) > 1) y *= (f.kind & 1) ? ahead.x[tid] : B.x;
+                    fetch(jm + kTcUnit + js);
+                    const uint64_t u = ((uint64_t)uv.y << 32) | uv.x;
+                    const uint64_t v = (((uint64_t)uv.w << 32) | uv.z) - kPhaseOffset;
+                    const uint64_t uh = u >> 1;
+                    // the middle of the first of 16 coarse blocks of cols bins, and the first of 32 fine offsets
+                    uint64_t pa = v + (uint64_t)(f.k0 + (uint32_t)(16 * grp * f.cols) + (uint32_t)nb) * u - uh;
+                    uint64_t pb = (uint64_t)(32 * grp) * u + uh;
+                    if (twice) {
+                        pa <<= 1;
+                        pb <<= 1;
+                        e1 = csquare(e1);
+                        E = csquare(E);
+                    }
+                    if (uses > 0) ok = ok && tc::mbar_wait(&empty[set], (uses - 1) & 1);
+                    ++uses;
+                    {
+                        float2 z = turn_cos_sin(pa);
+                        z.x *= y;
+                        z.y *= y;
+                        const float2 E2 = csquare(E), E4 = csquare(E2), E8 = csquare(E4);
+                        Pair p[4];
+                        powers8(z, E, E2, E4, p);
+                        unsigned char* re = Ah + 2 * grp * kSbo;
+                        unsigned char* im = re + 8 * kSbo;
+                        store_group(p, re, re + kAbytes, im, im + kAbytes);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) p[i] = mul_pair(p[i], E8);
+                        store_group(p, re + kSbo, re + kSbo + kAbytes, im + kSbo, im + kSbo + kAbytes);
+                    }
+                    if (32 * grp < nb) {
+                        const float2 e2 = csquare(e1), e4 = csquare(e2), e8 = csquare(e4);
+                        Pair p[4];
+                        powers8(turn_cos_sin(pb), e1, e2, e4, p);
+                        unsigned char* co = Bh + 4 * grp * kSbo;
+                        unsigned char* si = co + (nb >> 3) * kSbo;
+                        store_group(p, co, co + kBbytes, si, si + kBbytes);
+                        for (int b = 32 * grp + 8; b < min(nb, 32 * grp + 32); b += 8) {
+                            co += kSbo;
+                            si += kSbo;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) p[i] = mul_pair(p[i], e8);
+                            store_group(p, co, co + kBbytes, si, si + kBbytes);
+                        }
+                    }
+                    tc::fence_operands();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&filled[set]);
+                }
+                if (m > 0) drain(group - 1);
+                if (m > 0 && (m / kTcUnit) % kRunUnits == 0) {
+                    flush(m / kTcUnit > kRunUnits);
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) run[i] = 0.f;
+                }
+            }
+            drain(group - 1);
+            flush(left > kRunUnits * kTcUnit);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+    }
+    // every MMA has been waited for with its unit
+    if (!ok && a.status) atomicOr(a.status, kStatusWait);
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_free(tb, 512);
+}
+
+// The slots of a tile's pieces, in CTA order (the CTAs that got at least one
+// unit of it), and their number; every thread of the CTA calls it.
+struct Pieces {
+    int n;
+    int slot[kTcMaxCtas];
+};
+
+__device__ void find_pieces(const TcArgs& a, int tile, int64_t n, int cols, Pieces& out) {
+    const int64_t units = (n + kTcUnit - 1) / kTcUnit, c = tc_unit_cost(cols);
+    const int64_t p = a.tiles ? a.pre[tile] : (int64_t)tile * units * c;
+    const int i0 = tc_cta_of(a.work, a.ctas, p), i1 = tc_cta_of(a.work, a.ctas, p + (units - 1) * c);
+    if (threadIdx.x < 32) {
+        int at = 0;
+        for (int i = i0; i <= i1; i += 32) {
+            const int me = i + (int)threadIdx.x;
+            int64_t u0 = 0, u1 = 0;
+            if (me <= i1) tc_units(p, units, c, tc_bound(a.work, a.ctas, me), tc_bound(a.work, a.ctas, me + 1), &u0, &u1);
+            const unsigned has = __ballot_sync(0xffffffffu, u0 < u1);
+            if (u0 < u1) out.slot[at + __popc(has & ((1u << threadIdx.x) - 1u))] = tile + me;
+            at += __popc(has);
+        }
+        if (threadIdx.x == 0) out.n = at;
+    }
+}
+
+// The complex sums at f_a + f_b and f_a - f_b of S tiles, from a tile's four
+// entries each, the pieces added in order with compensated FP32 sums; four
+// pieces of every tile are loaded before any of them is added.
+template <int S>
+__device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces (&q)[S], int nb, int ra, int rb,
+                                          float2 (&plus)[S], float2 (&minus)[S]) {
+    float s[S][4] = {}, c[S][4] = {};
+    // sum y (Re A, Im A) cos, then sin
+    const size_t at[4] = {(size_t)rb * 128 + ra, (size_t)rb * 128 + 64 + ra, (size_t)(nb + rb) * 128 + ra,
+                          (size_t)(nb + rb) * 128 + 64 + ra};
+    int most = q[0].n;
+#pragma unroll
+    for (int x = 1; x < S; ++x) most = max(most, q[x].n);
+    for (int i0 = 0; i0 < most; i0 += 4) {
+        float v[S][4][4];
+#pragma unroll
+        for (int x = 0; x < S; ++x)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float* d = a.part + (size_t)q[x].slot[min(i0 + u, q[x].n - 1)] * (size_t)a.slot_floats;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[x][u][i] = i0 + u < q[x].n ? d[at[i]] : 0.f;
+            }
+#pragma unroll
+        for (int x = 0; x < S; ++x)
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float y = v[x][u][i], t = s[x][i] + y;
+                    c[x][i] += fabsf(s[x][i]) >= fabsf(y) ? (s[x][i] - t) + y : (y - t) + s[x][i];
+                    s[x][i] = t;
+                }
+    }
+#pragma unroll
+    for (int x = 0; x < S; ++x) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[x][i] += c[x][i];
+        plus[x] = make_float2(s[x][0] - s[x][3], s[x][1] + s[x][2]);
+        minus[x] = make_float2(s[x][0] + s[x][3], s[x][1] - s[x][2]);
+    }
+}
+
+// Where the smaller eigenvalue of the floating-mean form's second moments is
+// below this (f T under about a third, or an alias of it), P divides by a
+// difference that the tensor cores' truncated sums leave with too few digits
+// (the two sums it is taken from do not share their rounding errors: 1.7e-3 of
+// P at f T = 0.1, where sums formed together keep 1.9e-4): such bins are formed
+// again, sample by sample.
+constexpr float kGlsRefine = 0x1p-5f;
+
+// P of the floating-mean form from Z = sum w x' e, C = sum w e, W = sum w e^2:
+// dev::gls_value's two terms over their common denominator, where the square
+// root and three of its four divisions cancel.  With M = W - C^2 (= A + iB, the
+// centred CC - SS + 2i CS) and T = 1 - |C|^2 (CC + SS),
+//     p = 2 (|Z|^2 T - Re(conj(M) Z^2)) / (T^2 - |M|^2).
+// FP64 but for the reciprocal's seed: one Newton step takes FP32's 2^-24 to
+// 2^-47 (25 FP64 operations instead of ~150).
+// *ill: the smaller eigenvalue, between (T^2 - |M|^2) / 4T and / 2T, may lie
+// below kGlsRefine.
+__device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, double n, bool* ill) {
+    const double zx = Zf.x, zy = Zf.y, cx = Cf.x, cy = Cf.y;
+    const double A = fma(cy, cy, fma(-cx, cx, (double)Wf.x)), B = fma(-2.0 * cx, cy, (double)Wf.y);
+    const double T = fma(-cy, cy, fma(-cx, cx, 1.0));
+    const double D = fma(-B, B, fma(-A, A, T * T));
+    const double sx = zx * zx, sy = zy * zy;
+    const double num = fma(-B, 2.0 * zx * zy, fma(-A, sx - sy, T * (sx + sy)));
+    *ill = !(D >= 4.0 * kGlsRefine * T);
+    const double r0 = (double)(1.f / (float)D);
+    const double r = fma(r0, fma(-D, r0, 1.0), r0);
+    return fmaxf((float)(n * num * r), 0.f);
+}
+
+// The six sums at frequency k over samples b + i0, b + i0 + step, ... < b + n,
+// in compensated FP32 (s + c), from the same c~ = q cos, s~ = q sin.
+__device__ __forceinline__ void direct_gls(const TcArgs& a, int64_t b, int64_t n, const float* x, uint32_t k, int i0,
+                                           int step, float (&s)[6], float (&c)[6]) {
+#pragma unroll 4
+    for (int64_t j = b + i0; j < b + n; j += step) {
+        const uint4 A = a.recA[j];
+        const uint64_t u = ((uint64_t)A.y << 32) | A.x;
+        const uint64_t v = (((uint64_t)A.w << 32) | A.z) - kPhaseOffset;
+        const float2 e = turn_cos_sin(v + (uint64_t)k * u);
+        const float q = a.q[j], xj = x ? x[j] : a.recB[j].x;
+        const float co = q * e.x, si = q * e.y;
+        const float f[6] = {xj, xj, q, q, co, co}, g[6] = {co, si, co, si, co, si};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const float y = fmaf(f[i], g[i], c[i]), t = s[i] + y;
+            c[i] = y - (t - s[i]);
+            s[i] = t;
+        }
+    }
+}
+
+constexpr int kFinB = 4;  // fine offsets of one finalize CTA
+constexpr int kFinThreads = kTcRows * kFinB;
+
+// One CTA: a data tile's 64 coarse frequencies x 4 fine offsets, both signs, a
+// pair of frequencies a thread.  Reads run along the coarse frequencies
+// (contiguous in a slot); P is gathered in shared memory and written in runs of
+// 4 bins.
+template <int FORM>
+__global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, const TcFinal f) {
+    __shared__ float sp[kTcRows][2 * kFinB + 1];
+    constexpr int S = FORM == kTcClassic ? 2 : 3;
+    __shared__ Pieces q[S];
+    __shared__ unsigned long long s_red[kFinThreads / 32];
+    const int tid = threadIdx.x;
+    int curve = 0, real = 0, fb, cols, td, tw, tcx;
+    int64_t n, nf;
+    if (a.tiles) {
+        td = f.data_tiles[blockIdx.x];
+        const TcTile w = a.tiles[td];
+        curve = w.curve;
+        real = w.real;
+        fb = w.fblock;
+        cols = w.cols;
+        tw = w.wtile;
+        tcx = w.ctile;
+        n = a.off[curve + 1] - a.off[curve];
+        nf = f.nf[curve];
+    } else {
+        td = (int)blockIdx.x;
+        fb = a.fb0 + td;
+        cols = a.cols;
+        tw = td + a.nblk;
+        tcx = td + 2 * a.nblk;
+        n = a.n0;
+        nf = f.nf0;
+    }
+    const int nb = cols >> 1;
+    const int b0 = (int)blockIdx.y * kFinB;
+    if (b0 >= nb) return;
+    const int64_t k0 = (int64_t)fb * kTcRows * cols;
+    find_pieces(a, td, n, cols, q[0]);
+    find_pieces(a, tw, n, cols, q[1]);
+    if constexpr (S > 2) find_pieces(a, tcx, n, cols, q[2]);
+    __syncthreads();
+    const int ra = tid & (kTcRows - 1), bi = tid / kTcRows;
+    if (k0 + (int64_t)ra * cols < nf) {  // not a padding row
+        float2 zp[S], zm[S];
+        tile_sums<S>(a, q, nb, ra, b0 + bi, zp, zm);
+        float vp, vm;
+        if constexpr (FORM == kTcClassic) {
+            vp = dev::periodogram_value2(zp[0].x, zp[0].y, zp[1].x, zp[1].y, (float)n);
+            vm = dev::periodogram_value2(zm[0].x, zm[0].y, zm[1].x, zm[1].y, (float)n);
+        } else {
+            bool lp, lm;
+            vp = gls_power(zp[0], zp[2], zp[1], (double)n, &lp);
+            vm = gls_power(zm[0], zm[2], zm[1], (double)n, &lm);
+#pragma unroll 1
+            for (int s = 0; s < 2; ++s) {
+                const int64_t k = k0 + (int64_t)ra * cols + (s ? nb + b0 + bi : nb - 1 - b0 - bi);
+                if (!(s ? lp : lm) || k >= nf) continue;
+                float p = -1.f;  // left to launch_tc_refine
+                const unsigned at = atomicAdd(f.n_bins, 1u);
+                if (at < (unsigned)kTcBins) {
+                    f.bins[at] = TcBin{curve, real, (uint32_t)k, 0u};
+                } else {  // the list is full
+                    float d[6] = {}, e[6] = {};
+                    direct_gls(a, a.tiles ? a.off[curve] : 0, n,
+                               a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr, (uint32_t)k, 0, 1, d, e);
+                    p = dev::gls_value((double)d[0] + e[0], (double)d[1] + e[1], (double)d[2] + e[2],
+                                       (double)d[3] + e[3], (double)d[4] + e[4], (double)d[5] + e[5], (double)n);
+                }
+                (s ? vp : vm) = p;
+            }
+        }
+        sp[ra][kFinB - 1 - bi] = vm;
+        sp[ra][kFinB + bi] = vp;
+    }
+    __syncthreads();
+    // bin of slot i of row r: the minus run ends below the middle, the plus run starts above it
+    float* P = f.P;
+    if (P && f.P_off) P += (size_t)real * (size_t)f.P_total + f.P_off[curve];
+    unsigned long long best = 0ull;
+    for (int x = tid; x < kTcRows * 2 * kFinB; x += kFinThreads) {
+        const int r = x / (2 * kFinB), i = x % (2 * kFinB);
+        const int fine = i < kFinB ? nb - b0 - kFinB + i : nb + b0 + (i - kFinB);
+        const int64_t k = k0 + (int64_t)r * cols + fine;
+        if (k < nf) {
+            const float p = sp[r][i];
+            if (FORM == kTcGls && p < 0.f) continue;
+            if (P) P[k] = p;
+            const unsigned long long key =
+                ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~(uint32_t)k);
+            best = key > best ? key : best;
+        }
+    }
+    if (!f.maxkey) return;
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_down_sync(0xffffffffu, best, o);
+        best = y > best ? y : best;
+    }
+    if ((tid & 31) == 0) s_red[tid >> 5] = best;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kFinThreads / 32; ++w) best = s_red[w] > best ? s_red[w] : best;
+        if (best) atomicMax(&f.maxkey[(size_t)real * (size_t)f.n_curves + curve], best);
+    }
+}
+
+constexpr int kRefineThreads = 512;
+
+// s + c += t + d, s and t the leading parts (FP64 adds are slow on this part).
+__device__ __forceinline__ void add_pair(float& s, float& c, float t, float d) {
+    const float y = s + t, z = y - s;
+    c += ((s - (y - z)) + (t - z)) + d;
+    s = y;
+}
+
+// One cluster of CL CTAs per listed bin: the six sums over all samples, then P.
+// A single curve lists a few bins of many samples (CL = 8: 100,000 samples in
+// one CTA are 40 us of arithmetic), a batch many bins of shorter curves (CL = 1).
+template <int CL>
+__global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs a, const TcFinal f) {
+    __shared__ float2 sh[kRefineThreads / 32][6];
+    __shared__ float2 part[CL][6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0;
+    const unsigned count = min(*f.n_bins, (unsigned)kTcBins);
+    for (unsigned i = blockIdx.x / CL; i < count; i += gridDim.x / CL) {
+        const TcBin w = f.bins[i];
+        const int64_t b = a.off ? a.off[w.curve] : 0, n = a.off ? a.off[w.curve + 1] - b : a.n0;
+        float s[6] = {}, c[6] = {};
+        direct_gls(a, b, n, a.xr ? a.xr + (size_t)w.real * (size_t)a.total : nullptr, w.k,
+                   rank * kRefineThreads + (int)threadIdx.x, CL * kRefineThreads, s, c);
+        auto join = [&](int width) {
+            for (int o = width / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int x = 0; x < 6; ++x)
+                    add_pair(s[x], c[x], __shfl_down_sync(0xffffffffu, s[x], o),
+                             __shfl_down_sync(0xffffffffu, c[x], o));
+        };
+        join(32);
+        if (lane == 0)
+#pragma unroll
+            for (int x = 0; x < 6; ++x) sh[warp][x] = make_float2(s[x], c[x]);
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int x = 0; x < 6; ++x) {
+                const float2 v = lane < kRefineThreads / 32 ? sh[lane][x] : make_float2(0.f, 0.f);
+                s[x] = v.x;
+                c[x] = v.y;
+            }
+            join(kRefineThreads / 32);
+        }
+        if constexpr (CL > 1) {
+            if (threadIdx.x == 0) {
+                float2* first = cooperative_groups::this_cluster().map_shared_rank(&part[0][0], 0);
+#pragma unroll
+                for (int x = 0; x < 6; ++x) first[rank * 6 + x] = make_float2(s[x], c[x]);
+            }
+            cooperative_groups::this_cluster().sync();
+            if (threadIdx.x == 0 && rank == 0) {
+                for (int r = 1; r < CL; ++r)
+#pragma unroll
+                    for (int x = 0; x < 6; ++x) add_pair(s[x], c[x], part[r][x].x, part[r][x].y);
+            }
+        }
+        {
+            if (threadIdx.x == 0 && rank == 0) {
+                double d[6];
+#pragma unroll
+                for (int x = 0; x < 6; ++x) d[x] = (double)s[x] + (double)c[x];
+                const float p = dev::gls_value(d[0], d[1], d[2], d[3], d[4], d[5], (double)n);
+                if (f.P) f.P[(size_t)w.real * (size_t)f.P_total + (f.P_off ? f.P_off[w.curve] : 0) + w.k] = p;
+                if (f.maxkey)
+                    atomicMax(&f.maxkey[(size_t)w.real * (size_t)f.n_curves + w.curve],
+                              ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~w.k));
+            }
+        }
+        if constexpr (CL > 1) cooperative_groups::this_cluster().sync();
+        else __syncthreads();
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, int sms, cudaStream_t st) {
+    if (a.off) {
+        tc_refine_kernel<1><<<2 * sms, kRefineThreads, 0, st>>>(a, f);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 8;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(64);
+    cfg.blockDim = dim3(kRefineThreads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, tc_refine_kernel<8>, a, f);
+}
+
+cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(tc_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    if (e != cudaSuccess) return e;
+    tc_sums_kernel<<<a.ctas, kTcThreads, kSmem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st) {
+    const int n_data = a.tiles ? f.n_data : a.nblk;
+    if (n_data < 1) return cudaSuccess;
+    const int max_cols = (int)(a.slot_floats / 128);
+    dim3 grid((unsigned)n_data, (unsigned)((max_cols / 2 + kFinB - 1) / kFinB));
+    if (form == kTcClassic) tc_final_kernel<kTcClassic><<<grid, kFinThreads, 0, st>>>(a, f);
+    else tc_final_kernel<kTcGls><<<grid, kFinThreads, 0, st>>>(a, f);
+    return cudaGetLastError();
+}
+
+}  // namespace lsp

@@ -1,0 +1,130 @@
+// tc_sums.cuh -- the tensor-core evaluation of the periodogram's sums: work
+// list, launch interface and the closed-form split of the work over the CTAs
+// (shared by the kernels of tc_sums.cu and their callers).
+#pragma once
+
+#include "lsp_kernels.cuh"
+
+namespace lsp {
+
+// What a tile sums over its curve's samples j, for a block of frequencies:
+// sum_j y_j exp(2 pi i h phase_j(k)).
+enum : int {
+    kTcOne2 = 1,  // y = 1, h = 2: CC - SS + 2i CS
+    kTcRec = 2,   // y = x_hat of the records, h = 1: XC + i XS
+    kTcRow = 3,   // y = x_hat of a realization's row, h = 1
+    kTcW1 = 4,    // y = q^2, h = 1: the floating-mean form's C + i S
+    kTcW2 = 5,    // y = q^2, h = 2
+    kTcRecQ = 6,  // y = q x_hat of the records, h = 1
+    kTcRowQ = 7   // y = q x_hat of a realization's row, h = 1
+};
+
+// One tile: kTcRows coarse frequencies x cols fine offsets of one sum.  wtile
+// and ctile: the tiles with the same frequencies that hold the h = 2 sum and
+// the floating-mean form's (C, S) for the finalize kernel (data tiles only).
+struct TcTile {
+    int32_t curve, real, fblock, kind, wtile, ctile, cols, pad;
+};
+
+constexpr int kTcRows = 64;        // coarse frequencies of a tile (128 operand rows: real and imaginary parts)
+constexpr int kTcMaxCols = 256;    // fine offsets of a tile, at most
+constexpr int kTcUnit = 128;       // samples of one unit of work
+constexpr int kTcThreads = 640;
+constexpr int kTcMaxCtas = 512;   // CTAs (one per SM) that a launch is split over, at most
+
+// Cost of a unit of a tile, in sixteenths of the columns: the MMA time is
+// proportional to the columns above 144 and constant (75 cycles) below.
+__host__ __device__ inline int tc_unit_cost(int cols) { return (cols > 144 ? cols : 144) / 16; }
+
+// Fine offsets per coarse frequency for a grid of N_f bins: the number of
+// blocks (of 64 coarse frequencies) and columns (a multiple of 16, 32 .. 256)
+// whose cost is least.
+__host__ __device__ inline int tc_cols(int64_t N_f) {
+    const int64_t b0 = (N_f + kTcRows * kTcMaxCols - 1) / (kTcRows * kTcMaxCols);
+    int best = kTcMaxCols;
+    int64_t best_cost = INT64_MAX;
+    for (int64_t b = b0 < 1 ? 1 : b0; b <= b0 + 2; ++b) {
+        const int64_t per = (N_f + b * kTcRows - 1) / (b * kTcRows);
+        int c = (int)((per + 15) / 16 * 16);
+        if (c < 32) c = 32;
+        const int64_t blocks = (N_f + (int64_t)c * kTcRows - 1) / ((int64_t)c * kTcRows);
+        const int64_t cost = blocks * tc_unit_cost(c);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
+struct TcArgs {
+    // tiles: a list with the prefix sums of their costs (pre[0..n_tiles]), or,
+    // for a single curve (tiles == nullptr), sum s of block fb0 + b is tile
+    // s * nblk + b with kinds[s], every tile of the same cost
+    const TcTile* tiles;
+    const int64_t* pre;
+    int n_tiles, nblk, fb0, cols;
+    int kinds[3];
+    int64_t n0;                 // samples of the single curve
+    int64_t work;               // total cost
+    int ctas;                   // CTAs the work is split over
+    const int64_t* off;         // curves' sample offsets (list form)
+    const uint4* recA;
+    const float4* recB;
+    const float2* recE;         // (cos, sin)(2 pi cols u)
+    const float* q;             // sqrt weights (floating mean)
+    const float* qmax;          // largest q of each curve
+    const float* xr;            // realization rows
+    int64_t total;              // row stride of xr
+    float* part;                // slots of slot_floats: tile t's piece by CTA i is slot t + i
+    int64_t slot_floats;
+    int* status;
+};
+
+// Where the work coordinate of CTA i starts.
+__host__ __device__ inline int64_t tc_bound(int64_t work, int ctas, int i) { return work * i / ctas; }
+// The CTA whose range holds coordinate x.
+__host__ __device__ inline int tc_cta_of(int64_t work, int ctas, int64_t x) {
+    return (int)(((x + 1) * ctas - 1) / work);
+}
+// Units [u0, u1) of a tile that starts at coordinate p (n units of cost c each)
+// whose starts lie in [lo, hi).
+__host__ __device__ inline void tc_units(int64_t p, int64_t n, int64_t c, int64_t lo, int64_t hi, int64_t* u0,
+                                         int64_t* u1) {
+    const int64_t a = lo <= p ? 0 : (lo - p + c - 1) / c, b = hi <= p ? 0 : (hi - p + c - 1) / c;
+    *u0 = a < n ? a : n;
+    *u1 = b < n ? b : n;
+}
+
+// The finalize pass over the data tiles (kTcRec, kTcRow, kTcRecQ, kTcRowQ): P of
+// every frequency.
+// A bin of the floating-mean form whose sums are formed again by
+// launch_tc_refine: realization `real` of `curve`, frequency k.
+struct TcBin {
+    int32_t curve, real;
+    uint32_t k, pad;
+};
+constexpr int kTcBins = 1 << 16;  // bins the list holds
+
+struct TcFinal {
+    const int* data_tiles;      // list form: indices of the data tiles
+    int n_data;
+    const int64_t* nf;          // list form
+    int64_t nf0;                // single curve
+    float* P;                   // may be null
+    const int64_t* P_off;
+    int64_t P_total;
+    unsigned long long* maxkey; // may be null
+    int n_curves;
+    TcBin* bins;                // floating mean: list of ill-conditioned bins and
+    unsigned* n_bins;           // its counter (zeroed by launch_prep_stats, after qmax)
+};
+
+enum : int { kTcClassic = 0, kTcGls = 1 };
+
+cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st);
+cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st);
+// Floating mean: the listed bins, after every launch_tc_final of the call.
+cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, int sms, cudaStream_t st);
+
+}  // namespace lsp
