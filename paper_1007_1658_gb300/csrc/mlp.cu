@@ -32,43 +32,72 @@ __device__ __forceinline__ float gelu_grad(float z) {
 // EPI 0: C[m*ldc+n] = acc (+ bias[n] if bias)
 // EPI 1: Z = acc + bias[n]; C[m*ldc+n] = Z; D[m*ldc+n] = GELU(Z)
 // EPI 2: C[m*ldc+n] = acc * GELU'(Zs[m*ldc+n])
+// Every output adds its k in order, so the tiling does not show in the bits.
+// Operands are read along their contiguous dimension (ak1: A's is k, else m; bn1:
+// B's is n, else k), the next K step's into registers while the current one is
+// multiplied from one of two shared-memory buffers.  With gridDim.z > 1 (EPI 0,
+// no bias) slice z sums k in [z kc, (z + 1) kc) into C + z M ldc.
 template <typename TA, typename TB, typename TD, int EPI>
 __global__ void __launch_bounds__(kGemmThreads)
-gemm_kernel(int M, int N, int K, const TA* __restrict__ A, int64_t sAm, int64_t sAk, const TB* __restrict__ B,
-            int64_t sBk, int64_t sBn, const float* __restrict__ bias, float* __restrict__ C, int64_t ldc,
-            TD* __restrict__ D, const float* __restrict__ Zs) {
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
+gemm_kernel(int M, int N, int K, int kc, bool ak1, bool bn1, const TA* __restrict__ A, int64_t sAm, int64_t sAk,
+            const TB* __restrict__ B, int64_t sBk, int64_t sBn, const float* __restrict__ bias, float* __restrict__ C,
+            int64_t ldc, TD* __restrict__ D, const float* __restrict__ Zs) {
+    __shared__ __align__(16) float As[2][BK][BM + 4];
+    __shared__ __align__(16) float Bs[2][BK][BN + 4];
+    constexpr int kEach = BM * BK / kGemmThreads;  // elements of each operand a thread brings per step
+    static_assert(BM == BN && BM * BK % kGemmThreads == 0, "square tiles");
     const int tid = threadIdx.x;
     const int tm = tid / 16, tn = tid % 16;  // 16 x 16 threads, 4 x 4 outputs each
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int k_lo = blockIdx.z * kc, k_hi = min(K, k_lo + kc);
+    // element q of this thread: its place in the tile (m or n, k) and its address
+    int am[kEach], ak[kEach], bn[kEach], bk[kEach];
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) {
+        const int i = tid + q * kGemmThreads;
+        am[q] = ak1 ? i / BK : i % BM;
+        ak[q] = ak1 ? i % BK : i / BM;
+        bn[q] = bn1 ? i % BN : i / BK;
+        bk[q] = bn1 ? i / BN : i % BK;
+    }
+    float ra[kEach], rb[kEach];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < kEach; ++q) {
+            const int gm = m0 + am[q], gk = k0 + ak[q], gn = n0 + bn[q], hk = k0 + bk[q];
+            ra[q] = (gm < M && gk < k_hi) ? to_f(A[(int64_t)gm * sAm + (int64_t)gk * sAk]) : 0.f;
+            rb[q] = (gn < N && hk < k_hi) ? to_f(B[(int64_t)hk * sBk + (int64_t)gn * sBn]) : 0.f;
+        }
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int q = 0; q < kEach; ++q) {
+            As[buf][ak[q]][am[q]] = ra[q];
+            Bs[buf][bk[q]][bn[q]] = rb[q];
+        }
+    };
     float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int i = tid; i < BM * BK; i += kGemmThreads) {
-            const int mm = i / BK, kk = i % BK;
-            const int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < M && gk < K) ? to_f(A[(int64_t)gm * sAm + (int64_t)gk * sAk]) : 0.f;
-        }
-        for (int i = tid; i < BN * BK; i += kGemmThreads) {
-            const int nn = i % BN, kk = i / BN;
-            const int gn = n0 + nn, gk = k0 + kk;
-            Bs[kk][nn] = (gn < N && gk < K) ? to_f(B[(int64_t)gk * sBk + (int64_t)gn * sBn]) : 0.f;
-        }
-        __syncthreads();
+    load(k_lo);
+    store(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = k_lo; k0 < k_hi; k0 += BK, buf ^= 1) {
+        const bool more = k0 + BK < k_hi;
+        if (more) load(k0 + BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][tm * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tn * 4 + j];
+            const float4 av = *reinterpret_cast<const float4*>(&As[buf][kk][tm * 4]);
+            const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tn * 4]);
+            const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
+        if (more) store(buf ^ 1);
         __syncthreads();
     }
+    C += (size_t)blockIdx.z * (size_t)M * (size_t)ldc;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int gm = m0 + tm * 4 + i;
@@ -91,6 +120,16 @@ gemm_kernel(int M, int N, int K, const TA* __restrict__ A, int64_t sAm, int64_t 
             }
         }
     }
+}
+
+// Sum of S slices of n values, in order.
+__global__ void slices_kernel(int S, int64_t n, const float* __restrict__ part, float* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int z = 0; z < S; ++z) s += part[(size_t)z * (size_t)n + i];
+    out[i] = s;
 }
 
 // Gather B rows: X = (features[row % n_pat] - mu) / sigma, counts, y[row].
@@ -157,19 +196,26 @@ __global__ void head_kernel(int Bn, const float* __restrict__ z, const float* __
     }
 }
 
-// Column sums of a rows x cols matrix (bias gradients), fixed order per column.
-__global__ void colsum_kernel(int rows, int cols, const float* __restrict__ G, float* __restrict__ out) {
-    const int c = blockIdx.x;
-    __shared__ float sh[256];
+// Column sums of a rows x cols matrix (bias gradients), fixed order per column:
+// a warp reads 32 neighbouring columns of a row, 32 warps take every 32nd row.
+constexpr int kColThreads = 1024;
+__global__ void __launch_bounds__(kColThreads)
+colsum_kernel(int rows, int cols, const float* __restrict__ G, float* __restrict__ out) {
+    __shared__ float sh[32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) s += G[(int64_t)r * cols + c];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
+    if (c < cols) {
+#pragma unroll 8
+        for (int r = w; r < rows; r += 32) s += G[(int64_t)r * cols + c];
     }
-    if (threadIdx.x == 0) out[c] = sh[0];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && c < cols) {
+        float t = 0.f;
+        for (int x = 0; x < 32; ++x) t += sh[x][lane];
+        out[c] = t;
+    }
 }
 
 // Mean of n values (one CTA, fixed order).
@@ -244,7 +290,33 @@ template <typename TA, typename TB, typename TD, int EPI>
 cudaError_t gemm(int M, int N, int K, const TA* A, int64_t sAm, int64_t sAk, const TB* B, int64_t sBk,
                  int64_t sBn, const float* bias, float* C, int64_t ldc, TD* D, const float* Zs, cudaStream_t st) {
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-    gemm_kernel<TA, TB, TD, EPI><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, sAm, sAk, B, sBk, sBn, bias, C, ldc, D, Zs);
+    gemm_kernel<TA, TB, TD, EPI><<<grid, kGemmThreads, 0, st>>>(M, N, K, K, sAk == 1, sBn == 1, A, sAm, sAk, B, sBk,
+                                                                sBn, bias, C, ldc, D, Zs);
+    return cudaGetLastError();
+}
+
+// A weight gradient: few output tiles (16 of 64 x 64 at H = 256) and a sum over
+// the whole minibatch, so k is cut into slices of at least kMinSlice until about
+// kSliceCtas CTAs have work; the slices are added in order.  256 x 256 x 4096: 873
+// us in one slice.
+constexpr int kSliceCtas = 304, kMinSlice = 64;
+template <typename TA>
+cudaError_t gemm_weight_grad(int M, int N, int K, const TA* A, int64_t sAm, int64_t sAk, const float* B, float* part,
+                             float* C, cudaStream_t st) {
+    dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
+    const int tiles = (int)(grid.x * grid.y);
+    int S = kSliceCtas / tiles;
+    if (S > (K + kMinSlice - 1) / kMinSlice) S = (K + kMinSlice - 1) / kMinSlice;
+    if (S < 1) S = 1;
+    const int kc = ((K + S - 1) / S + BK - 1) / BK * BK;
+    S = (K + kc - 1) / kc;
+    grid.z = (unsigned)S;
+    gemm_kernel<TA, float, float, 0><<<grid, kGemmThreads, 0, st>>>(M, N, K, kc, sAk == 1, true, A, sAm, sAk, B, N, 1,
+                                                                    nullptr, S > 1 ? part : C, N, nullptr, nullptr);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || S == 1) return e;
+    const int64_t n = (int64_t)M * N;
+    slices_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(S, n, part, C);
     return cudaGetLastError();
 }
 
@@ -294,7 +366,8 @@ cudaError_t mlp_gather(int Bn, const int32_t* rows, int n_pat, const float* feat
 }
 
 // Forward (and with y, loss + backward into grad).  Workspace layout in `ws`
-// (floats): Z[3][B][H], dZ[2][B][H], zo[B][9], dzo[B][9], loss_row[B]; acts
+// (floats): Z[3][B][H], dZ[2][B][H], zo[B][9], dzo[B][9], loss_row[B], slices of a
+// weight gradient (at most kSliceCtas tiles of 64 x 64 in all); acts
 // in `act` (3 x B x H, BF16 or FP32 by `fp32`).
 template <typename TD>
 static cudaError_t mlp_run(int H, int Bn, const float* params, const float* X, const float* cnt, const float* y,
@@ -307,6 +380,7 @@ static cudaError_t mlp_run(int H, int Bn, const float* params, const float* X, c
     float* zo = ws + 5 * BH;
     float* dzo = zo + (int64_t)Bn * 9;
     float* lrow = dzo + (int64_t)Bn * 9;
+    float* part = lrow + (int64_t)Bn;  // slices of a weight gradient
     TD* Aa[3] = {act, act + BH, act + 2 * BH};
     const float* W[4] = {params + o[0], params + o[2], params + o[4], params + o[6]};
     const float* b[4] = {params + o[1], params + o[3], params + o[5], params + o[7]};
@@ -324,9 +398,9 @@ static cudaError_t mlp_run(int H, int Bn, const float* params, const float* X, c
     float* gW[4] = {grad + o[0], grad + o[2], grad + o[4], grad + o[6]};
     float* gb[4] = {grad + o[1], grad + o[3], grad + o[5], grad + o[7]};
     // output layer
-    e = gemm<TD, float, float, 0>(H, 9, Bn, Aa[2], 1, H, dzo, 9, 1, nullptr, gW[3], 9, (float*)nullptr, nullptr, st);
+    e = gemm_weight_grad<TD>(H, 9, Bn, Aa[2], 1, H, dzo, part, gW[3], st);
     if (e == cudaSuccess) {
-        colsum_kernel<<<9, 256, 0, st>>>(Bn, 9, dzo, gb[3]);
+        colsum_kernel<<<1, kColThreads, 0, st>>>(Bn, 9, dzo, gb[3]);
         e = cudaGetLastError();
     }
     // dZ3 = (dzo W4^T) * gelu'(Z3)
@@ -336,13 +410,11 @@ static cudaError_t mlp_run(int H, int Bn, const float* params, const float* X, c
     for (int l = 2; l >= 0 && e == cudaSuccess; --l) {
         // weight gradient: A_{l-1}^T dZ_l (the input X for l = 0)
         if (l > 0)
-            e = gemm<TD, float, float, 0>(l == 0 ? 32 : H, H, Bn, Aa[l - 1], 1, H, dZ[cur], H, 1, nullptr, gW[l], H,
-                                          (float*)nullptr, nullptr, st);
+            e = gemm_weight_grad<TD>(H, H, Bn, Aa[l - 1], 1, H, dZ[cur], part, gW[l], st);
         else
-            e = gemm<float, float, float, 0>(32, H, Bn, X, 1, 32, dZ[cur], H, 1, nullptr, gW[0], H, (float*)nullptr,
-                                             nullptr, st);
+            e = gemm_weight_grad<float>(32, H, Bn, X, 1, 32, dZ[cur], part, gW[0], st);
         if (e != cudaSuccess) break;
-        colsum_kernel<<<H, 256, 0, st>>>(Bn, H, dZ[cur], gb[l]);
+        colsum_kernel<<<(H + 31) / 32, kColThreads, 0, st>>>(Bn, H, dZ[cur], gb[l]);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if (l > 0) {
             e = gemm<float, float, float, 2>(Bn, H, H, dZ[cur], H, 1, W[l], 1, H, nullptr, dZ[cur ^ 1], H,
@@ -353,7 +425,9 @@ static cudaError_t mlp_run(int H, int Bn, const float* params, const float* X, c
     return e;
 }
 
-size_t mlp_workspace_floats(int H, int Bn) { return (size_t)5 * Bn * H + (size_t)Bn * 19 + 64; }
+size_t mlp_workspace_floats(int H, int Bn) {
+    return (size_t)5 * Bn * H + (size_t)Bn * 19 + (size_t)kSliceCtas * BM * BN + 64;
+}
 size_t mlp_act_bytes(int H, int Bn, bool fp32) { return (size_t)3 * Bn * H * (fp32 ? 4 : 2); }
 
 cudaError_t mlp_forward_backward(int H, int Bn, bool fp32, const float* params, const float* X, const float* cnt,
