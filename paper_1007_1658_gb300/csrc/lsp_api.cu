@@ -162,13 +162,13 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
     const int64_t per = (int64_t)lsp::kTcRows * cols, blocks = (N_f + per - 1) / per;
     const int sums = gls ? 3 : 2;
     const int64_t units = (N + lsp::kTcUnit - 1) / lsp::kTcUnit;
-    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    const int pairs = lsp::tc_pairs(ctx->sms);
     lsp::TcArgs a{};
-    a.slot_floats = 128 * (int64_t)cols;
+    a.slot_floats = lsp::tc_slot_floats(cols);
     // at most 1 GiB of partial tiles at a time
-    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - sms) / sums);
+    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - pairs) / sums);
     const int64_t step = std::min(blocks, most);
-    lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)(step * sums + sms) * (size_t)a.slot_floats * 4);
+    lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)(step * sums + pairs) * (size_t)a.slot_floats * 4);
     if (rs != LSP_OK || !launch) return rs;
     a.cols = cols;
     a.kinds[0] = gls ? lsp::kTcRecQ : lsp::kTcRec;
@@ -188,7 +188,7 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
         a.nblk = (int)std::min(step, blocks - fb);
         a.n_tiles = a.nblk * sums;
         a.work = (int64_t)a.n_tiles * units * lsp::tc_unit_cost(cols);
-        a.ctas = (int)std::min<int64_t>(sms, (int64_t)a.n_tiles * units);
+        a.pairs = (int)std::min<int64_t>(pairs, (int64_t)a.n_tiles * units);
         LSP_CUDA(ctx, lsp::launch_tc_sums(a, ctx->stream));
         if (timing && fb + step >= blocks) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
         lsp::TcFinal f{};
@@ -199,7 +199,7 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
         LSP_CUDA(ctx, lsp::launch_tc_final(gls ? lsp::kTcGls : lsp::kTcClassic, a, f, ctx->stream));
         *launches += 2;
         if (gls && fb + step >= blocks) {
-            LSP_CUDA(ctx, lsp::launch_tc_refine(a, f, sms, ctx->stream));
+            LSP_CUDA(ctx, lsp::launch_tc_refine(a, f, ctx->stream));
             ++*launches;
         }
     }
@@ -244,15 +244,15 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
                                      const std::vector<int64_t>& nf, int n_real) {
     TcPlan p;
     const int shared = form == lsp::kTcClassic ? 1 : 2;
-    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    const int pairs = lsp::tc_pairs(ctx->sms);
     // at most 4 GiB of partial tiles at a time
-    const int64_t most = (int64_t(1) << 30) / (128 * lsp::kTcMaxCols) - sms;
+    const int64_t most = (int64_t(1) << 30) / lsp::tc_slot_floats(lsp::kTcMaxCols) - pairs;
     TcChunk cur{0, 0, 0, 0, 0, 0};
     p.pre.push_back(0);
     auto flush = [&]() {
         if (cur.n == 0) return;
         p.chunks.push_back(cur);
-        p.max_slot_floats = std::max(p.max_slot_floats, (cur.n + sms) * 128 * (int64_t)cur.cols);
+        p.max_slot_floats = std::max(p.max_slot_floats, (cur.n + pairs) * lsp::tc_slot_floats(cur.cols));
         cur = TcChunk{(int64_t)p.tiles.size(), 0, (int64_t)p.data.size(), 0, 0, 0};
         p.pre.push_back(0);
     };
@@ -298,7 +298,7 @@ cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d
     const lsp::TcTile* tiles = (const lsp::TcTile*)d_plan;
     const int64_t* pre = (const int64_t*)(tiles + p.tiles.size());
     const int* data = (const int*)(pre + p.pre.size());
-    const int sms = std::min(std::max(1, ctx->sms), lsp::kTcMaxCtas);
+    const int pairs = lsp::tc_pairs(ctx->sms);
     for (size_t x = 0; x < p.chunks.size(); ++x) {
         const TcChunk& c = p.chunks[x];
         a.tiles = tiles + c.t0;
@@ -306,15 +306,15 @@ cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d
         a.n_tiles = (int)c.n;
         a.cols = c.cols;
         a.work = c.work;
-        a.ctas = (int)std::min<int64_t>(sms, c.work / lsp::tc_unit_cost(0));
-        a.slot_floats = 128 * (int64_t)c.cols;
+        a.pairs = (int)std::min<int64_t>(pairs, std::max<int64_t>(1, c.work / lsp::tc_unit_cost(c.cols)));
+        a.slot_floats = lsp::tc_slot_floats(c.cols);
         f.data_tiles = data + c.d0;
         f.n_data = (int)c.nd;
         cudaError_t e = lsp::launch_tc_sums(a, st);
         if (e == cudaSuccess) e = lsp::launch_tc_final(form, a, f, st);
         if (e != cudaSuccess) return e;
     }
-    if (form == lsp::kTcGls && !p.chunks.empty()) return lsp::launch_tc_refine(a, f, sms, st);
+    if (form == lsp::kTcGls && !p.chunks.empty()) return lsp::launch_tc_refine(a, f, st);
     return cudaSuccess;
 }
 

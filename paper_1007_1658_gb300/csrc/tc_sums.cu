@@ -7,8 +7,8 @@
 // are a real matrix product A^T B with A[j][2a, 2a+1] = y_j (cos, sin)(2 pi f_a
 // t_j) and B[j][2b, 2b+1] = (cos, sin)(2 pi f_b t_j); its four entries for
 // (a, b) give the complex sums at f_a + f_b and f_a - f_b, so a term still
-// costs two multiply-adds per sum, and the operands cost 64 + cols/2 complex
-// values per sample for 64 cols terms.  With y = x_hat this is XC + i XS; the
+// costs two multiply-adds per sum, and the operands cost 128 + cols/2 complex
+// values per sample for 128 cols terms.  With y = x_hat this is XC + i XS; the
 // tau sums CC - SS + 2i CS are the same product with y = 1 at doubled phases.
 // Phases are the exact 64-bit fixed-point turns of the strip kernels.
 //
@@ -22,8 +22,12 @@
 // to running sums in registers while the next unit accumulates in the other
 // half of tensor memory.
 //
+// The product runs on CTA pairs (256 x cols x 16 an instruction): a CTA makes and
+// holds half of the rows of A and half of the columns of B, so its operands per
+// term are two thirds of a single CTA's, in the making and in shared memory.
+//
 // What bounds it: with cols = 256 the three MMAs of 16 samples take 390 cycles
-// (24 a sample for 16,384 terms), the operands 192 complex values a sample.
+// (24 a sample for 32,768 terms), the operands 128 complex values a sample and CTA.
 #include "ls_device.cuh"
 #include "tc_device.cuh"
 #include "tc_sums.cuh"
@@ -34,13 +38,16 @@
 namespace lsp {
 namespace {
 
-constexpr int kStage = 64;                         // samples of one operand stage
-constexpr int kAbytes = 128 * kStage * 2;          // one half (hi or lo) of A: 128 rows
-constexpr int kBbytes = kTcMaxCols * kStage * 2;   // one half of B
+constexpr int kStage = 32;                        // samples of one operand stage
+constexpr int kSets = kTcUnit / kStage;           // sets of warps, each filling every kSets-th stage
+constexpr int kBufs = 6;                          // stage buffers
+constexpr int kAbytes = 128 * kStage * 2;         // one half (hi or lo) of A: 128 rows
+constexpr int kBbytes = kTcMaxCols / 2 * kStage * 2;  // one half of a CTA's columns of B
 constexpr int kStageBytes = 2 * kAbytes + 2 * kBbytes;
-constexpr int kSbo = kStage * 16;                  // bytes of one 8-row group of an operand
+constexpr int kSbo = kStage * 16;                 // bytes of one 8-row group of an operand
 constexpr int kGenWarps = 16;
-constexpr size_t kSmem = 2 * (size_t)kStageBytes + sizeof(float) * 12 * kGenWarps * 32;
+constexpr int kSetWarps = kGenWarps / kSets;
+constexpr size_t kSmem = kBufs * (size_t)kStageBytes + sizeof(float) * 12 * kGenWarps * 32;
 
 // (cos, sin) of a 64-bit fixed-point turn: quadrant and 30-bit remainder of the
 // top word, then the Taylor series on [-pi/4, pi/4] (truncation below 2e-9).
@@ -181,40 +188,49 @@ constexpr float kUnitGain = 1.f + 0x1.8p-22f;
 // result's norm from the 64-bit one, against 4e-7 with the strip kernels).
 constexpr int kRunUnits = 128;
 
-// Sixteen warps form the operands and drain the accumulators, in two sets that
-// take every other stage (a set's fixed latencies -- waits, record fetch, proxy
-// fence -- then pass while the other works), each thread 16 coarse rows and up
-// to 32 fine offsets of one sample; warp 16 issues the MMAs (issuing blocks
-// while the queue is full, so a warp that also forms operands would make the
-// two take turns: 5.4 us for 128 samples against 3.7).  The register split
-// comes from setmaxnreg: 640 threads at 96 registers launch, 512 x 112 + 128 x
-// 24 of those 61,440 are kept.  Barriers, two of each: filled and empty
-// (operand stages), full and drained (accumulators).  Nothing waits for another
-// CTA, and every wait has a limit, after which the CTA stops waiting, says so
-// in the status word and runs to its end.
-__global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) {
+// In each CTA of the pair, sixteen warps form the operands (its 64 coarse
+// frequencies, its half of the fine offsets) and drain its accumulators, in
+// four sets of four: a set fills every fourth stage of 32 samples, a thread 16
+// coarse rows and up to 16 fine offsets of one sample, so that the four warps
+// of an SM sub-partition are at different points of their work and hide each
+// other's waits; six stage buffers leave a set two stages ahead of the MMAs.
+// Warp 16 of the first CTA issues the MMAs of both (issuing blocks while the
+// queue is full, so in a warp that also forms operands the two would take
+// turns), all its lanes together but for the instruction itself.  The register split comes from setmaxnreg: 640 threads at 96
+// registers launch, 512 x 112 + 128 x 32 are those 61,440.  Barriers:
+// filled (a stage, counted at the first CTA) and empty, full (an accumulator, a
+// unit's MMAs done) and drained (counted at the first CTA).  No pair waits for
+// another pair, and every wait has a limit, after which the CTA stops waiting,
+// says so in the status word and runs to its end.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) {
     extern __shared__ __align__(128) unsigned char stages[];
-    Ahead& ahead = *reinterpret_cast<Ahead*>(stages + 2 * kStageBytes);
-    __shared__ uint64_t filled[2], empty[2], full[2], drained[2];
+    Ahead& ahead = *reinterpret_cast<Ahead*>(stages + kBufs * kStageBytes);
+    __shared__ uint64_t filled[kBufs], empty[kBufs], full[2], drained[2];
     __shared__ uint32_t tbase;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int rank = (int)tc::pair_rank(), pair = blockIdx.x >> 1;
     if (tid == 0) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&filled[i], kGenWarps / 2);
+        for (int i = 0; i < kBufs; ++i) {
+            tc::mbar_init(&filled[i], 2 * kSetWarps);
             tc::mbar_init(&empty[i], 1);
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&drained[i], kGenWarps);
         }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&drained[i], 2 * kGenWarps);
+        }
+        tc::mbar_init_done();
     }
     if (warp == 0) tc::tmem_alloc(&tbase, 512);
     tc::fence_operands();
     tc::fence_before_sync();
     __syncthreads();
+    tc::pair_sync();
     tc::fence_after_sync();
     const uint32_t tb = tbase;
 
-    const int64_t lo = tc_bound(a.work, a.ctas, blockIdx.x), hi = tc_bound(a.work, a.ctas, blockIdx.x + 1);
+    const int64_t lo = tc_bound(a.work, a.pairs, pair), hi = tc_bound(a.work, a.pairs, pair + 1);
     const int64_t cost0 = a.tiles ? 0 : (a.n0 + kTcUnit - 1) / kTcUnit * tc_unit_cost(a.cols);
     // first tile that reaches beyond lo
     int t = 0;
@@ -229,8 +245,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
         t = (int)(lo / cost0);
     }
     bool ok = true;
-    uint32_t group = 0;  // units so far
-    // the next piece of a tile in this CTA's range: its tile, first sample and length
+    uint32_t group = 0, it = 0;  // units and stages so far
+    // the next piece of a tile in this pair's range: its tile, first sample and length
     TileInfo f;
     int64_t j0 = 0;
     int left = 0;
@@ -250,48 +266,49 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
     };
 
     if (warp >= kGenWarps) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
-        if (warp == kGenWarps && lane == 0) {
-            uint32_t uses[2] = {0, 0};
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+        if (warp == kGenWarps && rank == 0) {
+            uint32_t buf = 0, phase = 0;
             for (; next_piece(); ++t) {
                 const uint32_t id = tc::instr_desc(f.cols);
                 for (int m = 0; m < left; m += kTcUnit, ++group) {
                     const uint32_t d = tb + (group & 1) * 256u;
                     if (group >= 2) ok = ok && tc::mbar_wait(&drained[group & 1], ((group >> 1) - 1) & 1);
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        const int rest = left - m - s * kStage;
-                        if (rest <= 0) break;
-                        ok = ok && tc::mbar_wait(&filled[s], uses[s]++ & 1);
+                    for (int q = m; q < min(left, m + kTcUnit); q += kStage) {
+                        ok = ok && tc::mbar_wait(&filled[buf], phase);
+                        __syncwarp();
                         tc::fence_after_sync();
-                        const uint32_t sa = tc::smem_addr(stages) + s * kStageBytes, sb = sa + 2 * kAbytes;
-                        const int ks = (min(rest, kStage) + 15) / 16;
-                        uint32_t acc = s;
-                        for (int pass = 0; pass < 3; ++pass) {  // hi lo, lo hi, hi hi
-                            const uint32_t qa = sa + (pass == 1 ? kAbytes : 0), qb = sb + (pass == 0 ? kBbytes : 0);
-                            for (int k = 0; k < ks; ++k) {
-                                tc::mma_f16(d, tc::operand_desc(qa + k * 256, 128, kSbo),
-                                            tc::operand_desc(qb + k * 256, 128, kSbo), id, acc);
-                                acc = 1;
-                            }
+                        const uint64_t da = tc::operand_desc(tc::smem_addr(stages) + buf * kStageBytes, 128, kSbo);
+                        const uint64_t db = da + (2 * kAbytes >> 4);
+                        constexpr uint64_t al = kAbytes >> 4, bl = kBbytes >> 4, k1 = 256 >> 4;
+                        const bool two = left - q > 16;  // the second 16 samples of the stage
+                        if (tc::elect_one()) {
+                            tc::mma_f16(d, da, db + bl, id, q > m);  // hi lo
+                            if (two) tc::mma_f16(d, da + k1, db + bl + k1, id, 1);
+                            tc::mma_f16(d, da + al, db, id, 1);      // lo hi
+                            if (two) tc::mma_f16(d, da + al + k1, db + k1, id, 1);
+                            tc::mma_f16(d, da, db, id, 1);           // hi hi
+                            if (two) tc::mma_f16(d, da + k1, db + k1, id, 1);
+                            tc::mma_commit(&empty[buf]);
+                            if (q + kStage >= min(left, m + kTcUnit)) tc::mma_commit(&full[group & 1]);
                         }
-                        tc::mma_commit(&empty[s]);
+                        __syncwarp();
+                        if (++buf == kBufs) {
+                            buf = 0;
+                            phase ^= 1;
+                        }
                     }
-                    tc::mma_commit(&full[group & 1]);
                 }
             }
         }
         __syncwarp();
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
-        const int set = tid / (kStage * 4), grp = (tid / kStage) & 3, js = tid & (kStage - 1);
-        const int quad = warp & 3, cg = warp >> 2;  // this warp's lanes and columns of the accumulators
-        unsigned char* const Ah = stages + set * kStageBytes + js * 16;
-        unsigned char* const Bh = Ah + 2 * kAbytes;
-        uint32_t uses = 0;
+        // this warp's set, its group of rows and offsets, its lanes and columns of the accumulators
+        const int set = warp >> 2, grp = warp & 3, quad = grp, cg = set;
         for (; next_piece(); ++t) {
             const bool twice = f.kind == kTcOne2 || f.kind == kTcW2;
-            const int nb = f.cols >> 1;  // fine offsets of one sign
+            const int hb = f.cols >> 2;  // fine offsets (of one sign) of this CTA
             auto fetch = [&](int j) {    // sample j of the piece
                 if (j < left) {
                     dev::cp_async16(&ahead.uv[tid], a.recA + j0 + j);
@@ -317,7 +334,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
                 tc::fence_after_sync();
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    if (cg * 64 + c * 32 < f.cols) {  // columns from f.cols on are read as they are and never stored
+                    if (cg * 64 + c * 32 < f.cols) {
                         uint32_t r[32];
                         tc::tmem_ld32(r, tb + (g & 1) * 256u + ((uint32_t)quad << 21) + (uint32_t)(cg * 64 + c * 32));
 #pragma unroll
@@ -327,18 +344,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
                 }
                 tc::fence_before_sync();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&drained[g & 1]);
+                if (lane == 0) tc::mbar_arrive_first(&drained[g & 1]);
             };
             // the running sums into this piece's slot: columns of the tile, rows contiguous
-            float* const out = a.part + (size_t)(t + (int)blockIdx.x) * (size_t)a.slot_floats +
-                               (size_t)(cg * 64) * 128 + quad * 32 + lane;
             auto flush = [&](bool add) {
+                float* const out = a.part + (size_t)(t + pair) * (size_t)a.slot_floats +
+                                   (size_t)rank * (size_t)(a.slot_floats / 2) + (size_t)(cg * 64) * 128 + quad * 32 + lane;
                 const float inv = 1.f / f.scale;
 #pragma unroll
                 for (int i = 0; i < 64; ++i)
                     if (cg * 64 + i < f.cols) out[i * 128] = fmaf(run[i], inv, add ? out[i * 128] : 0.f);
             };
-            fetch(set * kStage + js);
+            fetch(set * kStage + lane);
             for (int m = 0; m < left; m += kTcUnit, ++group) {
                 const int jm = m + set * kStage;  // this set's stage of the unit
                 if (jm < left) {
@@ -346,28 +363,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
                     const uint4 uv = ahead.uv[tid];
                     const float4 B = ahead.B[tid];
                     float2 e1 = make_float2(B.y, B.z), E = ahead.E[tid];
-                    float y = jm + js < left ? f.scale : 0.f;
+                    float y = jm + lane < left ? f.scale : 0.f;
                     if (f.kind >= kTcW1) {
                         const float q = ahead.q[tid];
                         y *= q;
                         if (f.kind <= kTcW2) y *= q;
                     }
                     if ((f.kind & 3) > 1) y *= (f.kind & 1) ? ahead.x[tid] : B.x;
-                    fetch(jm + kTcUnit + js);
+                    fetch(jm + kTcUnit + lane);
                     const uint64_t u = ((uint64_t)uv.y << 32) | uv.x;
                     const uint64_t v = (((uint64_t)uv.w << 32) | uv.z) - kPhaseOffset;
                     const uint64_t uh = u >> 1;
-                    // the middle of the first of 16 coarse blocks of cols bins, and the first of 32 fine offsets
-                    uint64_t pa = v + (uint64_t)(f.k0 + (uint32_t)(16 * grp * f.cols) + (uint32_t)nb) * u - uh;
-                    uint64_t pb = (uint64_t)(32 * grp) * u + uh;
+                    // the middle of the first of 16 coarse blocks of cols bins, and the first of 16 fine offsets
+                    uint64_t pa = v + (uint64_t)(f.k0 + (uint32_t)((64 * rank + 16 * grp) * f.cols + 2 * hb)) * u - uh;
+                    uint64_t pb = (uint64_t)(rank * hb + 16 * grp) * u + uh;
                     if (twice) {
                         pa <<= 1;
                         pb <<= 1;
                         e1 = csquare(e1);
                         E = csquare(E);
                     }
-                    if (uses > 0) ok = ok && tc::mbar_wait(&empty[set], (uses - 1) & 1);
-                    ++uses;
+                    const uint32_t si = it + set, buf = si % kBufs, use = si / kBufs;
+                    if (use > 0) ok = ok && tc::mbar_wait(&empty[buf], (use - 1) & 1);
+                    unsigned char* const Ah = stages + buf * kStageBytes + lane * 16;
                     {
                         float2 z = turn_cos_sin(pa);
                         z.x *= y;
@@ -382,25 +400,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
                         for (int i = 0; i < 4; ++i) p[i] = mul_pair(p[i], E8);
                         store_group(p, re + kSbo, re + kSbo + kAbytes, im + kSbo, im + kSbo + kAbytes);
                     }
-                    if (32 * grp < nb) {
+                    if (16 * grp < hb) {
                         const float2 e2 = csquare(e1), e4 = csquare(e2), e8 = csquare(e4);
                         Pair p[4];
                         powers8(turn_cos_sin(pb), e1, e2, e4, p);
-                        unsigned char* co = Bh + 4 * grp * kSbo;
-                        unsigned char* si = co + (nb >> 3) * kSbo;
-                        store_group(p, co, co + kBbytes, si, si + kBbytes);
-                        for (int b = 32 * grp + 8; b < min(nb, 32 * grp + 32); b += 8) {
-                            co += kSbo;
-                            si += kSbo;
+                        unsigned char* co = Ah + 2 * kAbytes + 2 * grp * kSbo;
+                        unsigned char* sn = co + (hb >> 3) * kSbo;
+                        store_group(p, co, co + kBbytes, sn, sn + kBbytes);
+                        if (16 * grp + 8 < hb) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) p[i] = mul_pair(p[i], e8);
-                            store_group(p, co, co + kBbytes, si, si + kBbytes);
+                            store_group(p, co + kSbo, co + kSbo + kBbytes, sn + kSbo, sn + kSbo + kBbytes);
                         }
                     }
                     tc::fence_operands();
                     __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(&filled[set]);
+                    if (lane == 0) tc::mbar_arrive_first(&filled[buf]);
                 }
+                it += (uint32_t)((min(left - m, kTcUnit) + kStage - 1) / kStage);
                 if (m > 0) drain(group - 1);
                 if (m > 0 && (m / kTcUnit) % kRunUnits == 0) {
                     flush(m / kTcUnit > kRunUnits);
@@ -413,30 +430,31 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) 
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
     }
-    // every MMA has been waited for with its unit
+    // every MMA has been waited for with its unit, by both CTAs
     if (!ok && a.status) atomicOr(a.status, kStatusWait);
     tc::fence_before_sync();
     __syncthreads();
+    tc::pair_sync();
     if (warp == 0) tc::tmem_free(tb, 512);
 }
 
-// The slots of a tile's pieces, in CTA order (the CTAs that got at least one
-// unit of it), and their number; every thread of the CTA calls it.
+// The slots of a tile's pieces, in order (the pairs that got at least one unit
+// of it), and their number; every thread of the CTA calls it.
 struct Pieces {
     int n;
-    int slot[kTcMaxCtas];
+    int slot[kTcMaxPairs];
 };
 
 __device__ void find_pieces(const TcArgs& a, int tile, int64_t n, int cols, Pieces& out) {
     const int64_t units = (n + kTcUnit - 1) / kTcUnit, c = tc_unit_cost(cols);
     const int64_t p = a.tiles ? a.pre[tile] : (int64_t)tile * units * c;
-    const int i0 = tc_cta_of(a.work, a.ctas, p), i1 = tc_cta_of(a.work, a.ctas, p + (units - 1) * c);
+    const int i0 = tc_pair_of(a.work, a.pairs, p), i1 = tc_pair_of(a.work, a.pairs, p + (units - 1) * c);
     if (threadIdx.x < 32) {
         int at = 0;
         for (int i = i0; i <= i1; i += 32) {
             const int me = i + (int)threadIdx.x;
             int64_t u0 = 0, u1 = 0;
-            if (me <= i1) tc_units(p, units, c, tc_bound(a.work, a.ctas, me), tc_bound(a.work, a.ctas, me + 1), &u0, &u1);
+            if (me <= i1) tc_units(p, units, c, tc_bound(a.work, a.pairs, me), tc_bound(a.work, a.pairs, me + 1), &u0, &u1);
             const unsigned has = __ballot_sync(0xffffffffu, u0 < u1);
             if (u0 < u1) out.slot[at + __popc(has & ((1u << threadIdx.x) - 1u))] = tile + me;
             at += __popc(has);
@@ -449,12 +467,12 @@ __device__ void find_pieces(const TcArgs& a, int tile, int64_t n, int cols, Piec
 // entries each, the pieces added in order with compensated FP32 sums; four
 // pieces of every tile are loaded before any of them is added.
 template <int S>
-__device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces (&q)[S], int nb, int ra, int rb,
+__device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces (&q)[S], int hb, int half, int ra, int rb,
                                           float2 (&plus)[S], float2 (&minus)[S]) {
     float s[S][4] = {}, c[S][4] = {};
-    // sum y (Re A, Im A) cos, then sin
-    const size_t at[4] = {(size_t)rb * 128 + ra, (size_t)rb * 128 + 64 + ra, (size_t)(nb + rb) * 128 + ra,
-                          (size_t)(nb + rb) * 128 + 64 + ra};
+    // sum y (Re A, Im A) cos, then sin; columns: cos, sin of the first CTA's hb offsets, then of the second's
+    const size_t co = (size_t)(rb < hb ? rb : hb + rb) * 128 + (size_t)half * (size_t)(a.slot_floats / 2) + ra;
+    const size_t at[4] = {co, co + 64, co + (size_t)hb * 128, co + (size_t)hb * 128 + 64};
     int most = q[0].n;
 #pragma unroll
     for (int x = 1; x < S; ++x) most = max(most, q[x].n);
@@ -541,15 +559,16 @@ __device__ __forceinline__ void direct_gls(const TcArgs& a, int64_t b, int64_t n
 }
 
 constexpr int kFinB = 4;  // fine offsets of one finalize CTA
-constexpr int kFinThreads = kTcRows * kFinB;
+constexpr int kFinRows = kTcRows / 2;
+constexpr int kFinThreads = kFinRows * kFinB;
 
-// One CTA: a data tile's 64 coarse frequencies x 4 fine offsets, both signs, a
+// One CTA: 64 of a data tile's coarse frequencies x 4 fine offsets, both signs, a
 // pair of frequencies a thread.  Reads run along the coarse frequencies
 // (contiguous in a slot); P is gathered in shared memory and written in runs of
 // 4 bins.
 template <int FORM>
 __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, const TcFinal f) {
-    __shared__ float sp[kTcRows][2 * kFinB + 1];
+    __shared__ float sp[kFinRows][2 * kFinB + 1];
     constexpr int S = FORM == kTcClassic ? 2 : 3;
     __shared__ Pieces q[S];
     __shared__ unsigned long long s_red[kFinThreads / 32];
@@ -557,7 +576,7 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
     int curve = 0, real = 0, fb, cols, td, tw, tcx;
     int64_t n, nf;
     if (a.tiles) {
-        td = f.data_tiles[blockIdx.x];
+        td = f.data_tiles[blockIdx.x >> 1];
         const TcTile w = a.tiles[td];
         curve = w.curve;
         real = w.real;
@@ -568,7 +587,7 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
         n = a.off[curve + 1] - a.off[curve];
         nf = f.nf[curve];
     } else {
-        td = (int)blockIdx.x;
+        td = (int)blockIdx.x >> 1;
         fb = a.fb0 + td;
         cols = a.cols;
         tw = td + a.nblk;
@@ -576,18 +595,18 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
         n = a.n0;
         nf = f.nf0;
     }
-    const int nb = cols >> 1;
+    const int nb = cols >> 1, half = (int)blockIdx.x & 1;
     const int b0 = (int)blockIdx.y * kFinB;
-    if (b0 >= nb) return;
-    const int64_t k0 = (int64_t)fb * kTcRows * cols;
+    const int64_t k0 = ((int64_t)fb * kTcRows + half * kFinRows) * cols;
+    if (b0 >= nb || k0 >= nf) return;
     find_pieces(a, td, n, cols, q[0]);
     find_pieces(a, tw, n, cols, q[1]);
     if constexpr (S > 2) find_pieces(a, tcx, n, cols, q[2]);
     __syncthreads();
-    const int ra = tid & (kTcRows - 1), bi = tid / kTcRows;
+    const int ra = tid & (kFinRows - 1), bi = tid / kFinRows;
     if (k0 + (int64_t)ra * cols < nf) {  // not a padding row
         float2 zp[S], zm[S];
-        tile_sums<S>(a, q, nb, ra, b0 + bi, zp, zm);
+        tile_sums<S>(a, q, nb >> 1, half, ra, b0 + bi, zp, zm);
         float vp, vm;
         if constexpr (FORM == kTcClassic) {
             vp = dev::periodogram_value2(zp[0].x, zp[0].y, zp[1].x, zp[1].y, (float)n);
@@ -622,7 +641,7 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
     float* P = f.P;
     if (P && f.P_off) P += (size_t)real * (size_t)f.P_total + f.P_off[curve];
     unsigned long long best = 0ull;
-    for (int x = tid; x < kTcRows * 2 * kFinB; x += kFinThreads) {
+    for (int x = tid; x < kFinRows * 2 * kFinB; x += kFinThreads) {
         const int r = x / (2 * kFinB), i = x % (2 * kFinB);
         const int fine = i < kFinB ? nb - b0 - kFinB + i : nb + b0 + (i - kFinB);
         const int64_t k = k0 + (int64_t)r * cols + fine;
@@ -726,9 +745,9 @@ __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs 
 
 }  // namespace
 
-cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, int sms, cudaStream_t st) {
+cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st) {
     if (a.off) {
-        tc_refine_kernel<1><<<2 * sms, kRefineThreads, 0, st>>>(a, f);
+        tc_refine_kernel<1><<<304, kRefineThreads, 0, st>>>(a, f);
         return cudaGetLastError();
     }
     cudaLaunchAttribute at;
@@ -747,15 +766,15 @@ cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, int sms, cudaStr
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(tc_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    tc_sums_kernel<<<a.ctas, kTcThreads, kSmem, st>>>(a);
+    tc_sums_kernel<<<2 * a.pairs, kTcThreads, kSmem, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st) {
     const int n_data = a.tiles ? f.n_data : a.nblk;
     if (n_data < 1) return cudaSuccess;
-    const int max_cols = (int)(a.slot_floats / 128);
-    dim3 grid((unsigned)n_data, (unsigned)((max_cols / 2 + kFinB - 1) / kFinB));
+    const int max_cols = (int)(a.slot_floats / tc_slot_floats(1));
+    dim3 grid((unsigned)n_data * 2u, (unsigned)((max_cols / 2 + kFinB - 1) / kFinB));
     if (form == kTcClassic) tc_final_kernel<kTcClassic><<<grid, kFinThreads, 0, st>>>(a, f);
     else tc_final_kernel<kTcGls><<<grid, kFinThreads, 0, st>>>(a, f);
     return cudaGetLastError();

@@ -26,18 +26,19 @@ struct TcTile {
     int32_t curve, real, fblock, kind, wtile, ctile, cols, pad;
 };
 
-constexpr int kTcRows = 64;        // coarse frequencies of a tile (128 operand rows: real and imaginary parts)
+constexpr int kTcRows = 128;       // coarse frequencies of a tile (real and imaginary parts: 128 operand rows a CTA)
 constexpr int kTcMaxCols = 256;    // fine offsets of a tile, at most
 constexpr int kTcUnit = 128;       // samples of one unit of work
 constexpr int kTcThreads = 640;
-constexpr int kTcMaxCtas = 512;   // CTAs (one per SM) that a launch is split over, at most
+constexpr int kTcMaxPairs = 256;  // CTA pairs that a launch is split over, at most
 
-// Cost of a unit of a tile, in sixteenths of the columns: the MMA time is
-// proportional to the columns above 144 and constant (75 cycles) below.
-__host__ __device__ inline int tc_unit_cost(int cols) { return (cols > 144 ? cols : 144) / 16; }
+// Cost of a unit of a tile: the operands (64 complex values a sample for a CTA's
+// coarse frequencies and cols / 4 for its fine offsets) take longer than the MMAs
+// (proportional to cols) below 256 columns.
+__host__ __device__ inline int tc_unit_cost(int cols) { return 8 + cols / 32; }
 
 // Fine offsets per coarse frequency for a grid of N_f bins: the number of
-// blocks (of 64 coarse frequencies) and columns (a multiple of 16, 32 .. 256)
+// blocks (of 128 coarse frequencies) and columns (a multiple of 32 up to 256)
 // whose cost is least.
 __host__ __device__ inline int tc_cols(int64_t N_f) {
     const int64_t b0 = (N_f + kTcRows * kTcMaxCols - 1) / (kTcRows * kTcMaxCols);
@@ -45,8 +46,7 @@ __host__ __device__ inline int tc_cols(int64_t N_f) {
     int64_t best_cost = INT64_MAX;
     for (int64_t b = b0 < 1 ? 1 : b0; b <= b0 + 2; ++b) {
         const int64_t per = (N_f + b * kTcRows - 1) / (b * kTcRows);
-        int c = (int)((per + 15) / 16 * 16);
-        if (c < 32) c = 32;
+        const int c = per > 32 ? (int)((per + 31) / 32 * 32) : 32;
         const int64_t blocks = (N_f + (int64_t)c * kTcRows - 1) / ((int64_t)c * kTcRows);
         const int64_t cost = blocks * tc_unit_cost(c);
         if (cost < best_cost) {
@@ -67,7 +67,7 @@ struct TcArgs {
     int kinds[3];
     int64_t n0;                 // samples of the single curve
     int64_t work;               // total cost
-    int ctas;                   // CTAs the work is split over
+    int pairs;                  // CTA pairs the work is split over
     const int64_t* off;         // curves' sample offsets (list form)
     const uint4* recA;
     const float4* recB;
@@ -76,17 +76,21 @@ struct TcArgs {
     const float* qmax;          // largest q of each curve
     const float* xr;            // realization rows
     int64_t total;              // row stride of xr
-    float* part;                // slots of slot_floats: tile t's piece by CTA i is slot t + i
-    int64_t slot_floats;
+    float* part;                // slots of slot_floats: tile t's piece by pair i is slot t + i, the halves of its
+    int64_t slot_floats;        // two CTAs one after the other, each [cols][128 rows]
     int* status;
 };
 
-// Where the work coordinate of CTA i starts.
-__host__ __device__ inline int64_t tc_bound(int64_t work, int ctas, int i) { return work * i / ctas; }
-// The CTA whose range holds coordinate x.
-__host__ __device__ inline int tc_cta_of(int64_t work, int ctas, int64_t x) {
-    return (int)(((x + 1) * ctas - 1) / work);
+// Where the work coordinate of pair i starts.
+__host__ __device__ inline int64_t tc_bound(int64_t work, int pairs, int i) { return work * i / pairs; }
+// The pair whose range holds coordinate x.
+__host__ __device__ inline int tc_pair_of(int64_t work, int pairs, int64_t x) {
+    return (int)(((x + 1) * pairs - 1) / work);
 }
+// Floats of a slot for tiles of up to cols columns.
+__host__ __device__ inline int64_t tc_slot_floats(int cols) { return 256 * (int64_t)cols; }
+// Pairs on a GPU of `sms` SMs.
+inline int tc_pairs(int sms) { return sms < 2 ? 1 : sms / 2 < kTcMaxPairs ? sms / 2 : kTcMaxPairs; }
 // Units [u0, u1) of a tile that starts at coordinate p (n units of cost c each)
 // whose starts lie in [lo, hi).
 __host__ __device__ inline void tc_units(int64_t p, int64_t n, int64_t c, int64_t lo, int64_t hi, int64_t* u0,
@@ -125,6 +129,6 @@ enum : int { kTcClassic = 0, kTcGls = 1 };
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st);
 cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st);
 // Floating mean: the listed bins, after every launch_tc_final of the call.
-cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, int sms, cudaStream_t st);
+cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st);
 
 }  // namespace lsp
