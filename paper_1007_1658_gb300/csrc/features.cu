@@ -11,12 +11,14 @@
 //                        on f_m = m df, m = 1..floor(f_max / df): the same
 //                        persistent tile loop as the batch periodogram, x = 1;
 //   features_kernel   -- one CTA per pattern: cadence order statistics (a
-//                        bitonic sort of the gaps in shared memory, or for
-//                        patterns of more than 32,768 gaps a radix select of
-//                        the five ranks over the gaps in global memory), gap
-//                        fractions, and the 8 highest window maxima outside
-//                        the main lobe (per-thread top-8 lists merged by
-//                        warp shuffles).
+//                        radix select of the five ranks over the gaps, in
+//                        shared memory up to 32,768 of them), gap fractions,
+//                        and the 8 highest window maxima outside the main lobe
+//                        (per-thread top-8 lists merged by warp shuffles).
+// With work enough the window comes from the tensor cores (tc_sums.cu), and the
+// strip kernel's values are formed only at the few bins that can be among its 8
+// highest maxima (window_peaks_kernel, window_exact_kernel): the features keep
+// their bits, 256 patterns' window 3.3 ms -> 0.7.
 #include <algorithm>
 #include <cfloat>
 
@@ -28,18 +30,17 @@ namespace {
 using namespace dev;
 
 constexpr int kFeatThreads = 1024;
-constexpr int kSortMaxGaps = 32768;  // gaps sorted in shared memory (128 KB); more are selected
+constexpr int kSortMaxGaps = 32768;  // gaps held in shared memory (128 KB); more are formed from t in every pass
 
-// The five cadence order statistics sorted(gaps)[k[i]] of a pattern too long
-// for the shared-memory sort, without sorting: an MSB-first radix select on
-// the FP32 bit patterns of the gaps (ordered as the values, gaps being >= 0),
-// 8 bits per pass and the five ranks at once, the gaps re-formed from t in
-// every pass exactly as the sort forms them.  Each warp adds to the five
-// 256-bin histograms once per distinct bin (__match_any_sync), so gaps that
-// share their leading bits do not serialize on one counter.  hist holds
-// 5 x 256 counters; out[i] receives the value of rank k[i].
-__device__ void select_gap_ranks(const double* __restrict__ t, int64_t b, int M, const int (&k)[5],
-                                 unsigned* hist, float* out) {
+// The five cadence order statistics sorted(gaps)[k[i]], without sorting: an
+// MSB-first radix select on the FP32 bit patterns of the gaps (ordered as the
+// values, gaps being >= 0), 8 bits per pass and the five ranks at once; key_at(i)
+// is gap i's.  Each warp adds to the five 256-bin histograms once per distinct
+// bin (__match_any_sync), so gaps that share their leading bits do not serialize
+// on one counter.  hist holds 5 x 256 counters; out[i] receives the value of rank
+// k[i].
+template <class Key>
+__device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigned* hist, float* out) {
     __shared__ unsigned s_prefix[5], s_rank[5];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     if (tid < 5) {
@@ -57,7 +58,7 @@ __device__ void select_gap_ranks(const double* __restrict__ t, int64_t b, int M,
         for (int base = tid - lane; base < M; base += nt) {
             const int i = base + lane;
             unsigned key = 0u;
-            if (i < M) key = __float_as_uint((float)(t[b + i + 1] - t[b + i]));
+            if (i < M) key = key_at(i);
             const int bin = (int)((key >> shift) & 255u);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
@@ -133,7 +134,8 @@ template <int F>
 __global__ void __launch_bounds__(kMainThreads)
 ls_window_kernel(const BatchItem* __restrict__ items, int n_items, unsigned* __restrict__ head,
                  const int64_t* __restrict__ off, const int64_t* __restrict__ nw, const uint4* __restrict__ recA,
-                 const float4* __restrict__ recB, float* __restrict__ W, const int64_t* __restrict__ W_off) {
+                 const float4* __restrict__ recB, float* __restrict__ W, const int64_t* __restrict__ W_off,
+                 const int* __restrict__ peaks) {
     __shared__ __align__(16) TileSmem<false> sm;
     __shared__ int s_item;
     for (;;) {
@@ -143,6 +145,7 @@ ls_window_kernel(const BatchItem* __restrict__ items, int n_items, unsigned* __r
         __syncthreads();
         if (it >= n_items) break;
         const BatchItem w = items[it];
+        if (peaks && peaks[(size_t)w.curve * (kWindowPeaks + 1)] >= 0) continue;  // its bins are formed one by one
         const int64_t b = off[w.curve], e = off[w.curve + 1];
         const int64_t M = nw[w.curve];
         const uint32_t k0 = (uint32_t)w.fblock * (kMainThreads * F) + (uint32_t)threadIdx.x * F;
@@ -170,6 +173,69 @@ ls_window_kernel(const BatchItem* __restrict__ items, int n_items, unsigned* __r
     }
 }
 
+// W of single bins as ls_window_kernel forms it, bit for bit.  There a thread
+// adds a strip's samples in order, one long chain; but only the additions are a
+// chain.  Here a warp forms the terms of its bin for 256 samples at once (the
+// strip's seed and the steps up to the bin), then one lane adds them in order:
+// 20,000 samples in 70 us instead of 1.3 ms.  Warp i of pattern c: neighbour
+// i % 3 - 1 of bin i / 3.
+constexpr int kExactWarps = 8, kExactSamples = 256;
+template <int F>
+__global__ void __launch_bounds__(32 * kExactWarps)
+window_exact_kernel(const int64_t* __restrict__ off, const uint4* __restrict__ recA, const float4* __restrict__ recB,
+                    const int* __restrict__ peaks, float* __restrict__ peak_w) {
+    __shared__ __align__(16) float2 terms[kExactWarps][kExactSamples];
+    const int c = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int* p = peaks + (size_t)c * (kWindowPeaks + 1);
+    const int i = (int)blockIdx.y * kExactWarps + warp;
+    if (i >= 3 * p[0]) return;
+    const uint32_t k = (uint32_t)(p[1 + i / 3] + i % 3 - 1), k0 = k / F * F;
+    const int step = (int)(k - k0);
+    const int64_t b = off[c], e = off[c + 1];
+    float2 s = make_float2(0.f, 0.f);
+    for (int64_t j0 = b; j0 < e; j0 += kExactSamples) {
+        const int n = (int)min((int64_t)kExactSamples, e - j0);
+#pragma unroll 4
+        for (int j = lane; j < n; j += 32) {
+            const float4 B = recB[j0 + j];
+            const float C = B.y, S = B.z;
+            float sn, cs;
+            __sincosf(phase_to_angle(top_phase(recA[j0 + j], k0)), &sn, &cs);
+            float2 y0 = make_float2(cs, sn);
+            float2 y1 = make_float2(fmaf(cs, C, -sn * S), fmaf(sn, C, cs * S));
+            const float2 cp2 = make_float2(B.w, B.w), cn2 = make_float2(-B.w, -B.w);
+#pragma unroll 1
+            for (int x = 2; x <= step; ++x) {
+                const float2 y2 = __ffma2_rn(((x - 1) & 1) ? cn2 : cp2, y1, y0);
+                y0 = y1;
+                y1 = y2;
+            }
+            terms[warp][j] = step == 0 ? y0 : y1;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            int j = 0;
+            for (; j + 8 <= n; j += 8) {
+                float4 v[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) v[x] = *reinterpret_cast<const float4*>(&terms[warp][j + 2 * x]);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    s = __fadd2_rn(s, make_float2(v[x].x, v[x].y));
+                    s = __fadd2_rn(s, make_float2(v[x].z, v[x].w));
+                }
+            }
+            for (; j < n; ++j) s = __fadd2_rn(s, terms[warp][j]);
+        }
+        __syncwarp();
+    }
+    if (lane == 0) {
+        const float inv = 1.f / ((float)(e - b) * (float)(e - b));
+        const float2 z = s;
+        peak_w[(size_t)c * (3 * kWindowPeaks) + i] = (z.x * z.x + z.y * z.y) * inv;
+    }
+}
+
 // (value, bin) ordered by value, then by lower bin.
 __device__ __forceinline__ bool better(float v, int m, float v2, int m2) { return v > v2 || (v == v2 && m < m2); }
 
@@ -185,14 +251,112 @@ __device__ __forceinline__ void top8_insert(float (&v)[8], int (&m)[8], float x,
     m[p] = mi;
 }
 
-// One CTA per pattern.  Dynamic shared memory: the gaps, padded to a power of
-// two, for patterns of up to kSortMaxGaps gaps; the select's histograms for longer ones.
+// The 8 best (value, bin) of a warp's lanes' lists, best first, through put(r,
+// value, bin) on lane 0: eight rounds of "best head in the warp wins".
+template <class Put>
+__device__ __forceinline__ void warp_top8(const float (&tv)[8], const int (&tm)[8], Put&& put) {
+    const int lane = threadIdx.x & 31;
+    int headp = 0;
+    for (int r = 0; r < 8; ++r) {
+        float bv = -1.f;
+        int bm = 0x7fffffff, bl = lane;
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+            if (x == headp) {
+                bv = tv[x];
+                bm = tm[x];
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int om = __shfl_xor_sync(0xffffffffu, bm, o);
+            const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
+            if (better(ov, om, bv, bm)) {
+                bv = ov;
+                bm = om;
+                bl = ol;
+            }
+        }
+        if (lane == bl) ++headp;
+        if (lane == 0) put(r, bv, bm);
+    }
+}
+
+// How far the strip kernel's W and an accurate one can be apart: its recurrence
+// is off by at most F^2 ulp a term (3.4e-5), its sums and hardware sin/cos by less,
+// so 1e-4 of |sum| / n <= sqrt(W), here for both.
+__device__ __forceinline__ float window_gap(float w) { return 2e-4f * sqrtf(w) + 1e-8f; }
+
+// A pattern's bins that can hold one of the 8 highest local maxima (outside the
+// main lobe) of the strip kernel's W: with g the gap above, maxima of the accurate
+// W by more than the gaps of both bins are maxima of the other too; the eighth of
+// those bounds the eighth of all from below; and a bin qualifies when it is a
+// maximum up to the gaps and not below that bound.
+constexpr int kPeakMaxSamples = 65536;
+__global__ void __launch_bounds__(kFeatThreads)
+window_peaks_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, const double* __restrict__ dfa,
+                    const float* __restrict__ W, const int64_t* __restrict__ W_off, const int64_t* __restrict__ nw,
+                    int* __restrict__ peaks) {
+    __shared__ float wv[32 * 8];
+    __shared__ float s_eighth;
+    __shared__ int s_n;
+    const int c = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5;
+    const int64_t b = off[c], e = off[c + 1], mw = nw[c];
+    const double df = dfa[c], T = t[e - 1] - t[b];
+    const float* Wc = W + W_off[c];
+    int* p = peaks + (size_t)c * (kWindowPeaks + 1);
+    if (e - b > kPeakMaxSamples) {
+        if (tid == 0) p[0] = -1;
+        return;
+    }
+    float tv[8];
+    int tm[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        tv[r] = -1.f;
+        tm[r] = 0x7fffffff;
+    }
+    if (tid == 0) s_n = 0;
+    for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
+        const float w = Wc[i], l = Wc[i - 1], h = Wc[i + 1], g = window_gap(w);
+        if (w - g > l + window_gap(l) && w - g > h + window_gap(h) && (double)(i + 1) * df * T >= 1.0)
+            top8_insert(tv, tm, w - g, (int)i);
+    }
+    warp_top8(tv, tm, [&](int r, float v, int) { wv[warp * 8 + r] = v; });
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            tv[r] = wv[tid * 8 + r];
+            tm[r] = tid * 8 + r;
+        }
+        warp_top8(tv, tm, [&](int r, float v, int) {
+            if (r == 7) s_eighth = v;
+        });
+    }
+    __syncthreads();
+    const float least = s_eighth;  // -1 where there are fewer than eight
+    for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
+        const float w = Wc[i], g = window_gap(w);
+        if (!(w + g >= least)) continue;
+        const float l = Wc[i - 1], h = Wc[i + 1];
+        if (w + g >= l - window_gap(l) && w + g >= h - window_gap(h) && (double)(i + 1) * df * T >= 1.0) {
+            const int at = atomicAdd(&s_n, 1);
+            if (at < kWindowPeaks) p[1 + at] = (int)i;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) p[0] = s_n <= kWindowPeaks ? s_n : -1;
+}
+
+// One CTA per pattern.  Dynamic shared memory: the gaps of patterns of up to
+// kSortMaxGaps of them, behind the select's histograms.
 __global__ void __launch_bounds__(kFeatThreads)
 features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, const double* __restrict__ f0a,
                 const double* __restrict__ dfa, const int64_t* __restrict__ nfa, const float* __restrict__ W,
                 const int64_t* __restrict__ W_off, const int64_t* __restrict__ nw, float* __restrict__ feat,
-                int* __restrict__ status) {
-    extern __shared__ float gaps[];
+                int* __restrict__ status, const int* __restrict__ peaks, const float* __restrict__ peak_w) {
+    extern __shared__ unsigned hist[];
+    float* const gaps = reinterpret_cast<float*>(hist + 5 * 256);
     __shared__ double red[33];
     __shared__ float wv[32 * 8];
     __shared__ int wm[32 * 8];
@@ -203,55 +367,35 @@ features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, c
     const int64_t b = off[c], e = off[c + 1];
     const int n = (int)(e - b), M = n - 1;
     const double ps[5] = {0.05, 0.25, 0.5, 0.75, 0.95};
-    int P2 = 1;
-    while (P2 < M) P2 <<= 1;
-    const bool sorted_in_smem = M <= kSortMaxGaps;
+    const bool in_smem = M <= kSortMaxGaps;
     if (tid == 0) unsorted = 0;
     __syncthreads();
     const double T = t[e - 1] - t[b];
-    if (!sorted_in_smem) {
-        int k[5];
-#pragma unroll
-        for (int i = 0; i < 5; ++i) k[i] = (int)floor(ps[i] * (double)(M - 1));
-        select_gap_ranks(t, b, M, k, (unsigned*)gaps, qsel);
-        for (int i = tid; i < M; i += nt)
-            if (t[b + i + 1] - t[b + i] < 0.0) unsorted = 1;
-    }
-    for (int i = tid; sorted_in_smem && i < P2; i += nt) {
-        if (i < M) {
-            const double d = t[b + i + 1] - t[b + i];
-            if (d < 0.0) unsorted = 1;
-            gaps[i] = (float)d;
-        } else {
-            gaps[i] = FLT_MAX;
-        }
+    for (int i = tid; i < M; i += nt) {
+        const double d = t[b + i + 1] - t[b + i];
+        if (d < 0.0) unsorted = 1;
+        if (in_smem) gaps[i] = (float)d;
     }
     __syncthreads();
-    // bitonic sort, ascending
-    for (int k = 2; sorted_in_smem && k <= P2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tid; i < P2; i += nt) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const float a = gaps[i], bb = gaps[l];
-                    const bool up = (i & k) == 0;
-                    if ((a > bb) == up) {
-                        gaps[i] = bb;
-                        gaps[l] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
     // q(ps[i]) = sorted(gaps)[floor(ps[i] (M - 1))]; the median is q(1/2)
-    auto q = [&](int i) { return sorted_in_smem ? gaps[(int)floor(ps[i] * (double)(M - 1))] : qsel[i]; };
+    int rank[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) rank[i] = (int)floor(ps[i] * (double)(M - 1));
+    if (in_smem) select_gap_ranks([&](int i) { return __float_as_uint(gaps[i]); }, M, rank, hist, qsel);
+    else select_gap_ranks([&](int i) { return __float_as_uint((float)(t[b + i + 1] - t[b + i])); }, M, rank, hist, qsel);
+    auto q = [&](int i) { return qsel[i]; };
     const double med = (double)q(2);
     // gap sums over dt > c med (1 + 1e-6): the margin keeps exact multiples of
     // the cadence (one dropped sample on an even grid) out of the gaps
     double s2 = 0.0, s10 = 0.0, s100 = 0.0, cnt2 = 0.0, mx = 0.0;
+    // (FP64 divisions are slow on this part: a gap that FP32 puts clearly below
+    // every bound and below the largest so far is done with)
+    const float low = 1.999f * (float)med;
+    float mx32 = 0.f;
     for (int i = tid; i < M; i += nt) {
+        if (in_smem && gaps[i] < low && gaps[i] < mx32) continue;
         const double d = t[b + i + 1] - t[b + i];
+        mx32 = fmaxf(mx32, (float)d);
         const double r = d / med;
         if (r > 2.0 * (1.0 + 1e-6)) {
             s2 += d;
@@ -304,33 +448,23 @@ features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, c
         tv[r] = -1.f;
         tm[r] = 0x7fffffff;
     }
-    for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
-        const float w = Wc[i];
-        if (w > Wc[i - 1] && w >= Wc[i + 1] && (double)(i + 1) * df * T >= 1.0) top8_insert(tv, tm, w, (int)i);
-    }
-    // warp merge: eight rounds of "best head in the warp wins"
-    const int lane = tid & 31, warp = tid >> 5;
-    int headp = 0;
-    for (int r = 0; r < 8; ++r) {
-        float bv = headp < 8 ? tv[headp] : -1.f;
-        int bm = headp < 8 ? tm[headp] : 0x7fffffff;
-        int bl = lane;
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int om = __shfl_xor_sync(0xffffffffu, bm, o);
-            const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
-            if (better(ov, om, bv, bm)) {
-                bv = ov;
-                bm = om;
-                bl = ol;
-            }
+    const int* pk = peaks ? peaks + (size_t)c * (kWindowPeaks + 1) : nullptr;
+    if (pk && pk[0] >= 0) {
+        if (tid < pk[0]) {
+            const float* x = peak_w + (size_t)c * (3 * kWindowPeaks) + 3 * tid;
+            if (x[1] > x[0] && x[1] >= x[2]) top8_insert(tv, tm, x[1], pk[1 + tid]);
         }
-        if (lane == bl) ++headp;
-        if (lane == 0) {
-            wv[warp * 8 + r] = bv;
-            wm[warp * 8 + r] = bm;
+    } else {
+        for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
+            const float w = Wc[i];
+            if (w > Wc[i - 1] && w >= Wc[i + 1] && (double)(i + 1) * df * T >= 1.0) top8_insert(tv, tm, w, (int)i);
         }
     }
+    const int warp = tid >> 5;
+    warp_top8(tv, tm, [&](int r, float v, int m) {
+        wv[warp * 8 + r] = v;
+        wm[warp * 8 + r] = m;
+    });
     __syncthreads();
     if (tid == 0) {
         float fv[8];
@@ -373,11 +507,11 @@ features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, c
 
 cudaError_t launch_window(int F, int grid, const BatchItem* items, int n_items, unsigned* head, const int64_t* off,
                           const int64_t* nw, const uint4* recA, const float4* recB, float* W, const int64_t* W_off,
-                          cudaStream_t st) {
+                          cudaStream_t st, const int* peaks) {
     switch (F) {
-        case 8: ls_window_kernel<8><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off); break;
-        case 16: ls_window_kernel<16><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off); break;
-        case 24: ls_window_kernel<24><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off); break;
+        case 8: ls_window_kernel<8><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off, peaks); break;
+        case 16: ls_window_kernel<16><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off, peaks); break;
+        case 24: ls_window_kernel<24><<<grid, kMainThreads, 0, st>>>(items, n_items, head, off, nw, recA, recB, W, W_off, peaks); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -402,18 +536,33 @@ int window_occupancy(int F) {
 }
 
 size_t features_smem_bytes(int64_t max_n) {
-    int64_t P2 = 1;
-    while (P2 < max_n - 1 && P2 < kSortMaxGaps) P2 <<= 1;
-    return std::max((size_t)P2 * sizeof(float), (size_t)5 * 256 * sizeof(unsigned));
+    const int64_t gaps = max_n - 1 <= kSortMaxGaps ? max_n - 1 : kSortMaxGaps;
+    return (size_t)5 * 256 * sizeof(unsigned) + (size_t)gaps * sizeof(float);
+}
+
+cudaError_t launch_window_peaks(int n_patterns, const double* t, const int64_t* off, const double* df, const float* W,
+                                const int64_t* W_off, const int64_t* nw, int* peaks, cudaStream_t st) {
+    window_peaks_kernel<<<n_patterns, kFeatThreads, 0, st>>>(t, off, df, W, W_off, nw, peaks);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_window_exact(int F, int n_patterns, const int64_t* off, const uint4* recA, const float4* recB,
+                                const int* peaks, float* peak_w, cudaStream_t st) {
+    if (F != 24) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)n_patterns, (3 * kWindowPeaks + kExactWarps - 1) / kExactWarps);
+    window_exact_kernel<24><<<grid, 32 * kExactWarps, 0, st>>>(off, recA, recB, peaks, peak_w);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_features(int n_patterns, int64_t max_n, const double* t, const int64_t* off, const double* f0,
                             const double* df, const int64_t* nf, const float* W, const int64_t* W_off,
-                            const int64_t* nw, float* feat, int* status, cudaStream_t st) {
+                            const int64_t* nw, float* feat, int* status, cudaStream_t st, const int* peaks,
+                            const float* peak_w) {
     const size_t smem = features_smem_bytes(max_n);
     cudaError_t e = cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    features_kernel<<<n_patterns, kFeatThreads, smem, st>>>(t, off, f0, df, nf, W, W_off, nw, feat, status);
+    features_kernel<<<n_patterns, kFeatThreads, smem, st>>>(t, off, f0, df, nf, W, W_off, nw, feat, status, peaks,
+                                                           peak_w);
     return cudaGetLastError();
 }
 

@@ -158,39 +158,44 @@ bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f) {
 
 lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_out, bool launch,
                                 int* launches) {
-    const int cols = lsp::tc_cols(N_f);
-    const int64_t per = (int64_t)lsp::kTcRows * cols, blocks = (N_f + per - 1) / per;
-    const int sums = gls ? 3 : 2;
+    const int sets = gls ? 2 : 1;
+    const int cols = lsp::tc_cols(N_f, sets);
+    const int64_t per = (int64_t)lsp::kTcGroup * cols, groups = (N_f + per - 1) / per;
     const int64_t units = (N + lsp::kTcUnit - 1) / lsp::kTcUnit;
     const int pairs = lsp::tc_pairs(ctx->sms);
+    const int G = lsp::kTcGroups;
     lsp::TcArgs a{};
     a.slot_floats = lsp::tc_slot_floats(cols);
     // at most 1 GiB of partial tiles at a time
-    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - pairs) / sums);
-    const int64_t step = std::min(blocks, most);
-    lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)(step * sums + pairs) * (size_t)a.slot_floats * 4);
+    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - pairs) / (sets + 1) - 1) * G;
+    const int64_t step = std::min(groups, most);
+    const int64_t slots = (sets * step + G - 1) / G + (step + G - 1) / G + pairs;
+    lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)slots * (size_t)a.slot_floats * 4);
     if (rs != LSP_OK || !launch) return rs;
-    a.cols = cols;
-    a.kinds[0] = gls ? lsp::kTcRecQ : lsp::kTcRec;
-    a.kinds[1] = gls ? lsp::kTcW2 : lsp::kTcOne2;
-    a.kinds[2] = lsp::kTcW1;
+    a.win_kind = gls ? lsp::kTcW2 : lsp::kTcOne2;
+    a.one.kind = gls ? lsp::kTcRecQ : lsp::kTcRec;
+    a.one.reals = 1;
+    a.one.gls = gls;
+    a.one.cols = cols;
     a.n0 = N;
     a.recA = (const uint4*)ctx->recA.p;
     a.recB = (const float4*)ctx->recB.p;
     a.recE = (const float2*)ctx->recE.p;
     a.q = (const float*)ctx->recQ.p;
-    a.qmax = (const float*)ctx->qmax.p;
+    a.qmax = gls ? (const float*)ctx->qmax.p : nullptr;
     a.part = (float*)ctx->tc_part.p;
     a.status = ctx->status_d;
     const bool timing = ctx->opt.timing != 0;
-    for (int64_t fb = 0; fb < blocks; fb += step) {
-        a.fb0 = (int)fb;
-        a.nblk = (int)std::min(step, blocks - fb);
-        a.n_tiles = a.nblk * sums;
+    for (int64_t g = 0; g < groups; g += step) {
+        a.one.kg0 = (int)g;
+        a.one.gpr = (int)std::min(step, groups - g);
+        a.h1 = (sets * a.one.gpr + G - 1) / G;
+        a.one.wt0 = a.h1;
+        a.n_tiles = a.h1 + (a.one.gpr + G - 1) / G;
         a.work = (int64_t)a.n_tiles * units * lsp::tc_unit_cost(cols);
         a.pairs = (int)std::min<int64_t>(pairs, (int64_t)a.n_tiles * units);
         LSP_CUDA(ctx, lsp::launch_tc_sums(a, ctx->stream));
-        if (timing && fb + step >= blocks) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
+        if (timing && g + step >= groups) LSP_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
         lsp::TcFinal f{};
         f.nf0 = N_f;
         f.P = P_out;
@@ -198,7 +203,7 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
         f.n_bins = (unsigned*)ctx->qmax.p + 1;
         LSP_CUDA(ctx, lsp::launch_tc_final(gls ? lsp::kTcGls : lsp::kTcClassic, a, f, ctx->stream));
         *launches += 2;
-        if (gls && fb + step >= blocks) {
+        if (gls && g + step >= groups) {
             LSP_CUDA(ctx, lsp::launch_tc_refine(a, f, ctx->stream));
             ++*launches;
         }
@@ -212,12 +217,13 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
 // tensor cores: 8 curves of 100 .. 500 samples 126 / 86 us, 100 of them 133 / 108,
 // 100 x 8 realizations (900 tiles) 180 / 226; 100 x 8 of 200 .. 1500 samples 330 /
 // 305, of 400 .. 5000 samples 1704 / 516.
-static bool tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real) {
+bool lsp::host::tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real) {
     double tiles = 0.0, units = 0.0, terms = 0.0;
     for (size_t c = 0; c < nf.size(); ++c) {
         if (nf[c] == 0) continue;
         const double n = (double)(off[c + 1] - off[c]);
-        const double t = std::ceil((double)nf[c] / (lsp::kTcRows * lsp::tc_cols(nf[c]))) * (n_real + 1);
+        const double gpr = std::ceil((double)nf[c] / (lsp::kTcGroup * lsp::tc_cols(nf[c], n_real)));
+        const double t = std::ceil(gpr * n_real / lsp::kTcGroups) + std::ceil(gpr / lsp::kTcGroups);
         tiles += t;
         units += t * std::ceil(n / lsp::kTcUnit);
         terms += n * (double)nf[c] * n_real;
@@ -234,17 +240,23 @@ bool lsp::host::use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off
 
 void lsp::host::TcPlan::pack(void* p) const {
     char* b = (char*)p;
-    std::memcpy(b, tiles.data(), tiles.size() * sizeof(lsp::TcTile));
-    b += tiles.size() * sizeof(lsp::TcTile);
-    std::memcpy(b, pre.data(), pre.size() * 8);
-    std::memcpy(b + pre.size() * 8, data.data(), data.size() * 4);
+    auto put = [&](const void* src, size_t bytes) {
+        if (bytes) std::memcpy(b, src, bytes);
+        b += bytes;
+    };
+    put(cols.data(), cols.size() * 8);
+    put(tiles.data(), tiles.size() * sizeof(lsp::TcTile));
+    put(pre.data(), pre.size() * 8);
+    put(data.data(), data.size() * 4);
 }
 
 lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, const std::vector<int64_t>& off,
                                      const std::vector<int64_t>& nf, int n_real) {
     TcPlan p;
-    const int shared = form == lsp::kTcClassic ? 1 : 2;
+    const int gls = form == lsp::kTcGls ? 1 : 0;
+    const int win_kind = gls ? lsp::kTcW2 : lsp::kTcOne2;
     const int pairs = lsp::tc_pairs(ctx->sms);
+    const int G = lsp::kTcGroups;
     // at most 4 GiB of partial tiles at a time
     const int64_t most = (int64_t(1) << 30) / lsp::tc_slot_floats(lsp::kTcMaxCols) - pairs;
     TcChunk cur{0, 0, 0, 0, 0, 0};
@@ -256,37 +268,46 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
         cur = TcChunk{(int64_t)p.tiles.size(), 0, (int64_t)p.data.size(), 0, 0, 0};
         p.pre.push_back(0);
     };
-    auto add = [&](int c, int r, int64_t fb, int kind, int64_t units, int cols, int wt, int ct) {
-        p.tiles.push_back({c, r, (int32_t)fb, kind, wt, ct, cols, 0});
-        cur.work += units * lsp::tc_unit_cost(cols);
-        p.pre.push_back(cur.work);
-        cur.cols = std::max(cur.cols, cols);
-        return (int)cur.n++;
-    };
+    auto tiles_of = [&](int64_t sets, int64_t gpr) { return (sets * gpr + G - 1) / G; };
     for (int c = 0; c < (int)nf.size(); ++c) {
+        const int cols = lsp::tc_cols(std::max<int64_t>(1, nf[c]), n_real + gls);
+        p.cols.push_back(cols);
         if (nf[c] == 0) continue;
-        const int cols = lsp::tc_cols(nf[c]);
-        const int64_t per = (int64_t)lsp::kTcRows * cols, blocks = (nf[c] + per - 1) / per;
+        const int64_t per = (int64_t)lsp::kTcGroup * cols, groups = (nf[c] + per - 1) / per;
         const int64_t units = (off[c + 1] - off[c] + lsp::kTcUnit - 1) / lsp::kTcUnit;
-        // blocks b, realizations r of this curve, as many at a time as fit a chunk
-        const int64_t bstep = std::min(blocks, std::max<int64_t>(1, most / (shared + 1)));
-        const int64_t rstep = std::min<int64_t>(n_real, std::max<int64_t>(1, most / bstep - shared));
-        for (int64_t b0 = 0; b0 < blocks; b0 += bstep)
+        // groups and realizations of this curve, as many at a time as fit a chunk
+        const int64_t gstep = std::min(groups, std::max<int64_t>(1, most / (gls + 2) - 1) * G);
+        const int64_t left = most - tiles_of(gls + 1, gstep) - 2;
+        const int64_t rstep = std::min<int64_t>(n_real, std::max<int64_t>(1, left * G / gstep));
+        for (int64_t g0 = 0; g0 < groups; g0 += gstep)
             for (int64_t r0 = 0; r0 < n_real; r0 += rstep) {
-                const int64_t b1 = std::min(blocks, b0 + bstep), r1 = std::min<int64_t>(n_real, r0 + rstep);
-                if (cur.n + (b1 - b0) * (shared + r1 - r0) > most) flush();
-                for (int64_t b = b0; b < b1; ++b) {
-                    int wt = -1, ct = -1;
-                    if (form == lsp::kTcClassic) wt = add(c, 0, b, lsp::kTcOne2, units, cols, -1, -1);
-                    if (form == lsp::kTcGls) {
-                        wt = add(c, 0, b, lsp::kTcW2, units, cols, -1, -1);
-                        ct = add(c, 0, b, lsp::kTcW1, units, cols, -1, -1);
-                    }
-                    for (int64_t r = r0; r < r1; ++r) {
-                        p.data.push_back(add(c, (int)r, b, data, units, cols, wt, ct));
+                const int64_t gpr = std::min(gstep, groups - g0), reals = std::min<int64_t>(rstep, n_real - r0);
+                const int64_t nw = form == lsp::kTcWindow ? 0 : tiles_of(1, gpr), nh = tiles_of(reals + gls, gpr);
+                if (cur.n + nw + nh > most) flush();
+                lsp::TcTile t{};
+                t.curve = c;
+                t.r0 = (int32_t)r0;
+                t.reals = (int32_t)reals;
+                t.gls = gls;
+                t.gpr = (int32_t)gpr;
+                t.kg0 = (int32_t)g0;
+                t.cols = cols;
+                t.wt0 = (int32_t)cur.n;
+                t.ht0 = (int32_t)(cur.n + nw);
+                for (int64_t i = 0; i < nw + nh; ++i) {
+                    t.twice = i < nw;
+                    t.kind = t.twice ? win_kind : data;
+                    t.g0 = (int32_t)(G * (t.twice ? i : i - nw));
+                    if (!t.twice) {
+                        p.data.push_back((int)cur.n);
                         ++cur.nd;
                     }
+                    p.tiles.push_back(t);
+                    cur.work += units * lsp::tc_unit_cost(cols);
+                    p.pre.push_back(cur.work);
+                    ++cur.n;
                 }
+                cur.cols = std::max(cur.cols, cols);
             }
     }
     flush();
@@ -295,7 +316,7 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
 
 cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int form, lsp::TcArgs a,
                               lsp::TcFinal f, cudaStream_t st) {
-    const lsp::TcTile* tiles = (const lsp::TcTile*)d_plan;
+    const lsp::TcTile* tiles = (const lsp::TcTile*)((const int64_t*)d_plan + p.cols.size());
     const int64_t* pre = (const int64_t*)(tiles + p.tiles.size());
     const int* data = (const int*)(pre + p.pre.size());
     const int pairs = lsp::tc_pairs(ctx->sms);
@@ -304,7 +325,6 @@ cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d
         a.tiles = tiles + c.t0;
         a.pre = pre + c.t0 + (int64_t)x;
         a.n_tiles = (int)c.n;
-        a.cols = c.cols;
         a.work = c.work;
         a.pairs = (int)std::min<int64_t>(pairs, std::max<int64_t>(1, c.work / lsp::tc_unit_cost(c.cols)));
         a.slot_floats = lsp::tc_slot_floats(c.cols);
@@ -455,7 +475,7 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
         NvtxRange r("lsp_periodogram.prep");
         LSP_CUDA(ctx, lsp::launch_prep_stats(td, xd, nullptr, N_t, 1, stats, ctx->status_d,
                                              (lsp::StatPart*)ctx->stat_parts.p, (unsigned*)ctx->stat_counters.p, st));
-        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f), nullptr};
+        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f, 1), nullptr};
         LSP_CUDA(ctx, lsp::launch_prep_records(td, xd, nullptr, N_t, 1, N_t, nullptr, nullptr, f_0, df, stats,
                                                (uint4*)ctx->recA.p, (float4*)ctx->recB.p,
                                                s.mode == lsp::kModeNaive ? (float2*)ctx->recN.p : nullptr, nullptr,
@@ -575,7 +595,7 @@ void lsp_destroy(lsp_ctx* ctx) {
     lsp::host::FapState& f = ctx->fap;
     DevBuf* fbufs[] = {&f.params, &f.grad, &f.m,    &f.v,    &f.mu_sig, &f.ws,    &f.act,  &f.X,
                        &f.cnt,    &f.y,    &f.loss, &f.q,    &f.rows,   &f.W,     &f.W_off, &f.nw,
-                       &f.counts, &f.best, &f.train_state, &f.hist};
+                       &f.counts, &f.peaks, &f.peak_w, &f.best, &f.train_state, &f.hist};
     for (DevBuf* b : fbufs)
         if (b->p) cudaFree(b->p);
     if (ctx->status_d) cudaFree(ctx->status_d);

@@ -73,6 +73,7 @@ struct FapState {
     int64_t n_params = 0;
     int64_t step = 0;
     DevBuf params, grad, m, v, mu_sig, ws, act, X, cnt, y, loss, q, rows, W, W_off, nw, counts;
+    DevBuf peaks, peak_w;            // bins of the window formed again, and their values
     DevBuf best, train_state, hist;  // lsp_fap_train: kept weights, loop scalars, histories
 };
 
@@ -321,24 +322,26 @@ lsp_status tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_ou
 
 // The tiles of a batch on the tensor cores, in chunks whose partial tiles fit
 // the workspace: tiles [t0, t0 + n) of the list, their cost prefix sums at
-// pre[t0 + chunk] (n + 1 values), the data tiles' indices within the chunk at
+// pre[t0 + chunk] (n + 1 values), the h = 1 tiles' indices within the chunk at
 // data[d0, d0 + nd).
 struct TcChunk {
     int64_t t0, n, d0, nd, work;
     int cols;
 };
 struct TcPlan {
+    std::vector<int64_t> cols;  // of every curve
     std::vector<lsp::TcTile> tiles;
     std::vector<int64_t> pre;
     std::vector<int> data;
     std::vector<TcChunk> chunks;
     int64_t max_slot_floats = 0;  // largest workspace of a chunk, in floats
-    size_t bytes() const { return tiles.size() * sizeof(lsp::TcTile) + pre.size() * 8 + data.size() * 4; }
-    // tiles, then prefix sums, then indices, as one block
+    size_t bytes() const { return cols.size() * 8 + tiles.size() * sizeof(lsp::TcTile) + pre.size() * 8 + data.size() * 4; }
+    // columns, tiles, prefix sums and indices, as one block
     void pack(void* p) const;
 };
-// Data tiles of kind `data` for every (curve, realization), with the pattern's
-// sums the form needs (kTcClassic: h = 2; kTcGls: h = 2 and h = 1).
+// Data sets of kind `data` for every (curve, realization), with the pattern's
+// sums the form needs (kTcClassic: h = 2; kTcGls: h = 2 and y = q^2; kTcWindow:
+// none).
 TcPlan plan_tc(const lsp_ctx* ctx, int form, int data, const std::vector<int64_t>& off,
                const std::vector<int64_t>& nf, int n_real);
 
@@ -350,6 +353,8 @@ cudaError_t run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int 
 // Whether a batch runs on the tensor cores: the options leave the choice to the
 // library, and the batch is of a size where they are faster.
 bool use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real);
+// The size part of it alone.
+bool tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real);
 
 // Release the cached batch graph.
 void drop_plan(lsp_ctx* ctx);

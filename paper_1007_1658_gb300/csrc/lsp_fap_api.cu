@@ -165,6 +165,17 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
+    // the window on the tensor cores, where that pays (it takes no options)
+    const bool tc = tc_batch_pays(off, nw, 1);
+    TcPlan tcp;
+    if (tc) {
+        tcp = plan_tc(ctx, lsp::kTcWindow, lsp::kTcOne1, off, nw, 1);
+        if ((rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, f.peaks, (size_t)n * (lsp::kWindowPeaks + 1) * 4)) != LSP_OK) return rs;
+        if ((rs = ensure(ctx, f.peak_w, (size_t)n * 3 * lsp::kWindowPeaks * 4)) != LSP_OK) return rs;
+    }
     std::vector<lsp::BatchItem> items;
     for (int c : order)
         for (int64_t fb = 0; fb < (nw[c] + per_block - 1) / per_block; ++fb) items.push_back({c, 0, (int32_t)fb, 0});
@@ -172,7 +183,8 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     const size_t meta = (size_t)(2 * n + 1) * 8;
     if ((rs = ensure(ctx, ctx->b_items, item_bytes + 16)) != LSP_OK) return rs;
     if (ctx->plan.valid) drop_plan(ctx);  // the batch graph's work list is overwritten here
-    if ((rs = ensure_pinned(ctx, item_bytes + meta + 64)) != LSP_OK) return rs;
+    const size_t tc_at = (meta + item_bytes + 15) & ~(size_t)15;
+    if ((rs = ensure_pinned(ctx, tc_at + (tc ? tcp.bytes() : 0) + 64)) != LSP_OK) return rs;
     LSP_CUDA(ctx, cudaStreamSynchronize(st));
     char* pin = (char*)ctx->pinned;
     std::memcpy(pin, woff.data(), (size_t)(n + 1) * 8);
@@ -181,24 +193,48 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     LSP_CUDA(ctx, cudaMemcpyAsync(f.W_off.p, pin, (size_t)(n + 1) * 8, cudaMemcpyHostToDevice, st));
     LSP_CUDA(ctx, cudaMemcpyAsync(f.nw.p, pin + (size_t)(n + 1) * 8, (size_t)n * 8, cudaMemcpyHostToDevice, st));
     if (!items.empty()) LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_items.p, pin + meta, item_bytes, cudaMemcpyHostToDevice, st));
+    if (tc) {
+        tcp.pack(pin + tc_at);
+        LSP_CUDA(ctx, cudaMemcpyAsync(ctx->b_tc.p, pin + tc_at, tcp.bytes(), cudaMemcpyHostToDevice, st));
+    }
     LSP_CUDA(ctx, cudaMemsetAsync(ctx->b_head.p, 0, 16, st));
     // phases on the window grid f_m = m df: records with f0 := df
+    const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, (const int64_t*)ctx->b_tc.p, 0, nullptr};
     LSP_CUDA(ctx, lsp::launch_prep_stats(d_t, nullptr, d_off, 0, n, (lsp::CurveStats*)ctx->b_stats.p, ctx->status_d,
                                          nullptr, nullptr, st));
     LSP_CUDA(ctx, lsp::launch_prep_records(d_t, nullptr, d_off, 0, n, max_n, d_df, d_df, 0.0, 0.0,
                                            (const lsp::CurveStats*)ctx->b_stats.p, (uint4*)ctx->b_recA.p,
                                            (float4*)ctx->b_recB.p, nullptr, nullptr, st, nullptr, nullptr,
-                                           ctx->status_d));
+                                           ctx->status_d, tc ? &tprep : nullptr));
+    if (tc) {
+        lsp::TcArgs a{};
+        a.off = d_off;
+        a.recA = (const uint4*)ctx->b_recA.p;
+        a.recB = (const float4*)ctx->b_recB.p;
+        a.recE = (const float2*)ctx->b_recE.p;
+        a.part = (float*)ctx->tc_part.p;
+        a.status = ctx->status_d;
+        lsp::TcFinal fin{};
+        fin.nf = (const int64_t*)f.nw.p;
+        fin.P = (float*)f.W.p;
+        fin.P_off = (const int64_t*)f.W_off.p;
+        LSP_CUDA(ctx, run_tc(ctx, tcp, ctx->b_tc.p, lsp::kTcWindow, a, fin, st));
+        LSP_CUDA(ctx, lsp::launch_window_peaks(n, d_t, d_off, d_df, (const float*)f.W.p, (const int64_t*)f.W_off.p,
+                                               (const int64_t*)f.nw.p, (int*)f.peaks.p, st));
+        LSP_CUDA(ctx, lsp::launch_window_exact(F, n, d_off, (const uint4*)ctx->b_recA.p, (const float4*)ctx->b_recB.p,
+                                               (const int*)f.peaks.p, (float*)f.peak_w.p, st));
+    }
     if (!items.empty()) {
         const int grid = (int)std::min<int64_t>((int64_t)lsp::window_occupancy(F) * ctx->sms, (int64_t)items.size());
         LSP_CUDA(ctx, lsp::launch_window(F, grid, (const lsp::BatchItem*)ctx->b_items.p, (int)items.size(),
                                          (unsigned*)ctx->b_head.p, d_off, (const int64_t*)f.nw.p,
                                          (const uint4*)ctx->b_recA.p, (const float4*)ctx->b_recB.p, (float*)f.W.p,
-                                         (const int64_t*)f.W_off.p, st));
+                                         (const int64_t*)f.W_off.p, st, tc ? (const int*)f.peaks.p : nullptr));
     }
     LSP_CUDA(ctx, lsp::launch_features(n, max_n, d_t, d_off, d_f0, d_df, d_nf, (const float*)f.W.p,
-                                       (const int64_t*)f.W_off.p, (const int64_t*)f.nw.p, d_feat, ctx->status_d, st));
-    ctx->last_launches = 4;
+                                       (const int64_t*)f.W_off.p, (const int64_t*)f.nw.p, d_feat, ctx->status_d, st,
+                                       tc ? (const int*)f.peaks.p : nullptr, (const float*)f.peak_w.p));
+    ctx->last_launches = 4 + (tc ? 2 + 2 * (int)tcp.chunks.size() : 0);
     if (feat_host) {
         LSP_CUDA(ctx, cudaMemcpyAsync(features, d_feat, (size_t)n * kNFeat * 4, cudaMemcpyDeviceToHost, st));
         return lsp_sync(ctx, -1.0);

@@ -118,7 +118,7 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
         LSP_CUDA(ctx, lsp::launch_prep_stats(td, xd, nullptr, N_t, 1, stats, ctx->status_d,
                                              (lsp::StatPart*)ctx->stat_parts.p, (unsigned*)ctx->stat_counters.p, st,
                                              dyd, tc ? (float*)ctx->qmax.p : nullptr));
-        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f), (float*)ctx->qmax.p};
+        const lsp::TcPrep tp{(float2*)ctx->recE.p, nullptr, lsp::tc_cols(N_f, 2), (float*)ctx->qmax.p};
         LSP_CUDA(ctx, lsp::launch_prep_records(td, xd, nullptr, N_t, 1, N_t, nullptr, nullptr, f_0, df, stats,
                                                (uint4*)ctx->recA.p, (float4*)ctx->recB.p, nullptr, nullptr, st, dyd,
                                                (float*)ctx->recQ.p, ctx->status_d, tc ? &tp : nullptr));
@@ -303,7 +303,7 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
     lsp::CurveStats* stats = (lsp::CurveStats*)ctx->b_stats.p;
     LSP_CUDA(ctx, lsp::launch_prep_stats(d_t, d_X, d_off, 0, n_curves, stats, ctx->status_d, nullptr, nullptr, st,
                                          d_dy, tc ? (float*)ctx->b_qmax.p : nullptr));
-    const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, d_nf, 0, (float*)ctx->b_qmax.p};
+    const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, (const int64_t*)ctx->b_tc.p, 0, (float*)ctx->b_qmax.p};
     const int64_t max_n = off[order[0] + 1] - off[order[0]];
     LSP_CUDA(ctx, lsp::launch_prep_records(d_t, d_X, d_off, 0, n_curves, max_n, d_f0, d_df, 0.0, 0.0, stats,
                                            (uint4*)ctx->b_recA.p, (float4*)ctx->b_recB.p, nullptr, nullptr, st,

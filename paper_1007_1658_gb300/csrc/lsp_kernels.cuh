@@ -57,12 +57,12 @@ cudaError_t launch_prep_stats(const double* t, const double* X, const int64_t* o
                               float* qmax = nullptr);
 
 // What the tensor-core path needs beside the records: recE[j] = (cos, sin)(2 pi
-// cols u_j) with cols the curve's fine offsets (`cols`, or from nf[curve]), and
+// cols u_j) with cols the bins of a coarse frequency (`cols`, or by curve), and
 // the largest q of each curve (n_curves floats and one word more, zeroed by
 // launch_prep_stats).
 struct TcPrep {
     float2* recE;
-    const int64_t* nf;
+    const int64_t* curve_cols;
     int cols;
     float* qmax;
 };
@@ -263,16 +263,31 @@ cudaError_t launch_noise_prep(const int64_t* off, int n_curves, int n_real, cons
 
 // ---- false-alarm surrogate (features.cu, mlp.cu) ----
 
-// Spectral window of each pattern on its own window grid (persistent items).
+// Spectral window of each pattern on its own window grid (persistent items), by
+// the strip kernel; with `peaks`, only of the patterns it gives up (below).
 cudaError_t launch_window(int F, int grid, const BatchItem* items, int n_items, unsigned* head, const int64_t* off,
                           const int64_t* nw, const uint4* recA, const float4* recB, float* W, const int64_t* W_off,
-                          cudaStream_t st);
+                          cudaStream_t st, const int* peaks = nullptr);
 int window_occupancy(int F);
+// From a window W that is accurate but not the strip kernel's bit for bit: the
+// bins that can be among the 8 highest local maxima of that one, as
+// peaks[c][1 ..], their number in peaks[c][0]; -1 gives the pattern up (more than
+// kWindowPeaks of them, or too long a pattern).
+constexpr int kWindowPeaks = 127;
+cudaError_t launch_window_peaks(int n_patterns, const double* t, const int64_t* off, const double* df, const float* W,
+                                const int64_t* W_off, const int64_t* nw, int* peaks, cudaStream_t st);
+// The strip kernel's W, bit for bit, at each such bin and its two neighbours:
+// peak_w[c][3 i ..], i < peaks[c][0].
+cudaError_t launch_window_exact(int F, int n_patterns, const int64_t* off, const uint4* recA, const float4* recB,
+                                const int* peaks, float* peak_w, cudaStream_t st);
 // Dynamic shared memory of the features kernel for patterns of up to max_n samples.
 size_t features_smem_bytes(int64_t max_n);
+// The window's maxima come from peaks and peak_w where they are given and the
+// pattern is not given up, else from W.
 cudaError_t launch_features(int n_patterns, int64_t max_n, const double* t, const int64_t* off, const double* f0,
                             const double* df, const int64_t* nf, const float* W, const int64_t* W_off,
-                            const int64_t* nw, float* feat, int* status, cudaStream_t st);
+                            const int64_t* nw, float* feat, int* status, cudaStream_t st, const int* peaks = nullptr,
+                            const float* peak_w = nullptr);
 
 int64_t mlp_param_count(int H);
 cudaError_t mlp_init(int H, uint64_t seed, float* params, cudaStream_t st);

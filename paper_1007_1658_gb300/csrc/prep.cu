@@ -8,7 +8,6 @@
 #include <cmath>
 
 #include "lsp_kernels.cuh"
-#include "tc_sums.cuh"
 
 namespace lsp {
 namespace {
@@ -244,7 +243,7 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // 1/sqrt(sum of weights): the weight sum from the stats, or N without errors
     const float isw = qout ? (float)rsqrt(dy ? st.pad : (double)(e - b)) : 0.f;
-    const int cols = tc.recE ? (tc.nf ? tc_cols(tc.nf[c]) : tc.cols) : 0;
+    const int cols = tc.recE ? (tc.curve_cols ? (int)tc.curve_cols[c] : tc.cols) : 0;
     float qm = 0.f;
     for (int64_t j = b + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < e; j += stride) {
         const double tt = t[j] - st.t_ref;

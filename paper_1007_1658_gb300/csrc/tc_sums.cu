@@ -135,47 +135,65 @@ struct Ahead {
     float q[kGenWarps * 32], x[kGenWarps * 32];
 };
 
+// The tile of a launch, and the samples of its curve.
 struct TileInfo {
-    int64_t b, n;       // samples [b, b + n)
-    uint32_t k0;        // first frequency index
-    int cols, kind;
-    float scale;        // power of two on y, so that its FP16 halves keep their bits
-    const float* x;     // realization row
+    TcTile w;
+    int64_t b, n;
 };
+
+__device__ __forceinline__ TcTile tile_of(const TcArgs& a, int t) {
+    if (a.tiles) return a.tiles[t];
+    TcTile w = a.one;
+    if (t < a.h1) {
+        w.g0 = kTcGroups * t;
+    } else {
+        w.g0 = kTcGroups * (t - a.h1);
+        w.kind = a.win_kind;
+        w.twice = 1;
+    }
+    return w;
+}
 
 __device__ __forceinline__ TileInfo tile_info(const TcArgs& a, int t) {
     TileInfo f;
-    int curve = 0, real = 0, fb;
-    if (a.tiles) {
-        const TcTile w = a.tiles[t];
-        curve = w.curve;
-        real = w.real;
-        fb = w.fblock;
-        f.kind = w.kind;
-        f.cols = w.cols;
-        f.b = a.off[curve];
-        f.n = a.off[curve + 1] - f.b;
+    f.w = tile_of(a, t);
+    f.b = a.off ? a.off[f.w.curve] : 0;
+    f.n = a.off ? a.off[f.w.curve + 1] - f.b : a.n0;
+    return f;
+}
+
+// A group of a tile: what its rows sum (y = 0 beyond the last set), the grid's
+// group, the realization, and the power of two on y that keeps the bits of its
+// FP16 halves.
+struct Group {
+    int kind, kg, real;
+    bool live;
+    float scale;
+};
+
+__device__ __forceinline__ Group group_of(const TcArgs& a, const TileInfo& f, int g) {
+    Group r;
+    const int G = f.w.g0 + g, set = G / f.w.gpr;
+    r.kg = f.w.kg0 + (G - set * f.w.gpr);
+    r.kind = f.w.kind;
+    r.real = f.w.r0 + set;
+    if (f.w.twice) {
+        r.live = set == 0;
     } else {
-        const int s = t / a.nblk;
-        fb = a.fb0 + (t - s * a.nblk);
-        f.kind = s == 0 ? a.kinds[0] : s == 1 ? a.kinds[1] : a.kinds[2];
-        f.cols = a.cols;
-        f.b = 0;
-        f.n = a.n0;
+        r.live = set < f.w.reals + f.w.gls;
+        if (f.w.gls && set >= f.w.reals) r.kind = kTcW1;
     }
-    f.k0 = (uint32_t)fb * (uint32_t)(kTcRows * f.cols);
-    f.x = a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr;
     // |x_hat| <= sqrt(n); |q x_hat| <= qmax; q^2 <= qmax^2: scaled to at most 2^14
     int ex = 0;
-    if (f.kind == kTcRec || f.kind == kTcRow) {
+    if (r.kind == kTcRec || r.kind == kTcRow) {
         ex = 14 - (33 - __clz((int)min(f.n, (int64_t)0x7fffffff))) / 2;
-    } else if (f.kind >= kTcW1) {
+    } else if (r.kind >= kTcW1 && a.qmax) {
         int eq;
-        frexpf(a.qmax[curve], &eq);  // qmax < 2^eq
-        ex = 14 - (f.kind >= kTcRecQ ? eq : 2 * eq);
+        frexpf(a.qmax[f.w.curve], &eq);  // qmax < 2^eq
+        ex = 14 - (r.kind >= kTcRecQ ? eq : 2 * eq);
     }
-    f.scale = ldexpf(1.f, min(max(ex, -100), 100));
-    return f;
+    r.scale = ldexpf(1.f, min(max(ex, -100), 100));
+    return r;
 }
 
 // The factor that undoes the mean shrinking of a unit's accumulation (see
@@ -231,7 +249,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
     const uint32_t tb = tbase;
 
     const int64_t lo = tc_bound(a.work, a.pairs, pair), hi = tc_bound(a.work, a.pairs, pair + 1);
-    const int64_t cost0 = a.tiles ? 0 : (a.n0 + kTcUnit - 1) / kTcUnit * tc_unit_cost(a.cols);
+    const int64_t cost0 = a.tiles ? 0 : (a.n0 + kTcUnit - 1) / kTcUnit * tc_unit_cost(a.one.cols);
     // first tile that reaches beyond lo
     int t = 0;
     if (a.tiles) {
@@ -256,7 +274,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
             if (p >= hi) return false;
             f = tile_info(a, t);
             int64_t u0, u1;
-            tc_units(p, (f.n + kTcUnit - 1) / kTcUnit, tc_unit_cost(f.cols), lo, hi, &u0, &u1);
+            tc_units(p, (f.n + kTcUnit - 1) / kTcUnit, tc_unit_cost(f.w.cols), lo, hi, &u0, &u1);
             if (u0 >= u1) continue;
             j0 = f.b + u0 * kTcUnit;
             left = (int)(min(f.n, u1 * kTcUnit) - u0 * kTcUnit);
@@ -270,7 +288,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
         if (warp == kGenWarps && rank == 0) {
             uint32_t buf = 0, phase = 0;
             for (; next_piece(); ++t) {
-                const uint32_t id = tc::instr_desc(f.cols);
+                const uint32_t id = tc::instr_desc(f.w.cols);
                 for (int m = 0; m < left; m += kTcUnit, ++group) {
                     const uint32_t d = tb + (group & 1) * 256u;
                     if (group >= 2) ok = ok && tc::mbar_wait(&drained[group & 1], ((group >> 1) - 1) & 1);
@@ -307,15 +325,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
         // this warp's set, its group of rows and offsets, its lanes and columns of the accumulators
         const int set = warp >> 2, grp = warp & 3, quad = grp, cg = set;
         for (; next_piece(); ++t) {
-            const bool twice = f.kind == kTcOne2 || f.kind == kTcW2;
-            const int hb = f.cols >> 2;  // fine offsets (of one sign) of this CTA
+            const bool twice = f.w.twice;
+            const int cols = f.w.cols, hb = cols >> 2;  // fine offsets (of one sign) of this CTA: hb
+            const Group r = group_of(a, f, 4 * rank + grp);
+            const float yscale = r.live ? r.scale : 0.f;
+            const float* xrow = a.xr ? a.xr + (size_t)r.real * (size_t)a.total : nullptr;
             auto fetch = [&](int j) {    // sample j of the piece
                 if (j < left) {
                     dev::cp_async16(&ahead.uv[tid], a.recA + j0 + j);
                     dev::cp_async16(&ahead.B[tid], a.recB + j0 + j);
                     dev::cp_async8(&ahead.E[tid], a.recE + j0 + j);
-                    if (f.kind >= kTcW1) dev::cp_async4(&ahead.q[tid], a.q + j0 + j);
-                    if (f.kind == kTcRow || f.kind == kTcRowQ) dev::cp_async4(&ahead.x[tid], f.x + j0 + j);
+                    if (r.kind >= kTcW1) dev::cp_async4(&ahead.q[tid], a.q + j0 + j);
+                    if (r.live && (r.kind == kTcRow || r.kind == kTcRowQ)) dev::cp_async4(&ahead.x[tid], xrow + j0 + j);
                 } else {  // beyond the piece: zeros, and y = 0 below
                     ahead.uv[tid] = make_uint4(0, 0, 0, 0);
                     ahead.B[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -334,7 +355,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                 tc::fence_after_sync();
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    if (cg * 64 + c * 32 < f.cols) {
+                    if (cg * 64 + c * 32 < cols) {
                         uint32_t r[32];
                         tc::tmem_ld32(r, tb + (g & 1) * 256u + ((uint32_t)quad << 21) + (uint32_t)(cg * 64 + c * 32));
 #pragma unroll
@@ -350,10 +371,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
             auto flush = [&](bool add) {
                 float* const out = a.part + (size_t)(t + pair) * (size_t)a.slot_floats +
                                    (size_t)rank * (size_t)(a.slot_floats / 2) + (size_t)(cg * 64) * 128 + quad * 32 + lane;
-                const float inv = 1.f / f.scale;
+                // rows of a CTA: real parts of its four groups, then imaginary parts
+                const float inv = 1.f / group_of(a, f, 4 * rank + (2 * quad + (lane >> 4) & 3)).scale;
 #pragma unroll
                 for (int i = 0; i < 64; ++i)
-                    if (cg * 64 + i < f.cols) out[i * 128] = fmaf(run[i], inv, add ? out[i * 128] : 0.f);
+                    if (cg * 64 + i < cols) out[i * 128] = fmaf(run[i], inv, add ? out[i * 128] : 0.f);
             };
             fetch(set * kStage + lane);
             for (int m = 0; m < left; m += kTcUnit, ++group) {
@@ -363,19 +385,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                     const uint4 uv = ahead.uv[tid];
                     const float4 B = ahead.B[tid];
                     float2 e1 = make_float2(B.y, B.z), E = ahead.E[tid];
-                    float y = jm + lane < left ? f.scale : 0.f;
-                    if (f.kind >= kTcW1) {
-                        const float q = ahead.q[tid];
-                        y *= q;
-                        if (f.kind <= kTcW2) y *= q;
+                    float y = jm + lane < left ? yscale : 0.f;
+                    if (r.live) {
+                        if (r.kind >= kTcW1) {
+                            const float q = ahead.q[tid];
+                            y *= q;
+                            if (r.kind <= kTcW2) y *= q;
+                        }
+                        if ((r.kind & 3) > 1) y *= (r.kind & 1) ? ahead.x[tid] : B.x;
                     }
-                    if ((f.kind & 3) > 1) y *= (f.kind & 1) ? ahead.x[tid] : B.x;
                     fetch(jm + kTcUnit + lane);
                     const uint64_t u = ((uint64_t)uv.y << 32) | uv.x;
                     const uint64_t v = (((uint64_t)uv.w << 32) | uv.z) - kPhaseOffset;
                     const uint64_t uh = u >> 1;
                     // the middle of the first of 16 coarse blocks of cols bins, and the first of 16 fine offsets
-                    uint64_t pa = v + (uint64_t)(f.k0 + (uint32_t)((64 * rank + 16 * grp) * f.cols + 2 * hb)) * u - uh;
+                    uint64_t pa = v + (uint64_t)((uint32_t)r.kg * (uint32_t)(kTcGroup * cols) + (uint32_t)(2 * hb)) * u - uh;
                     uint64_t pb = (uint64_t)(rank * hb + 16 * grp) * u + uh;
                     if (twice) {
                         pa <<= 1;
@@ -439,63 +463,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
 }
 
 // The slots of a tile's pieces, in order (the pairs that got at least one unit
-// of it), and their number; every thread of the CTA calls it.
+// of it), and their number; one warp calls it.
 struct Pieces {
     int n;
     int slot[kTcMaxPairs];
 };
 
 __device__ void find_pieces(const TcArgs& a, int tile, int64_t n, int cols, Pieces& out) {
+    const int lane = threadIdx.x & 31;
     const int64_t units = (n + kTcUnit - 1) / kTcUnit, c = tc_unit_cost(cols);
     const int64_t p = a.tiles ? a.pre[tile] : (int64_t)tile * units * c;
     const int i0 = tc_pair_of(a.work, a.pairs, p), i1 = tc_pair_of(a.work, a.pairs, p + (units - 1) * c);
-    if (threadIdx.x < 32) {
-        int at = 0;
+    int at = 0;
+    if (i0 == i1) {
+        if (lane == 0) out.slot[0] = tile + i0;
+        at = 1;
+    } else {
         for (int i = i0; i <= i1; i += 32) {
-            const int me = i + (int)threadIdx.x;
+            const int me = i + lane;
             int64_t u0 = 0, u1 = 0;
             if (me <= i1) tc_units(p, units, c, tc_bound(a.work, a.pairs, me), tc_bound(a.work, a.pairs, me + 1), &u0, &u1);
             const unsigned has = __ballot_sync(0xffffffffu, u0 < u1);
-            if (u0 < u1) out.slot[at + __popc(has & ((1u << threadIdx.x) - 1u))] = tile + me;
+            if (u0 < u1) out.slot[at + __popc(has & ((1u << lane) - 1u))] = tile + me;
             at += __popc(has);
         }
-        if (threadIdx.x == 0) out.n = at;
     }
+    if (lane == 0) out.n = at;
 }
 
 // The complex sums at f_a + f_b and f_a - f_b of S tiles, from a tile's four
-// entries each, the pieces added in order with compensated FP32 sums; four
-// pieces of every tile are loaded before any of them is added.
+// entries each (at[x], cos, real part; the others 64 and hb columns on), the
+// pieces added in order with compensated FP32 sums; four pieces of every tile
+// are loaded before any of them is added.
 template <int S>
-__device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces (&q)[S], int hb, int half, int ra, int rb,
+__device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces* const (&q)[S], const size_t (&at)[S], int hb,
                                           float2 (&plus)[S], float2 (&minus)[S]) {
     float s[S][4] = {}, c[S][4] = {};
-    // sum y (Re A, Im A) cos, then sin; columns: cos, sin of the first CTA's hb offsets, then of the second's
-    const size_t co = (size_t)(rb < hb ? rb : hb + rb) * 128 + (size_t)half * (size_t)(a.slot_floats / 2) + ra;
-    const size_t at[4] = {co, co + 64, co + (size_t)hb * 128, co + (size_t)hb * 128 + 64};
-    int most = q[0].n;
+    const size_t step[4] = {0, 64, (size_t)hb * 128, (size_t)hb * 128 + 64};
+    int most = q[0]->n;
 #pragma unroll
-    for (int x = 1; x < S; ++x) most = max(most, q[x].n);
-    for (int i0 = 0; i0 < most; i0 += 4) {
-        float v[S][4][4];
+    for (int x = 1; x < S; ++x) most = max(most, q[x]->n);
+    if (most == 1) {  // a tile of one pair: nothing to add
 #pragma unroll
         for (int x = 0; x < S; ++x)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float* d = a.part + (size_t)q[x].slot[min(i0 + u, q[x].n - 1)] * (size_t)a.slot_floats;
+            for (int i = 0; i < 4; ++i)
+                s[x][i] = a.part[(size_t)q[x]->slot[0] * (size_t)a.slot_floats + at[x] + step[i]];
+    } else {
+        for (int i0 = 0; i0 < most; i0 += 4) {
+            float v[S][4][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[x][u][i] = i0 + u < q[x].n ? d[at[i]] : 0.f;
-            }
+            for (int x = 0; x < S; ++x)
 #pragma unroll
-        for (int x = 0; x < S; ++x)
+                for (int u = 0; u < 4; ++u) {
+                    const float* d = a.part + (size_t)q[x]->slot[min(i0 + u, q[x]->n - 1)] * (size_t)a.slot_floats + at[x];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float y = v[x][u][i], t = s[x][i] + y;
-                    c[x][i] += fabsf(s[x][i]) >= fabsf(y) ? (s[x][i] - t) + y : (y - t) + s[x][i];
-                    s[x][i] = t;
+                    for (int i = 0; i < 4; ++i) v[x][u][i] = i0 + u < q[x]->n ? d[step[i]] : 0.f;
                 }
+#pragma unroll
+            for (int x = 0; x < S; ++x)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float y = v[x][u][i], t = s[x][i] + y;
+                        c[x][i] += fabsf(s[x][i]) >= fabsf(y) ? (s[x][i] - t) + y : (y - t) + s[x][i];
+                        s[x][i] = t;
+                    }
+        }
     }
 #pragma unroll
     for (int x = 0; x < S; ++x) {
@@ -558,112 +593,133 @@ __device__ __forceinline__ void direct_gls(const TcArgs& a, int64_t b, int64_t n
     }
 }
 
-constexpr int kFinB = 4;  // fine offsets of one finalize CTA
-constexpr int kFinRows = kTcRows / 2;
+constexpr int kFinB = 4;  // fine offsets a CTA takes at a time
+constexpr int kFinRows = kTcGroups / 2 * kTcGroup;
 constexpr int kFinThreads = kFinRows * kFinB;
 
-// One CTA: 64 of a data tile's coarse frequencies x 4 fine offsets, both signs, a
-// pair of frequencies a thread.  Reads run along the coarse frequencies
-// (contiguous in a slot); P is gathered in shared memory and written in runs of
-// 4 bins.
+// One CTA: the 64 coarse frequencies of half a tile (four groups) and every
+// gridDim.y-th run of 4 fine offsets, both signs, a pair of frequencies a thread.
+// Reads run along the coarse frequencies (contiguous in a slot).  P, where it is
+// asked for, is gathered in shared memory and written in runs of 4 bins; the
+// maxima need no exchange until the end.
 template <int FORM>
 __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, const TcFinal f) {
     __shared__ float sp[kFinRows][2 * kFinB + 1];
-    constexpr int S = FORM == kTcClassic ? 2 : 3;
-    __shared__ Pieces q[S];
-    __shared__ unsigned long long s_red[kFinThreads / 32];
-    const int tid = threadIdx.x;
-    int curve = 0, real = 0, fb, cols, td, tw, tcx;
-    int64_t n, nf;
-    if (a.tiles) {
-        td = f.data_tiles[blockIdx.x >> 1];
-        const TcTile w = a.tiles[td];
-        curve = w.curve;
-        real = w.real;
-        fb = w.fblock;
-        cols = w.cols;
-        tw = w.wtile;
-        tcx = w.ctile;
-        n = a.off[curve + 1] - a.off[curve];
-        nf = f.nf[curve];
-    } else {
-        td = (int)blockIdx.x >> 1;
-        fb = a.fb0 + td;
-        cols = a.cols;
-        tw = td + a.nblk;
-        tcx = td + 2 * a.nblk;
-        n = a.n0;
-        nf = f.nf0;
+    constexpr int S = FORM == kTcWindow ? 1 : FORM == kTcClassic ? 2 : 3;
+    __shared__ Pieces pd, pw[4], pc[FORM == kTcGls ? 4 : 1];
+    __shared__ unsigned long long s_red[kFinB][4];
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int td = a.tiles ? f.data_tiles[blockIdx.x >> 1] : (int)blockIdx.x >> 1;
+    const int half = (int)blockIdx.x & 1;
+    const TileInfo t = tile_info(a, td);
+    const TcTile& w = t.w;
+    const int cols = w.cols, hb = cols >> 2, nb = cols >> 1;
+    const int64_t n = t.n, nf = a.tiles ? f.nf[w.curve] : f.nf0;
+    // this thread's row, its group's set and place in the grid, and the same
+    // frequencies' rows in the h = 2 tile and in the set y = q^2
+    const int ra = tid & (kFinRows - 1), bi = tid / kFinRows, grp = ra >> 4;
+    const int G = w.g0 + 4 * half + grp, set = G / w.gpr, kl = G - set * w.gpr, Gc = w.reals * w.gpr + kl;
+    const int64_t k0 = ((int64_t)(w.kg0 + kl) * kTcGroup + (ra & 15)) * cols;
+    const bool live = set < w.reals && k0 < nf;
+    const int real = w.r0 + set;
+    if (!__syncthreads_or(live)) return;
+    {
+        // warps 0 .. 3 find the h = 2 pieces of group `warp`, 4 .. 7 the y = q^2 ones, 0 the data tile's
+        const int g = warp & 3, Gg = w.g0 + 4 * half + g, sg = Gg / w.gpr, lg = Gg - sg * w.gpr;
+        if (FORM == kTcWindow) {
+        } else if (warp < 4) find_pieces(a, w.wt0 + lg / kTcGroups, n, cols, pw[g]);
+        else if (FORM == kTcGls) find_pieces(a, w.ht0 + (w.reals * w.gpr + lg) / kTcGroups, n, cols, pc[FORM == kTcGls ? g : 0]);
+        if (warp == 0) find_pieces(a, td, n, cols, pd);
     }
-    const int nb = cols >> 1, half = (int)blockIdx.x & 1;
-    const int b0 = (int)blockIdx.y * kFinB;
-    const int64_t k0 = ((int64_t)fb * kTcRows + half * kFinRows) * cols;
-    if (b0 >= nb || k0 >= nf) return;
-    find_pieces(a, td, n, cols, q[0]);
-    find_pieces(a, tw, n, cols, q[1]);
-    if constexpr (S > 2) find_pieces(a, tcx, n, cols, q[2]);
     __syncthreads();
-    const int ra = tid & (kFinRows - 1), bi = tid / kFinRows;
-    if (k0 + (int64_t)ra * cols < nf) {  // not a padding row
-        float2 zp[S], zm[S];
-        tile_sums<S>(a, q, nb >> 1, half, ra, b0 + bi, zp, zm);
-        float vp, vm;
-        if constexpr (FORM == kTcClassic) {
-            vp = dev::periodogram_value2(zp[0].x, zp[0].y, zp[1].x, zp[1].y, (float)n);
-            vm = dev::periodogram_value2(zm[0].x, zm[0].y, zm[1].x, zm[1].y, (float)n);
-        } else {
-            bool lp, lm;
-            vp = gls_power(zp[0], zp[2], zp[1], (double)n, &lp);
-            vm = gls_power(zm[0], zm[2], zm[1], (double)n, &lm);
+    const size_t half_slot = (size_t)(a.slot_floats / 2);
+    auto row_at = [&](int g) { return (size_t)((g & 7) >> 2) * half_slot + (size_t)((g & 3) << 4 | (ra & 15)); };
+    const size_t at_d = row_at(G - w.g0), at_w = row_at(kl), at_c = row_at(Gc);
+    float* P = f.P;
+    if (P && f.P_off) P += (size_t)real * (size_t)f.P_total + f.P_off[w.curve];
+    unsigned long long best = 0ull;
+    auto keep = [&](float p, int64_t k) {
+        const unsigned long long key = ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~(uint32_t)k);
+        if (k < nf && !(FORM == kTcGls && p < 0.f)) best = key > best ? key : best;
+    };
+    for (int b0 = (int)blockIdx.y * kFinB; b0 < nb; b0 += (int)gridDim.y * kFinB) {
+        const int rb = b0 + bi;
+        if (live) {
+            // columns: cos, sin of the first CTA's hb offsets, then of the second's
+            const size_t col = (size_t)(rb < hb ? rb : hb + rb) * 128;
+            const int64_t km = k0 + nb - 1 - rb, kp = k0 + nb + rb;
+            float2 zp[S], zm[S];
+            float vp, vm;
+            if constexpr (FORM == kTcWindow) {
+                const Pieces* const q[1] = {&pd};
+                const size_t at[1] = {at_d + col};
+                tile_sums<1>(a, q, at, hb, zp, zm);
+                const float inv = 1.f / ((float)n * (float)n);
+                vp = (zp[0].x * zp[0].x + zp[0].y * zp[0].y) * inv;
+                vm = (zm[0].x * zm[0].x + zm[0].y * zm[0].y) * inv;
+            } else if constexpr (FORM == kTcClassic) {
+                const Pieces* const q[2] = {&pd, &pw[grp]};
+                const size_t at[2] = {at_d + col, at_w + col};
+                tile_sums<2>(a, q, at, hb, zp, zm);
+                vp = dev::periodogram_value2(zp[0].x, zp[0].y, zp[1].x, zp[1].y, (float)n);
+                vm = dev::periodogram_value2(zm[0].x, zm[0].y, zm[1].x, zm[1].y, (float)n);
+            } else {
+                const Pieces* const q[3] = {&pd, &pw[grp], &pc[grp]};
+                const size_t at[3] = {at_d + col, at_w + col, at_c + col};
+                tile_sums<3>(a, q, at, hb, zp, zm);
+                bool lp, lm;
+                vp = gls_power(zp[0], zp[2], zp[1], (double)n, &lp);
+                vm = gls_power(zm[0], zm[2], zm[1], (double)n, &lm);
 #pragma unroll 1
-            for (int s = 0; s < 2; ++s) {
-                const int64_t k = k0 + (int64_t)ra * cols + (s ? nb + b0 + bi : nb - 1 - b0 - bi);
-                if (!(s ? lp : lm) || k >= nf) continue;
-                float p = -1.f;  // left to launch_tc_refine
-                const unsigned at = atomicAdd(f.n_bins, 1u);
-                if (at < (unsigned)kTcBins) {
-                    f.bins[at] = TcBin{curve, real, (uint32_t)k, 0u};
-                } else {  // the list is full
-                    float d[6] = {}, e[6] = {};
-                    direct_gls(a, a.tiles ? a.off[curve] : 0, n,
-                               a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr, (uint32_t)k, 0, 1, d, e);
-                    p = dev::gls_value((double)d[0] + e[0], (double)d[1] + e[1], (double)d[2] + e[2],
-                                       (double)d[3] + e[3], (double)d[4] + e[4], (double)d[5] + e[5], (double)n);
+                for (int s = 0; s < 2; ++s) {
+                    const int64_t k = s ? kp : km;
+                    if (!(s ? lp : lm) || k >= nf) continue;
+                    float p = -1.f;  // left to launch_tc_refine
+                    const unsigned at = atomicAdd(f.n_bins, 1u);
+                    if (at < (unsigned)kTcBins) {
+                        f.bins[at] = TcBin{w.curve, real, (uint32_t)k, 0u};
+                    } else {  // the list is full
+                        float d[6] = {}, e[6] = {};
+                        direct_gls(a, t.b, n, a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr, (uint32_t)k, 0, 1, d,
+                                   e);
+                        p = dev::gls_value((double)d[0] + e[0], (double)d[1] + e[1], (double)d[2] + e[2],
+                                           (double)d[3] + e[3], (double)d[4] + e[4], (double)d[5] + e[5], (double)n);
+                    }
+                    (s ? vp : vm) = p;
                 }
-                (s ? vp : vm) = p;
+            }
+            keep(vm, km);
+            keep(vp, kp);
+            sp[ra][kFinB - 1 - bi] = vm;
+            sp[ra][kFinB + bi] = vp;
+        }
+        if (!f.P) continue;
+        __syncthreads();
+        // bin i of a row: the minus run ends below the middle, the plus run starts above it; 8 threads a row
+        for (int x = tid; x < kFinRows * 2 * kFinB; x += kFinThreads) {
+            const int r = x / (2 * kFinB), i = x % (2 * kFinB);
+            const int Gr = w.g0 + 4 * half + (r >> 4), sr = Gr / w.gpr;
+            const int fine = i < kFinB ? nb - b0 - kFinB + i : nb + b0 + (i - kFinB);
+            const int64_t k = ((int64_t)(w.kg0 + Gr - sr * w.gpr) * kTcGroup + (r & 15)) * cols + fine;
+            if (sr < w.reals && k < nf) {
+                const float p = sp[r][i];
+                if (!(FORM == kTcGls && p < 0.f))
+                    f.P[(f.P_off ? (size_t)(w.r0 + sr) * (size_t)f.P_total + f.P_off[w.curve] : 0) + k] = p;
             }
         }
-        sp[ra][kFinB - 1 - bi] = vm;
-        sp[ra][kFinB + bi] = vp;
-    }
-    __syncthreads();
-    // bin of slot i of row r: the minus run ends below the middle, the plus run starts above it
-    float* P = f.P;
-    if (P && f.P_off) P += (size_t)real * (size_t)f.P_total + f.P_off[curve];
-    unsigned long long best = 0ull;
-    for (int x = tid; x < kFinRows * 2 * kFinB; x += kFinThreads) {
-        const int r = x / (2 * kFinB), i = x % (2 * kFinB);
-        const int fine = i < kFinB ? nb - b0 - kFinB + i : nb + b0 + (i - kFinB);
-        const int64_t k = k0 + (int64_t)r * cols + fine;
-        if (k < nf) {
-            const float p = sp[r][i];
-            if (FORM == kTcGls && p < 0.f) continue;
-            if (P) P[k] = p;
-            const unsigned long long key =
-                ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~(uint32_t)k);
-            best = key > best ? key : best;
-        }
+        __syncthreads();
     }
     if (!f.maxkey) return;
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_down_sync(0xffffffffu, best, o);
+    // the largest of each group: 16 lanes, then the four offsets
+    for (int o = 8; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_down_sync(0xffffffffu, best, o, 16);
         best = y > best ? y : best;
     }
-    if ((tid & 31) == 0) s_red[tid >> 5] = best;
+    if ((tid & 15) == 0) s_red[bi][grp] = best;
     __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < kFinThreads / 32; ++w) best = s_red[w] > best ? s_red[w] : best;
-        if (best) atomicMax(&f.maxkey[(size_t)real * (size_t)f.n_curves + curve], best);
+    if (bi == 0 && (ra & 15) == 0 && set < w.reals) {
+        for (int x = 1; x < kFinB; ++x) best = s_red[x][grp] > best ? s_red[x][grp] : best;
+        if (best) atomicMax(&f.maxkey[(size_t)real * (size_t)f.n_curves + w.curve], best);
     }
 }
 
@@ -771,12 +827,17 @@ cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st) {
-    const int n_data = a.tiles ? f.n_data : a.nblk;
+    const int n_data = a.tiles ? f.n_data : a.h1;
     if (n_data < 1) return cudaSuccess;
     const int max_cols = (int)(a.slot_floats / tc_slot_floats(1));
-    dim3 grid((unsigned)n_data * 2u, (unsigned)((max_cols / 2 + kFinB - 1) / kFinB));
+    // all runs of offsets in CTAs of their own, until there are some thousands of CTAs
+    int y = (max_cols / 2 + kFinB - 1) / kFinB;
+    const int most = 8192 / (2 * n_data);
+    y = y > most ? (most < 1 ? 1 : most) : y;
+    dim3 grid((unsigned)n_data * 2u, (unsigned)y);
     if (form == kTcClassic) tc_final_kernel<kTcClassic><<<grid, kFinThreads, 0, st>>>(a, f);
-    else tc_final_kernel<kTcGls><<<grid, kFinThreads, 0, st>>>(a, f);
+    else if (form == kTcGls) tc_final_kernel<kTcGls><<<grid, kFinThreads, 0, st>>>(a, f);
+    else tc_final_kernel<kTcWindow><<<grid, kFinThreads, 0, st>>>(a, f);
     return cudaGetLastError();
 }
 

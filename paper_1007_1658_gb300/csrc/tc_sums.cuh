@@ -10,6 +10,7 @@ namespace lsp {
 // What a tile sums over its curve's samples j, for a block of frequencies:
 // sum_j y_j exp(2 pi i h phase_j(k)).
 enum : int {
+    kTcOne1 = 0,  // y = 1, h = 1: the spectral window
     kTcOne2 = 1,  // y = 1, h = 2: CC - SS + 2i CS
     kTcRec = 2,   // y = x_hat of the records, h = 1: XC + i XS
     kTcRow = 3,   // y = x_hat of a realization's row, h = 1
@@ -19,14 +20,24 @@ enum : int {
     kTcRowQ = 7   // y = q x_hat of a realization's row, h = 1
 };
 
-// One tile: kTcRows coarse frequencies x cols fine offsets of one sum.  wtile
-// and ctile: the tiles with the same frequencies that hold the h = 2 sum and
-// the floating-mean form's (C, S) for the finalize kernel (data tiles only).
+// Work on a curve's sums is cut into groups of 16 coarse frequencies of cols bins
+// each, gpr of them for a grid; tiles are eight groups that share the fine
+// offsets.  Groups of the h = 1 sums run through the realizations in order and,
+// in the floating-mean form, end with the group set of y = q^2: group G is
+// coarse frequencies 16 (G mod gpr) .. of set G / gpr.  So a short grid's
+// realizations share tiles, whose cost hardly depends on how full they are.
 struct TcTile {
-    int32_t curve, real, fblock, kind, wtile, ctile, cols, pad;
+    int32_t curve, kind;    // kind of the data sets (h = 1) or of the tile (twice)
+    int32_t twice;          // an h = 2 tile: one set
+    int32_t g0;             // first group
+    int32_t r0, reals;      // data sets: realizations r0 .. r0 + reals
+    int32_t gls;            // an h = 1 tile's sets end with y = q^2
+    int32_t gpr, kg0, cols; // groups of a set, the grid's group that is its first, bins of a coarse frequency
+    int32_t wt0, ht0;       // first h = 2 and first h = 1 tile of these groups
 };
 
-constexpr int kTcRows = 128;       // coarse frequencies of a tile (real and imaginary parts: 128 operand rows a CTA)
+constexpr int kTcGroup = 16;       // coarse frequencies of a group
+constexpr int kTcGroups = 8;       // groups of a tile (four a CTA: 128 operand rows, real and imaginary parts)
 constexpr int kTcMaxCols = 256;    // fine offsets of a tile, at most
 constexpr int kTcUnit = 128;       // samples of one unit of work
 constexpr int kTcThreads = 640;
@@ -37,18 +48,15 @@ constexpr int kTcMaxPairs = 256;  // CTA pairs that a launch is split over, at m
 // (proportional to cols) below 256 columns.
 __host__ __device__ inline int tc_unit_cost(int cols) { return 8 + cols / 32; }
 
-// Fine offsets per coarse frequency for a grid of N_f bins: the number of
-// blocks (of 128 coarse frequencies) and columns (a multiple of 32 up to 256)
-// whose cost is least.
-__host__ __device__ inline int tc_cols(int64_t N_f) {
-    const int64_t b0 = (N_f + kTcRows * kTcMaxCols - 1) / (kTcRows * kTcMaxCols);
+// Bins per coarse frequency (a multiple of 32 up to 256) for a grid of N_f bins
+// and `sets` sets of its h = 1 sums: the one whose tiles cost least.
+inline int tc_cols(int64_t N_f, int64_t sets) {
     int best = kTcMaxCols;
     int64_t best_cost = INT64_MAX;
-    for (int64_t b = b0 < 1 ? 1 : b0; b <= b0 + 2; ++b) {
-        const int64_t per = (N_f + b * kTcRows - 1) / (b * kTcRows);
-        const int c = per > 32 ? (int)((per + 31) / 32 * 32) : 32;
-        const int64_t blocks = (N_f + (int64_t)c * kTcRows - 1) / ((int64_t)c * kTcRows);
-        const int64_t cost = blocks * tc_unit_cost(c);
+    for (int c = kTcMaxCols; c >= 32; c -= 32) {
+        const int64_t gpr = (N_f + kTcGroup * c - 1) / (kTcGroup * c);
+        const int64_t cost =
+            ((sets * gpr + kTcGroups - 1) / kTcGroups + (gpr + kTcGroups - 1) / kTcGroups) * tc_unit_cost(c);
         if (cost < best_cost) {
             best_cost = cost;
             best = c;
@@ -59,12 +67,12 @@ __host__ __device__ inline int tc_cols(int64_t N_f) {
 
 struct TcArgs {
     // tiles: a list with the prefix sums of their costs (pre[0..n_tiles]), or,
-    // for a single curve (tiles == nullptr), sum s of block fb0 + b is tile
-    // s * nblk + b with kinds[s], every tile of the same cost
+    // for a single curve (tiles == nullptr), `one` with g0 = 8 t for tile
+    // t < h1 and, twice and of kind win_kind, g0 = 8 (t - h1) from there on
     const TcTile* tiles;
     const int64_t* pre;
-    int n_tiles, nblk, fb0, cols;
-    int kinds[3];
+    int n_tiles, h1, win_kind;
+    TcTile one;
     int64_t n0;                 // samples of the single curve
     int64_t work;               // total cost
     int pairs;                  // CTA pairs the work is split over
@@ -100,8 +108,8 @@ __host__ __device__ inline void tc_units(int64_t p, int64_t n, int64_t c, int64_
     *u1 = b < n ? b : n;
 }
 
-// The finalize pass over the data tiles (kTcRec, kTcRow, kTcRecQ, kTcRowQ): P of
-// every frequency.
+// The finalize pass over the h = 1 tiles: P (kTcWindow: |sum|^2 / n^2) of every
+// frequency of their data sets.
 // A bin of the floating-mean form whose sums are formed again by
 // launch_tc_refine: realization `real` of `curve`, frequency k.
 struct TcBin {
@@ -111,7 +119,7 @@ struct TcBin {
 constexpr int kTcBins = 1 << 16;  // bins the list holds
 
 struct TcFinal {
-    const int* data_tiles;      // list form: indices of the data tiles
+    const int* data_tiles;      // list form: indices of the h = 1 tiles
     int n_data;
     const int64_t* nf;          // list form
     int64_t nf0;                // single curve
@@ -124,7 +132,7 @@ struct TcFinal {
     unsigned* n_bins;           // its counter (zeroed by launch_prep_stats, after qmax)
 };
 
-enum : int { kTcClassic = 0, kTcGls = 1 };
+enum : int { kTcClassic = 0, kTcGls = 1, kTcWindow = 2 };
 
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st);
 cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st);
