@@ -197,8 +197,17 @@ __device__ __forceinline__ Group group_of(const TcArgs& a, const TileInfo& f, in
 }
 
 // The factor that undoes the mean shrinking of a unit's accumulation (see
-// above): 1 + 3 ulp.
-constexpr float kUnitGain = 1.f + 0x1.8p-22f;
+// above): 1 + 4 ulp.  How much a sum shrinks depends on where its growth lies
+// between two powers of two, by a third either way; so four units in turn are
+// scaled by (about) 1, 2^1/4, 2^1/2, 2^3/4, which makes the mean the same for every
+// sum.  The scales are FP32 values whose product with their gains is 1 + 4 ulp to
+// 2e-9.
+__device__ __forceinline__ float unit_scale(int u) {
+    return u & 2 ? (u & 1 ? 0x1.ae7ee8p+0f : 0x1.6a09ecp+0f) : (u & 1 ? 0x1.30840ep+0f : 1.f);
+}
+__device__ __forceinline__ float unit_gain(int u) {
+    return u & 2 ? (u & 1 ? 0x1.3077bep-1f : 0x1.6a09ecp-1f) : (u & 1 ? 0x1.ae6d8p-1f : 0x1.000008p+0f);
+}
 
 // A running sum covers at most this many units (16,384 samples); then it is
 // added to the piece's slot, so that its rounding error does not grow with the
@@ -349,7 +358,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
 #pragma unroll
             for (int i = 0; i < 64; ++i) run[i] = 0.f;
             // adds a finished unit's accumulators to the running sums
-            auto drain = [&](uint32_t g) {
+            auto drain = [&](uint32_t g, int unit) {
+                const float gain = unit_gain(unit);
                 ok = ok && tc::mbar_wait(&full[g & 1], (g >> 1) & 1);
                 __syncwarp();
                 tc::fence_after_sync();
@@ -360,7 +370,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                         tc::tmem_ld32(r, tb + (g & 1) * 256u + ((uint32_t)quad << 21) + (uint32_t)(cg * 64 + c * 32));
 #pragma unroll
                         for (int i = 0; i < 32; ++i)
-                            run[c * 32 + i] = fmaf(__uint_as_float(r[i]), kUnitGain, run[c * 32 + i]);
+                            run[c * 32 + i] = fmaf(__uint_as_float(r[i]), gain, run[c * 32 + i]);
                     }
                 }
                 tc::fence_before_sync();
@@ -385,7 +395,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                     const uint4 uv = ahead.uv[tid];
                     const float4 B = ahead.B[tid];
                     float2 e1 = make_float2(B.y, B.z), E = ahead.E[tid];
-                    float y = jm + lane < left ? yscale : 0.f;
+                    float y = jm + lane < left ? yscale * unit_scale(m / kTcUnit) : 0.f;
                     if (r.live) {
                         if (r.kind >= kTcW1) {
                             const float q = ahead.q[tid];
@@ -442,14 +452,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                     if (lane == 0) tc::mbar_arrive_first(&filled[buf]);
                 }
                 it += (uint32_t)((min(left - m, kTcUnit) + kStage - 1) / kStage);
-                if (m > 0) drain(group - 1);
+                if (m > 0) drain(group - 1, m / kTcUnit - 1);
                 if (m > 0 && (m / kTcUnit) % kRunUnits == 0) {
                     flush(m / kTcUnit > kRunUnits);
 #pragma unroll
                     for (int i = 0; i < 64; ++i) run[i] = 0.f;
                 }
             }
-            drain(group - 1);
+            drain(group - 1, (left - 1) / kTcUnit);
             flush(left > kRunUnits * kTcUnit);
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
