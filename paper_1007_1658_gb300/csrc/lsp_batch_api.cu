@@ -274,7 +274,7 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         if (e == cudaSuccess) {
             const int64_t max_n = off[order[0] + 1] - off[order[0]];
             const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, (const int64_t*)ctx->b_tc.p, 0, nullptr};
-            e = lsp::launch_prep_records(d_t, d_X, d_off, 0, n_curves, max_n, d_f0, d_df, 0.0, 0.0,
+            e = lsp::launch_prep_records(d_t, d_X, d_off, total, n_curves, max_n, d_f0, d_df, 0.0, 0.0,
                                          (const lsp::CurveStats*)ctx->b_stats.p, (uint4*)ctx->b_recA.p,
                                          (float4*)ctx->b_recB.p, nullptr, noise ? nullptr : (float*)ctx->b_xr.p,
                                          cst, nullptr, nullptr, ctx->status_d, tc ? &tprep : nullptr);

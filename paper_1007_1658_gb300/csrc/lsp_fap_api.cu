@@ -202,7 +202,7 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, (const int64_t*)ctx->b_tc.p, 0, nullptr};
     LSP_CUDA(ctx, lsp::launch_prep_stats(d_t, nullptr, d_off, 0, n, (lsp::CurveStats*)ctx->b_stats.p, ctx->status_d,
                                          nullptr, nullptr, st));
-    LSP_CUDA(ctx, lsp::launch_prep_records(d_t, nullptr, d_off, 0, n, max_n, d_df, d_df, 0.0, 0.0,
+    LSP_CUDA(ctx, lsp::launch_prep_records(d_t, nullptr, d_off, total, n, max_n, d_df, d_df, 0.0, 0.0,
                                            (const lsp::CurveStats*)ctx->b_stats.p, (uint4*)ctx->b_recA.p,
                                            (float4*)ctx->b_recB.p, nullptr, nullptr, st, nullptr, nullptr,
                                            ctx->status_d, tc ? &tprep : nullptr));

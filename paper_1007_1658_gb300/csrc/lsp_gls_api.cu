@@ -305,7 +305,7 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
                                          d_dy, tc ? (float*)ctx->b_qmax.p : nullptr));
     const lsp::TcPrep tprep{(float2*)ctx->b_recE.p, (const int64_t*)ctx->b_tc.p, 0, (float*)ctx->b_qmax.p};
     const int64_t max_n = off[order[0] + 1] - off[order[0]];
-    LSP_CUDA(ctx, lsp::launch_prep_records(d_t, d_X, d_off, 0, n_curves, max_n, d_f0, d_df, 0.0, 0.0, stats,
+    LSP_CUDA(ctx, lsp::launch_prep_records(d_t, d_X, d_off, total, n_curves, max_n, d_f0, d_df, 0.0, 0.0, stats,
                                            (uint4*)ctx->b_recA.p, (float4*)ctx->b_recB.p, nullptr, nullptr, st,
                                            d_dy, (float*)ctx->b_xr.p, ctx->status_d, tc ? &tprep : nullptr));
     int launches = 2;

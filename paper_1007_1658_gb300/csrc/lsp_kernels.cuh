@@ -67,6 +67,7 @@ struct TcPrep {
     float* qmax;
 };
 
+// n0: samples of the single curve, or of all curves together.
 // X may be null (noise batches): then only t_ref is computed and x_hat = 0.
 // xout, if given, receives x_hat as a plain FP32 array (batch layout).
 // qout (floating-mean periodogram, stats from launch_prep_stats with the same
