@@ -195,17 +195,37 @@ prep_stats_kernel(const double* __restrict__ t, const double* __restrict__ X,
     }
 }
 
-// frac(a*b) as a 64-bit fixed-point number of turns, exact to ~1 unit of 2^-64:
-// the product is split into p + e exactly (Dekker/Ogita-Rump-Oishi TwoProduct
-// through fma), floor(p) is removed exactly, and both pieces are scaled by
-// 2^64 and added modulo 2^64.  Requires |a*b| < 2^52.
+// frac(a*b) as a 64-bit fixed-point number of turns, rounded to the nearest unit
+// of 2^-64, for finite a and b: the 106-bit product of the mantissas, shifted to
+// the binary point; what lies above it is whole turns and falls off.  Integer
+// arithmetic throughout: FP64 runs at two operations per clock and SM here, and
+// the same phase by a TwoProduct, floor and two conversions took nine of them.
 __device__ __forceinline__ uint64_t frac_turns64(double a, double b) {
-    const double p = __dmul_rn(a, b);
-    const double e = fma(a, b, -p);
-    const double fr = p - floor(p);
-    const uint64_t U = __double2ull_rn(fr * 0x1p64);
-    const int64_t E = __double2ll_rn(e * 0x1p64);
-    return U + (uint64_t)E;
+    const uint64_t xa = (uint64_t)__double_as_longlong(a), xb = (uint64_t)__double_as_longlong(b);
+    const int fa = (int)(xa >> 52) & 2047, fb = (int)(xb >> 52) & 2047;
+    const uint64_t frac = (1ull << 52) - 1;
+    const uint64_t ma = (xa & frac) | (fa ? frac + 1 : 0), mb = (xb & frac) | (fb ? frac + 1 : 0);
+    const uint64_t lo = ma * mb, hi = __umul64hi(ma, mb);
+    // a b = +- (hi 2^64 + lo) 2^(s - 64)
+    const int s = (fa ? fa : 1) + (fb ? fb : 1) - 2 * 1075 + 64;
+    uint64_t r;
+    if (s >= 0) {
+        r = s < 64 ? lo << s : 0;
+    } else if (s > -64) {
+        r = (hi << (64 + s)) + (lo >> -s) + ((lo >> (-s - 1)) & 1);
+    } else if (s > -128) {
+        r = s == -64 ? hi + (lo >> 63) : (hi >> (-s - 64)) + ((hi >> (-s - 65)) & 1);
+    } else {
+        r = 0;
+    }
+    return (xa ^ xb) >> 63 ? 0 - r : r;
+}
+
+// Whether |a b| may reach 2^51: only then is the product itself formed to see
+// whether it reaches 2^52, where frac_turns64's caller gives up.
+__device__ __forceinline__ bool beyond_phase(double a, double b) {
+    const int e = ((int)(__double2hiint(a) >> 20) & 2047) + ((int)(__double2hiint(b) >> 20) & 2047);
+    return e >= 2 * 1023 + 50 && !(fabs(a * b) < 0x1p52);
 }
 
 // cos/sin(2 pi u) of a 64-bit fixed-point turn u (read as signed, so the turn
@@ -298,7 +318,7 @@ prep_records_kernel(const double* __restrict__ t, const double* __restrict__ X,
             xh = X ? (float)((X[j] - st.mean) * st.inv_sd) : 0.f;
         }
         // frac_turns64's range: beyond 2^52 turns the phase is not exact
-        if (!(fabs(tt * df) < 0x1p52) || !(fabs(tt * f0) < 0x1p52)) {
+        if (beyond_phase(tt, df) || beyond_phase(tt, f0)) {
             xh = __int_as_float(0x7fc00000);
             if (status) atomicOr(status, kStatusPhaseRange);
         }
