@@ -96,8 +96,11 @@ __device__ __forceinline__ Pair mul_pair(const Pair& z, float2 e) {
 // halves, 16 bytes each.
 __device__ __forceinline__ void split_pair(float2 v, uint32_t& hi, uint32_t& lo) {
     const __half2 a = __floats2half2_rn(v.x, v.y);
-    const float2 f = __half22float2(a);
-    const float2 d = __ffma2_rn(f, make_float2(-1.f, -1.f), v);
+    float2 d;  // v - a, exact, by FP32 additions that take an FP16 operand
+    asm("{\n .reg .b16 p, q, m;\n mov.b32 {p, q}, %4;\n mov.b16 m, 0xBC00;\n"
+        " fma.rn.f32.f16 %0, p, m, %2;\n fma.rn.f32.f16 %1, q, m, %3;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(v.x), "f"(v.y), "r"(*reinterpret_cast<const uint32_t*>(&a)));
     const __half2 b = __floats2half2_rn(d.x, d.y);
     hi = *reinterpret_cast<const uint32_t*>(&a);
     lo = *reinterpret_cast<const uint32_t*>(&b);
@@ -553,10 +556,9 @@ __device__ __forceinline__ void tile_sums(const TcArgs& a, const Pieces* const (
 
 // Where the smaller eigenvalue of the floating-mean form's second moments is
 // below this (f T under about a third, or an alias of it), P divides by a
-// difference that the tensor cores' truncated sums leave with too few digits
-// (the two sums it is taken from do not share their rounding errors: 1.7e-3 of
-// P at f T = 0.1, where sums formed together keep 1.9e-4): such bins are formed
-// again, sample by sample.
+// difference that separately rounded sums leave with too few digits (1.7e-3 of P
+// at f T = 0.1; the strip kernels' sums, formed together, keep 1.9e-4): such bins
+// are formed again, sample by sample and from moments that do not cancel.
 constexpr float kGlsRefine = 0x1p-5f;
 
 // P of the floating-mean form from Z = sum w x' e, C = sum w e, W = sum w e^2:
@@ -581,26 +583,59 @@ __device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, doub
     return fmaxf((float)(n * num * r), 0.f);
 }
 
-// The six sums at frequency k over samples b + i0, b + i0 + step, ... < b + n,
-// in compensated FP32 (s + c), from the same c~ = q cos, s~ = q sin.
+// Sums over samples b + i0, b + i0 + step, ... < b + n at frequency k from which
+// the centred moments of such a bin can be had without cancellation, with s =
+// sin and v = 1 - cos of the phase (small where the phases are, and formed as
+// such): w s, w v, w s^2, w v^2, w s v, w x' s, w x' v, w x'.  Compensated FP32
+// (s + c).
+constexpr int kMoments = 8;
 __device__ __forceinline__ void direct_gls(const TcArgs& a, int64_t b, int64_t n, const float* x, uint32_t k, int i0,
-                                           int step, float (&s)[6], float (&c)[6]) {
+                                           int step, float (&s)[kMoments], float (&c)[kMoments]) {
 #pragma unroll 4
     for (int64_t j = b + i0; j < b + n; j += step) {
         const uint4 A = a.recA[j];
         const uint64_t u = ((uint64_t)A.y << 32) | A.x;
-        const uint64_t v = (((uint64_t)A.w << 32) | A.z) - kPhaseOffset;
-        const float2 e = turn_cos_sin(v + (uint64_t)k * u);
+        const uint64_t ph = (((uint64_t)A.w << 32) | A.z) - kPhaseOffset + (uint64_t)k * u;
+        const float2 e = turn_cos_sin(ph);
+        // within an eighth of a turn 1 - cos by its series, from the signed turn
+        const float h = (float)(int32_t)(uint32_t)(ph >> 32) * 1.4629180792671596e-9f, h2 = h * h;  // 2 pi / 2^32
+        float v = fmaf(h2, 2.7557319223985888e-7f, -2.4801587301587302e-5f);
+        v = fmaf(h2, v, 1.3888888888888889e-3f);
+        v = fmaf(h2, v, -4.1666666666666664e-2f);
+        v = h2 * fmaf(h2, v, 0.5f);
+        if (fabsf(h) > 0.78f) v = 1.f - e.x;
         const float q = a.q[j], xj = x ? x[j] : a.recB[j].x;
-        const float co = q * e.x, si = q * e.y;
-        const float f[6] = {xj, xj, q, q, co, co}, g[6] = {co, si, co, si, co, si};
+        const float si = q * e.y, vi = q * v;
+        const float f[kMoments] = {q, q, si, vi, si, xj, xj, xj}, g[kMoments] = {si, vi, si, vi, vi, si, vi, q};
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
+        for (int i = 0; i < kMoments; ++i) {
             const float y = fmaf(f[i], g[i], c[i]), t = s[i] + y;
             c[i] = y - (t - s[i]);
             s[i] = t;
         }
     }
+}
+
+// P from those sums: dev::gls_value with the moments centred in FP64.  The
+// smaller eigenvalue comes from the determinant, so that it keeps its digits; a
+// direction whose eigenvalue is at most 2^-24 adds nothing, as there.
+__device__ float moments_value(const float (&s)[kMoments], const float (&c)[kMoments], double n) {
+    double m[kMoments];
+#pragma unroll
+    for (int i = 0; i < kMoments; ++i) m[i] = (double)s[i] + (double)c[i];
+    const double ss = m[2] - m[0] * m[0], vv = m[3] - m[1] * m[1], sv = m[4] - m[0] * m[1];
+    const double ys = m[5] - m[7] * m[0], yv = m[6] - m[7] * m[1];
+    // cos = 1 - v: CC = vv, SS = ss, CS = -sv, YC = -yv, YS = ys
+    const double T = vv + ss, A = vv - ss, B = -2.0 * sv, R = sqrt(A * A + B * B);
+    const double big = 0.5 * (T + R), det = vv * ss - sv * sv, thr = 0x1p-24;
+    if (!(big > thr)) return 0.f;
+    if (det > thr * big) {
+        const double p = (yv * yv * ss + ys * ys * vv - 2.0 * sv * yv * ys) / det;
+        return (float)(0.5 * n * fmax(p, 0.0));
+    }
+    // the projection on the larger direction
+    const double z2 = yv * yv + ys * ys, cross = R > 0.0 ? (A * (yv * yv - ys * ys) - 2.0 * B * yv * ys) / R : z2;
+    return (float)(0.5 * n * fmax(0.5 * (z2 + cross), 0.0) / big);
 }
 
 constexpr int kFinB = 4;  // fine offsets a CTA takes at a time
@@ -689,11 +724,10 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
                     if (at < (unsigned)kTcBins) {
                         f.bins[at] = TcBin{w.curve, real, (uint32_t)k, 0u};
                     } else {  // the list is full
-                        float d[6] = {}, e[6] = {};
+                        float d[kMoments] = {}, e[kMoments] = {};
                         direct_gls(a, t.b, n, a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr, (uint32_t)k, 0, 1, d,
                                    e);
-                        p = dev::gls_value((double)d[0] + e[0], (double)d[1] + e[1], (double)d[2] + e[2],
-                                           (double)d[3] + e[3], (double)d[4] + e[4], (double)d[5] + e[5], (double)n);
+                        p = moments_value(d, e, (double)n);
                     }
                     (s ? vp : vm) = p;
                 }
@@ -742,37 +776,37 @@ __device__ __forceinline__ void add_pair(float& s, float& c, float t, float d) {
     s = y;
 }
 
-// One cluster of CL CTAs per listed bin: the six sums over all samples, then P.
+// One cluster of CL CTAs per listed bin: its sums over all samples, then P.
 // A single curve lists a few bins of many samples (CL = 8: 100,000 samples in
 // one CTA are 40 us of arithmetic), a batch many bins of shorter curves (CL = 1).
 template <int CL>
 __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs a, const TcFinal f) {
-    __shared__ float2 sh[kRefineThreads / 32][6];
-    __shared__ float2 part[CL][6];
+    __shared__ float2 sh[kRefineThreads / 32][kMoments];
+    __shared__ float2 part[CL][kMoments];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0;
     const unsigned count = min(*f.n_bins, (unsigned)kTcBins);
     for (unsigned i = blockIdx.x / CL; i < count; i += gridDim.x / CL) {
         const TcBin w = f.bins[i];
         const int64_t b = a.off ? a.off[w.curve] : 0, n = a.off ? a.off[w.curve + 1] - b : a.n0;
-        float s[6] = {}, c[6] = {};
+        float s[kMoments] = {}, c[kMoments] = {};
         direct_gls(a, b, n, a.xr ? a.xr + (size_t)w.real * (size_t)a.total : nullptr, w.k,
                    rank * kRefineThreads + (int)threadIdx.x, CL * kRefineThreads, s, c);
         auto join = [&](int width) {
             for (int o = width / 2; o > 0; o >>= 1)
 #pragma unroll
-                for (int x = 0; x < 6; ++x)
+                for (int x = 0; x < kMoments; ++x)
                     add_pair(s[x], c[x], __shfl_down_sync(0xffffffffu, s[x], o),
                              __shfl_down_sync(0xffffffffu, c[x], o));
         };
         join(32);
         if (lane == 0)
 #pragma unroll
-            for (int x = 0; x < 6; ++x) sh[warp][x] = make_float2(s[x], c[x]);
+            for (int x = 0; x < kMoments; ++x) sh[warp][x] = make_float2(s[x], c[x]);
         __syncthreads();
         if (warp == 0) {
 #pragma unroll
-            for (int x = 0; x < 6; ++x) {
+            for (int x = 0; x < kMoments; ++x) {
                 const float2 v = lane < kRefineThreads / 32 ? sh[lane][x] : make_float2(0.f, 0.f);
                 s[x] = v.x;
                 c[x] = v.y;
@@ -783,21 +817,18 @@ __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs 
             if (threadIdx.x == 0) {
                 float2* first = cooperative_groups::this_cluster().map_shared_rank(&part[0][0], 0);
 #pragma unroll
-                for (int x = 0; x < 6; ++x) first[rank * 6 + x] = make_float2(s[x], c[x]);
+                for (int x = 0; x < kMoments; ++x) first[rank * kMoments + x] = make_float2(s[x], c[x]);
             }
             cooperative_groups::this_cluster().sync();
             if (threadIdx.x == 0 && rank == 0) {
                 for (int r = 1; r < CL; ++r)
 #pragma unroll
-                    for (int x = 0; x < 6; ++x) add_pair(s[x], c[x], part[r][x].x, part[r][x].y);
+                    for (int x = 0; x < kMoments; ++x) add_pair(s[x], c[x], part[r][x].x, part[r][x].y);
             }
         }
         {
             if (threadIdx.x == 0 && rank == 0) {
-                double d[6];
-#pragma unroll
-                for (int x = 0; x < 6; ++x) d[x] = (double)s[x] + (double)c[x];
-                const float p = dev::gls_value(d[0], d[1], d[2], d[3], d[4], d[5], (double)n);
+                const float p = moments_value(s, c, (double)n);
                 if (f.P) f.P[(size_t)w.real * (size_t)f.P_total + (f.P_off ? f.P_off[w.curve] : 0) + w.k] = p;
                 if (f.maxkey)
                     atomicMax(&f.maxkey[(size_t)w.real * (size_t)f.n_curves + w.curve],
