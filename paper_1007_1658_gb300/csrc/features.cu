@@ -18,7 +18,7 @@
 // With work enough the window comes from the tensor cores (tc_sums.cu), and the
 // strip kernel's values are formed only at the few bins that can be among its 8
 // highest maxima (window_peaks_kernel, window_exact_kernel): the features keep
-// their bits, 256 patterns' window 3.3 ms -> 0.7.
+// their bits; 256 patterns of up to 20,000 samples, the call 3.4 ms -> 1.4.
 #include <algorithm>
 #include <cfloat>
 
@@ -37,8 +37,8 @@ constexpr int kSortMaxGaps = 32768;  // gaps held in shared memory (128 KB); mor
 // values, gaps being >= 0), 8 bits per pass and the five ranks at once; key_at(i)
 // is gap i's.  Each warp adds to the five 256-bin histograms once per distinct
 // bin (__match_any_sync), so gaps that share their leading bits do not serialize
-// on one counter.  hist holds 5 x 256 counters; out[i] receives the value of rank
-// k[i].
+// on one counter; ranks whose leading bits a warp's gaps do not have cost it one
+// vote.  hist holds 5 x 256 counters; out[i] receives the value of rank k[i].
 template <class Key>
 __device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigned* hist, float* out) {
     __shared__ unsigned s_prefix[5], s_rank[5];
@@ -62,23 +62,41 @@ __device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigne
             const int bin = (int)((key >> shift) & 255u);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
+                if (q && !mask) break;  // the first pass counts the same for all five
                 const int mine = (i < M && (key & mask) == prefix[q]) ? bin : -1;
+                if (!__any_sync(0xffffffffu, mine >= 0)) continue;
                 const unsigned peers = __match_any_sync(0xffffffffu, mine);
                 if (mine >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[q * 256 + mine], (unsigned)__popc(peers));
             }
         }
         __syncthreads();
-        if (tid < 5) {
-            // the bin holding rank s_rank: ranks below it move to the next pass's count
-            unsigned r = s_rank[tid], acc = 0u;
-            int bin = 0;
-            for (; bin < 255; ++bin) {
-                const unsigned c = hist[tid * 256 + bin];
-                if (acc + c > r) break;
-                acc += c;
+        if (tid < 5 * 32) {
+            // warp q: the bin holding rank s_rank[q], lane l counting bins 8 l .. 8 l + 7;
+            // ranks below it move to the next pass's count
+            const int w = tid >> 5;
+            const unsigned* h = hist + (mask ? w * 256 : 0) + 8 * lane;
+            const unsigned r = s_rank[w];
+            unsigned cnt[8], sum = 0u;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) sum += cnt[x] = h[x];
+            unsigned acc = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, acc, o);
+                if (lane >= o) acc += v;
             }
-            s_rank[tid] = r - acc;
-            s_prefix[tid] |= (unsigned)bin << shift;
+            const unsigned past = __ballot_sync(0xffffffffu, acc > r);
+            if (lane == (past ? __ffs(past) - 1 : 31)) {
+                acc -= sum;
+                int x = 0;
+#pragma unroll
+                for (int y = 0; y < 7; ++y)
+                    if (x == y && acc + cnt[y] <= r) {
+                        acc += cnt[y];
+                        x = y + 1;
+                    }
+                s_rank[w] = r - acc;
+                s_prefix[w] |= (unsigned)(8 * lane + x) << shift;
+            }
         }
         mask |= 255u << shift;
         __syncthreads();
@@ -175,64 +193,82 @@ ls_window_kernel(const BatchItem* __restrict__ items, int n_items, unsigned* __r
 
 // W of single bins as ls_window_kernel forms it, bit for bit.  There a thread
 // adds a strip's samples in order, one long chain; but only the additions are a
-// chain.  Here a warp forms the terms of its bin for 256 samples at once (the
-// strip's seed and the steps up to the bin), then one lane adds them in order:
-// 20,000 samples in 70 us instead of 1.3 ms.  Warp i of pattern c: neighbour
-// i % 3 - 1 of bin i / 3.
-constexpr int kExactWarps = 8, kExactSamples = 256;
+// chain.  Here a warp takes a bin and its two neighbours: for 128 samples at a
+// time its lanes form the terms (the strip's seed and the steps up to the last of
+// them, four samples abreast; a second strip's where the three straddle one's
+// end), then three lanes add one bin's terms each, in order.
+constexpr int kExactWarps = 8, kExactSamples = 128;
 template <int F>
 __global__ void __launch_bounds__(32 * kExactWarps)
 window_exact_kernel(const int64_t* __restrict__ off, const uint4* __restrict__ recA, const float4* __restrict__ recB,
                     const int* __restrict__ peaks, float* __restrict__ peak_w) {
-    __shared__ __align__(16) float2 terms[kExactWarps][kExactSamples];
+    __shared__ __align__(16) float2 terms[kExactWarps][3][kExactSamples + 2];
     const int c = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int* p = peaks + (size_t)c * (kWindowPeaks + 1);
     const int i = (int)blockIdx.y * kExactWarps + warp;
-    if (i >= 3 * p[0]) return;
-    const uint32_t k = (uint32_t)(p[1 + i / 3] + i % 3 - 1), k0 = k / F * F;
-    const int step = (int)(k - k0);
+    if (i >= p[0]) return;
+    const uint32_t kf = (uint32_t)(p[1 + i] - 1);  // the first of the three bins
     const int64_t b = off[c], e = off[c + 1];
+    constexpr int U = kExactSamples / 32;
     float2 s = make_float2(0.f, 0.f);
     for (int64_t j0 = b; j0 < e; j0 += kExactSamples) {
         const int n = (int)min((int64_t)kExactSamples, e - j0);
-#pragma unroll 4
-        for (int j = lane; j < n; j += 32) {
-            const float4 B = recB[j0 + j];
-            const float C = B.y, S = B.z;
-            float sn, cs;
-            __sincosf(phase_to_angle(top_phase(recA[j0 + j], k0)), &sn, &cs);
-            float2 y0 = make_float2(cs, sn);
-            float2 y1 = make_float2(fmaf(cs, C, -sn * S), fmaf(sn, C, cs * S));
-            const float2 cp2 = make_float2(B.w, B.w), cn2 = make_float2(-B.w, -B.w);
-#pragma unroll 1
-            for (int x = 2; x <= step; ++x) {
-                const float2 y2 = __ffma2_rn(((x - 1) & 1) ? cn2 : cp2, y1, y0);
-                y0 = y1;
-                y1 = y2;
+        // strips of the three bins: first .. first + 2 of k0 = F (kf / F), or partly the next one
+        for (uint32_t k0 = kf / F * F; k0 <= kf + 2; k0 += F) {
+            const int first = (int)kf - (int)k0, last = min(first + 2, F - 1);  // steps of the bins in this strip
+            float2 y0[U], y1[U];
+            float c2[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t j = min(j0 + lane + 32 * u, e - 1);
+                const float4 B = recB[j];
+                float sn, cs;
+                __sincosf(phase_to_angle(top_phase(recA[j], k0)), &sn, &cs);
+                y0[u] = make_float2(cs, sn);
+                y1[u] = make_float2(fmaf(cs, B.y, -sn * B.z), fmaf(sn, B.y, cs * B.z));
+                c2[u] = B.w;
             }
-            terms[warp][j] = step == 0 ? y0 : y1;
+            auto put = [&](int step, const float2 (&y)[U]) {
+                if (step < first || step > last) return;
+#pragma unroll
+                for (int u = 0; u < U; ++u) terms[warp][step - first][lane + 32 * u] = y[u];
+            };
+            put(0, y0);
+            put(1, y1);
+#pragma unroll 1
+            for (int x = 2; x <= last; ++x) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float cx = ((x - 1) & 1) ? -c2[u] : c2[u];
+                    const float2 y2 = __ffma2_rn(make_float2(cx, cx), y1[u], y0[u]);
+                    y0[u] = y1[u];
+                    y1[u] = y2;
+                }
+                put(x, y1);
+            }
         }
         __syncwarp();
-        if (lane == 0) {
+        if (lane < 3) {
+            const float2* y = terms[warp][lane];
             int j = 0;
             for (; j + 8 <= n; j += 8) {
                 float4 v[4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) v[x] = *reinterpret_cast<const float4*>(&terms[warp][j + 2 * x]);
+                for (int x = 0; x < 4; ++x) v[x] = *reinterpret_cast<const float4*>(&y[j + 2 * x]);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     s = __fadd2_rn(s, make_float2(v[x].x, v[x].y));
                     s = __fadd2_rn(s, make_float2(v[x].z, v[x].w));
                 }
             }
-            for (; j < n; ++j) s = __fadd2_rn(s, terms[warp][j]);
+            for (; j < n; ++j) s = __fadd2_rn(s, y[j]);
         }
         __syncwarp();
     }
-    if (lane == 0) {
+    if (lane < 3) {
         const float inv = 1.f / ((float)(e - b) * (float)(e - b));
         const float2 z = s;
-        peak_w[(size_t)c * (3 * kWindowPeaks) + i] = (z.x * z.x + z.y * z.y) * inv;
+        peak_w[(size_t)c * (3 * kWindowPeaks) + 3 * i + lane] = (z.x * z.x + z.y * z.y) * inv;
     }
 }
 
@@ -466,40 +502,46 @@ features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, c
         wm[warp * 8 + r] = m;
     });
     __syncthreads();
-    if (tid == 0) {
-        float fv[8];
-        int fm[8];
+    if (tid < 32) {
+        // the warps' lists, then one output a lane: 11 logarithms and as many
+        // divisions in FP64 take one thread longer than a pass over the gaps
+        __shared__ float fv[8];
+        __shared__ int fm[8];
+        const bool has = tid < (nt >> 5);
+#pragma unroll
         for (int r = 0; r < 8; ++r) {
-            fv[r] = -1.f;
-            fm[r] = 0x7fffffff;
+            tv[r] = has ? wv[tid * 8 + r] : -1.f;
+            tm[r] = has ? wm[tid * 8 + r] : 0x7fffffff;
         }
-        for (int i = 0; i < (nt >> 5) * 8; ++i)
-            if (wv[i] >= 0.f) top8_insert(fv, fm, wv[i], wm[i]);
+        warp_top8(tv, tm, [&](int r, float v, int m) {
+            fv[r] = v;
+            fm[r] = m;
+        });
+        __syncwarp();
         float* o = feat + (size_t)c * 32;
-        const float nanv = __int_as_float(0x7fc00000);
         if (unsorted || !(T > 0.0) || M < 1) {
-            for (int i = 0; i < 32; ++i) o[i] = nanv;
-            atomicOr(status, kStatusNonFinite);
+            o[tid] = __int_as_float(0x7fc00000);
+            if (tid == 0) atomicOr(status, kStatusNonFinite);
             return;
         }
-        const double meanGap = T / (double)M;
-        o[0] = (float)log((double)n);
-        o[1] = (float)log(T);
-        o[2] = (float)log((double)nf);
-        o[3] = (float)log(1.0 / (df * T));
-        o[4] = (float)log(f_max * T / (double)n);
-        o[5] = (float)log1p(f0 / df);
-        for (int i = 0; i < 5; ++i) o[6 + i] = (float)log(fmax((double)q(i), 1e-12 * T) / meanGap);
-        o[11] = (float)(s2 / T);
-        o[12] = (float)(s10 / T);
-        o[13] = (float)(s100 / T);
-        o[14] = (float)(mx / T);
-        o[15] = (float)(cnt2 / (double)M);
-        for (int r = 0; r < 8; ++r) {
-            const bool ok = fv[r] >= 0.f;
-            o[16 + r] = ok ? fv[r] : 0.f;
-            o[24 + r] = ok ? (float)((double)(fm[r] + 1) * df / f_max) : 0.f;
-        }
+        // lane 0 .. 5: log n, log T, log N_f, log 1/(df T), log f_max T / n, log(1 + f0 / df);
+        // 6 .. 10: log gap quantile / mean gap; 11 .. 15: shares; 16 .. 23: heights; 24 .. 31: places
+        const int r = tid & 7;
+        const bool ok = fv[r] >= 0.f;
+        double num = 1.0, den = 1.0;
+        if (tid == 0) num = (double)n;
+        else if (tid == 1) num = T;
+        else if (tid == 2) num = (double)nf;
+        else if (tid == 3) den = df * T;
+        else if (tid == 4) num = f_max * T, den = (double)n;
+        else if (tid == 5) num = f0, den = df;
+        else if (tid <= 10) num = fmax((double)qsel[tid - 6], 1e-12 * T), den = T / (double)M;
+        else if (tid <= 14) num = tid == 11 ? s2 : tid == 12 ? s10 : tid == 13 ? s100 : mx, den = T;
+        else if (tid == 15) num = cnt2, den = (double)M;
+        else if (tid >= 24) num = ok ? (double)(fm[r] + 1) * df : 0.0, den = f_max;
+        const double x = num / den;
+        o[tid] = tid == 5 ? (float)log1p(x) : tid <= 10 ? (float)log(x) : tid <= 15 || (tid >= 24 && ok) ? (float)x
+                 : ok && tid < 24 ? fv[r] : 0.f;
     }
 }
 
@@ -549,7 +591,7 @@ cudaError_t launch_window_peaks(int n_patterns, const double* t, const int64_t* 
 cudaError_t launch_window_exact(int F, int n_patterns, const int64_t* off, const uint4* recA, const float4* recB,
                                 const int* peaks, float* peak_w, cudaStream_t st) {
     if (F != 24) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)n_patterns, (3 * kWindowPeaks + kExactWarps - 1) / kExactWarps);
+    dim3 grid((unsigned)n_patterns, (kWindowPeaks + kExactWarps - 1) / kExactWarps);
     window_exact_kernel<24><<<grid, 32 * kExactWarps, 0, st>>>(off, recA, recB, peaks, peak_w);
     return cudaGetLastError();
 }
