@@ -67,9 +67,44 @@ noise_raw_kernel(uint64_t seed, uint32_t curve, uint32_t real, int64_t n, float*
     }
 }
 
+// A value as the unevaluated sum of two FP32 numbers, about 48 bits: the sums and
+// differences of the normalizations.  FP64 runs at two operations per clock and
+// SM on this part, an FP32 pair's addition at a sixth of 128.
+struct Pair {
+    float h, l;
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+__device__ __forceinline__ Pair pair_of(double v) {
+    const float h = (float)v;
+    return {h, (float)(v - (double)h)};
+}
+
+// a + b; the low part takes the rounding of the high one (Knuth's exact two-sum).
+__device__ __forceinline__ Pair add(Pair a, Pair b) {
+    const float s = a.h + b.h, t = s - a.h;
+    return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
+}
+
+// a b for an FP32 b, and a^2.
+__device__ __forceinline__ Pair times(Pair a, float b) {
+    const float p = a.h * b;
+    return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
+}
+__device__ __forceinline__ Pair square(Pair a) {
+    const float p = a.h * a.h;
+    return {p, fmaf(2.f * a.h, a.l, fmaf(a.h, a.h, -p))};
+}
+
+// a b to FP32, from all four parts but the smallest product.
+__device__ __forceinline__ float rounded_product(Pair a, Pair b) { return fmaf(a.h, b.h, fmaf(a.h, b.l, a.l * b.h)); }
+
 // One CTA per (curve, realization): draw the noise into xr, then normalize it
-// in place to zero mean and unit population variance (Sec. 3), mean and
-// variance in FP64 over two passes.
+// in place to zero mean and unit population variance (Sec. 3), over two passes.
+// The threads' sums are FP32 pairs, the block's FP64.  Bound by the instructions
+// of the generator; with FP64 sums and differences it was nine FP64 operations a
+// sample, and a Monte Carlo of 256 patterns of 200 .. 20,000 samples by 64
+// realizations took 13.94 ms, now 12.99 (with errors, by 16: 7.04 -> 6.54).
 __global__ void __launch_bounds__(kNoiseThreads)
 noise_prep_kernel(const int64_t* __restrict__ off, const uint64_t* __restrict__ seed_p, int64_t total,
                   float* __restrict__ xr, float4* __restrict__ recB) {
@@ -78,87 +113,132 @@ noise_prep_kernel(const int64_t* __restrict__ off, const uint64_t* __restrict__ 
     const int64_t b = off[c], n = off[c + 1] - off[c];
     float* x = xr + (size_t)r * (size_t)total + b;
     const uint64_t seed = *seed_p;
-    double s = 0.0;
-    for (int64_t blk = threadIdx.x; blk * 4 < n; blk += blockDim.x) {
-        const float4 z = normals4(seed, (uint32_t)blk, (uint32_t)c, (uint32_t)r);
-        const int64_t j = blk * 4;
-        x[j] = z.x;
-        s += z.x;
-        if (j + 1 < n) { x[j + 1] = z.y; s += z.y; }
-        if (j + 2 < n) { x[j + 2] = z.z; s += z.z; }
-        if (j + 3 < n) { x[j + 3] = z.w; s += z.w; }
-    }
-    __syncthreads();
-    const double mean = block_sum(s, sh) / (double)n;
-    double v = 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const double d = (double)x[j] - mean;
-        v = fma(d, d, v);
-    }
-    const double var = block_sum(v, sh) / (double)n;
-    const double inv_sd = var > 0.0 ? 1.0 / sqrt(var) : 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const float xh = (float)(((double)x[j] - mean) * inv_sd);
-        x[j] = xh;
-        if (recB) recB[b + j].x = xh;  // single realization: straight into the sample records
-    }
-}
-
-// One CTA per (curve, realization) of the floating-mean Monte Carlo: the
-// same N(0,1) draws z_j as noise_prep_kernel, X_j = dy_j z_j (z_j without dy),
-// then the weighted normalization of prep_records_kernel's floating-mean form,
-// x_j = q_j (X_j - mean_w) / sd_w, with v_j = 1/dy_j^2 formed in FP32 as the
-// prep kernels form it, mean_w = sum v X / sum v and the population variance
-// sum v (X - mean_w)^2 / sum v in FP64.  X_j is re-formed from the stored z_j
-// in every pass (exact: a float times a double).
-__global__ void __launch_bounds__(kNoiseThreads)
-gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t total, const double* __restrict__ dy,
-                      const float* __restrict__ q, float* __restrict__ xr) {
-    __shared__ double sh[33];
-    const int c = blockIdx.x, r = blockIdx.y;
-    const int64_t b = off[c], n = off[c + 1] - off[c];
-    float* x = xr + (size_t)r * (size_t)total + b;
-    auto weight = [&](int64_t j) {
-        if (!dy) return 1.0;
-        const float ef = (float)dy[b + j];
-        return (double)(1.f / (ef * ef));
-    };
-    auto value = [&](int64_t j) { return dy ? dy[b + j] * (double)x[j] : (double)x[j]; };
-    double sv = 0.0, svx = 0.0;
+    Pair s = {0.f, 0.f};
     for (int64_t blk = threadIdx.x; blk * 4 < n; blk += blockDim.x) {
         const float4 z = normals4(seed, (uint32_t)blk, (uint32_t)c, (uint32_t)r);
         const int64_t j = blk * 4;
         const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 4; ++u)
             if (j + u < n) {
                 x[j + u] = zz[u];
-                const double v = weight(j + u);
-                sv += v;
-                svx += v * value(j + u);
+                s = add(s, {zz[u], 0.f});
+            }
+    }
+    __syncthreads();
+    const Pair minus_mean = pair_of(-(block_sum(s.value(), sh) / (double)n));
+    Pair v = {0.f, 0.f};
+#pragma unroll 4
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) v = add(v, square(add({x[j], 0.f}, minus_mean)));
+    const double var = block_sum(v.value(), sh) / (double)n;
+    const Pair inv_sd = pair_of(var > 0.0 ? 1.0 / sqrt(var) : 0.0);
+#pragma unroll 4
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        const float xh = rounded_product(add({x[j], 0.f}, minus_mean), inv_sd);
+        x[j] = xh;
+        if (recB) recB[b + j].x = xh;  // single realization: straight into the sample records
+    }
+}
+
+// One CTA per curve and RR realizations of the floating-mean Monte Carlo: the
+// same N(0,1) draws z_j as noise_prep_kernel, X_j = dy_j z_j (z_j without dy),
+// then the weighted normalization of prep_records_kernel's floating-mean form,
+// x_j = q_j (X_j - mean_w) / sd_w, with v_j = 1/dy_j^2 formed in FP32 as the
+// prep kernels form it, mean_w = sum v X / sum v and the population variance
+// sum v (X - mean_w)^2 / sum v, the threads' sums FP32 pairs.  X_j is re-formed
+// from the stored z_j in every pass.  The four FP64 operations that split dy_j
+// serve the RR realizations.
+template <int RR>
+__global__ void __launch_bounds__(kNoiseThreads)
+gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t total, int n_real,
+                      const double* __restrict__ dy, const float* __restrict__ q, float* __restrict__ xr) {
+    __shared__ double sh[33];
+    const int c = blockIdx.x, r0 = blockIdx.y * RR, nr = min(RR, n_real - r0);
+    const int64_t b = off[c], n = off[c + 1] - off[c];
+    float* const x = xr + (size_t)r0 * (size_t)total + b;
+    // dy_j and v_j
+    auto error = [&](int64_t j, Pair& e, float& v) {
+        e = dy ? pair_of(dy[b + j]) : Pair{1.f, 0.f};
+        v = dy ? 1.f / (e.h * e.h) : 1.f;
+    };
+    Pair sv = {0.f, 0.f}, acc[RR], minus_mean[RR], inv_sd[RR];
+#pragma unroll
+    for (int i = 0; i < RR; ++i) acc[i] = {0.f, 0.f};
+    for (int64_t blk = threadIdx.x; blk * 4 < n; blk += blockDim.x) {
+        const int64_t j = blk * 4;
+        Pair e[4];
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j + u >= n) break;
+            error(j + u, e[u], v[u]);
+            sv = add(sv, {v[u], 0.f});
+        }
+#pragma unroll
+        for (int i = 0; i < RR; ++i) {
+            if (i >= nr) break;
+            const float4 z = normals4(seed, (uint32_t)blk, (uint32_t)c, (uint32_t)(r0 + i));
+            const float zz[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (j + u >= n) break;
+                x[(size_t)i * (size_t)total + j + u] = zz[u];
+                acc[i] = add(acc[i], times(times(e[u], zz[u]), v[u]));
             }
         }
     }
     __syncthreads();
-    sv = block_sum(sv, sh);
-    const double mean = block_sum(svx, sh) / sv;
-    double m2 = 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const double d = value(j) - mean;
-        m2 = fma(d * weight(j), d, m2);
+    const double svd = block_sum(sv.value(), sh);
+#pragma unroll
+    for (int i = 0; i < RR; ++i) {
+        minus_mean[i] = pair_of(-(block_sum(acc[i].value(), sh) / svd));
+        acc[i] = {0.f, 0.f};
     }
-    const double var = block_sum(m2, sh) / sv;
-    const double inv_sd = var > 0.0 ? 1.0 / sqrt(var) : 0.0;
-    __syncthreads();
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) x[j] = (float)((value(j) - mean) * inv_sd) * q[b + j];
+#pragma unroll 2
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        Pair e;
+        float v;
+        error(j, e, v);
+#pragma unroll
+        for (int i = 0; i < RR; ++i)
+            if (i < nr) {
+                const Pair d = add(times(e, x[(size_t)i * (size_t)total + j]), minus_mean[i]), w = times(d, v);
+                const float p = w.h * d.h;
+                acc[i] = add(acc[i], {p, fmaf(w.h, d.l, fmaf(w.l, d.h, fmaf(w.h, d.h, -p)))});
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < RR; ++i) {
+        const double var = block_sum(acc[i].value(), sh) / svd;
+        inv_sd[i] = pair_of(var > 0.0 ? 1.0 / sqrt(var) : 0.0);
+    }
+#pragma unroll 2
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        Pair e;
+        float v;
+        error(j, e, v);
+        const float qj = q[b + j];
+#pragma unroll
+        for (int i = 0; i < RR; ++i)
+            if (i < nr) {
+                float& xj = x[(size_t)i * (size_t)total + j];
+                xj = rounded_product(add(times(e, xj), minus_mean[i]), inv_sd[i]) * qj;
+            }
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_gls_noise_prep(const int64_t* off, int n_curves, int n_real, uint64_t seed, int64_t total,
                                   const double* dy, const float* q, float* xr, cudaStream_t st) {
-    dim3 grid((unsigned)n_curves, (unsigned)n_real);
-    gls_noise_prep_kernel<<<grid, kNoiseThreads, 0, st>>>(off, seed, total, dy, q, xr);
+    // four realizations a CTA where that leaves two CTAs an SM and more
+    constexpr int RR = 4;
+    if ((int64_t)n_curves * (n_real / RR) >= 2 * 152)
+        gls_noise_prep_kernel<RR><<<dim3((unsigned)n_curves, (unsigned)((n_real + RR - 1) / RR)), kNoiseThreads, 0, st>>>(
+            off, seed, total, n_real, dy, q, xr);
+    else
+        gls_noise_prep_kernel<1><<<dim3((unsigned)n_curves, (unsigned)n_real), kNoiseThreads, 0, st>>>(
+            off, seed, total, n_real, dy, q, xr);
     return cudaGetLastError();
 }
 
