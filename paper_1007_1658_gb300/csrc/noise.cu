@@ -12,6 +12,7 @@
 #include <cfloat>
 
 #include "lsp_kernels.cuh"
+#include "pair.cuh"
 #include "philox.cuh"
 
 namespace lsp {
@@ -19,6 +20,8 @@ namespace {
 
 constexpr int kNoiseThreads = 256;
 
+using dev::Pair;
+using dev::pair_of;
 using dev::philox4x32_10;
 
 __device__ __forceinline__ float unit_uniform(uint32_t w) { return (float)(2u * (w >> 9) + 1u) * 0x1p-24f; }
@@ -67,38 +70,6 @@ noise_raw_kernel(uint64_t seed, uint32_t curve, uint32_t real, int64_t n, float*
     }
 }
 
-// A value as the unevaluated sum of two FP32 numbers, about 48 bits: the sums and
-// differences of the normalizations.  FP64 runs at two operations per clock and
-// SM on this part, an FP32 pair's addition at a sixth of 128.
-struct Pair {
-    float h, l;
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
-
-__device__ __forceinline__ Pair pair_of(double v) {
-    const float h = (float)v;
-    return {h, (float)(v - (double)h)};
-}
-
-// a + b; the low part takes the rounding of the high one (Knuth's exact two-sum).
-__device__ __forceinline__ Pair add(Pair a, Pair b) {
-    const float s = a.h + b.h, t = s - a.h;
-    return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
-}
-
-// a b for an FP32 b, and a^2.
-__device__ __forceinline__ Pair times(Pair a, float b) {
-    const float p = a.h * b;
-    return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
-}
-__device__ __forceinline__ Pair square(Pair a) {
-    const float p = a.h * a.h;
-    return {p, fmaf(2.f * a.h, a.l, fmaf(a.h, a.h, -p))};
-}
-
-// a b to FP32, from all four parts but the smallest product.
-__device__ __forceinline__ float rounded_product(Pair a, Pair b) { return fmaf(a.h, b.h, fmaf(a.h, b.l, a.l * b.h)); }
-
 // One CTA per (curve, realization): draw the noise into xr, then normalize it
 // in place to zero mean and unit population variance (Sec. 3), over two passes.
 // The threads' sums are FP32 pairs, the block's FP64.  Bound by the instructions
@@ -122,19 +93,22 @@ noise_prep_kernel(const int64_t* __restrict__ off, const uint64_t* __restrict__ 
         for (int u = 0; u < 4; ++u)
             if (j + u < n) {
                 x[j + u] = zz[u];
-                s = add(s, {zz[u], 0.f});
+                s = s + Pair{zz[u], 0.f};
             }
     }
     __syncthreads();
     const Pair minus_mean = pair_of(-(block_sum(s.value(), sh) / (double)n));
     Pair v = {0.f, 0.f};
 #pragma unroll 4
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) v = add(v, square(add({x[j], 0.f}, minus_mean)));
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        const Pair d = Pair{x[j], 0.f} + minus_mean;
+        v = v + d * d;
+    }
     const double var = block_sum(v.value(), sh) / (double)n;
     const Pair inv_sd = pair_of(var > 0.0 ? 1.0 / sqrt(var) : 0.0);
 #pragma unroll 4
     for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const float xh = rounded_product(add({x[j], 0.f}, minus_mean), inv_sd);
+        const float xh = rounded_product(Pair{x[j], 0.f} + minus_mean, inv_sd);
         x[j] = xh;
         if (recB) recB[b + j].x = xh;  // single realization: straight into the sample records
     }
@@ -172,7 +146,7 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
         for (int u = 0; u < 4; ++u) {
             if (j + u >= n) break;
             error(j + u, e[u], v[u]);
-            sv = add(sv, {v[u], 0.f});
+            sv = sv + Pair{v[u], 0.f};
         }
 #pragma unroll
         for (int i = 0; i < RR; ++i) {
@@ -183,7 +157,7 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
             for (int u = 0; u < 4; ++u) {
                 if (j + u >= n) break;
                 x[(size_t)i * (size_t)total + j + u] = zz[u];
-                acc[i] = add(acc[i], times(times(e[u], zz[u]), v[u]));
+                acc[i] = acc[i] + e[u] * zz[u] * v[u];
             }
         }
     }
@@ -202,9 +176,8 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
 #pragma unroll
         for (int i = 0; i < RR; ++i)
             if (i < nr) {
-                const Pair d = add(times(e, x[(size_t)i * (size_t)total + j]), minus_mean[i]), w = times(d, v);
-                const float p = w.h * d.h;
-                acc[i] = add(acc[i], {p, fmaf(w.h, d.l, fmaf(w.l, d.h, fmaf(w.h, d.h, -p)))});
+                const Pair d = e * x[(size_t)i * (size_t)total + j] + minus_mean[i];
+                acc[i] = acc[i] + d * v * d;
             }
     }
 #pragma unroll
@@ -222,7 +195,7 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
         for (int i = 0; i < RR; ++i)
             if (i < nr) {
                 float& xj = x[(size_t)i * (size_t)total + j];
-                xj = rounded_product(add(times(e, xj), minus_mean[i]), inv_sd[i]) * qj;
+                xj = rounded_product(e * xj + minus_mean[i], inv_sd[i]) * qj;
             }
     }
 }

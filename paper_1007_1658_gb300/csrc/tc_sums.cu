@@ -29,6 +29,7 @@
 // What bounds it: with cols = 256 the three MMAs of 16 samples take 390 cycles
 // (24 a sample for 32,768 terms), the operands 128 complex values a sample and CTA.
 #include "ls_device.cuh"
+#include "pair.cuh"
 #include "tc_device.cuh"
 #include "tc_sums.cuh"
 
@@ -566,21 +567,23 @@ constexpr float kGlsRefine = 0x1p-5f;
 // root and three of its four divisions cancel.  With M = W - C^2 (= A + iB, the
 // centred CC - SS + 2i CS) and T = 1 - |C|^2 (CC + SS),
 //     p = 2 (|Z|^2 T - Re(conj(M) Z^2)) / (T^2 - |M|^2).
-// FP64 but for the reciprocal's seed: one Newton step takes FP32's 2^-24 to
-// 2^-47 (25 FP64 operations instead of ~150).
+// In FP32 pairs, whose 2^-48 the differences leave enough of: D >= T / 8 >= 1/64
+// where the result is used.  The quotient is corrected once by its remainder.
 // *ill: the smaller eigenvalue, between (T^2 - |M|^2) / 4T and / 2T, may lie
-// below kGlsRefine.
-__device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, double n, bool* ill) {
-    const double zx = Zf.x, zy = Zf.y, cx = Cf.x, cy = Cf.y;
-    const double A = fma(cy, cy, fma(-cx, cx, (double)Wf.x)), B = fma(-2.0 * cx, cy, (double)Wf.y);
-    const double T = fma(-cy, cy, fma(-cx, cx, 1.0));
-    const double D = fma(-B, B, fma(-A, A, T * T));
-    const double sx = zx * zx, sy = zy * zy;
-    const double num = fma(-B, 2.0 * zx * zy, fma(-A, sx - sy, T * (sx + sy)));
-    *ill = !(D >= 4.0 * kGlsRefine * T);
-    const double r0 = (double)(1.f / (float)D);
-    const double r = fma(r0, fma(-D, r0, 1.0), r0);
-    return fmaxf((float)(n * num * r), 0.f);
+// below kGlsRefine.  n: the sample count.
+__device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, dev::Pair n, bool* ill) {
+    using dev::Pair;
+    using dev::product;
+    const Pair cx2 = product(Cf.x, Cf.x), cy2 = product(Cf.y, Cf.y);
+    const Pair A = Pair{Wf.x, 0.f} + (cy2 + -cx2), B = Pair{Wf.y, 0.f} + product(-2.f * Cf.x, Cf.y);
+    const Pair T = Pair{1.f, 0.f} + -(cx2 + cy2);
+    const Pair D = T * T + -(A * A + B * B);
+    const Pair sx = product(Zf.x, Zf.x), sy = product(Zf.y, Zf.y);
+    const Pair num = T * (sx + sy) + -(A * (sx + -sy) + B * product(2.f * Zf.x, Zf.y));
+    *ill = !(D.h + D.l >= (float)(4.0 * kGlsRefine) * (T.h + T.l));
+    const float r = 1.f / D.h, q = num.h * r;
+    const float rest = (fmaf(-q, D.h, num.h) + num.l) - q * D.l;
+    return fmaxf(rounded_product(Pair{q, rest * r}, n), 0.f);
 }
 
 // Sums over samples b + i0, b + i0 + step, ... < b + n at frequency k from which
@@ -713,8 +716,8 @@ __global__ void __launch_bounds__(kFinThreads) tc_final_kernel(const TcArgs a, c
                 const size_t at[3] = {at_d + col, at_w + col, at_c + col};
                 tile_sums<3>(a, q, at, hb, zp, zm);
                 bool lp, lm;
-                vp = gls_power(zp[0], zp[2], zp[1], (double)n, &lp);
-                vm = gls_power(zm[0], zm[2], zm[1], (double)n, &lm);
+                vp = gls_power(zp[0], zp[2], zp[1], dev::pair_of((double)n), &lp);
+                vm = gls_power(zm[0], zm[2], zm[1], dev::pair_of((double)n), &lm);
 #pragma unroll 1
                 for (int s = 0; s < 2; ++s) {
                     const int64_t k = s ? kp : km;
