@@ -18,7 +18,7 @@
 // With work enough the window comes from the tensor cores (tc_sums.cu), and the
 // strip kernel's values are formed only at the few bins that can be among its 8
 // highest maxima (window_peaks_kernel, window_exact_kernel): the features keep
-// their bits; 256 patterns of up to 20,000 samples, the call 3.4 ms -> 1.4.
+// their bits; 256 patterns of up to 20,000 samples, the call 3.4 ms -> 1.1.
 #include <algorithm>
 #include <cfloat>
 
@@ -35,10 +35,9 @@ constexpr int kSortMaxGaps = 32768;  // gaps held in shared memory (128 KB); mor
 // The five cadence order statistics sorted(gaps)[k[i]], without sorting: an
 // MSB-first radix select on the FP32 bit patterns of the gaps (ordered as the
 // values, gaps being >= 0), 8 bits per pass and the five ranks at once; key_at(i)
-// is gap i's.  Each warp adds to the five 256-bin histograms once per distinct
-// bin (__match_any_sync), so gaps that share their leading bits do not serialize
-// on one counter; ranks whose leading bits a warp's gaps do not have cost it one
-// vote.  hist holds 5 x 256 counters; out[i] receives the value of rank k[i].
+// is gap i's.  A warp whose gaps all fall into one bin adds to it once, so the
+// equal gaps of an even cadence do not serialize on one counter; ranks whose
+// leading bits a warp's gaps do not have cost it one vote.  hist holds 5 x 256 counters; out[i] receives the value of rank k[i].
 template <class Key>
 __device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigned* hist, float* out) {
     __shared__ unsigned s_prefix[5], s_rank[5];
@@ -54,7 +53,7 @@ __device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigne
         unsigned prefix[5];
 #pragma unroll
         for (int q = 0; q < 5; ++q) prefix[q] = s_prefix[q];
-        // the whole warp steps together so that every lane takes part in the match
+        // the whole warp steps together so that every lane takes part in the votes
         for (int base = tid - lane; base < M; base += nt) {
             const int i = base + lane;
             unsigned key = 0u;
@@ -64,9 +63,15 @@ __device__ void select_gap_ranks(Key&& key_at, int M, const int (&k)[5], unsigne
             for (int q = 0; q < 5; ++q) {
                 if (q && !mask) break;  // the first pass counts the same for all five
                 const int mine = (i < M && (key & mask) == prefix[q]) ? bin : -1;
-                if (!__any_sync(0xffffffffu, mine >= 0)) continue;
-                const unsigned peers = __match_any_sync(0xffffffffu, mine);
-                if (mine >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[q * 256 + mine], (unsigned)__popc(peers));
+                const unsigned some = __ballot_sync(0xffffffffu, mine >= 0);
+                if (!some) continue;
+                const int lead = __ffs(some) - 1;
+                const unsigned peers = __ballot_sync(0xffffffffu, mine == __shfl_sync(0xffffffffu, mine, lead));
+                if (peers != some) {
+                    if (mine >= 0) atomicAdd(&hist[q * 256 + mine], 1u);
+                } else if (lane == lead) {
+                    atomicAdd(&hist[q * 256 + mine], (unsigned)__popc(some));
+                }
             }
         }
         __syncthreads();
@@ -193,82 +198,93 @@ ls_window_kernel(const BatchItem* __restrict__ items, int n_items, unsigned* __r
 
 // W of single bins as ls_window_kernel forms it, bit for bit.  There a thread
 // adds a strip's samples in order, one long chain; but only the additions are a
-// chain.  Here a warp takes a bin and its two neighbours: for 128 samples at a
-// time its lanes form the terms (the strip's seed and the steps up to the last of
-// them, four samples abreast; a second strip's where the three straddle one's
-// end), then three lanes add one bin's terms each, in order.
-constexpr int kExactWarps = 8, kExactSamples = 128;
+// chain.  Here a CTA takes a bin and its two neighbours: three warps form the
+// terms of the next 384 samples (the strip's seed and the steps up to the last of
+// the bins, four samples abreast; a second strip's where the three straddle one's
+// end) while three lanes of the first warp add this chunk's, a bin each, in order.
+// Bound by that chain, 20,000 additions for the largest patterns; with one warp
+// forming and adding in turn 256 patterns took 463 us here, now 154; 48 362, now 79.
+constexpr int kExactThreads = 128, kExactU = 4, kExactSamples = (kExactThreads - 32) * kExactU;
 template <int F>
-__global__ void __launch_bounds__(32 * kExactWarps)
+__global__ void __launch_bounds__(kExactThreads)
 window_exact_kernel(const int64_t* __restrict__ off, const uint4* __restrict__ recA, const float4* __restrict__ recB,
                     const int* __restrict__ peaks, float* __restrict__ peak_w) {
-    __shared__ __align__(16) float2 terms[kExactWarps][3][kExactSamples + 2];
-    const int c = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ __align__(16) float2 terms[2][3][kExactSamples + 2];
+    const int c = blockIdx.x, tid = threadIdx.x, i = blockIdx.y;
     const int* p = peaks + (size_t)c * (kWindowPeaks + 1);
-    const int i = (int)blockIdx.y * kExactWarps + warp;
     if (i >= p[0]) return;
     const uint32_t kf = (uint32_t)(p[1 + i] - 1);  // the first of the three bins
     const int64_t b = off[c], e = off[c + 1];
-    constexpr int U = kExactSamples / 32;
+    constexpr int U = kExactU;
     float2 s = make_float2(0.f, 0.f);
-    for (int64_t j0 = b; j0 < e; j0 += kExactSamples) {
-        const int n = (int)min((int64_t)kExactSamples, e - j0);
-        // strips of the three bins: first .. first + 2 of k0 = F (kf / F), or partly the next one
-        for (uint32_t k0 = kf / F * F; k0 <= kf + 2; k0 += F) {
-            const int first = (int)kf - (int)k0, last = min(first + 2, F - 1);  // steps of the bins in this strip
-            float2 y0[U], y1[U];
-            float c2[U];
+    const int chunks = (int)((e - b + kExactSamples - 1) / kExactSamples);
+    for (int x0 = 0; x0 <= chunks; ++x0) {
+        if (tid >= 32 && x0 < chunks) {
+            const int64_t j0 = b + (int64_t)x0 * kExactSamples;
+            const int at = tid - 32;
+            float2(&out)[3][kExactSamples + 2] = terms[x0 & 1];
+            uint4 A[U];
+            float4 B[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int64_t j = min(j0 + lane + 32 * u, e - 1);
-                const float4 B = recB[j];
-                float sn, cs;
-                __sincosf(phase_to_angle(top_phase(recA[j], k0)), &sn, &cs);
-                y0[u] = make_float2(cs, sn);
-                y1[u] = make_float2(fmaf(cs, B.y, -sn * B.z), fmaf(sn, B.y, cs * B.z));
-                c2[u] = B.w;
+                const int64_t j = min(j0 + at + (kExactThreads - 32) * u, e - 1);
+                A[u] = recA[j];
+                B[u] = recB[j];
             }
-            auto put = [&](int step, const float2 (&y)[U]) {
-                if (step < first || step > last) return;
-#pragma unroll
-                for (int u = 0; u < U; ++u) terms[warp][step - first][lane + 32 * u] = y[u];
-            };
-            put(0, y0);
-            put(1, y1);
-#pragma unroll 1
-            for (int x = 2; x <= last; ++x) {
+            // strips of the three bins: k0 = F (kf / F), and the next one where they reach into it
+            for (uint32_t k0 = kf / F * F; k0 <= kf + 2; k0 += F) {
+                const int first = (int)kf - (int)k0, last = min(first + 2, F - 1);  // the bins' steps in this strip
+                float2 y0[U], y1[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const float cx = ((x - 1) & 1) ? -c2[u] : c2[u];
-                    const float2 y2 = __ffma2_rn(make_float2(cx, cx), y1[u], y0[u]);
-                    y0[u] = y1[u];
-                    y1[u] = y2;
+                    float sn, cs;
+                    __sincosf(phase_to_angle(top_phase(A[u], k0)), &sn, &cs);
+                    y0[u] = make_float2(cs, sn);
+                    y1[u] = make_float2(fmaf(cs, B[u].y, -sn * B[u].z), fmaf(sn, B[u].y, cs * B[u].z));
                 }
-                put(x, y1);
+                auto put = [&](int step, const float2 (&y)[U]) {
+                    if (step < first || step > last) return;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) out[step - first][at + (kExactThreads - 32) * u] = y[u];
+                };
+                put(0, y0);
+                put(1, y1);
+#pragma unroll 1
+                for (int x = 2; x <= last; ++x) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const float cx = ((x - 1) & 1) ? -B[u].w : B[u].w;
+                        const float2 y2 = __ffma2_rn(make_float2(cx, cx), y1[u], y0[u]);
+                        y0[u] = y1[u];
+                        y1[u] = y2;
+                    }
+                    put(x, y1);
+                }
             }
         }
-        __syncwarp();
-        if (lane < 3) {
-            const float2* y = terms[warp][lane];
+        if (tid < 3 && x0) {
+            const int64_t j0 = b + (int64_t)(x0 - 1) * kExactSamples;
+            const int n = (int)min((int64_t)kExactSamples, e - j0);
+            const float2* y = terms[(x0 - 1) & 1][tid];
             int j = 0;
-            for (; j + 8 <= n; j += 8) {
-                float4 v[4];
+            for (; j + 16 <= n; j += 16) {
+                float4 v[8];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) v[x] = *reinterpret_cast<const float4*>(&y[j + 2 * x]);
+                for (int x = 0; x < 8; ++x) v[x] = *reinterpret_cast<const float4*>(&y[j + 2 * x]);
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < 8; ++x) {
                     s = __fadd2_rn(s, make_float2(v[x].x, v[x].y));
                     s = __fadd2_rn(s, make_float2(v[x].z, v[x].w));
                 }
             }
             for (; j < n; ++j) s = __fadd2_rn(s, y[j]);
         }
-        __syncwarp();
+        __syncthreads();
     }
-    if (lane < 3) {
+    if (tid < 3) {
         const float inv = 1.f / ((float)(e - b) * (float)(e - b));
         const float2 z = s;
-        peak_w[(size_t)c * (3 * kWindowPeaks) + 3 * i + lane] = (z.x * z.x + z.y * z.y) * inv;
+        peak_w[(size_t)c * (3 * kWindowPeaks) + 3 * i + tid] = (z.x * z.x + z.y * z.y) * inv;
     }
 }
 
@@ -591,8 +607,8 @@ cudaError_t launch_window_peaks(int n_patterns, const double* t, const int64_t* 
 cudaError_t launch_window_exact(int F, int n_patterns, const int64_t* off, const uint4* recA, const float4* recB,
                                 const int* peaks, float* peak_w, cudaStream_t st) {
     if (F != 24) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)n_patterns, (kWindowPeaks + kExactWarps - 1) / kExactWarps);
-    window_exact_kernel<24><<<grid, 32 * kExactWarps, 0, st>>>(off, recA, recB, peaks, peak_w);
+    dim3 grid((unsigned)n_patterns, kWindowPeaks);
+    window_exact_kernel<24><<<grid, kExactThreads, 0, st>>>(off, recA, recB, peaks, peak_w);
     return cudaGetLastError();
 }
 
