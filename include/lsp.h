@@ -195,7 +195,8 @@ lsp_status lsp_batch_gls(lsp_ctx *ctx, int32_t n_curves, const int64_t *t_off, c
  * frequency block) items; each (frequency, realization) is computed exactly
  * as the one-at-a-time kernel with the same strip length would.  Runs the
  * packed three-term strip (sin/cos mode AUTO or RECUR3_X2; other modes return
- * UNSUPPORTED).
+ * UNSUPPORTED).  Under AUTO with automatic groups, batches with work enough
+ * run on the tensor cores (as lsp_batch's), a realization's sums apart.
  * Pointers host or device; any host output makes the call blocking.
  * Errors: INVALID_ARG, NONFINITE, UNSUPPORTED, OOM, CUDA.
  */
@@ -292,8 +293,9 @@ lsp_status lsp_grid(double t_min, double t_max, int64_t N_t, double F_over, doub
  * re-seed length) and N_t splits on a synthetic series of this size, keep
  * only candidates within 2e-5 max P of the all-hardware-sin/cos result, and
  * remember the fastest for this (log2 N_t, log2 N_f) bucket: later calls with
- * LSP_SINCOS_AUTO and automatic F/split use it.  *chosen (may be NULL)
- * receives the winning options.  Blocks; allocates temporary buffers.
+ * LSP_SINCOS_AUTO and automatic F/split use it (in place of the tensor cores
+ * too, where the size would take them).  *chosen (may be NULL) receives the
+ * winning options.  Blocks; allocates temporary buffers.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 lsp_status lsp_autotune(lsp_ctx *ctx, int64_t N_t, int64_t N_f, lsp_options *chosen);

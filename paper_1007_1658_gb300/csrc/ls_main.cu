@@ -35,7 +35,8 @@
 //   RECUR3 x2 -- the same arithmetic in packed FP32x2 FMA (FFMA2), the
 //             (cos, sin) pair of a frequency in the two lanes: (XC, XS),
 //             (CC, CS) and the step one FFMA2 each per term, half the issue
-//             slots; sums bit-identical to RECUR3 at the same F.  The default.
+//             slots; sums bit-identical to RECUR3 at the same F.  The default
+//             of the calls that tc_sums.cu does not take.
 // NAIVE_FP32 -- the paper's own single-precision phase f*t - rintf(f*t)
 //             (Sec. 4.3), kept as a comparator.
 #include "ls_device.cuh"

@@ -105,8 +105,8 @@ MainShape lsp::host::choose_shape(const lsp_ctx* ctx, int64_t N, int64_t N_f) {
 // ceil(CTAs / slots) x chunk sample-steps, each costing (ops F + 16) issue
 // slots for every warp sharing a sub-partition; the partial sums of the
 // chunks are written and read back once (at ~4 TB/s).  Chunks stay within
-// kMaxChunk samples (precision) and above kMinChunk.  On the 100k x 200k
-// periodogram this picks 65 chunks over 7 waves (main kernel 3.74 ms) where
+// kMaxChunk samples (precision) and above kMinChunk.  On a 100k x 200k
+// periodogram by strips this picks 65 chunks over 7 waves (main kernel 3.74 ms) where
 // filling a single wave as fully as possible took 9 chunks (3.88 ms: 2,349 of
 // 2,432 slots busy).
 void lsp::host::finish_shape(const lsp_ctx* ctx, MainShape& s, int occ_in, int64_t N, int64_t N_f, int split,

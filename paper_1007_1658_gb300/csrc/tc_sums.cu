@@ -26,8 +26,10 @@
 // holds half of the rows of A and half of the columns of B, so its operands per
 // term are two thirds of a single CTA's, in the making and in shared memory.
 //
-// What bounds it: with cols = 256 the three MMAs of 16 samples take 390 cycles
-// (24 a sample for 32,768 terms), the operands 128 complex values a sample and CTA.
+// What bounds it: with cols = 256 the three MMAs of 16 samples take 390 cycles (24
+// a sample for 32,768 terms), the operands 128 complex values a sample and CTA.  A
+// unit of 128 samples takes a pair 3750 cycles, its MMAs alone 3120.  100,000
+// samples by 200,000 frequencies: this kernel 285 us, the FP32 strips 3605.
 #include "ls_device.cuh"
 #include "pair.cuh"
 #include "tc_device.cuh"
