@@ -52,9 +52,20 @@ def _peaks():
     if os.path.exists(p):
         with open(p) as fh:
             return json.load(fh), "measured"
-    return {"sm_max_mhz": 2070.0}, "fallback"
+    return {"sm_max_mhz": 2070.0, "bf16_tflops": 1900.0}, "fallback"
 
 
+def tensor_roof(sets, peaks, peak_src):
+    """(basis, terms/s) of the tensor-core sums: a term takes one complex product
+    of each set of values (data, window, weights) as 4 real multiply-adds for two
+    frequencies, three FP16 products each: 12 flops a set."""
+    flops = 12 * sets
+    tflops = float(peaks.get("bf16_tflops", 1900.0))
+    return ("tensor cores: %d flops per term (%d sets of sums, three 16-bit products) at %.0f TFLOP/s (%s bf16 burst)"
+            % (flops, sets, tflops, peak_src), tflops * 1e12 / flops)
+
+
+TENSOR_SOURCES = ("tc_sums.cu", "tc_sums.cuh", "tc_device.cuh")
 MAIN_SOURCES = ("ls_main.cu", "ls_device.cuh", "lsp_kernels.cuh")
 GLS_SOURCES = ("gls.cu", "ls_device.cuh", "lsp_kernels.cuh")
 
@@ -245,7 +256,8 @@ def run_gpu(args, rank, world, dist):
         return 0
     peaks, peak_src = _peaks()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    # the library's AUTO choice is the packed three-term strip
+    # the library's AUTO choice at this size is the tensor-core sums
+    tensor = not args.mode and not args.F
     mode = args.mode if args.mode else lsp.SINCOS_RECUR3_X2
     F = args.F if args.F else {lsp.SINCOS_MUFU: 8, lsp.SINCOS_RECUR: 16, lsp.SINCOS_RECUR3: 24,
                                lsp.SINCOS_RECUR3_X2: 24}[mode]
@@ -258,21 +270,25 @@ def run_gpu(args, rank, world, dist):
                                       "128/clk/SM", 128.0 / 6)}[mode]
     terms_per_clk = roof[2]
     peak = terms_per_clk * sms * peaks["sm_max_mhz"] * 1e6
+    basis = "%s: %.2f terms/clk/SM x %d SMs x %.0f MHz (%s sm_max_mhz)" % (roof[1], terms_per_clk, sms,
+                                                                         peaks["sm_max_mhz"], peak_src)
     achieved = terms / (float(np.mean(main_ms)) * 1e-3)
     kernel = "ls_main_kernel<%d,%d>" % (F, {1: 1, 2: 2, 3: 4, 4: 5}[mode])
+    if tensor:
+        kernel, (basis, peak) = "tc_sums_kernel", tensor_roof(2, peaks, peak_src)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD, "N_t": int(c.t.size), "N_f": int(c.nf), "terms_per_step": terms,
-                   "sincos": {1: "mufu", 2: "recurrence", 3: "three-term recurrence",
-                              4: "three-term recurrence, packed FP32x2"}[mode], "F": F,
+                   "sincos": "tensor-core sums" if tensor else {1: "mufu", 2: "recurrence", 3: "three-term recurrence",
+                              4: "three-term recurrence, packed FP32x2"}[mode], "F": 0 if tensor else F,
                    "phase": "fixed64",
                    "l2": "flushed between steps (256 MB write)", "parallelism": "frequency shards x%d" % world},
-        "roofline": {"bound": "alu", "kernel": kernel, "achieved": achieved / 1e9, "peak": peak / 1e9,
-                     "unit": "Gterms/s", "frac": achieved / peak, "traffic": _recorded_traffic(kernel),
-                     "peak_basis": "%s: %.2f terms/clk/SM x %d SMs x %.0f MHz (%s sm_max_mhz)" % (
-                         roof[1], terms_per_clk, sms, peaks["sm_max_mhz"], peak_src),
+        "roofline": {"bound": "tensor" if tensor else "alu", "kernel": kernel, "achieved": achieved / 1e9,
+                     "peak": peak / 1e9, "unit": "Gterms/s", "frac": achieved / peak,
+                     "traffic": _recorded_traffic(kernel, files=TENSOR_SOURCES if tensor else MAIN_SOURCES),
+                     "peak_basis": basis,
                      "main_ms": float(np.mean(main_ms))},
         "e2e": None if e2e_val is None else {
             "value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": int(c.t.nbytes + c.X.nbytes),
@@ -342,9 +358,10 @@ def run_cadence_bench(torch, dev, stream, args, peaks, peak_src, sms, with_oracl
     out = {"workload": "cadence_65k: N_t = %d, N_f = %d (%.3g terms)" % (c.t.size, c.nf, terms)}
     res = {}
     with ClockSampler(dev.index or 0) as clk:
-        for name, opts, per_clk, basis in (
-                ("fixed64", dict(), 128.0 / 6, "FMA pipe, 6 ops/term"),
-                ("naive_fp32", dict(phase_mode=lsp.PHASE_NAIVE_FP32), 16.0 / 2, "SFU, 2 ops/term")):
+        for name, opts, (basis, peak) in (
+                ("fixed64", dict(), tensor_roof(2, peaks, peak_src)),
+                ("naive_fp32", dict(phase_mode=lsp.PHASE_NAIVE_FP32),
+                 ("SFU, 2 ops/term, %s sm_max_mhz" % peak_src, 16.0 / 2 * sms * peaks["sm_max_mhz"] * 1e6))):
             cctx = lsp.Context(dev.index or 0, stream=stream, timing=1, **opts)
             P_d = torch.empty(c.nf, dtype=torch.float32, device=dev)
             main = []
@@ -355,11 +372,10 @@ def run_cadence_bench(torch, dev, stream, args, peaks, peak_src, sms, with_oracl
             ms = _time_calls(torch, stream, fn, 2, max(3, args.steps // 2), flush)
             cctx.sync(120.0)
             main_ms = float(np.median(main[2:]))
-            peak = per_clk * sms * peaks["sm_max_mhz"] * 1e6
             res[name] = P_d.cpu().numpy().astype(np.float64)
             out[name] = {"ms": ms, "terms_per_s": terms / (ms * 1e-3), "main_ms": main_ms,
                          "frac_of_roof": terms / (main_ms * 1e-3) / peak,
-                         "roof": "%s, %s sm_max_mhz" % (basis, peak_src)}
+                         "roof": basis}
             cctx.close()
     out["clocks"] = clk.summary()
     if with_oracle:
@@ -498,7 +514,8 @@ def run_gls_bench(torch, dev, stream, args, peaks, peak_src, sms):
     P_d = torch.empty(c.nf, dtype=torch.float32, device=dev)
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device=dev)
     mode = args.mode if args.mode else lsp.SINCOS_RECUR3_X2
-    gctx = lsp.Context(dev.index or 0, stream=stream, timing=1, sincos_mode=mode,
+    tensor = not args.mode and args.F not in (8, 16)
+    gctx = lsp.Context(dev.index or 0, stream=stream, timing=1, sincos_mode=args.mode,
                        freqs_per_thread=args.F if args.F in (8, 16) else 0)
     F = args.F if args.F in (8, 16) else (8 if mode == lsp.SINCOS_MUFU else 16)
     steps = max(3, args.steps)
@@ -528,6 +545,10 @@ def run_gls_bench(torch, dev, stream, args, peaks, peak_src, sms):
     peak = roof[1] * sms * peaks["sm_max_mhz"] * 1e6
     achieved = terms / (float(np.mean(main_ms)) * 1e-3)
     kernel = "gls_main_kernel<%d,%d>" % (F, {1: 1, 2: 2, 3: 4, 4: 5}[mode])
+    basis = "%s: %.2f terms/clk/SM x %d SMs x %.0f MHz (%s sm_max_mhz)" % (roof[0], roof[1], sms,
+                                                                         peaks["sm_max_mhz"], peak_src)
+    if tensor:
+        kernel, (basis, peak) = "tc_sums_kernel", tensor_roof(3, peaks, peak_src)
     # many curves: the Monte-Carlo batch's 4096 sampling patterns as measured curves with errors
     b = synth.noise_batch(n_curves=args.batch_curves)
     rng = np.random.default_rng(17)
@@ -560,11 +581,11 @@ def run_gls_bench(torch, dev, stream, args, peaks, peak_src, sms):
                         % (c.t.size, c.nf),
             "batch": batch_line,
             "ms_per_call": step_ms, "terms_per_s": terms / (step_ms * 1e-3),
-            "roofline": {"bound": "alu", "kernel": kernel,
+            "roofline": {"bound": "tensor" if tensor else "alu", "kernel": kernel,
                          "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gterms/s", "frac": achieved / peak,
-                         "traffic": _recorded_traffic(kernel, "gls_main_gapped_100k_errors.md", GLS_SOURCES),
-                         "peak_basis": "%s: %.2f terms/clk/SM x %d SMs x %.0f MHz (%s sm_max_mhz)" % (
-                             roof[0], roof[1], sms, peaks["sm_max_mhz"], peak_src),
+                         "traffic": _recorded_traffic(kernel, "gls_main_gapped_100k_errors.md",
+                                                      TENSOR_SOURCES if tensor else GLS_SOURCES),
+                         "peak_basis": basis,
                          "main_ms": float(np.mean(main_ms))},
             "clocks": clk.summary()}
 
@@ -601,10 +622,11 @@ def mrhs_ops_per_term(R, n_real):
     return 2.0 + 4.0 / R
 
 
-def run_mrhs_bench(torch, dev, stream, n_patterns=256, n_real=64, groups=(1, 2, 4, 8), clk_sm=None):
+def run_mrhs_bench(torch, dev, stream, n_patterns=256, n_real=64, groups=(0, 1, 2, 4, 8), clk_sm=None):
     """Many realizations per pattern (the surrogate's training shape: 256
     noise_batch patterns x 64 realizations, one lsp_batch call) for each
-    multi-RHS group size; every result is bit-identical across group sizes.
+    multi-RHS group size (results bit-identical across group sizes) and for the
+    library's own choice (0, the tensor-core sums).
     With clk_sm (SMs x clock in Hz) each group also gets its FMA-pipe roof
     (128 lanes/clk/SM over mrhs_ops_per_term) and the fraction reached."""
     from paper_1007_1658_gb300 import lsp, synth
@@ -629,7 +651,7 @@ def run_mrhs_bench(torch, dev, stream, n_patterns=256, n_real=64, groups=(1, 2, 
         mctx.close()
         row = {"batch_rhs": rhs, "ms": ms, "periodograms_per_s": n_real * b.n / (ms * 1e-3),
                "terms_per_s": n_real * b.terms / (ms * 1e-3)}
-        if clk_sm:
+        if clk_sm and rhs:
             ops = mrhs_ops_per_term(min(rhs, n_real), n_real)
             row["ops_per_term"] = ops
             row["frac_of_roof"] = row["terms_per_s"] / (128.0 / ops * clk_sm)
@@ -729,7 +751,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--mode", type=int, default=0,
-                    help="sin/cos mode: 0 auto (= 4), 1 MUFU, 2 recurrence, 3 three-term recurrence, "
+                    help="sin/cos mode: 0 auto (tensor-core sums at these sizes), 1 MUFU, 2 recurrence, 3 three-term recurrence, "
                          "4 three-term recurrence in packed FP32x2")
     ap.add_argument("--F", type=int, default=0, help="frequencies per thread (0 = auto)")
     ap.add_argument("--ref-bins", type=int, default=2048, help="reference arm: oracle frequencies per step")
