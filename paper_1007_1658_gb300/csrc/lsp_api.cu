@@ -145,9 +145,11 @@ void lsp::host::finish_shape(const lsp_ctx* ctx, MainShape& s, int occ_in, int64
 }
 
 // Terms of a call from which the tensor cores run it.  Whole calls, strips
-// against tensor cores: 3000 x 6000 50.1 / 54.7 us, 5000 x 10,000 62.9 / 62.2,
-// 7000 x 14,000 77.9 / 67.8, 10,000 x 20,000 96.8 / 68.6; floating mean 5000 x
-// 10,000 84.3 / 85.0, 7000 x 14,000 97.2 / 91.8; 100,000 x 300 98.5 / 102.7.
+// against tensor cores: 4000 x 8000 55.9 / 60.1 us, 5000 x 10,000 61.6 / 66.1,
+// 6000 x 12,000 68.0 / 67.7, 7000 x 14,000 76.0 / 61.0, 10,000 x 20,000 94.4 / 63.0;
+// floating mean 5000 x 10,000 83.3 / 86.8, 6000 x 12,000 93.5 / 83.7.  Short curves on
+// long grids gain earlier (500 x 100,000 55.3 / 44.7), long ones on short grids
+// later (100,000 x 500 95.5 / 97.4).
 static constexpr double kTcMinTerms = 6e7;
 bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f) {
     const lsp_options& o = ctx->opt;
@@ -214,9 +216,8 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
 // A tile costs about one unit's time beside its units, so many short curves stay
 // with the strips; a few of them do not fill the GPU either way, and there a
 // strip's serial pass over its curve is the longer.  Whole calls, strips against
-// tensor cores: 8 curves of 100 .. 500 samples 126 / 86 us, 100 of them 133 / 108,
-// 100 x 8 realizations (900 tiles) 180 / 226; 100 x 8 of 200 .. 1500 samples 330 /
-// 305, of 400 .. 5000 samples 1704 / 516.
+// tensor cores: 8 curves of 100 .. 500 samples 124 / 83 us, 100 of them 132 / 109,
+// 100 of 50 .. 200 85 / 98, 100 x 8 realizations of 200 .. 1500 322 / 183.
 bool lsp::host::tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real) {
     double tiles = 0.0, units = 0.0, terms = 0.0;
     for (size_t c = 0; c < nf.size(); ++c) {

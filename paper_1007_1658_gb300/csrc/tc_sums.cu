@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(kFinThreads, FORM == kTcGls ? 2 : 4) tc_final_
     }
 }
 
-constexpr int kRefineThreads = 512;
+constexpr int64_t kRefineAlone = 4096;
 
 // s + c += t + d, s and t the leading parts (FP64 adds are slow on this part).
 __device__ __forceinline__ void add_pair(float& s, float& c, float t, float d) {
@@ -797,11 +797,15 @@ __device__ __forceinline__ void add_pair(float& s, float& c, float t, float d) {
 }
 
 // One cluster of CL CTAs per listed bin: its sums over all samples, then P.
-// A single curve lists a few bins of many samples (CL = 8: 100,000 samples in
-// one CTA are 40 us of arithmetic), a batch many bins of shorter curves (CL = 1).
-template <int CL>
-__global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs a, const TcFinal f) {
-    __shared__ float2 sh[kRefineThreads / 32][kMoments];
+// A single long curve lists a few bins of many samples (CL = 8: 100,000 samples in
+// one CTA are 40 us of arithmetic), a batch many bins of shorter curves (CL = 1),
+// and a single short curve far beyond its mean Nyquist frequency thousands of bins
+// with a sample or a few for each of 128 threads (500 samples, 100,000 frequencies
+// on a nightly cadence, the finalize stage: CL = 8 78 us, 128 threads 20; 20,000
+// samples, 2000 frequencies 31 and 68, 6000 by 12,000 31 and 39).
+template <int CL, int kThreads>
+__global__ void __launch_bounds__(kThreads) tc_refine_kernel(const TcArgs a, const TcFinal f) {
+    __shared__ float2 sh[kThreads / 32][kMoments];
     __shared__ float2 part[CL][kMoments];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0;
@@ -811,7 +815,7 @@ __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs 
         const int64_t b = a.off ? a.off[w.curve] : 0, n = a.off ? a.off[w.curve + 1] - b : a.n0;
         float s[kMoments] = {}, c[kMoments] = {};
         direct_gls(a, b, n, a.xr ? a.xr + (size_t)w.real * (size_t)a.total : nullptr, w.k,
-                   rank * kRefineThreads + (int)threadIdx.x, CL * kRefineThreads, s, c);
+                   rank * kThreads + (int)threadIdx.x, CL * kThreads, s, c);
         auto join = [&](int width) {
             for (int o = width / 2; o > 0; o >>= 1)
 #pragma unroll
@@ -827,11 +831,11 @@ __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs 
         if (warp == 0) {
 #pragma unroll
             for (int x = 0; x < kMoments; ++x) {
-                const float2 v = lane < kRefineThreads / 32 ? sh[lane][x] : make_float2(0.f, 0.f);
+                const float2 v = lane < kThreads / 32 ? sh[lane][x] : make_float2(0.f, 0.f);
                 s[x] = v.x;
                 c[x] = v.y;
             }
-            join(kRefineThreads / 32);
+            join(kThreads / 32);
         }
         if constexpr (CL > 1) {
             if (threadIdx.x == 0) {
@@ -863,8 +867,9 @@ __global__ void __launch_bounds__(kRefineThreads) tc_refine_kernel(const TcArgs 
 }  // namespace
 
 cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st) {
-    if (a.off) {
-        tc_refine_kernel<1><<<304, kRefineThreads, 0, st>>>(a, f);
+    if (a.off || a.n0 <= kRefineAlone) {
+        if (a.off) tc_refine_kernel<1, 512><<<304, 512, 0, st>>>(a, f);
+        else tc_refine_kernel<1, 128><<<152 * 8, 128, 0, st>>>(a, f);
         return cudaGetLastError();
     }
     cudaLaunchAttribute at;
@@ -873,11 +878,11 @@ cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st)
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(64);
-    cfg.blockDim = dim3(kRefineThreads);
+    cfg.blockDim = dim3(512);
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_refine_kernel<8>, a, f);
+    return cudaLaunchKernelEx(&cfg, tc_refine_kernel<8, 512>, a, f);
 }
 
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st) {
