@@ -769,7 +769,7 @@ def main():
     ap.add_argument("--batch-reps", type=int, default=3)
     ap.add_argument("--mrhs-patterns", type=int, default=256, help="multi-realization leg: sampling patterns")
     ap.add_argument("--mrhs-real", type=int, default=64, help="multi-realization leg: realizations per pattern")
-    ap.add_argument("--mrhs-groups", default="1,2,4,8", help="multi-realization leg: group sizes to time")
+    ap.add_argument("--mrhs-groups", default="0,1,2,4,8", help="multi-realization leg: group sizes to time")
     ap.add_argument("--no-mc", dest="mc", action="store_false",
                     help="skip the 4096-curve graph-vs-plain leg (keeps the multi-realization leg)")
     args = ap.parse_args()
