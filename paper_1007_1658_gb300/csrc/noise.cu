@@ -119,9 +119,11 @@ noise_prep_kernel(const int64_t* __restrict__ off, const uint64_t* __restrict__ 
 // then the weighted normalization of prep_records_kernel's floating-mean form,
 // x_j = q_j (X_j - mean_w) / sd_w, with v_j = 1/dy_j^2 formed in FP32 as the
 // prep kernels form it, mean_w = sum v X / sum v and the population variance
-// sum v (X - mean_w)^2 / sum v, the threads' sums FP32 pairs.  X_j is re-formed
-// from the stored z_j in every pass.  The four FP64 operations that split dy_j
-// serve the RR realizations.
+// sum v (X - mean_w)^2 / sum v, the threads' sums FP32 pairs but for sum v: errors
+// around 1e-19 (fluxes in cgs units) have weights of 1e38, which only FP64 can add
+// up; every other sum is of the size of dy, of 1/dy or of 1.  X_j is re-formed
+// from the stored z_j in every pass.  The four FP64 operations that split dy_j and
+// the one that adds v_j serve the RR realizations.
 template <int RR>
 __global__ void __launch_bounds__(kNoiseThreads)
 gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t total, int n_real,
@@ -133,9 +135,10 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
     // dy_j and v_j
     auto error = [&](int64_t j, Pair& e, float& v) {
         e = dy ? pair_of(dy[b + j]) : Pair{1.f, 0.f};
-        v = dy ? 1.f / (e.h * e.h) : 1.f;
+        v = dy ? dev::error_weight(e.h) : 1.f;
     };
-    Pair sv = {0.f, 0.f}, acc[RR], minus_mean[RR], inv_sd[RR];
+    double sv = 0.0;
+    Pair acc[RR], minus_mean[RR], inv_sd[RR];
 #pragma unroll
     for (int i = 0; i < RR; ++i) acc[i] = {0.f, 0.f};
     for (int64_t blk = threadIdx.x; blk * 4 < n; blk += blockDim.x) {
@@ -146,7 +149,7 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
         for (int u = 0; u < 4; ++u) {
             if (j + u >= n) break;
             error(j + u, e[u], v[u]);
-            sv = sv + Pair{v[u], 0.f};
+            sv += (double)v[u];
         }
 #pragma unroll
         for (int i = 0; i < RR; ++i) {
@@ -162,7 +165,7 @@ gls_noise_prep_kernel(const int64_t* __restrict__ off, uint64_t seed, int64_t to
         }
     }
     __syncthreads();
-    const double svd = block_sum(sv.value(), sh);
+    const double svd = block_sum(sv, sh);
 #pragma unroll
     for (int i = 0; i < RR; ++i) {
         minus_mean[i] = pair_of(-(block_sum(acc[i].value(), sh) / svd));

@@ -43,6 +43,15 @@ __device__ __forceinline__ Pair operator*(Pair a, Pair b) {
     return {p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
 }
 
+// 1 / e^2, a sample's weight from its error, in FP32 (FP64 division is slow on this
+// part).  Below 2^-60 e is scaled first: its square would be subnormal and short
+// of digits, the weight itself stays below 2^128 down to e = 2^-64.
+__device__ __forceinline__ float error_weight(float e) {
+    const bool tiny = fabsf(e) < 0x1p-60f;
+    const float m = tiny ? e * 0x1p62f : e, v = 1.f / (m * m);
+    return tiny ? v * 0x1p62f * 0x1p62f : v;
+}
+
 // a b to FP32.
 __device__ __forceinline__ float rounded_product(Pair a, Pair b) { return fmaf(a.h, b.h, fmaf(a.h, b.l, a.l * b.h)); }
 

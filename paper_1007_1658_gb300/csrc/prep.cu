@@ -8,6 +8,7 @@
 #include <cmath>
 
 #include "lsp_kernels.cuh"
+#include "pair.cuh"
 
 namespace lsp {
 namespace {
@@ -95,10 +96,8 @@ prep_stats_kernel(const double* __restrict__ t, const double* __restrict__ X,
         const double x = X ? X[j] : 0.0, tj = t[j];
         bad |= !(isfinite(x) && isfinite(tj));
         if (dy) {
-            // weights in FP32 (relative error ~1e-7; FP64 division is slow on this part)
             const double ej = dy[j];
-            const float ef = (float)ej;
-            const double wj = (double)(1.f / (ef * ef));
+            const double wj = (double)dev::error_weight((float)ej);
             badw |= !(isfinite(ej) && ej > 0.0 && isfinite(wj) && wj > 0.0);
             ws += wj;
             s += wj * x;
@@ -119,8 +118,7 @@ prep_stats_kernel(const double* __restrict__ t, const double* __restrict__ X,
         for (int64_t j = sb + threadIdx.x; j < se; j += blockDim.x) {
             const double d = X[j] - mean_g;
             if (dy) {
-                const float ef = (float)dy[j];
-                v = fma(d * (double)(1.f / (ef * ef)), d, v);
+                v = fma(d * (double)dev::error_weight((float)dy[j]), d, v);
             } else {
                 v = fma(d, d, v);
             }
