@@ -215,10 +215,15 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
 
 // A tile costs about one unit's time beside its units, so many short curves stay
 // with the strips; a few of them do not fill the GPU either way, and there a
-// strip's serial pass over its curve is the longer.  Whole calls, strips against
-// tensor cores: 8 curves of 100 .. 500 samples 124 / 83 us, 100 of them 132 / 109,
-// 100 of 50 .. 200 85 / 98, 100 x 8 realizations of 200 .. 1500 322 / 183.
-bool lsp::host::tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real) {
+// strip's serial pass over its curve is the longer.  How few depends on how much
+// the strips have to do for a curve, that is on its sets of h = 1 sums.  Whole
+// calls, strips against tensor cores (us), N_f = 2 N_t:
+//   units a tile  1.3: one set 40, 60, 100 curves (two tiles each) 81 / 89, 80 / 90,
+//     82 / 98, but N_f = 10 N_t 92 / 83, 91 / 87, 95 / 95; two or three sets 60, 100
+//     curves 133 / 117, 134 / 130; four sets 100 curves 117 / 104
+//   units a tile  2.4: one set 60, 100, 148 curves 115 / 90, 118 / 95, 117 / 107
+bool lsp::host::tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real,
+                              double few) {
     double tiles = 0.0, units = 0.0, terms = 0.0;
     for (size_t c = 0; c < nf.size(); ++c) {
         if (nf[c] == 0) continue;
@@ -229,14 +234,15 @@ bool lsp::host::tc_batch_pays(const std::vector<int64_t>& off, const std::vector
         units += t * std::ceil(n / lsp::kTcUnit);
         terms += n * (double)nf[c] * n_real;
     }
-    return terms >= 1e6 && (tiles <= 300.0 || units >= 5.0 * tiles);
+    return terms >= 1e6 && (tiles <= few || (tiles <= 300.0 && units > 2.0 * tiles) || units >= 5.0 * tiles);
 }
 
 bool lsp::host::use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf,
-                             int n_real) {
+                             int n_real, bool gls) {
     const lsp_options& o = ctx->opt;
+    const int sets = n_real + (gls ? 1 : 0);
     return o.sincos_mode == LSP_SINCOS_AUTO && o.phase_mode == LSP_PHASE_FIXED64 && !o.freqs_per_thread &&
-           !o.batch_rhs && tc_batch_pays(off, nf, n_real);
+           !o.batch_rhs && tc_batch_pays(off, nf, n_real, sets == 1 ? 100.0 : sets <= 3 ? 160.0 : 300.0);
 }
 
 void lsp::host::TcPlan::pack(void* p) const {

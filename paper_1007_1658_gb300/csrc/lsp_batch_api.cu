@@ -106,7 +106,7 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
             tile = lsp::kTile;
         }
     }
-    const bool tc = !shape && use_tc_batch(ctx, off, nf, n_real);
+    const bool tc = !shape && use_tc_batch(ctx, off, nf, n_real, false);
     TcPlan tcp;
     if (tc) {
         mode = lsp::kModeTensor;

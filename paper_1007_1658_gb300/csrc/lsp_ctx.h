@@ -352,9 +352,11 @@ cudaError_t run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int 
 
 // Whether a batch runs on the tensor cores: the options leave the choice to the
 // library, and the batch is of a size where they are faster.
-bool use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real);
-// The size part of it alone.
-bool tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real);
+bool use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real,
+                  bool gls);
+// The size part of it alone; few: the tiles up to which a batch of curves of any
+// length is taken.
+bool tc_batch_pays(const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real, double few = 300.0);
 
 // Release the cached batch graph.
 void drop_plan(lsp_ctx* ctx);

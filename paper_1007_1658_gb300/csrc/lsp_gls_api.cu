@@ -237,7 +237,7 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         if (R > 1 && lsp::gls_mrhs_occupancy(F, R) <= 0)
             return fail(ctx, LSP_ERR_UNSUPPORTED, "batch_rhs = %d is not built for the floating-mean form", R);
     }
-    const bool tc = use_tc_batch(ctx, off, nf, n_real);
+    const bool tc = use_tc_batch(ctx, off, nf, n_real, true);
     TcPlan tcp;
     const int64_t per_block = lsp::gls_batch_freqs_per_block(F);
     std::vector<int> order(n_curves);
