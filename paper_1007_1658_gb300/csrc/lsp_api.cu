@@ -151,11 +151,11 @@ void lsp::host::finish_shape(const lsp_ctx* ctx, MainShape& s, int occ_in, int64
 // long grids gain earlier (500 x 100,000 55.3 / 44.7), long ones on short grids
 // later (100,000 x 500 95.5 / 97.4).
 static constexpr double kTcMinTerms = 6e7;
-bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f) {
+bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f, bool gls) {
     const lsp_options& o = ctx->opt;
     if (o.sincos_mode != LSP_SINCOS_AUTO || o.phase_mode != LSP_PHASE_FIXED64 || o.freqs_per_thread || o.split)
         return false;
-    return (double)N * (double)N_f >= kTcMinTerms && !tuned(ctx, N, N_f);
+    return (double)N * (double)N_f >= kTcMinTerms && (gls || !tuned(ctx, N, N_f));
 }
 
 lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_out, bool launch,
@@ -441,7 +441,7 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
     if ((rs = where(ctx, t, &t_dev)) != LSP_OK || (rs = where(ctx, X, &x_dev)) != LSP_OK ||
         (rs = where(ctx, P_out, &p_dev)) != LSP_OK)
         return rs;
-    const bool tc = use_tc(ctx, N_t, N_f);
+    const bool tc = use_tc(ctx, N_t, N_f, false);
     MainShape s{};
     int tc_launches = 2;
     if (tc) {

@@ -312,8 +312,8 @@ const TuneEntry* tuned(const lsp_ctx* ctx, int64_t N, int64_t N_f);
 
 // Whether a single-curve call of this size runs on the tensor cores: the
 // options leave the choice to the library (AUTO, no strip length, no split) and
-// the tuning table has no entry for it.
-bool use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f);
+// the tuning table, whose entries are of the classic form, has none for it.
+bool use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f, bool gls);
 
 // The sums and the finalize pass of one curve on the tensor cores, its records
 // and recE in place, in blocks of frequencies whose partial tiles fit the

@@ -67,7 +67,7 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
             return ws;
     }
     lsp_status rs;
-    const bool tc = use_tc(ctx, N_t, N_f);
+    const bool tc = use_tc(ctx, N_t, N_f, true);
     MainShape s{};
     int tc_launches = 2;
     if (tc) {
