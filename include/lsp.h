@@ -52,7 +52,7 @@ typedef enum lsp_status {
 typedef enum lsp_sincos_mode {
     LSP_SINCOS_AUTO = 0,   /* the library's choice: RECUR3_X2 on small calls, and on larger
                               ones, when freqs_per_thread, split and batch_rhs are 0 too
-                              and the tuning table has no entry for the size, the same
+                              and the tuning table does not say otherwise, the same
                               sums as a matrix product on the tensor cores (FP32
                               accuracy from split FP16 operands)                     */
     LSP_SINCOS_MUFU = 1,   /* hardware sin/cos (SFU) of every phase (Sec. 4.3's choice)  */
@@ -292,10 +292,13 @@ lsp_status lsp_grid(double t_min, double t_max, int64_t N_t, double F_over, doub
  * Autotuner: time the sin/cos modes, strip lengths F (also the recurrence's
  * re-seed length) and N_t splits on a synthetic series of this size, keep
  * only candidates within 2e-5 max P of the all-hardware-sin/cos result, and
- * remember the fastest for this (log2 N_t, log2 N_f) bucket: later calls with
- * LSP_SINCOS_AUTO and automatic F/split use it (in place of the tensor cores
- * too, where the size would take them).  *chosen (may be NULL) receives the
- * winning options.  Blocks; allocates temporary buffers.
+ * remember the fastest for this (log2 N_t, log2 N_f) bucket: later
+ * lsp_periodogram calls with LSP_SINCOS_AUTO and automatic F/split use it.  Where
+ * AUTO would take the tensor cores they are timed too: if they win, the bucket is
+ * left without an entry (and loses one it had), so that AUTO goes on taking
+ * them; an entry that was not timed against them, such as one of a file of an
+ * earlier version, does not keep a call from them.  *chosen (may be NULL)
+ * receives the winning options.  Blocks; allocates temporary buffers.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 lsp_status lsp_autotune(lsp_ctx *ctx, int64_t N_t, int64_t N_f, lsp_options *chosen);
@@ -315,7 +318,10 @@ lsp_status lsp_autotune(lsp_ctx *ctx, int64_t N_t, int64_t N_f, lsp_options *cho
  * remembered for this batch's size bucket (log2 of its terms per
  * realization, log2 of its mean N_t, its realization count 1 / 2-3 / 4-7 / 8+):
  * later lsp_batch calls in that bucket use it when the options leave the
- * choice to the library (AUTO sin/cos, freqs_per_thread 0, batch_rhs 0).
+ * choice to the library (AUTO sin/cos, freqs_per_thread 0, batch_rhs 0).  Only
+ * strips are timed: a tuned bucket runs them also where an untuned one takes the
+ * tensor cores, which are faster there (4096 curves of 200 .. 20,000 samples
+ * 9.4 ms against 63), so tune batches that are to be summed term by term.
  * *chosen (may be NULL) receives the winner as options.  Arrays as lsp_batch
  * (host or device).  Blocks; allocates temporary buffers.
  * Errors: INVALID_ARG, OOM, CUDA.

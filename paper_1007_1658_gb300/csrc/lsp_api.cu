@@ -155,7 +155,9 @@ bool lsp::host::use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f, bool gls) {
     const lsp_options& o = ctx->opt;
     if (o.sincos_mode != LSP_SINCOS_AUTO || o.phase_mode != LSP_PHASE_FIXED64 || o.freqs_per_thread || o.split)
         return false;
-    return (double)N * (double)N_f >= kTcMinTerms && (gls || !tuned(ctx, N, N_f));
+    if ((double)N * (double)N_f < kTcMinTerms) return false;
+    const TuneEntry* te = gls ? nullptr : tuned(ctx, N, N_f);
+    return !(te && te->beat_tensor);
 }
 
 lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, float* P_out, bool launch,

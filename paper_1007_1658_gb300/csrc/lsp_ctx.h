@@ -37,11 +37,14 @@ struct BatchPlan {
     int kernels = 0;
 };
 
-// One autotuned choice for a (log2 N_t, log2 N_f) size bucket.
+// One autotuned choice for a (log2 N_t, log2 N_f) size bucket.  beat_tensor: it was
+// timed against the tensor cores too and won; without that it is the fastest strip
+// only and does not keep a call from them.
 struct TuneEntry {
     int nt_bucket, nf_bucket;
     int sincos, F, split;
     float ms;
+    int beat_tensor;
 };
 
 // Launch shape of lsp_batch: kernel mode (kMode*), strip length, realizations
@@ -312,7 +315,8 @@ const TuneEntry* tuned(const lsp_ctx* ctx, int64_t N, int64_t N_f);
 
 // Whether a single-curve call of this size runs on the tensor cores: the
 // options leave the choice to the library (AUTO, no strip length, no split) and
-// the tuning table, whose entries are of the classic form, has none for it.
+// the tuning table, whose entries are of the classic form, has none for it that
+// was measured to be faster.
 bool use_tc(const lsp_ctx* ctx, int64_t N, int64_t N_f, bool gls);
 
 // The sums and the finalize pass of one curve on the tensor cores, its records

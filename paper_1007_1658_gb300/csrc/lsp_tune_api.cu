@@ -1,6 +1,7 @@
 // lsp_tune_api.cu -- lsp_autotune: pick the sin/cos mode, strip length F
 // (which is also the recurrence's re-seed length K) and N_t split for a
-// problem size by timing candidates on the device, behind a precision gate.
+// problem size by timing candidates on the device, behind a precision gate; the
+// tensor cores are a candidate where AUTO would take them.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -127,7 +128,12 @@ extern "C" lsp_status lsp_autotune(lsp_ctx* ctx, int64_t N_t, int64_t N_f, lsp_o
     const Cand cands[] = {{LSP_SINCOS_RECUR3_X2, 24}, {LSP_SINCOS_RECUR3_X2, 16}, {LSP_SINCOS_RECUR3_X2, 8},
                           {LSP_SINCOS_RECUR3_X2, 4},  {LSP_SINCOS_RECUR3, 24},    {LSP_SINCOS_RECUR, 16},
                           {LSP_SINCOS_RECUR, 8},      {LSP_SINCOS_MUFU, 8}};
-    TuneEntry best{bucket(N_t), bucket(N_f), 0, 0, 0, 1e30f};
+    TuneEntry best{bucket(N_t), bucket(N_f), 0, 0, 0, 1e30f, 0};
+    auto max_err = [&]() {
+        float err = 0.f;
+        for (size_t k = 0; k < got.size(); ++k) err = std::max(err, std::fabs(got[k] - ref[k]));
+        return err;
+    };
     for (const Cand& c : cands) {
         // the heuristic split of this candidate, then half and double of it
         ctx->opt = saved;
@@ -144,24 +150,39 @@ extern "C" lsp_status lsp_autotune(lsp_ctx* ctx, int64_t N_t, int64_t N_f, lsp_o
                 release();
                 return rs;
             }
-            float err = 0.f;
-            for (size_t k = 0; k < got.size(); ++k) err = std::max(err, std::fabs(got[k] - ref[k]));
+            const float err = max_err();
             const bool pass = std::isfinite(err) && err <= 2e-5f * pmax;  // a fifth of the parity budget
-            if (pass && ms < best.ms) best = TuneEntry{bucket(N_t), bucket(N_f), c.sincos, c.F, splits[si], ms};
+            if (pass && ms < best.ms) best = TuneEntry{bucket(N_t), bucket(N_f), c.sincos, c.F, splits[si], ms, 0};
         }
     }
+    // the tensor cores, with the table out of the way; where they win, no entry is left
+    bool tensor = false;
+    std::vector<TuneEntry> table;
+    table.swap(ctx->tune);
+    ctx->opt = saved;
+    ctx->opt.sincos_mode = LSP_SINCOS_AUTO;
+    ctx->opt.phase_mode = LSP_PHASE_FIXED64;
+    ctx->opt.freqs_per_thread = ctx->opt.split = 0;
+    if (use_tc(ctx, N_t, N_f, false)) {
+        rs = run(LSP_SINCOS_AUTO, 0, 0, &got, &ms);
+        const float err = rs == LSP_OK ? max_err() : 0.f;
+        tensor = rs == LSP_OK && std::isfinite(err) && err <= 2e-5f * pmax && ms < best.ms;
+        best.beat_tensor = !tensor;
+    }
+    ctx->tune.swap(table);
     ctx->opt = saved;
     release();
-    if (best.sincos == 0) return fail(ctx, LSP_ERR_CUDA, "autotune: no candidate passed the precision gate");
+    if (rs != LSP_OK) return rs;
+    if (best.sincos == 0 && !tensor) return fail(ctx, LSP_ERR_CUDA, "autotune: no candidate passed the precision gate");
     ctx->tune.erase(std::remove_if(ctx->tune.begin(), ctx->tune.end(),
                                    [&](const TuneEntry& e) { return e.nt_bucket == best.nt_bucket && e.nf_bucket == best.nf_bucket; }),
                     ctx->tune.end());
-    ctx->tune.push_back(best);
+    if (!tensor) ctx->tune.push_back(best);
     if (chosen) {
         *chosen = saved;
-        chosen->sincos_mode = best.sincos;
-        chosen->freqs_per_thread = best.F;
-        chosen->split = best.split;
+        chosen->sincos_mode = tensor ? LSP_SINCOS_AUTO : best.sincos;
+        chosen->freqs_per_thread = tensor ? 0 : best.F;
+        chosen->split = tensor ? 0 : best.split;
     }
     return LSP_OK;
 }
@@ -307,8 +328,10 @@ extern "C" lsp_status lsp_tune_save(lsp_ctx* ctx, const char* path) {
     fprintf(f, "{\"lsp_tune\": 1, \"device\": \"%s\", \"entries\": [\n", device_name(ctx->device).c_str());
     size_t n = 0, total = ctx->tune.size() + ctx->tune_batch.size();
     for (const TuneEntry& e : ctx->tune)
-        fprintf(f, "{\"kind\": 1, \"nt\": %d, \"nf\": %d, \"sincos\": %d, \"F\": %d, \"split\": %d, \"ms\": %.6g}%s\n",
-                e.nt_bucket, e.nf_bucket, e.sincos, e.F, e.split, e.ms, ++n < total ? "," : "");
+        fprintf(f,
+                "{\"kind\": 1, \"nt\": %d, \"nf\": %d, \"sincos\": %d, \"F\": %d, \"split\": %d, \"ms\": %.6g, "
+                "\"beat_tensor\": %d}%s\n",
+                e.nt_bucket, e.nf_bucket, e.sincos, e.F, e.split, e.ms, e.beat_tensor, ++n < total ? "," : "");
     for (const BatchTuneEntry& e : ctx->tune_batch)
         fprintf(f,
                 "{\"kind\": 2, \"terms\": %d, \"mean_nt\": %d, \"real\": %d, \"mode\": %d, \"F\": %d, \"R\": %d, "
@@ -341,7 +364,7 @@ extern "C" lsp_status lsp_tune_load(lsp_ctx* ctx, const char* path, int32_t* n_l
         const double kind = field(line, "kind");
         if (kind == 1) {
             TuneEntry e{(int)field(line, "nt"), (int)field(line, "nf"), (int)field(line, "sincos"), (int)field(line, "F"),
-                        (int)field(line, "split"), (float)field(line, "ms")};
+                        (int)field(line, "split"), (float)field(line, "ms"), field(line, "beat_tensor") == 1.0};
             lsp_options o = ctx->opt;
             o.sincos_mode = e.sincos;
             o.freqs_per_thread = e.F;

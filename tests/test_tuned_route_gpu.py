@@ -60,3 +60,28 @@ def test_floating_mean_calls_do_not_follow_a_classic_entry(lsp, data, tmp_path):
     with lsp.Context(0) as ctx:
         assert ctx.tune_load(path) == 1
         assert np.array_equal(_run(ctx, data, True), want)
+
+
+def test_an_entry_not_timed_against_the_tensor_cores_leaves_them(lsp, data, tmp_path):
+    """A file of a version that timed strips only, and one whose strip won."""
+    tensor, strips = _default(lsp, data, False), _default(lsp, data, False, sincos_mode=lsp.SINCOS_RECUR3_X2, split=10)
+    assert not np.array_equal(tensor, strips)
+    path = tmp_path / "tune.json"
+    for more, want in (({}, tensor), ({"beat_tensor": 1}, strips)):
+        _strip_file(lsp, path, **more)
+        with lsp.Context(0) as ctx:
+            assert ctx.tune_load(path) == 1
+            assert np.array_equal(_run(ctx, data, False), want)
+
+
+def test_tuning_a_large_size_keeps_the_tensor_cores(lsp, data, tmp_path):
+    want = _default(lsp, data, False)
+    path = tmp_path / "tune.json"
+    _strip_file(lsp, path)
+    with lsp.Context(0) as ctx:
+        ctx.tune_load(path)
+        chosen = ctx.autotune(N, NF)
+        assert (chosen["sincos_mode"], chosen["freqs_per_thread"], chosen["split"]) == (lsp.SINCOS_AUTO, 0, 0)
+        assert np.array_equal(_run(ctx, data, False), want)
+        ctx.tune_save(path)
+    assert '"kind"' not in path.read_text()
