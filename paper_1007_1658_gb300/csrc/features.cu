@@ -333,10 +333,15 @@ __device__ __forceinline__ void warp_top8(const float (&tv)[8], const int (&tm)[
     }
 }
 
-// How far the strip kernel's W and an accurate one can be apart: its recurrence
-// is off by at most F^2 ulp a term (3.4e-5), its sums and hardware sin/cos by less,
-// so 1e-4 of |sum| / n <= sqrt(W), here for both.
-__device__ __forceinline__ float window_gap(float w) { return 2e-4f * sqrtf(w) + 1e-8f; }
+// How far the strip kernel's W and an accurate one can be apart, for n samples: its
+// recurrence is off by at most F^2 ulp a term (3.4e-5) and its hardware sin/cos by
+// less, 1e-4 of |sum| / n <= sqrt(W) together; and each of its FP32 additions by
+// half an ulp of the running sum, 2^-24 j after j samples, n 2^-25 of the whole
+// (where the terms repeat, on a cadence at its aliases, those roundings have one
+// sign: up to 1.3e-4 and 3.7e-4 of n at 20,000 and 32,700 samples).  e bounds
+// ||sum| - |sum'|| / n, so |W - W'| <= e (2 sqrt(W) + e).
+__device__ __forceinline__ float window_error(int64_t n) { return 1e-4f + (float)n * 0x1p-25f; }
+__device__ __forceinline__ float window_gap(float w, float e) { return e * (2.f * sqrtf(w) + e); }
 
 // A pattern's bins that can hold one of the 8 highest local maxima (outside the
 // main lobe) of the strip kernel's W: with g the gap above, maxima of the accurate
@@ -360,6 +365,7 @@ window_peaks_kernel(const double* __restrict__ t, const int64_t* __restrict__ of
         if (tid == 0) p[0] = -1;
         return;
     }
+    const float err = window_error(e - b);
     float tv[8];
     int tm[8];
 #pragma unroll
@@ -369,8 +375,8 @@ window_peaks_kernel(const double* __restrict__ t, const int64_t* __restrict__ of
     }
     if (tid == 0) s_n = 0;
     for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
-        const float w = Wc[i], l = Wc[i - 1], h = Wc[i + 1], g = window_gap(w);
-        if (w - g > l + window_gap(l) && w - g > h + window_gap(h) && (double)(i + 1) * df * T >= 1.0)
+        const float w = Wc[i], l = Wc[i - 1], h = Wc[i + 1], g = window_gap(w, err);
+        if (w - g > l + window_gap(l, err) && w - g > h + window_gap(h, err) && (double)(i + 1) * df * T >= 1.0)
             top8_insert(tv, tm, w - g, (int)i);
     }
     warp_top8(tv, tm, [&](int r, float v, int) { wv[warp * 8 + r] = v; });
@@ -388,10 +394,10 @@ window_peaks_kernel(const double* __restrict__ t, const int64_t* __restrict__ of
     __syncthreads();
     const float least = s_eighth;  // -1 where there are fewer than eight
     for (int64_t i = 1 + tid; i + 1 < mw; i += nt) {
-        const float w = Wc[i], g = window_gap(w);
+        const float w = Wc[i], g = window_gap(w, err);
         if (!(w + g >= least)) continue;
         const float l = Wc[i - 1], h = Wc[i + 1];
-        if (w + g >= l - window_gap(l) && w + g >= h - window_gap(h) && (double)(i + 1) * df * T >= 1.0) {
+        if (w + g >= l - window_gap(l, err) && w + g >= h - window_gap(h, err) && (double)(i + 1) * df * T >= 1.0) {
             const int at = atomicAdd(&s_n, 1);
             if (at < kWindowPeaks) p[1 + at] = (int)i;
         }
