@@ -587,8 +587,9 @@ constexpr float kGlsRefine = 0x1p-5f;
 // In FP32 pairs, whose 2^-48 the differences leave enough of: D >= T / 8 >= 1/64
 // where the result is used.  The quotient is corrected once by its remainder.
 // *ill: the smaller eigenvalue, between (T^2 - |M|^2) / 4T and / 2T, may lie
-// below kGlsRefine (not where the sums are NaN, of errors that the statistics
-// refuse: P is 0 then, whichever way).  n: the sample count.
+// below kGlsRefine; so it does where T does, whose sign is then lost in the sums'
+// rounding.  (Not where the sums are NaN, of errors that the statistics refuse: P
+// is 0 then, whichever way.)  n: the sample count.
 __device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, dev::Pair n, bool* ill) {
     using dev::Pair;
     using dev::product;
@@ -598,7 +599,7 @@ __device__ __forceinline__ float gls_power(float2 Zf, float2 Cf, float2 Wf, dev:
     const Pair D = T * T + -(A * A + B * B);
     const Pair sx = product(Zf.x, Zf.x), sy = product(Zf.y, Zf.y);
     const Pair num = T * (sx + sy) + -(A * (sx + -sy) + B * product(2.f * Zf.x, Zf.y));
-    *ill = D.h + D.l < (float)(4.0 * kGlsRefine) * (T.h + T.l);
+    *ill = T.h < kGlsRefine || D.h + D.l < (float)(4.0 * kGlsRefine) * (T.h + T.l);
     const float r = 1.f / D.h, q = num.h * r;
     const float rest = (fmaf(-q, D.h, num.h) + num.l) - q * D.l;
     return fmaxf(rounded_product(Pair{q, rest * r}, n), 0.f);
