@@ -175,6 +175,8 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
     const int64_t step = std::min(groups, most);
     const int64_t slots = (sets * step + G - 1) / G + (step + G - 1) / G + pairs;
     lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)slots * (size_t)a.slot_floats * 4);
+    if (rs == LSP_OK && gls)
+        rs = ensure_zeroed(ctx, ctx->tc_mask, (size_t)lsp::tc_mask_words((sets * step + G - 1) / G, cols) * 4);
     if (rs != LSP_OK || !launch) return rs;
     a.win_kind = gls ? lsp::kTcW2 : lsp::kTcOne2;
     a.one.kind = gls ? lsp::kTcRecQ : lsp::kTcRec;
@@ -205,9 +207,11 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
         f.P = P_out;
         f.bins = (lsp::TcBin*)ctx->tc_bins.p;
         f.n_bins = (unsigned*)ctx->qmax.p + 1;
+        f.mask = (unsigned*)ctx->tc_mask.p;
+        if (gls && g > 0) LSP_CUDA(ctx, cudaMemsetAsync(f.n_bins, 0, 4, ctx->stream));
         LSP_CUDA(ctx, lsp::launch_tc_final(gls ? lsp::kTcGls : lsp::kTcClassic, a, f, ctx->stream));
         *launches += 2;
-        if (gls && g + step >= groups) {
+        if (gls) {
             LSP_CUDA(ctx, lsp::launch_tc_refine(a, f, ctx->stream));
             ++*launches;
         }
@@ -274,6 +278,7 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
         if (cur.n == 0) return;
         p.chunks.push_back(cur);
         p.max_slot_floats = std::max(p.max_slot_floats, (cur.n + pairs) * lsp::tc_slot_floats(cur.cols));
+        p.max_mask_words = std::max(p.max_mask_words, lsp::tc_mask_words(cur.nd, cur.cols));
         cur = TcChunk{(int64_t)p.tiles.size(), 0, (int64_t)p.data.size(), 0, 0, 0};
         p.pre.push_back(0);
     };
@@ -339,11 +344,13 @@ cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d
         a.slot_floats = lsp::tc_slot_floats(c.cols);
         f.data_tiles = data + c.d0;
         f.n_data = (int)c.nd;
+        const bool gls = form == lsp::kTcGls;
         cudaError_t e = lsp::launch_tc_sums(a, st);
+        if (e == cudaSuccess && gls && x > 0) e = cudaMemsetAsync(f.n_bins, 0, 4, st);
         if (e == cudaSuccess) e = lsp::launch_tc_final(form, a, f, st);
+        if (e == cudaSuccess && gls) e = lsp::launch_tc_refine(a, f, st);
         if (e != cudaSuccess) return e;
     }
-    if (form == lsp::kTcGls && !p.chunks.empty()) return lsp::launch_tc_refine(a, f, st);
     return cudaSuccess;
 }
 
@@ -592,7 +599,7 @@ void lsp_destroy(lsp_ctx* ctx) {
     DeviceGuard guard(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_plan(ctx);
-    DevBuf* bufs[] = {&ctx->recE, &ctx->qmax, &ctx->tc_part, &ctx->tc_bins, &ctx->b_recE, &ctx->b_qmax, &ctx->b_tc, &ctx->recQ,   &ctx->dy_stage, &ctx->pr_acc, &ctx->pr_z0, &ctx->pr_z1,
+    DevBuf* bufs[] = {&ctx->recE, &ctx->qmax, &ctx->tc_part, &ctx->tc_bins, &ctx->tc_mask, &ctx->b_recE, &ctx->b_qmax, &ctx->b_tc, &ctx->recQ,   &ctx->dy_stage, &ctx->pr_acc, &ctx->pr_z0, &ctx->pr_z1,
                       &ctx->recA,   &ctx->recB,   &ctx->recN,   &ctx->part,    &ctx->stats,  &ctx->t_stage,
                       &ctx->x_stage, &ctx->p_stage, &ctx->stat_parts, &ctx->stat_counters, &ctx->b_recA,
                       &ctx->b_recB,  &ctx->b_xr,   &ctx->b_stats, &ctx->b_items, &ctx->b_head, &ctx->b_maxkey,

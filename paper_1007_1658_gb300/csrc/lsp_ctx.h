@@ -94,7 +94,8 @@ struct lsp_ctx {
     // single-curve workspace
     lsp::host::DevBuf recA, recB, recN, part, stats, t_stage, x_stage, p_stage, stat_parts, stat_counters;
     lsp::host::DevBuf recQ, dy_stage;  // floating-mean periodogram: sqrt(w_j), staged errors
-    lsp::host::DevBuf recE, qmax, tc_part, tc_bins;  // tensor-core path: coarse rotations, largest q, partial tiles, bins formed again
+    lsp::host::DevBuf recE, qmax, tc_part;  // tensor-core path: coarse rotations, largest q, partial tiles
+    lsp::host::DevBuf tc_bins, tc_mask;     // floating mean: list and bit map of the bins formed again
     lsp::host::DevBuf b_recE, b_qmax, b_tc;  // its batch form: the same per curve, and the packed tile list
     lsp::host::DevBuf pr_acc, pr_z0, pr_z1;  // Press-Rybicki: FP64 grid, FFT ping-pong buffers
     // batch workspace
@@ -339,6 +340,7 @@ struct TcPlan {
     std::vector<int> data;
     std::vector<TcChunk> chunks;
     int64_t max_slot_floats = 0;  // largest workspace of a chunk, in floats
+    int64_t max_mask_words = 0;   // and bit map (kTcGls)
     size_t bytes() const { return cols.size() * 8 + tiles.size() * sizeof(lsp::TcTile) + pre.size() * 8 + data.size() * 4; }
     // columns, tiles, prefix sums and indices, as one block
     void pack(void* p) const;

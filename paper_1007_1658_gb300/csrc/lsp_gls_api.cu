@@ -270,6 +270,7 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         if ((rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->b_qmax, (size_t)n_curves * 4 + 4)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins)) != LSP_OK) return rs;
+        if ((rs = ensure_zeroed(ctx, ctx->tc_mask, (size_t)tcp.max_mask_words * 4 + 16)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
     } else if ((rs = ensure(ctx, ctx->b_items, items.size() * sizeof(lsp::BatchItem) + 16)) != LSP_OK) {
@@ -337,8 +338,9 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         f.n_curves = n_curves;
         f.bins = (lsp::TcBin*)ctx->tc_bins.p;
         f.n_bins = (unsigned*)ctx->b_qmax.p + n_curves;
+        f.mask = (unsigned*)ctx->tc_mask.p;
         LSP_CUDA(ctx, run_tc(ctx, tcp, ctx->b_tc.p, lsp::kTcGls, a, f, st));
-        launches += 2 * (int)tcp.chunks.size() + 1;
+        launches += 3 * (int)tcp.chunks.size();
     } else if (!items.empty()) {
         NvtxRange r("lsp_batch_gls.main");
         // the packed form when the work is many times the longest curve's, per

@@ -741,17 +741,15 @@ __global__ void __launch_bounds__(kFinThreads, FORM == kTcGls ? 2 : 4) tc_final_
                 for (int s = 0; s < 2; ++s) {
                     const int64_t k = s ? kp : km;
                     if (!(s ? lp : lm) || k >= nf) continue;
-                    float p = -1.f;  // left to launch_tc_refine
                     const unsigned at = atomicAdd(f.n_bins, 1u);
                     if (at < (unsigned)kTcBins) {
                         f.bins[at] = TcBin{w.curve, real, (uint32_t)k, 0u};
                     } else {  // the list is full
-                        float d[kMoments] = {}, e[kMoments] = {};
-                        direct_gls(a, t.b, n, a.xr ? a.xr + (size_t)real * (size_t)a.total : nullptr, (uint32_t)k, 0, 1, d,
-                                   e);
-                        p = moments_value(d, e, (double)n);
+                        const int fine = s ? nb + rb : nb - 1 - rb;
+                        const int64_t row = (int64_t)blockIdx.x * kFinRows + ra;  // of the launch's h = 1 tiles
+                        atomicOr(&f.mask[row * (a.slot_floats / tc_slot_floats(32)) + (fine >> 5)], 1u << (fine & 31));
                     }
-                    (s ? vp : vm) = p;
+                    (s ? vp : vm) = -1.f;  // left to launch_tc_refine
                 }
             }
             keep(vm, km);
@@ -798,34 +796,79 @@ __device__ __forceinline__ void add_pair(float& s, float& c, float t, float d) {
     s = y;
 }
 
-// One cluster of CL CTAs per listed bin: its sums over all samples, then P.
-// A single long curve lists a few bins of many samples (CL = 8: 100,000 samples in
+// Joins the sums of the first `width` lanes in lane 0.
+__device__ __forceinline__ void join_lanes(float (&s)[kMoments], float (&c)[kMoments], int width) {
+    for (int o = width / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int x = 0; x < kMoments; ++x)
+            add_pair(s[x], c[x], __shfl_down_sync(0xffffffffu, s[x], o), __shfl_down_sync(0xffffffffu, c[x], o));
+}
+
+// One cluster of CL CTAs per bin: its sums over all samples, then P.  A single long
+// curve lists a few bins of many samples (CL = 8: 100,000 samples in
 // one CTA are 40 us of arithmetic), a batch many bins of shorter curves (CL = 1),
 // and a single short curve far beyond its mean Nyquist frequency thousands of bins
 // with a sample or a few for each of 128 threads (500 samples, 100,000 frequencies
 // on a nightly cadence, the finalize stage: CL = 8 78 us, 128 threads 20; 20,000
 // samples, 2000 frequencies 31 and 68, 6000 by 12,000 31 and 39).
+// With more bins than the list holds (a grid below 1 / 3T, one sample whose weight
+// exceeds all others') a warp takes a bin, those listed and then those in the bit
+// map: 100,000 samples by 200,000 such bins 72 ms, by clusters 135; 2000 patterns of
+// 200 .. 1000 samples by 64 realizations, about one such bin each, the call 11.8 ms,
+// by CTAs 14.3.  So how a bin is summed depends on the number of them, not on the
+// order in which they came.
 template <int CL, int kThreads>
 __global__ void __launch_bounds__(kThreads) tc_refine_kernel(const TcArgs a, const TcFinal f) {
     __shared__ float2 sh[kThreads / 32][kMoments];
     __shared__ float2 part[CL][kMoments];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0;
-    const unsigned count = min(*f.n_bins, (unsigned)kTcBins);
-    for (unsigned i = blockIdx.x / CL; i < count; i += gridDim.x / CL) {
-        const TcBin w = f.bins[i];
+    const unsigned found = *f.n_bins;
+    auto sums = [&](const TcBin& w, int i0, int step, float (&s)[kMoments], float (&c)[kMoments]) {
         const int64_t b = a.off ? a.off[w.curve] : 0, n = a.off ? a.off[w.curve + 1] - b : a.n0;
-        float s[kMoments] = {}, c[kMoments] = {};
-        direct_gls(a, b, n, a.xr ? a.xr + (size_t)w.real * (size_t)a.total : nullptr, w.k,
-                   rank * kThreads + (int)threadIdx.x, CL * kThreads, s, c);
-        auto join = [&](int width) {
-            for (int o = width / 2; o > 0; o >>= 1)
 #pragma unroll
-                for (int x = 0; x < kMoments; ++x)
-                    add_pair(s[x], c[x], __shfl_down_sync(0xffffffffu, s[x], o),
-                             __shfl_down_sync(0xffffffffu, c[x], o));
+        for (int x = 0; x < kMoments; ++x) s[x] = c[x] = 0.f;
+        direct_gls(a, b, n, a.xr ? a.xr + (size_t)w.real * (size_t)a.total : nullptr, w.k, i0, step, s, c);
+    };
+    auto put = [&](const TcBin& w, const float (&s)[kMoments], const float (&c)[kMoments]) {
+        const int64_t n = a.off ? a.off[w.curve + 1] - a.off[w.curve] : a.n0;
+        const float p = moments_value(s, c, (double)n);
+        if (f.P) f.P[(size_t)w.real * (size_t)f.P_total + (f.P_off ? f.P_off[w.curve] : 0) + w.k] = p;
+        if (f.maxkey)
+            atomicMax(&f.maxkey[(size_t)w.real * (size_t)f.n_curves + w.curve],
+                      ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~w.k));
+    };
+    float s[kMoments], c[kMoments];
+    if (found > (unsigned)kTcBins) {
+        auto form = [&](const TcBin& w) {
+            sums(w, lane, 32, s, c);
+            join_lanes(s, c, 32);
+            if (lane == 0) put(w, s, c);
         };
-        join(32);
+        const int me = blockIdx.x * (kThreads / 32) + warp, all = gridDim.x * (kThreads / 32);
+        for (int i = me; i < kTcBins; i += all) form(f.bins[i]);
+        const int per_row = (int)(a.slot_floats / tc_slot_floats(32));  // words
+        const int64_t words = tc_mask_words(a.tiles ? f.n_data : a.h1, 32 * per_row);
+        // an odd number of warps: such bins are often the first of every row, a fixed number of words apart
+        for (int64_t word = me; word < words && me < all - 1; word += all - 1) {
+            unsigned bits = f.mask[word];
+            if (!bits) continue;
+            __syncwarp();
+            if (lane == 0) f.mask[word] = 0u;
+            const int64_t row = word / per_row;
+            const int tile = (int)(row / (2 * kFinRows)), r = (int)(row % (2 * kFinRows));
+            const TcTile w = tile_of(a, a.tiles ? f.data_tiles[tile] : tile);
+            const int G = w.g0 + r / kTcGroup, set = G / w.gpr;
+            const uint32_t k0 = (uint32_t)(((int64_t)(w.kg0 + G - set * w.gpr) * kTcGroup + r % kTcGroup) * w.cols +
+                                           word % per_row * 32);
+            for (; bits; bits &= bits - 1) form(TcBin{w.curve, w.r0 + set, k0 + (uint32_t)__ffs(bits) - 1u, 0u});
+        }
+        return;
+    }
+    for (unsigned i = blockIdx.x / CL; i < found; i += gridDim.x / CL) {
+        const TcBin w = f.bins[i];
+        sums(w, rank * kThreads + (int)threadIdx.x, CL * kThreads, s, c);
+        join_lanes(s, c, 32);
         if (lane == 0)
 #pragma unroll
             for (int x = 0; x < kMoments; ++x) sh[warp][x] = make_float2(s[x], c[x]);
@@ -837,7 +880,7 @@ __global__ void __launch_bounds__(kThreads) tc_refine_kernel(const TcArgs a, con
                 s[x] = v.x;
                 c[x] = v.y;
             }
-            join(kThreads / 32);
+            join_lanes(s, c, kThreads / 32);
         }
         if constexpr (CL > 1) {
             if (threadIdx.x == 0) {
@@ -852,15 +895,7 @@ __global__ void __launch_bounds__(kThreads) tc_refine_kernel(const TcArgs a, con
                     for (int x = 0; x < kMoments; ++x) add_pair(s[x], c[x], part[r][x].x, part[r][x].y);
             }
         }
-        {
-            if (threadIdx.x == 0 && rank == 0) {
-                const float p = moments_value(s, c, (double)n);
-                if (f.P) f.P[(size_t)w.real * (size_t)f.P_total + (f.P_off ? f.P_off[w.curve] : 0) + w.k] = p;
-                if (f.maxkey)
-                    atomicMax(&f.maxkey[(size_t)w.real * (size_t)f.n_curves + w.curve],
-                              ((unsigned long long)__float_as_uint(p) << 32) | (unsigned long long)(~w.k));
-            }
-        }
+        if (threadIdx.x == 0 && rank == 0) put(w, s, c);
         if constexpr (CL > 1) cooperative_groups::this_cluster().sync();
         else __syncthreads();
     }
@@ -879,7 +914,7 @@ cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st)
     at.val.clusterDim.x = 8;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(64);
+    cfg.gridDim = dim3(304);
     cfg.blockDim = dim3(512);
     cfg.stream = st;
     cfg.attrs = &at;

@@ -116,7 +116,9 @@ struct TcBin {
     int32_t curve, real;
     uint32_t k, pad;
 };
-constexpr int kTcBins = 1 << 16;  // bins the list holds
+constexpr int kTcBins = 1 << 16;  // bins the list holds; the others of a launch are marked in a bit map of its h = 1 tiles
+// Words of the bit map of n h = 1 tiles of up to cols columns: 128 rows (coarse frequencies) of cols bits each.
+__host__ __device__ inline int64_t tc_mask_words(int64_t n, int cols) { return n * 128 * (cols / 32); }
 
 struct TcFinal {
     const int* data_tiles;      // list form: indices of the h = 1 tiles
@@ -130,13 +132,15 @@ struct TcFinal {
     int n_curves;
     TcBin* bins;                // floating mean: list of ill-conditioned bins and
     unsigned* n_bins;           // its counter (zeroed by launch_prep_stats, after qmax)
+    unsigned* mask;             // bit map of the others (zero before and after)
 };
 
 enum : int { kTcClassic = 0, kTcGls = 1, kTcWindow = 2 };
 
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st);
 cudaError_t launch_tc_final(int form, const TcArgs& a, const TcFinal& f, cudaStream_t st);
-// Floating mean: the listed bins, after every launch_tc_final of the call.
+// Floating mean: the bins that the launch_tc_final before it, with the same
+// arguments, listed and marked.  n_bins is to be zero before the next one.
 cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st);
 
 }  // namespace lsp
