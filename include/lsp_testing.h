@@ -38,6 +38,14 @@ int32_t lsp_test_pointer_kind(int32_t memory_type, int32_t pointer_device, int32
 lsp_status lsp_test_fail_allocation(lsp_ctx *ctx, int32_t n);
 
 /*
+ * While `on` is not 0, every wait of the tensor-core kernel of `ctx` gives up at
+ * its first look, as if its limit of about a second had passed.  A call in which
+ * one does ends normally, its outputs NaN, and lsp_sync returns LSP_ERR_CUDA.
+ * Errors: INVALID_ARG (null context).
+ */
+lsp_status lsp_test_give_up_waits(lsp_ctx *ctx, int32_t on);
+
+/*
  * Launch shape of the context's last lsp_batch plan: shape[0..4] = kernel
  * mode (1 hardware sin/cos, 2 angle-addition recurrence, 4 three-term
  * recurrence, 5 its packed form), strip length F, realizations per pass R,

@@ -541,9 +541,10 @@ features_kernel(const double* __restrict__ t, const int64_t* __restrict__ off, c
         });
         __syncwarp();
         float* o = feat + (size_t)c * 32;
-        if (unsorted || !(T > 0.0) || M < 1) {
+        const bool lost = pk && (__ldcg(status) & kStatusWait);  // a window of a wait that ran out
+        if (unsorted || !(T > 0.0) || M < 1 || lost) {
             o[tid] = __int_as_float(0x7fc00000);
-            if (tid == 0) atomicOr(status, kStatusNonFinite);
+            if (tid == 0 && !lost) atomicOr(status, kStatusNonFinite);
             return;
         }
         // lane 0 .. 5: log n, log T, log N_f, log 1/(df T), log f_max T / n, log(1 + f0 / df);

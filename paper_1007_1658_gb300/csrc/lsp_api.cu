@@ -191,6 +191,7 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
     a.qmax = gls ? (const float*)ctx->qmax.p : nullptr;
     a.part = (float*)ctx->tc_part.p;
     a.status = ctx->status_d;
+    a.give_up = ctx->give_up;
     const bool timing = ctx->opt.timing != 0;
     for (int64_t g = 0; g < groups; g += step) {
         a.one.kg0 = (int)g;
@@ -334,6 +335,7 @@ cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d
     const int64_t* pre = (const int64_t*)(tiles + p.tiles.size());
     const int* data = (const int*)(pre + p.pre.size());
     const int pairs = lsp::tc_pairs(ctx->sms);
+    a.give_up = ctx->give_up;
     for (size_t x = 0; x < p.chunks.size(); ++x) {
         const TcChunk& c = p.chunks[x];
         a.tiles = tiles + c.t0;
@@ -589,6 +591,13 @@ lsp_status lsp_test_last_batch_shape(const lsp_ctx* ctx, int32_t shape[5]) {
 lsp_status lsp_test_fail_allocation(lsp_ctx* ctx, int32_t n) {
     if (!ctx || n < 0) return LSP_ERR_INVALID_ARG;
     ctx->fail_alloc_in = n;
+    return LSP_OK;
+}
+
+lsp_status lsp_test_give_up_waits(lsp_ctx* ctx, int32_t on) {
+    if (!ctx) return LSP_ERR_INVALID_ARG;
+    ctx->give_up = on != 0;
+    drop_plan(ctx);  // a captured batch holds what it was
     return LSP_OK;
 }
 

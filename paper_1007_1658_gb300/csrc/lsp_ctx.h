@@ -116,6 +116,7 @@ struct lsp_ctx {
     bool timing_valid = false;
     bool has_finalize = false;
     int last_launches = 0;
+    bool give_up = false;   // test hook: the tensor-core kernel's waits give up at once
     int fail_alloc_in = 0;  // test hook: the n-th workspace allocation from now fails (0: never)
 };
 

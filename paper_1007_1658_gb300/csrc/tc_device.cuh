@@ -75,6 +75,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity) {
         else if (now - t0 > kWaitClocks) return false;
     }
 }
+// Whether the phase is complete now.
+__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_addr(b)), "r"(parity)
+        : "memory");
+    return ok;
+}
 
 // Tensor memory: columns of 128 lanes x 32 bits; one warp of each CTA of the
 // pair allocates and frees.

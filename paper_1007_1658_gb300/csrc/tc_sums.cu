@@ -232,13 +232,17 @@ constexpr int kRunUnits = 128;
 // turns), all its lanes together but for the instruction itself.  The register split comes from setmaxnreg: 640 threads at 96
 // registers launch, 512 x 112 + 128 x 32 are those 61,440.  Barriers:
 // filled (a stage, counted at the first CTA) and empty, full (an accumulator, a
-// unit's MMAs done) and drained (counted at the first CTA).  No pair waits for
-// another pair, and every wait has a limit, after which the CTA stops waiting,
-// says so in the status word and runs to its end.
+// unit's MMAs done), drained (counted at the first CTA) and finished.  No pair
+// waits for another pair, and every wait has a limit.  Where one runs out, its warp
+// stops waiting, the issuing one issues no more, and the status word makes the
+// finalize pass write NaN; the tensor memory is given back and the CTAs end only
+// after `finished`, which every MMA issued so far completes.
+// GIVE_UP, for a test: every wait gives up at its first look.
+template <bool GIVE_UP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_sums_kernel(const TcArgs a) {
     extern __shared__ __align__(128) unsigned char stages[];
     Ahead& ahead = *reinterpret_cast<Ahead*>(stages + kBufs * kStageBytes);
-    __shared__ uint64_t filled[kBufs], empty[kBufs], full[2], drained[2];
+    __shared__ uint64_t filled[kBufs], empty[kBufs], full[2], drained[2], finished;
     __shared__ uint32_t tbase;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int rank = (int)tc::pair_rank(), pair = blockIdx.x >> 1;
@@ -253,6 +257,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&drained[i], 2 * kGenWarps);
         }
+        tc::mbar_init(&finished, 1);
         tc::mbar_init_done();
     }
     if (warp == 0) tc::tmem_alloc(&tbase, 512);
@@ -278,6 +283,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
         t = (int)(lo / cost0);
     }
     bool ok = true;
+    auto wait = [](uint64_t* b, uint32_t parity) {
+        return GIVE_UP ? tc::mbar_test(b, parity) : tc::mbar_wait(b, parity);
+    };
     uint32_t group = 0, it = 0;  // units and stages so far
     // the next piece of a tile in this pair's range: its tile, first sample and length
     TileInfo f;
@@ -306,16 +314,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                 const uint32_t id = tc::instr_desc(f.w.cols);
                 for (int m = 0; m < left; m += kTcUnit, ++group) {
                     const uint32_t d = tb + (group & 1) * 256u;
-                    if (group >= 2) ok = ok && tc::mbar_wait(&drained[group & 1], ((group >> 1) - 1) & 1);
+                    if (group >= 2) ok = ok && wait(&drained[group & 1], ((group >> 1) - 1) & 1);
                     for (int q = m; q < min(left, m + kTcUnit); q += kStage) {
-                        ok = ok && tc::mbar_wait(&filled[buf], phase);
+                        ok = ok && wait(&filled[buf], phase);
                         __syncwarp();
                         tc::fence_after_sync();
                         const uint64_t da = tc::operand_desc(tc::smem_addr(stages) + buf * kStageBytes, 128, kSbo);
                         const uint64_t db = da + (2 * kAbytes >> 4);
                         constexpr uint64_t al = kAbytes >> 4, bl = kBbytes >> 4, k1 = 256 >> 4;
                         const bool two = left - q > 16;  // the second 16 samples of the stage
-                        if (tc::elect_one()) {
+                        if (tc::elect_one() && ok) {
                             tc::mma_f16(d, da, db + bl, id, q > m);  // hi lo
                             if (two) tc::mma_f16(d, da + k1, db + bl + k1, id, 1);
                             tc::mma_f16(d, da + al, db, id, 1);      // lo hi
@@ -333,6 +341,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                     }
                 }
             }
+            if (tc::elect_one()) tc::mma_commit(&finished);
         }
         __syncwarp();
     } else {
@@ -366,7 +375,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
             // adds a finished unit's accumulators to the running sums
             auto drain = [&](uint32_t g, int unit) {
                 const float gain = unit_gain(unit);
-                ok = ok && tc::mbar_wait(&full[g & 1], (g >> 1) & 1);
+                ok = ok && wait(&full[g & 1], (g >> 1) & 1);
                 __syncwarp();
                 tc::fence_after_sync();
 #pragma unroll
@@ -424,7 +433,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
                         E = csquare(E);
                     }
                     const uint32_t si = it + set, buf = si % kBufs, use = si / kBufs;
-                    if (use > 0) ok = ok && tc::mbar_wait(&empty[buf], (use - 1) & 1);
+                    if (use > 0) ok = ok && wait(&empty[buf], (use - 1) & 1);
                     unsigned char* const Ah = stages + buf * kStageBytes + lane * 16;
                     {
                         float2 z = turn_cos_sin(pa);
@@ -470,7 +479,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) tc_su
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
     }
-    // every MMA has been waited for with its unit, by both CTAs
+    if (warp == 0) ok = tc::mbar_wait(&finished, 0) && ok;
     if (!ok && a.status) atomicOr(a.status, kStatusWait);
     tc::fence_before_sync();
     __syncthreads();
@@ -689,6 +698,7 @@ __global__ void __launch_bounds__(kFinThreads, FORM == kTcGls ? 2 : 4) tc_final_
     const int64_t k0 = ((int64_t)(w.kg0 + kl) * kTcGroup + (ra & 15)) * cols;
     const bool live = set < w.reals && k0 < nf;
     const int real = w.r0 + set;
+    const bool lost = a.status && (__ldcg(a.status) & kStatusWait);  // sums of a wait that ran out
     if (!__syncthreads_or(live)) return;
     {
         // warps 0 .. 3 find the h = 2 pieces of group `warp`, 4 .. 7 the y = q^2 ones, 0 the data tile's
@@ -740,7 +750,7 @@ __global__ void __launch_bounds__(kFinThreads, FORM == kTcGls ? 2 : 4) tc_final_
 #pragma unroll 1
                 for (int s = 0; s < 2; ++s) {
                     const int64_t k = s ? kp : km;
-                    if (!(s ? lp : lm) || k >= nf) continue;
+                    if (lost || !(s ? lp : lm) || k >= nf) continue;
                     const unsigned at = atomicAdd(f.n_bins, 1u);
                     if (at < (unsigned)kTcBins) {
                         f.bins[at] = TcBin{w.curve, real, (uint32_t)k, 0u};
@@ -752,6 +762,7 @@ __global__ void __launch_bounds__(kFinThreads, FORM == kTcGls ? 2 : 4) tc_final_
                     (s ? vp : vm) = -1.f;  // left to launch_tc_refine
                 }
             }
+            if (lost) vm = vp = __int_as_float(0x7fc00000);
             keep(vm, km);
             keep(vp, kp);
             sp[ra][kFinB - 1 - bi] = vm;
@@ -923,9 +934,10 @@ cudaError_t launch_tc_refine(const TcArgs& a, const TcFinal& f, cudaStream_t st)
 }
 
 cudaError_t launch_tc_sums(const TcArgs& a, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(tc_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    auto* const kernel = a.give_up ? tc_sums_kernel<true> : tc_sums_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    tc_sums_kernel<<<2 * a.pairs, kTcThreads, kSmem, st>>>(a);
+    kernel<<<2 * a.pairs, kTcThreads, kSmem, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,7 @@ struct TcArgs {
     float* part;                // slots of slot_floats: tile t's piece by pair i is slot t + i, the halves of its
     int64_t slot_floats;        // two CTAs one after the other, each [cols][128 rows]
     int* status;
+    bool give_up;               // a test: every wait on a barrier gives up at its first look
 };
 
 // Where the work coordinate of pair i starts.

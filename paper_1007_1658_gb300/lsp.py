@@ -148,6 +148,8 @@ def _extra_prototypes(lib):
         lib.lsp_test_pointer_kind.restype = i32
         lib.lsp_test_fail_allocation.argtypes = [p, i32]
         lib.lsp_test_fail_allocation.restype = ctypes.c_int
+        lib.lsp_test_give_up_waits.argtypes = [p, i32]
+        lib.lsp_test_give_up_waits.restype = ctypes.c_int
         lib.lsp_test_last_batch_shape.argtypes = [p, p]
         lib.lsp_test_last_batch_shape.restype = ctypes.c_int
 
@@ -460,6 +462,10 @@ class Context:
     def test_fail_allocation(self, n):
         """lsp_test_fail_allocation: the n-th workspace allocation from now fails (0 cancels)."""
         self._check(self._lib.lsp_test_fail_allocation(self.h, int(n)))
+
+    def test_give_up_waits(self, on):
+        """lsp_test_give_up_waits: the tensor-core kernel's waits give up at once."""
+        self._check(self._lib.lsp_test_give_up_waits(self.h, int(on)))
 
     def sync(self, timeout_s: float = -1.0):
         self._check(self._lib.lsp_sync(self.h, float(timeout_s)))
