@@ -183,7 +183,8 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
     const bool same = pl.valid && pl.n_curves == n_curves && pl.n_real == n_real && pl.mode == mode &&
                       pl.F == F && pl.R == R && pl.tailF == tailF && pl.tile == tile && pl.noise == noise &&
                       pl.ptrs == ptrs && pl.t_off == off &&
-                      pl.nf == nf && pl.f0 == f0v && pl.df == dfv && pl.p_off == poff;
+                      pl.nf == nf && pl.f0 == f0v && pl.df == dfv && pl.p_off == poff &&
+                      (!tc || ctx->tc_part.cap >= pl.part_bytes);
     if (!same) {
         NvtxRange r("lsp_batch.plan");
         drop_plan(ctx);
@@ -348,6 +349,7 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         pl.p_off = poff;
         pl.n_items = tc ? (int)tcp.tiles.size() : (int)n_main;
         pl.grid = grid;
+        pl.part_bytes = tc ? (size_t)tcp.max_slot_floats * 4 : 0;
         pl.kernels = 3 + (noise ? 1 : 0) + ((d_maxP || d_argmax) ? 1 : 0) + (n_main == 0 ? -1 : 0) + (n_win > 0 ? 1 : 0) +
                      2 * (int)tcp.chunks.size();
     }

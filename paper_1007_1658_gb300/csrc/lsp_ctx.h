@@ -33,6 +33,7 @@ struct BatchPlan {
     std::vector<int64_t> t_off, nf, p_off;
     std::vector<double> f0, df;
     int n_items = 0, grid = 0;
+    size_t part_bytes = 0;  // of the tensor-core partial tiles that the graph writes
     cudaGraphExec_t exec = nullptr;
     int kernels = 0;
 };

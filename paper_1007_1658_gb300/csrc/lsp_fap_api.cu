@@ -161,6 +161,7 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     float* d_feat = nullptr;
     bool feat_host = false;
     if ((rs = out_view(ctx, features, (size_t)n * kNFeat, ctx->b_maxP, &d_feat, &feat_host)) != LSP_OK) return rs;
+    if (ctx->plan.valid) drop_plan(ctx);  // the batch graph's work lists are overwritten here
     // work list for the window pass, longest pattern first
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
@@ -182,7 +183,6 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     const size_t item_bytes = items.size() * sizeof(lsp::BatchItem);
     const size_t meta = (size_t)(2 * n + 1) * 8;
     if ((rs = ensure(ctx, ctx->b_items, item_bytes + 16)) != LSP_OK) return rs;
-    if (ctx->plan.valid) drop_plan(ctx);  // the batch graph's work list is overwritten here
     const size_t tc_at = (meta + item_bytes + 15) & ~(size_t)15;
     if ((rs = ensure_pinned(ctx, tc_at + (tc ? tcp.bytes() : 0) + 64)) != LSP_OK) return rs;
     LSP_CUDA(ctx, cudaStreamSynchronize(st));
