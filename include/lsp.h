@@ -18,7 +18,9 @@
  *   after argument checks and kernel launches, and errors found on the device
  *   (non-finite data, zero variance) are reported by lsp_sync().
  * - The caller owns every array it passes; the library owns only the context
- *   and its workspace (grown on demand, freed by lsp_destroy).
+ *   and its workspace (grown on demand, freed by lsp_destroy).  The tensor-core
+ *   sums hold up to 1.25 GiB of it (single curves) or 5 GiB (batches, features);
+ *   a call for which that cannot be allocated runs the strip kernels instead.
  * - Every function returns an lsp_status; lsp_last_error() gives the text of
  *   the last failure on that context.  A failed call leaves outputs undefined.
  * - A context is not thread-safe: one host thread at a time.

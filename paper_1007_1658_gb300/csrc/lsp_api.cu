@@ -329,6 +329,17 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
     return p;
 }
 
+bool lsp::host::without_tc(lsp_ctx* ctx) {
+    ctx->err.clear();
+    drop_plan(ctx);
+    cudaStreamSynchronize(ctx->stream);
+    for (DevBuf* b : {&ctx->recE, &ctx->tc_part, &ctx->tc_bins, &ctx->tc_mask, &ctx->b_recE, &ctx->b_tc}) {
+        if (b->p) cudaFree(b->p);
+        *b = DevBuf{};
+    }
+    return false;
+}
+
 cudaError_t lsp::host::run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int form, lsp::TcArgs a,
                               lsp::TcFinal f, cudaStream_t st) {
     const lsp::TcTile* tiles = (const lsp::TcTile*)((const int64_t*)d_plan + p.cols.size());
@@ -452,16 +463,17 @@ lsp_status lsp_periodogram(lsp_ctx* ctx, const double* t, const double* X, int64
     if ((rs = where(ctx, t, &t_dev)) != LSP_OK || (rs = where(ctx, X, &x_dev)) != LSP_OK ||
         (rs = where(ctx, P_out, &p_dev)) != LSP_OK)
         return rs;
-    const bool tc = use_tc(ctx, N_t, N_f, false);
+    bool tc = use_tc(ctx, N_t, N_f, false);
     MainShape s{};
     int tc_launches = 2;
     if (tc) {
-        s.split = 1;
-        if ((rs = ensure(ctx, ctx->recE, (size_t)N_t * 8)) != LSP_OK) return rs;
-        if ((rs = tc_single(ctx, false, N_t, N_f, nullptr, false, nullptr)) != LSP_OK) return rs;
-    } else {
-        s = choose_shape(ctx, N_t, N_f);
+        rs = ensure(ctx, ctx->recE, (size_t)N_t * 8);
+        if (rs == LSP_OK) rs = tc_single(ctx, false, N_t, N_f, nullptr, false, nullptr);
+        if (rs == LSP_ERR_OOM) tc = without_tc(ctx);
+        else if (rs != LSP_OK) return rs;
     }
+    if (tc) s.split = 1;
+    else s = choose_shape(ctx, N_t, N_f);
     if ((rs = ensure(ctx, ctx->recA, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recB, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->stats, sizeof(CurveStats))) != LSP_OK) return rs;

@@ -25,7 +25,7 @@ void lsp::host::drop_plan(lsp_ctx* ctx) {
 lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, const double* t,
                                 const double* X, uint64_t seed, int32_t n_real, const double* f_0, const double* df,
                                 const int64_t* N_f, float* P_out, const int64_t* P_off, float* maxP_out,
-                                int32_t* argmax_out, const BatchShape* forced) {
+                                int32_t* argmax_out, const BatchShape* forced, bool tensor) {
     if (!ctx) return LSP_ERR_INVALID_ARG;
     ctx->err.clear();
     ctx->timing_valid = false;
@@ -106,7 +106,7 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
             tile = lsp::kTile;
         }
     }
-    const bool tc = !shape && use_tc_batch(ctx, off, nf, n_real, false);
+    const bool tc = tensor && !shape && use_tc_batch(ctx, off, nf, n_real, false);
     TcPlan tcp;
     if (tc) {
         mode = lsp::kModeTensor;
@@ -163,7 +163,12 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
     if (!p_dev && (rs = ensure(ctx, ctx->b_P, (size_t)n_real * (size_t)P_total * 4)) != LSP_OK) return rs;
     if (!m_dev && (rs = ensure(ctx, ctx->b_maxP, n_out * 4)) != LSP_OK) return rs;
     if (!a_dev && (rs = ensure(ctx, ctx->b_argmax, n_out * 4)) != LSP_OK) return rs;
-    if (tc && (rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
+    auto strips = [&]() {
+        without_tc(ctx);
+        return batch_run(ctx, n_curves, t_off, t, X, seed, n_real, f_0, df, N_f, P_out, P_off, maxP_out, argmax_out,
+                         forced, false);
+    };
+    if (tc && (rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs == LSP_ERR_OOM ? strips() : rs;
     if (use_win) {
         if ((rs = ensure(ctx, ctx->b_win, (size_t)nf_total * 8)) != LSP_OK) return rs;
         if ((rs = ensure(ctx, ctx->b_woff, ((size_t)n_curves + 1) * 8)) != LSP_OK) return rs;
@@ -201,8 +206,9 @@ lsp_status lsp::host::batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t
         if (tc) {
             tcp = plan_tc(ctx, lsp::kTcClassic, n_real == 1 ? lsp::kTcRec : lsp::kTcRow, off, nf, n_real);
             if (tcp.tiles.size() >= (size_t)(1u << 31)) return fail(ctx, LSP_ERR_INVALID_ARG, "batch too large");
-            if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
-            if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
+            rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16);
+            if (rs == LSP_OK) rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16);
+            if (rs != LSP_OK) return rs == LSP_ERR_OOM ? strips() : rs;
         }
         for (int c : order) {
             if (tc) break;

@@ -358,6 +358,10 @@ TcPlan plan_tc(const lsp_ctx* ctx, int form, int data, const std::vector<int64_t
 cudaError_t run_tc(const lsp_ctx* ctx, const TcPlan& p, const void* d_plan, int form, lsp::TcArgs args,
                    lsp::TcFinal fin, cudaStream_t st);
 
+// What a call does whose tensor-core workspace cannot be allocated: that
+// workspace is given back, and the strips run, which need less.  Returns false.
+bool without_tc(lsp_ctx* ctx);
+
 // Whether a batch runs on the tensor cores: the options leave the choice to the
 // library, and the batch is of a size where they are faster.
 bool use_tc_batch(const lsp_ctx* ctx, const std::vector<int64_t>& off, const std::vector<int64_t>& nf, int n_real,
@@ -373,11 +377,12 @@ BatchBucket batch_bucket(int n_curves, int64_t total_samples, int64_t total_freq
 // lsp_autotune_batch entry for this bucket, or null.
 const BatchTuneEntry* tuned_batch(const lsp_ctx* ctx, const BatchBucket& b);
 
-// lsp_batch with an optional forced launch shape (the autotuner's candidates).
+// lsp_batch with an optional forced launch shape (the autotuner's candidates);
+// tensor = false keeps it from the tensor cores.
 lsp_status batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, const double* t, const double* X,
                      uint64_t seed, int32_t n_real, const double* f_0, const double* df, const int64_t* N_f,
                      float* P_out, const int64_t* P_off, float* maxP_out, int32_t* argmax_out,
-                     const BatchShape* forced);
+                     const BatchShape* forced, bool tensor = true);
 
 }  // namespace host
 }  // namespace lsp

@@ -167,15 +167,17 @@ lsp_status lsp_fap_features(lsp_ctx* ctx, int32_t n, const int64_t* t_off, const
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
     // the window on the tensor cores, where that pays (it takes no options)
-    const bool tc = tc_batch_pays(off, nw, 1);
+    bool tc = tc_batch_pays(off, nw, 1);
     TcPlan tcp;
     if (tc) {
         tcp = plan_tc(ctx, lsp::kTcWindow, lsp::kTcOne1, off, nw, 1);
-        if ((rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, f.peaks, (size_t)n * (lsp::kWindowPeaks + 1) * 4)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, f.peak_w, (size_t)n * 3 * lsp::kWindowPeaks * 4)) != LSP_OK) return rs;
+        rs = ensure(ctx, ctx->b_recE, (size_t)total * 8);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16);
+        if (rs == LSP_OK) rs = ensure(ctx, f.peaks, (size_t)n * (lsp::kWindowPeaks + 1) * 4);
+        if (rs == LSP_OK) rs = ensure(ctx, f.peak_w, (size_t)n * 3 * lsp::kWindowPeaks * 4);
+        if (rs == LSP_ERR_OOM) tc = without_tc(ctx);
+        else if (rs != LSP_OK) return rs;
     }
     std::vector<lsp::BatchItem> items;
     for (int c : order)

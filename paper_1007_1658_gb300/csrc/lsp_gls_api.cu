@@ -67,18 +67,19 @@ lsp_status lsp_periodogram_gls(lsp_ctx* ctx, const double* t, const double* X, c
             return ws;
     }
     lsp_status rs;
-    const bool tc = use_tc(ctx, N_t, N_f, true);
+    bool tc = use_tc(ctx, N_t, N_f, true);
     MainShape s{};
     int tc_launches = 2;
     if (tc) {
-        s.split = 1;
-        if ((rs = ensure(ctx, ctx->recE, (size_t)N_t * 8)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->qmax, 16)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins)) != LSP_OK) return rs;
-        if ((rs = tc_single(ctx, true, N_t, N_f, nullptr, false, nullptr)) != LSP_OK) return rs;
-    } else {
-        s = choose_gls_shape(ctx, N_t, N_f);
+        rs = ensure(ctx, ctx->recE, (size_t)N_t * 8);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->qmax, 16);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins);
+        if (rs == LSP_OK) rs = tc_single(ctx, true, N_t, N_f, nullptr, false, nullptr);
+        if (rs == LSP_ERR_OOM) tc = without_tc(ctx);
+        else if (rs != LSP_OK) return rs;
     }
+    if (tc) s.split = 1;
+    else s = choose_gls_shape(ctx, N_t, N_f);
     if ((rs = ensure(ctx, ctx->recA, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recB, (size_t)N_t * 16)) != LSP_OK) return rs;
     if ((rs = ensure(ctx, ctx->recQ, (size_t)N_t * 4)) != LSP_OK) return rs;
@@ -161,7 +162,7 @@ namespace {
 lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, const double* t, const double* X,
                          const double* dy, uint64_t seed, int32_t n_real, const double* f_0, const double* df,
                          const int64_t* N_f, float* P_out, const int64_t* P_off, float* maxP_out,
-                         int32_t* argmax_out) {
+                         int32_t* argmax_out, bool tensor = true) {
     if (!ctx) return LSP_ERR_INVALID_ARG;
     ctx->err.clear();
     ctx->timing_valid = false;
@@ -237,7 +238,7 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
         if (R > 1 && lsp::gls_mrhs_occupancy(F, R) <= 0)
             return fail(ctx, LSP_ERR_UNSUPPORTED, "batch_rhs = %d is not built for the floating-mean form", R);
     }
-    const bool tc = use_tc_batch(ctx, off, nf, n_real, true);
+    const bool tc = tensor && use_tc_batch(ctx, off, nf, n_real, true);
     TcPlan tcp;
     const int64_t per_block = lsp::gls_batch_freqs_per_block(F);
     std::vector<int> order(n_curves);
@@ -267,12 +268,18 @@ lsp_status gls_batch_run(lsp_ctx* ctx, int32_t n_curves, const int64_t* t_off, c
     if ((rs = ensure(ctx, ctx->b_maxkey, n_out * 8)) != LSP_OK) return rs;
     if (noise && (rs = ensure(ctx, ctx->b_gx, (size_t)n_real * (size_t)total * 4)) != LSP_OK) return rs;
     if (tc) {
-        if ((rs = ensure(ctx, ctx->b_recE, (size_t)total * 8)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->b_qmax, (size_t)n_curves * 4 + 4)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins)) != LSP_OK) return rs;
-        if ((rs = ensure_zeroed(ctx, ctx->tc_mask, (size_t)tcp.max_mask_words * 4 + 16)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16)) != LSP_OK) return rs;
-        if ((rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16)) != LSP_OK) return rs;
+        rs = ensure(ctx, ctx->b_recE, (size_t)total * 8);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->b_qmax, (size_t)n_curves * 4 + 4);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->tc_bins, sizeof(lsp::TcBin) * lsp::kTcBins);
+        if (rs == LSP_OK) rs = ensure_zeroed(ctx, ctx->tc_mask, (size_t)tcp.max_mask_words * 4 + 16);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->b_tc, tcp.bytes() + 16);
+        if (rs == LSP_OK) rs = ensure(ctx, ctx->tc_part, (size_t)tcp.max_slot_floats * 4 + 16);
+        if (rs == LSP_ERR_OOM) {
+            without_tc(ctx);
+            return gls_batch_run(ctx, n_curves, t_off, t, X, dy, seed, n_real, f_0, df, N_f, P_out, P_off, maxP_out,
+                                 argmax_out, false);
+        }
+        if (rs != LSP_OK) return rs;
     } else if ((rs = ensure(ctx, ctx->b_items, items.size() * sizeof(lsp::BatchItem) + 16)) != LSP_OK) {
         return rs;
     }

@@ -1,7 +1,9 @@
-"""The tensor-core path's workspace, shared by the calls of a context, when it cannot be allocated.
+"""Calls that the tensor cores would run and whose workspace there cannot be allocated: the strip kernels run them.
 
-lsp_test_fail_allocation makes the n-th workspace allocation from then fail as
-cudaMalloc would.
+lsp_test_fail_allocation makes the n-th workspace allocation of a fresh context
+fail as cudaMalloc would; n covers the tensor-core path's own buffers, in the order
+the call asks for them.  The results are the strips' bit for bit, and the next call
+runs on the tensor cores again.
 """
 import numpy as np
 import pytest
@@ -46,6 +48,41 @@ def calls(lsp):
                 c.sync(60.0)
         assert not torch.equal(ref[k, lsp.SINCOS_AUTO], ref[k, lsp.SINCOS_RECUR3_X2]), k
     return out, ref, many
+
+
+@pytest.mark.parametrize("which,first,last", [("periodogram", 1, 2), ("gls", 1, 5), ("batch", 8, 10),
+                                              ("batch_gls_noise", 8, 13)])
+def test_without_the_workspace_the_strips_run(lsp, calls, which, first, last):
+    call, ref, _ = calls[0][which], calls[1], calls[2]
+    for nth in range(first, last + 1):
+        with lsp.Context(0) as ctx:
+            ctx.test_fail_allocation(nth)
+            got = call(ctx)
+            ctx.sync(60.0)
+            assert torch.equal(got, ref[which, lsp.SINCOS_RECUR3_X2]), nth
+            got = call(ctx)
+            ctx.sync(60.0)
+            assert torch.equal(got, ref[which, lsp.SINCOS_AUTO]), nth
+        # the allocation after them is one that every route needs
+    with lsp.Context(0) as ctx:
+        if which in ("periodogram", "gls"):
+            ctx.test_fail_allocation(last + 1)
+            with pytest.raises(lsp.LspError) as e:
+                call(ctx)
+            assert e.value.status == lsp.ERR_OOM
+
+
+@pytest.mark.parametrize("nth", [8, 9, 10, 11, 12])
+def test_features_without_the_workspace(lsp, calls, nth):
+    many = calls[2]
+    with lsp.Context(0) as ctx:
+        want = ctx.fap_features(*many).clone()
+        ctx.sync(60.0)
+    with lsp.Context(0) as ctx:
+        ctx.test_fail_allocation(nth)
+        got = ctx.fap_features(*many)
+        ctx.sync(60.0)
+        assert torch.equal(got, want)
 
 
 @pytest.mark.parametrize("other", ["features", "batch_gls"])
