@@ -38,6 +38,14 @@ int32_t lsp_test_pointer_kind(int32_t memory_type, int32_t pointer_device, int32
 lsp_status lsp_test_fail_allocation(lsp_ctx *ctx, int32_t n);
 
 /*
+ * Let a launch of the tensor-core sums take at most n tiles (n >= 4), as where
+ * its workspace holds no more; 0: the default.  Larger calls then run in several
+ * blocks of frequencies, curves or realizations.
+ * Errors: INVALID_ARG (null context, n < 4).
+ */
+lsp_status lsp_test_tensor_tiles(lsp_ctx *ctx, int32_t n);
+
+/*
  * While `on` is not 0, every wait of the tensor-core kernel of `ctx` gives up at
  * its first look, as if its limit of about a second had passed.  A call in which
  * one does ends normally, its outputs NaN, and lsp_sync returns LSP_ERR_CUDA.

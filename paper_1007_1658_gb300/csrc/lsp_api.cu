@@ -171,7 +171,8 @@ lsp_status lsp::host::tc_single(lsp_ctx* ctx, bool gls, int64_t N, int64_t N_f, 
     lsp::TcArgs a{};
     a.slot_floats = lsp::tc_slot_floats(cols);
     // at most 1 GiB of partial tiles at a time
-    const int64_t most = std::max<int64_t>(1, ((int64_t(1) << 28) / a.slot_floats - pairs) / (sets + 1) - 1) * G;
+    const int64_t tiles = ctx->max_tiles ? ctx->max_tiles : (int64_t(1) << 28) / a.slot_floats - pairs;
+    const int64_t most = std::max<int64_t>(1, tiles / (sets + 1) - 1) * G;
     const int64_t step = std::min(groups, most);
     const int64_t slots = (sets * step + G - 1) / G + (step + G - 1) / G + pairs;
     lsp_status rs = ensure(ctx, ctx->tc_part, (size_t)slots * (size_t)a.slot_floats * 4);
@@ -272,7 +273,8 @@ lsp::host::TcPlan lsp::host::plan_tc(const lsp_ctx* ctx, int form, int data, con
     const int pairs = lsp::tc_pairs(ctx->sms);
     const int G = lsp::kTcGroups;
     // at most 4 GiB of partial tiles at a time
-    const int64_t most = (int64_t(1) << 30) / lsp::tc_slot_floats(lsp::kTcMaxCols) - pairs;
+    const int64_t most =
+        ctx->max_tiles ? ctx->max_tiles : (int64_t(1) << 30) / lsp::tc_slot_floats(lsp::kTcMaxCols) - pairs;
     TcChunk cur{0, 0, 0, 0, 0, 0};
     p.pre.push_back(0);
     auto flush = [&]() {
@@ -603,6 +605,13 @@ lsp_status lsp_test_last_batch_shape(const lsp_ctx* ctx, int32_t shape[5]) {
 lsp_status lsp_test_fail_allocation(lsp_ctx* ctx, int32_t n) {
     if (!ctx || n < 0) return LSP_ERR_INVALID_ARG;
     ctx->fail_alloc_in = n;
+    return LSP_OK;
+}
+
+lsp_status lsp_test_tensor_tiles(lsp_ctx* ctx, int32_t n) {
+    if (!ctx || (n != 0 && n < 4)) return LSP_ERR_INVALID_ARG;
+    ctx->max_tiles = n;
+    drop_plan(ctx);
     return LSP_OK;
 }
 

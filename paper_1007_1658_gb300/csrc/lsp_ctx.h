@@ -117,6 +117,7 @@ struct lsp_ctx {
     bool timing_valid = false;
     bool has_finalize = false;
     int last_launches = 0;
+    int max_tiles = 0;      // test hook: tiles of one launch of the tensor-core sums, at most (0: by the workspace)
     bool give_up = false;   // test hook: the tensor-core kernel's waits give up at once
     int fail_alloc_in = 0;  // test hook: the n-th workspace allocation from now fails (0: never)
 };

@@ -148,6 +148,8 @@ def _extra_prototypes(lib):
         lib.lsp_test_pointer_kind.restype = i32
         lib.lsp_test_fail_allocation.argtypes = [p, i32]
         lib.lsp_test_fail_allocation.restype = ctypes.c_int
+        lib.lsp_test_tensor_tiles.argtypes = [p, i32]
+        lib.lsp_test_tensor_tiles.restype = ctypes.c_int
         lib.lsp_test_give_up_waits.argtypes = [p, i32]
         lib.lsp_test_give_up_waits.restype = ctypes.c_int
         lib.lsp_test_last_batch_shape.argtypes = [p, p]
@@ -462,6 +464,10 @@ class Context:
     def test_fail_allocation(self, n):
         """lsp_test_fail_allocation: the n-th workspace allocation from now fails (0 cancels)."""
         self._check(self._lib.lsp_test_fail_allocation(self.h, int(n)))
+
+    def test_tensor_tiles(self, n):
+        """lsp_test_tensor_tiles: tiles of one launch of the tensor-core sums, at most (0: the default)."""
+        self._check(self._lib.lsp_test_tensor_tiles(self.h, int(n)))
 
     def test_give_up_waits(self, on):
         """lsp_test_give_up_waits: the tensor-core kernel's waits give up at once."""
