@@ -44,8 +44,11 @@ def test_frequency_blocks_of_one_curve(lsp, nf, gls):
     with lsp.Context(0) as ctx:
         for tiles in (0, 4, 7):
             ctx.test_tensor_tiles(tiles)
-            P = ctx.periodogram_gls(*args, dy=_dev(dy)) if gls else ctx.periodogram(*args)
+            padded = torch.full((nf + 512,), -7.0, device="cuda")  # what lies around P stays as it was
+            P = padded[256:256 + nf]
+            ctx.periodogram_gls(*args, dy=_dev(dy), out=P) if gls else ctx.periodogram(*args, out=P)
             ctx.sync(60.0)
+            assert torch.all(padded[:256] == -7.0) and torch.all(padded[256 + nf:] == -7.0)
             out.append((P.cpu().numpy().astype(np.float64), ctx.last_launch_count()))
     assert nf < 70000 or out[1][1] > out[0][1]
     for P, _ in out[1:]:
