@@ -296,11 +296,11 @@ lsp_status lsp_grid(double t_min, double t_max, int64_t N_t, double F_over, doub
  * only candidates within 2e-5 max P of the all-hardware-sin/cos result, and
  * remember the fastest for this (log2 N_t, log2 N_f) bucket: later
  * lsp_periodogram calls with LSP_SINCOS_AUTO and automatic F/split use it.  Where
- * AUTO would take the tensor cores they are timed too: if they win, the bucket is
- * left without an entry (and loses one it had), so that AUTO goes on taking
- * them; an entry that was not timed against them, such as one of a file of an
- * earlier version, does not keep a call from them.  *chosen (may be NULL)
- * receives the winning options.  Blocks; allocates temporary buffers.
+ * AUTO would take the tensor cores they are timed too, and it goes on taking them
+ * unless the strip won; nor does an entry that was not timed against them, such
+ * as one of a file of an earlier version, keep a call from them.  *chosen (may be
+ * NULL) receives the fastest strip as options.  Blocks; allocates temporary
+ * buffers.
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 lsp_status lsp_autotune(lsp_ctx *ctx, int64_t N_t, int64_t N_f, lsp_options *chosen);

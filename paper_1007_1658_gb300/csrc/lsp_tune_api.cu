@@ -155,8 +155,7 @@ extern "C" lsp_status lsp_autotune(lsp_ctx* ctx, int64_t N_t, int64_t N_f, lsp_o
             if (pass && ms < best.ms) best = TuneEntry{bucket(N_t), bucket(N_f), c.sincos, c.F, splits[si], ms, 0};
         }
     }
-    // the tensor cores, with the table out of the way; where they win, no entry is left
-    bool tensor = false;
+    // the tensor cores, with the table out of the way
     std::vector<TuneEntry> table;
     table.swap(ctx->tune);
     ctx->opt = saved;
@@ -166,23 +165,22 @@ extern "C" lsp_status lsp_autotune(lsp_ctx* ctx, int64_t N_t, int64_t N_f, lsp_o
     if (use_tc(ctx, N_t, N_f, false)) {
         rs = run(LSP_SINCOS_AUTO, 0, 0, &got, &ms);
         const float err = rs == LSP_OK ? max_err() : 0.f;
-        tensor = rs == LSP_OK && std::isfinite(err) && err <= 2e-5f * pmax && ms < best.ms;
-        best.beat_tensor = !tensor;
+        best.beat_tensor = !(std::isfinite(err) && err <= 2e-5f * pmax && ms < best.ms);
     }
     ctx->tune.swap(table);
     ctx->opt = saved;
     release();
     if (rs != LSP_OK) return rs;
-    if (best.sincos == 0 && !tensor) return fail(ctx, LSP_ERR_CUDA, "autotune: no candidate passed the precision gate");
+    if (best.sincos == 0) return fail(ctx, LSP_ERR_CUDA, "autotune: no candidate passed the precision gate");
     ctx->tune.erase(std::remove_if(ctx->tune.begin(), ctx->tune.end(),
                                    [&](const TuneEntry& e) { return e.nt_bucket == best.nt_bucket && e.nf_bucket == best.nf_bucket; }),
                     ctx->tune.end());
-    if (!tensor) ctx->tune.push_back(best);
+    ctx->tune.push_back(best);
     if (chosen) {
         *chosen = saved;
-        chosen->sincos_mode = tensor ? LSP_SINCOS_AUTO : best.sincos;
-        chosen->freqs_per_thread = tensor ? 0 : best.F;
-        chosen->split = tensor ? 0 : best.split;
+        chosen->sincos_mode = best.sincos;
+        chosen->freqs_per_thread = best.F;
+        chosen->split = best.split;
     }
     return LSP_OK;
 }
