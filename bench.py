@@ -287,7 +287,8 @@ def run_gpu(args, rank, world, dist):
                    "l2": "flushed between steps (256 MB write)", "parallelism": "frequency shards x%d" % world},
         "roofline": {"bound": "tensor" if tensor else "alu", "kernel": kernel, "achieved": achieved / 1e9,
                      "peak": peak / 1e9, "unit": "Gterms/s", "frac": achieved / peak,
-                     "traffic": _recorded_traffic(kernel, files=TENSOR_SOURCES if tensor else MAIN_SOURCES),
+                     "traffic": (_recorded_traffic(kernel, "tensor_core_sums.md", TENSOR_SOURCES) if tensor
+                                 else _recorded_traffic(kernel)),
                      "peak_basis": basis,
                      "main_ms": float(np.mean(main_ms))},
         "e2e": None if e2e_val is None else {
@@ -583,8 +584,7 @@ def run_gls_bench(torch, dev, stream, args, peaks, peak_src, sms):
             "ms_per_call": step_ms, "terms_per_s": terms / (step_ms * 1e-3),
             "roofline": {"bound": "tensor" if tensor else "alu", "kernel": kernel,
                          "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gterms/s", "frac": achieved / peak,
-                         "traffic": _recorded_traffic(kernel, "gls_main_gapped_100k_errors.md",
-                                                      TENSOR_SOURCES if tensor else GLS_SOURCES),
+                         "traffic": _recorded_traffic(kernel, "gls_main_gapped_100k_errors.md", GLS_SOURCES),
                          "peak_basis": basis,
                          "main_ms": float(np.mean(main_ms))},
             "clocks": clk.summary()}

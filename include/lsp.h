@@ -198,7 +198,8 @@ lsp_status lsp_batch_gls(lsp_ctx *ctx, int32_t n_curves, const int64_t *t_off, c
  * as the one-at-a-time kernel with the same strip length would.  Runs the
  * packed three-term strip (sin/cos mode AUTO or RECUR3_X2; other modes return
  * UNSUPPORTED).  Under AUTO with automatic groups, batches with work enough
- * run on the tensor cores (as lsp_batch's), a realization's sums apart.
+ * run on the tensor cores (as lsp_batch's, whose word on last bits holds here too),
+ * a realization's sums apart.
  * Pointers host or device; any host output makes the call blocking.
  * Errors: INVALID_ARG, NONFINITE, UNSUPPORTED, OOM, CUDA.
  */
@@ -257,7 +258,10 @@ lsp_status lsp_press_rybicki(lsp_ctx *ctx, const double *t, const double *X, int
  * (frequency, realization) is computed exactly as the one-at-a-time kernel
  * with the same strip length would.
  * Under AUTO, batches with work enough run on the tensor cores, whose FP32
- * running sums cover at most 16,384 samples each.  A strip kernel's work item
+ * running sums cover at most 16,384 samples each.  Where these sums of a curve are
+ * cut depends on the whole call's work, so there the last bits of P depend on the
+ * other curves and on n_real (to the sums' rounding, about 1e-6 of max P); the same
+ * call gives the same bits.  A strip kernel's work item
  * sums over all samples of its curve in FP32 (the batch does not split N_t), so
  * with a sin/cos mode asked for curves far beyond 10^6 samples are better
  * served by lsp_periodogram.
