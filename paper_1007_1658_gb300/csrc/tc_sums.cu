@@ -870,9 +870,11 @@ __global__ void __launch_bounds__(kThreads) tc_refine_kernel(const TcArgs a, con
             const int tile = (int)(row / (2 * kFinRows)), r = (int)(row % (2 * kFinRows));
             const TcTile w = tile_of(a, a.tiles ? f.data_tiles[tile] : tile);
             const int G = w.g0 + r / kTcGroup, set = G / w.gpr;
-            const uint32_t k0 = (uint32_t)(((int64_t)(w.kg0 + G - set * w.gpr) * kTcGroup + r % kTcGroup) * w.cols +
-                                           word % per_row * 32);
-            for (; bits; bits &= bits - 1) form(TcBin{w.curve, w.r0 + set, k0 + (uint32_t)__ffs(bits) - 1u, 0u});
+            const int64_t k0 = ((int64_t)(w.kg0 + G - set * w.gpr) * kTcGroup + r % kTcGroup) * w.cols + word % per_row * 32;
+            // (a bit left by a call whose refine pass was never launched may lie beyond this grid)
+            const int64_t bins = set < w.reals ? (a.tiles ? f.nf[w.curve] : f.nf0) - k0 : 0;
+            if (bins < 32) bits &= bins > 0 ? (1u << (int)bins) - 1u : 0u;
+            for (; bits; bits &= bits - 1) form(TcBin{w.curve, w.r0 + set, (uint32_t)k0 + (uint32_t)__ffs(bits) - 1u, 0u});
         }
         return;
     }
